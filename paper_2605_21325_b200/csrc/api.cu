@@ -318,7 +318,10 @@ int chunk_scan_any(const void* Q, const void* K, const void* W, const void* U, c
       err = launch_chunk_scan(p, Qp, Km, Wm, tokens, stream, true);
     }
   } else {
+    // fp32 with a scalar gate has register-tiled products at the chunk size and key dimensions it keeps on chip
+    const bool f32 = !G && desc->kv_dtype == TRI_INV_F32 && desc->C == 64 && desc->d_k <= 128;
     err = (tc && !G) ? launch_chunk_scan(p, Q, K, W, tokens > 0 ? tokens : 1, stream)
+          : f32      ? launch_chunk_scan_f32(p, Q, K, W, desc->d_k, desc->d_v, stream)
                      : launch_chunk_scan_simt(p, Q, K, W, desc->d_k, desc->d_v, desc->C, desc->kv_dtype, stream);
   }
   if (err == cudaSuccess) g_launches.fetch_add(1, std::memory_order_relaxed);

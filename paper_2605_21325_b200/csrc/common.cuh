@@ -127,6 +127,8 @@ cudaError_t launch_chunk_scan(const ScanParams& p, const void* Q, const void* K,
 // ER = exp(G_ref), EX = exp(G_last - G_ref) ([slots,H,128] fp32), G_ref the middle row of each chunk, G_last its last.
 cudaError_t launch_kda_scan_prep(const ScanParams& p, const void* Q, const void* K, const void* W, void* Qp, void* Km, void* Wm,
                                  float* EL, float* ER, float* EX, int max_chunks_per_seq, cudaStream_t stream);
+// Single precision with a scalar gate at C = 64 and d_k <= 128 (scan_f32_kernel.cu).
+cudaError_t launch_chunk_scan_f32(const ScanParams& p, const void* Q, const void* K, const void* W, int d_k, int d_v, cudaStream_t stream);
 // The same scan on the CUDA cores, for every other shape and storage type (fp32 arithmetic).
 cudaError_t launch_chunk_scan_simt(const ScanParams& p, const void* Q, const void* K, const void* W, int d_k, int d_v, int C,
                                    int kv_dtype, cudaStream_t stream);

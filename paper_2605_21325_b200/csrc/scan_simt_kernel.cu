@@ -1,5 +1,6 @@
-// Chunk scan on the CUDA cores: the same chunk form as scan_kernel.cu for every shape and storage type the
-// tensor-core kernel does not take (fp32 tensors, d_k or d_v other than 128, C other than 64).  fp32 arithmetic.
+// Chunk scan on the CUDA cores: the same chunk form as scan_kernel.cu for every shape and storage type that neither the
+// tensor-core kernel nor scan_f32_kernel.cu takes (bf16 with d_k or d_v other than 128, C other than 64, fp32 with
+// d_k > 128, a per-channel gate outside the tensor-core shape).  fp32 arithmetic.
 //
 // One CTA of 256 threads per (sequence, head, slice of 32 value columns).  Shared memory holds the slice of the
 // state S [d_k][32], U~ [C][32], P [C][C+1] and the chunk's g; W, Q and K are read from global memory (one address

@@ -152,6 +152,22 @@ def test_chunk_scan_cuda_core_kernel_other_shapes(bnd, name, B, T, H, d_k, d_v, 
         assert max_ratio(bnd.to_numpy_f64(O2), O_rec) <= 1e-5 and max_ratio(bnd.to_numpy_f64(S2), S_rec) <= 1e-5
 
 
+# the register-tiled fp32 scan: key dimensions on both sides of its two instances (padded and full), a last value slice of
+# eight columns, one-token and empty sequences, a chunk that ends one token into the next, and the first d_k beyond it
+F32_SCAN_CASES = [
+    ("d8_v8", 1, 70, 1, 8, 8, None),
+    ("d64_v24_ragged", 1, 0, 3, 64, 24, np.array([0, 1, 65, 65, 192, 321], np.int32)),
+    ("d72_v128", 2, 3 * 64 + 1, 2, 72, 128, None),
+    ("d128_v16", 1, 63, 2, 128, 16, None),
+    ("d136_v40", 1, 130, 1, 136, 40, None),
+]
+
+
+@pytest.mark.parametrize("name,B,T,H,d_k,d_v,cu", F32_SCAN_CASES, ids=[c[0] for c in F32_SCAN_CASES])
+def test_chunk_scan_fp32_tiles(bnd, name, B, T, H, d_k, d_v, cu):
+    test_chunk_scan_cuda_core_kernel_other_shapes(bnd, name, B, T, H, d_k, d_v, 64, wl.F32, cu)
+
+
 # ---------------------------------------------------------------- full sizes, in the launch configuration bench.py times
 
 def test_layer_full_size_config2_sampled_and_restart(bnd):
