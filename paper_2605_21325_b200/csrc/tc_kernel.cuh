@@ -91,7 +91,14 @@ struct Cfg {
 // Byte offset of the 16-byte chunk holding features [f, f+8) of row r inside a swizzled tile.
 // VAR specialises two run-time switches away so that the common case carries less code (the instruction cache is shared
 // by four CTAs in different phases): 0 = fused / build call with substitution leaves, 1 = with series leaves,
-// 2 = tri_inv_wy (A read from memory), 3 = decided at run time.
+// 2 = tri_inv_wy (A read from memory), 3 = decided at run time, 4 = fused call with the decay-weighted W (substitution leaves).
+//
+// The decay of VAR 4 sits in the operand, not in the keys: W = (A diag(beta exp g)) K takes an operand A'' of its own, written
+// beside A' where the output staging will be (W is staged only after the product that reads A'' has completed).  That is 8 KB
+// of shared-memory stores; weighting the K tile's rows instead, as the RAW variant does, reads and writes 16 KB, takes a
+// barrier for the row factors in the gate and rounds to bf16 twice.  Without A wanted
+// (L2 flushed): B = 4, T = 4096, H = 16: 80.4 -> 67.6 us; B = 1, T = 32768, H = 32: 261 -> 223 us; 64 packed sequences of up
+// to 2048 tokens, H = 16: 285 -> 240 us.
 template <int C, int D, bool SER, bool RAW, bool BO, bool REF, bool H16, int VAR>
 __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SER, BO, REF, H16>::CTAS_PER_SM) tc_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmU,
                                                                              const __grid_constant__ CUtensorMap tmV, const __grid_constant__ KParams p) {
@@ -112,6 +119,8 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
   const uint32_t sK = smem_u32(smem + cfg::OFF_K);
   const uint32_t sV = smem_u32(smem + cfg::OFF_V);
   const uint32_t sAp = smem_u32(smem + cfg::OFF_AP);  // A' = A diag(beta), bf16 K-major swizzled operand
+  static_assert(VAR != 4 || (C == 64 && D == 128 && !SER && !RAW && !BO && !REF), "A'' lies in the staging tiles' space");
+  const uint32_t sApw = VAR == 4 ? smem_u32(smem + cfg::OFF_STAGE) : sAp;   // the operand of the W product
   const uint32_t bar_k = smem_u32(smem + cfg::OFF_BAR);  // K tile landed
   const uint32_t bar_mma = bar_k + 8;                    // a batch of MMAs completed
   const uint32_t bar_v = bar_k + 16;                     // V tile landed
@@ -922,12 +931,25 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
     // bf16 pair stores of one float4 of A scaled by beta: K-major, 128-byte swizzle, 64 tokens per row block
     // (a thread's columns j are the same in every pass: NT is a multiple of C / 4)
     const float4 beta_j = *reinterpret_cast<const float4*>(sBeta + 4 * (tid % (C / 4)));
+    float4 beta_w = beta_j;   // VAR 4: beta_j exp(g_j), the factors of A'' (shifted gate: exp(g_{j-1}), 1 for the first token)
+    if constexpr (VAR == 4) {
+      const int j = 4 * (tid % (C / 4));
+      float gw[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) gw[q] = (gshift && j + q == 0) ? 0.f : sG[j + q - gshift];
+      beta_w.x *= ex2_approx(gw[0]); beta_w.y *= ex2_approx(gw[1]); beta_w.z *= ex2_approx(gw[2]); beta_w.w *= ex2_approx(gw[3]);
+    }
     auto put_ap = [&](int i, int j, const float4& v) {
       const float4 b = beta_j;
       const uint32_t lo = pack_bf16(v.x * b.x, v.y * b.y), hi = pack_bf16(v.z * b.z, v.w * b.w);
       const uint32_t off = (uint32_t)((j >> 6) * (C * 128) + i * 128 + (((((j & 63) >> 3) ^ (i & 7)) << 4) | ((j & 7) * 2)));
-      if (TRI_INV_CHECK(p, off + 8 <= (uint32_t)(C * C * 2) && i < C && j + 4 <= C))
+      if (TRI_INV_CHECK(p, off + 8 <= (uint32_t)(C * C * 2) && i < C && j + 4 <= C)) {
         asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(sAp + off), "r"(lo), "r"(hi) : "memory");
+        if constexpr (VAR == 4) {
+          const uint32_t wlo = pack_bf16(v.x * beta_w.x, v.y * beta_w.y), whi = pack_bf16(v.z * beta_w.z, v.w * beta_w.w);
+          asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(sApw + off), "r"(wlo), "r"(whi) : "memory");
+        }
+      }
     };
     float4 xv[cfg::ALIAS ? 1 : NV];
     if constexpr (cfg::ALIAS) {
@@ -1041,19 +1063,19 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
       // side by side, U behind a commit of its own so that W is stored while U runs (and V's last box may still be on its way)
       static_assert(D == 128 || (D == 64 && C == 64), "head dimensions: 128, or 64 at C = 64");
       constexpr uint32_t idesc_wy = umma_idesc(C, D, 1);
-      auto issue_wy = [&](uint32_t b_tile, uint32_t d_col = 0, bool second = false) {
+      auto issue_wy = [&](uint32_t a_op, uint32_t b_tile, uint32_t d_col = 0, bool second = false) {
 #pragma unroll
         for (int ks = 0; ks < C / 16; ++ks) {
-          const uint64_t da = umma_desc(sAp + (ks >> 2) * (C * 128) + (ks & 3) * 32, 16, 1024);
+          const uint64_t da = umma_desc(a_op + (ks >> 2) * (C * 128) + (ks & 3) * 32, 16, 1024);
           const uint64_t db = umma_desc(b_tile + ks * 2048, cfg::BOX_BYTES, 1024);
           umma_bf16(tmem + d_col, da, db, idesc_wy, ks > 0);
         }
         umma_commit(second ? bar_mma_u : bar_mma);
       };
       if (tid == 0) {
-        if (wait(bar_k, ph_k)) { tc_fence_after(); issue_wy(sK); }
+        if (wait(bar_k, ph_k)) { tc_fence_after(); issue_wy(sApw, sK); }
         if (C == 128 && need_v) {
-          if (wait(bar_v, ph_v)) { tc_fence_after(); issue_wy(sV, D, true); }
+          if (wait(bar_v, ph_v)) { tc_fence_after(); issue_wy(sAp, sV, D, true); }
         }
       }
       // A goes to global memory while the W product runs (its registers are free again before W returns)
@@ -1082,7 +1104,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
         tc_fence_before();
         __syncthreads();  // every warp holds its rows of W in registers: U may overwrite the columns
         if (tid == 0) {
-          if (wait(bar_v, ph_v)) { tc_fence_after(); issue_wy(sV); }
+          if (wait(bar_v, ph_v)) { tc_fence_after(); issue_wy(sAp, sV); }
         }
         if (tid == kTidK && has_next) issue_k(nx_tok0, nx_h);  // K's last reader (the W product) is done
         store_frag_piece_bf16(f0, stage, lane, w_row0, row_stride, rows - row0, &tmW, h * D + 0, tok0 + row0);

@@ -657,3 +657,25 @@ def test_head_dimension_64_on_the_tensor_cores(bnd):
         A_simt, W_simt, U_simt = bnd.fused(dev["K"], dev["V"], dev["beta"], dev["g"], 64, method=bnd.FORCE_SIMT, cu_seqlens=cuq)
         torch.cuda.synchronize()
         assert float((A_simt - A).abs().max()) <= 4e-3 * float(A_simt.abs().max())
+
+
+@pytest.mark.parametrize("shift", [False, True])
+@pytest.mark.parametrize("T,cu", [(1, None), (63, None), (64, None), (129, None), (0, [0, 1, 17, 80, 80, 209])])
+def test_decay_weighted_w_from_its_own_operand(bnd, shift, T, cu):
+    """W_DECAY on prepared inputs at C = 64: A diag(beta exp g) is an operand of its own.  W against the general path (the
+    CUDA-core kernel: fp32 throughout, so the two differ by the operand's and the result's bf16 rounding: 2^-9 each per
+    term and element, 1e-2 of max|W| as for every bf16 W), U and A bit for bit what the call without the flag gives."""
+    cu = None if cu is None else np.array(cu, np.int32)
+    T = T if cu is None else int(cu[-1])
+    inp = wl.make("wd", 1, T, 3, 128, 128, 64, wl.BF16, seed=77, cu_seqlens=cu)
+    d = bnd.to_device(inp)
+    extra = bnd.GATE_SHIFTED if shift else 0
+    call = lambda m, want_A: bnd.fused(d["K"], d["V"], d["beta"], d["g"], 64, method=m | extra, cu_seqlens=cu, want_A=want_A)
+    A, W, U = call(bnd.W_DECAY, True)
+    none, W2, U2 = call(bnd.W_DECAY, False)
+    A0, _, U0 = call(0, True)
+    _, W_ref, _ = call(bnd.W_DECAY | bnd.FORCE_SIMT, True)
+    torch.cuda.synchronize()
+    assert bnd.last_device_status() == 0 and none is None
+    assert torch.equal(A, A0) and torch.equal(U, U0) and torch.equal(W, W2) and torch.equal(U, U2)
+    assert float((W.float() - W_ref.float()).abs().max()) <= 1e-2 * float(W_ref.float().abs().max())
