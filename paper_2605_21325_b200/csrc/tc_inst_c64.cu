@@ -4,9 +4,9 @@
 
 namespace tri_inv {
 cudaError_t launch_tc_c64_br(const KParams& p, cudaStream_t stream, bool raw) {
-  // the decay-weighted W on prepared inputs, U wanted too: its own instance (series leaves and the front end: the run-time form)
-  if (raw && !(p.ops & kRaw) && !(p.method & TRI_INV_LEAF_SERIES) && p.V) return launch_one<64, 128, false, false, false, false, false, 4>(p, stream);
-  if (raw) return launch_one<64, 128, false, true>(p, stream);
+  // row factors on the keys (front end, decay-weighted W): the prepared inputs' form has an instance without the front end's code
+  if (raw && !(p.ops & kRaw) && !(p.method & TRI_INV_LEAF_SERIES)) return launch_one<64, 128, false, false, false, false, false, 4>(p, stream);
+  if (raw) return launch_one<64, 128, false, true, false, false, false, 4>(p, stream);
   // the common calls get kernels of their own, without the code of the paths they do not take
   if (p.ops & kLoadA) return launch_one<64, 128, false, false, false, false, false, 2>(p, stream);
   if (p.method & TRI_INV_LEAF_SERIES) return launch_one<64, 128, false, false, false, false, false, 1>(p, stream);

@@ -91,9 +91,10 @@ struct Cfg {
 // Byte offset of the 16-byte chunk holding features [f, f+8) of row r inside a swizzled tile.
 // VAR specialises two run-time switches away so that the common case carries less code (the instruction cache is shared
 // by four CTAs in different phases): 0 = fused / build call with substitution leaves, 1 = with series leaves,
-// 2 = tri_inv_wy (A read from memory), 3 = decided at run time, 4 = fused call with the decay-weighted W (substitution leaves).
+// 2 = tri_inv_wy (A read from memory), 3 = decided at run time, 4 = fused call whose W has row factors on the keys: the
+// decay-weighted W (RAW = false: substitution leaves only) and the front end's 1 / |k_j| (RAW = true).
 //
-// The decay of VAR 4 sits in the operand, not in the keys: W = (A diag(beta exp g)) K takes an operand A'' of its own, written
+// The factors of VAR 4 sit in the operand, not in the keys: W = (A diag(beta exp g)) K takes an operand A'' of its own, written
 // beside A' where the output staging will be (W is staged only after the product that reads A'' has completed).  That is 8 KB
 // of shared-memory stores; weighting the K tile's rows instead, as the RAW variant does, reads and writes 16 KB, takes a
 // barrier for the row factors in the gate and rounds to bf16 twice.  Without A wanted
@@ -119,7 +120,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
   const uint32_t sK = smem_u32(smem + cfg::OFF_K);
   const uint32_t sV = smem_u32(smem + cfg::OFF_V);
   const uint32_t sAp = smem_u32(smem + cfg::OFF_AP);  // A' = A diag(beta), bf16 K-major swizzled operand
-  static_assert(VAR != 4 || (C == 64 && D == 128 && !SER && !RAW && !BO && !REF), "A'' lies in the staging tiles' space");
+  static_assert(VAR != 4 || (C == 64 && D == 128 && !SER && !BO && !REF), "A'' lies in the staging tiles' space");
   const uint32_t sApw = VAR == 4 ? smem_u32(smem + cfg::OFF_STAGE) : sAp;   // the operand of the W product
   const uint32_t bar_k = smem_u32(smem + cfg::OFF_BAR);  // K tile landed
   const uint32_t bar_mma = bar_k + 8;                    // a batch of MMAs completed
@@ -158,7 +159,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
   const bool do_wy = !BO && (p.ops & kDoWY) != 0;
   const bool need_v = do_wy && p.V != nullptr;
   const bool load_a = VAR == 3 ? (p.ops & kLoadA) != 0 : VAR == 2;
-  const bool leaf_series_on = VAR == 3 ? (p.method & TRI_INV_LEAF_SERIES) != 0 : VAR == 1;
+  const bool leaf_series_on = (VAR == 3 || (VAR == 4 && RAW)) ? (p.method & TRI_INV_LEAF_SERIES) != 0 : VAR == 1;
   // RAW compiles in the code that rewrites the K tile in shared memory before the WY step and the per-row
   // factors of the gate.  Two run-time uses: the front end (sigmoid, log-sigmoid + chunk cumsum, key
   // normalisation: kRaw) and the decay-weighted W (rows of K times exp(g_i): kWDecay).
@@ -931,8 +932,12 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
     // bf16 pair stores of one float4 of A scaled by beta: K-major, 128-byte swizzle, 64 tokens per row block
     // (a thread's columns j are the same in every pass: NT is a multiple of C / 4)
     const float4 beta_j = *reinterpret_cast<const float4*>(sBeta + 4 * (tid % (C / 4)));
-    float4 beta_w = beta_j;   // VAR 4: beta_j exp(g_j), the factors of A'' (shifted gate: exp(g_{j-1}), 1 for the first token)
-    if constexpr (VAR == 4) {
+    float4 beta_w = beta_j;   // VAR 4: the factors of A'': beta_j exp(g_j) (shifted gate: exp(g_{j-1}), 1 for the first token), times 1 / |k_j| with the front end
+    if constexpr (VAR == 4 && RAW) {
+      const float4 r = *reinterpret_cast<const float4*>(sR + 4 * (tid % (C / 4)));
+      beta_w.x *= r.x; beta_w.y *= r.y; beta_w.z *= r.z; beta_w.w *= r.w;
+    }
+    if (VAR == 4 && (!RAW || wdecay)) {
       const int j = 4 * (tid % (C / 4));
       float gw[4];
 #pragma unroll
@@ -1051,7 +1056,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
           const int i = e / (C / 4), j = 4 * (e - i * (C / 4));
           put_ap(i, j, xv[m]);
         }
-        if (raw && !cfg::RELOAD) rescale_k_tile();  // the Gram product, K's only reader so far, has completed
+        if (raw && !cfg::RELOAD && VAR != 4) rescale_k_tile();  // the Gram product, K's only reader so far, has completed
         fence_proxy_async();  // generic-proxy writes of A' become visible to the tensor core's reads
         __syncthreads();
       }
