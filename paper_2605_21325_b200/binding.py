@@ -4,6 +4,9 @@ Argument marshalling only: every step of the path runs in the CUDA kernels.
 torch is used for device memory and streams.  There is no CPU path: if the
 library is missing or a call fails, these functions raise.
 
+Outputs that a function allocates are not filled first: the kernels write every row of every token (each token belongs to
+a sequence), all columns of it.
+
 Tensors follow the header's layouts: K/V ``[B,T,H,d]`` (bf16 or fp32), beta/g
 ``[B,T,H]`` fp32, A ``[B,T,H,C]`` fp32, W/U like K/V.  All must be contiguous
 CUDA tensors on the current device.
@@ -162,15 +165,17 @@ def _p(t):
 
 
 def _stream(stream):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return ctypes.c_void_p(stream.cuda_stream)
+    # the current stream's handle without a Stream object around it (which costs more than the rest of the marshalling)
+    return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
 
 def build(K, beta, g, C, method=BLOCK_RECURSIVE, cu_seqlens=None, out=None, stream=None):
     """A = (I+N)^{-1} per chunk -> A [B,T,H,C] fp32 (rows of real tokens written)."""
     B, T, H, d_k = K.shape
     desc, keep = make_desc(B, T, H, d_k, d_k, C, _dtype_code(K), cu_seqlens)
-    A = torch.zeros((B, T, H, C), dtype=torch.float32, device=K.device) if out is None else out
+    A = torch.empty((B, T, H, C), dtype=torch.float32, device=K.device) if out is None else out
     rc = load().tri_inv_build(_p(K), _p(beta), _p(g), _p(A), ctypes.byref(desc), int(method), _stream(stream))
     if rc != OK:
         raise TriInvError("tri_inv_build", rc)
@@ -181,7 +186,7 @@ def build_kda(K, G, beta, C, method=BLOCK_RECURSIVE, cu_seqlens=None, out=None, 
     """Per-channel decay: A = (I+N)^{-1} with N_ij = beta_i sum_c K_ic K_jc exp(G_ic - G_jc); G [B,T,H,d] fp32."""
     B, T, H, d_k = K.shape
     desc, keep = make_desc(B, T, H, d_k, d_k, C, _dtype_code(K), cu_seqlens)
-    A = torch.zeros((B, T, H, C), dtype=torch.float32, device=K.device) if out is None else out
+    A = torch.empty((B, T, H, C), dtype=torch.float32, device=K.device) if out is None else out
     rc = load().tri_inv_build_kda(_p(K), _p(G), _p(beta), _p(A), ctypes.byref(desc), int(method), _stream(stream))
     if rc != OK:
         raise TriInvError("tri_inv_build_kda", rc)
@@ -210,7 +215,7 @@ def fused_kda(K, V, G, beta, C, method=BLOCK_RECURSIVE, cu_seqlens=None, out=Non
     d_v = V.shape[-1]
     desc, keep = make_desc(B, T, H, d_k, d_v, C, _dtype_code(K), cu_seqlens)
     if out is None:
-        out = (torch.zeros((B, T, H, C), dtype=torch.float32, device=K.device), torch.zeros_like(K), torch.zeros_like(V))
+        out = (torch.empty((B, T, H, C), dtype=torch.float32, device=K.device), torch.empty_like(K), torch.empty_like(V))
     A, W, U = out
     rc = load().tri_inv_fused_kda(_p(K), _p(V), _p(G), _p(beta), _p(A), _p(W), _p(U), ctypes.byref(desc), int(method), _stream(stream))
     if rc != OK:
@@ -246,8 +251,8 @@ def wy(A, K, V, beta, cu_seqlens=None, out=None, stream=None):
     d_v = V.shape[-1] if V is not None else d_k
     desc, keep = make_desc(B, T, H, d_k, d_v, C, _dtype_code(K), cu_seqlens)
     if out is None:
-        W = torch.zeros_like(K)
-        U = torch.zeros_like(V) if V is not None else None
+        W = torch.empty_like(K)
+        U = torch.empty_like(V) if V is not None else None
     else:
         W, U = out
     rc = load().tri_inv_wy(_p(A), _p(K), _p(V), _p(beta), _p(W), _p(U), ctypes.byref(desc), _stream(stream))
@@ -262,8 +267,8 @@ def fused(K, V, beta, g, C, method=BLOCK_RECURSIVE, cu_seqlens=None, want_A=True
     d_v = V.shape[-1]
     desc, keep = make_desc(B, T, H, d_k, d_v, C, _dtype_code(K), cu_seqlens)
     if out is None:
-        A = torch.zeros((B, T, H, C), dtype=torch.float32, device=K.device) if want_A else None
-        W, U = torch.zeros_like(K), torch.zeros_like(V)
+        A = torch.empty((B, T, H, C), dtype=torch.float32, device=K.device) if want_A else None
+        W, U = torch.empty_like(K), torch.empty_like(V)
     else:
         A, W, U = out
     rc = load().tri_inv_fused(_p(K), _p(V), _p(beta), _p(g), _p(A), _p(W), _p(U), ctypes.byref(desc), int(method), _stream(stream))
@@ -280,10 +285,10 @@ def fused_raw(K_raw, V, beta_logit, gate_logit, C, method=BLOCK_RECURSIVE, cu_se
     d_v = V.shape[-1]
     desc, keep = make_desc(B, T, H, d_k, d_v, C, _dtype_code(K_raw), cu_seqlens)
     if out is None:
-        A = torch.zeros((B, T, H, C), dtype=torch.float32, device=K_raw.device) if want_A else None
-        W, U = torch.zeros_like(K_raw), torch.zeros_like(V)
-        bo = torch.zeros((B, T, H), dtype=torch.float32, device=K_raw.device) if want_gates else None
-        go = torch.zeros((B, T, H), dtype=torch.float32, device=K_raw.device) if want_gates else None
+        A = torch.empty((B, T, H, C), dtype=torch.float32, device=K_raw.device) if want_A else None
+        W, U = torch.empty_like(K_raw), torch.empty_like(V)
+        bo = torch.empty((B, T, H), dtype=torch.float32, device=K_raw.device) if want_gates else None
+        go = torch.empty((B, T, H), dtype=torch.float32, device=K_raw.device) if want_gates else None
     else:
         A, W, U, bo, go = out
     rc = load().tri_inv_fused_raw(_p(K_raw), _p(V), _p(beta_logit), _p(gate_logit), _p(A), _p(W), _p(U), _p(bo), _p(go),
@@ -301,7 +306,7 @@ def fused_packed_static(K, V, beta, g, C, cu_seqlens, method=BLOCK_RECURSIVE, ou
     d_v = V.shape[-1]
     desc, keep = make_desc(B, T, H, d_k, d_v, C, _dtype_code(K), cu_seqlens)
     if out is None:
-        out = (torch.zeros((B, T, H, C), dtype=torch.float32, device=K.device), torch.zeros_like(K), torch.zeros_like(V))
+        out = (torch.empty((B, T, H, C), dtype=torch.float32, device=K.device), torch.empty_like(K), torch.empty_like(V))
     A, W, U = out
     rc = load().tri_inv_fused_packed_static(_p(K), _p(V), _p(beta), _p(g), _p(A), _p(W), _p(U), ctypes.byref(desc),
                                             int(method), _stream(stream))
