@@ -329,7 +329,8 @@ int tri_inv_selftest_wait_timeout(const void* K, const void* V, const float* bet
 /*
  * The same for the tensor-core chunk scan (bf16, d_k = d_v = 128, C = 64; no step of the paper's method): tri_inv_chunk_scan
  * (zero initial state, scale 1, final state not returned) with every device-side wait limited to wait_limit_ns nanoseconds
- * and with the first thread block -- sequence 0, head 0, the first slice of value columns -- leaving out the state-update
+ * and with the first thread block -- sequence 0, head 0, the first slice of value columns (all of them when there are more (sequence, head) pairs than
+ * half the SMs) -- leaving out the state-update
  * product of its second chunk.  The block's waits run out one after the other (each warp gives up at its next wait and
  * leaves its loop), it raises the status word, frees its tensor memory and returns; what it had written of O stays (its
  * first chunk), the rest of its columns of sequence 0, head 0 is undefined.  All other blocks finish as usual.  The limit

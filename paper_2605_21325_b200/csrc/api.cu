@@ -10,7 +10,7 @@
 namespace tri_inv {
 namespace {
 
-__device__ int g_device_status[128] = {0};  // word 0: raised by kernels that give up on a bounded wait
+__device__ int g_device_status[256] = {0};  // word 0: raised by kernels that give up on a bounded wait
 
 std::atomic<long long> g_launches{0};
 

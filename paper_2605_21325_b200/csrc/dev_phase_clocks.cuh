@@ -36,7 +36,7 @@ extern "C" int tri_inv_debug_counters(int* out) {
   cudaError_t err;
   int* word = tri_inv::status_word_for_current_device(&err);
   if (!word) return 3;
-  if (cudaMemcpy(out, word, 128 * sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return 3;
-  return cudaMemset(word, 0, 128 * sizeof(int)) == cudaSuccess ? 0 : 3;
+  if (cudaMemcpy(out, word, 256 * sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return 3;
+  return cudaMemset(word, 0, 256 * sizeof(int)) == cudaSuccess ? 0 : 3;
 }
 #endif

@@ -44,7 +44,7 @@ def main():
     if not hasattr(L, "tri_inv_debug_counters"):
         raise SystemExit("%s is not a development build" % b.LIB_PATH)
     flush = torch.empty(256 << 20, dtype=torch.uint8, device="cuda")
-    words = (ctypes.c_int * 128)()
+    words = (ctypes.c_int * 256)()
     for _ in range(4):
         flush.fill_(1)
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -77,10 +77,10 @@ def main():
     print("SMs by number of CTAs they ran:", np.bincount(np.bincount(sm.astype(int))).tolist())
 
 
-SCAN_COMPUTE = ["loop top", "last chunk's O written", "P1 seen", "chain: U tile seen | output: P loads done", "chain: W S loaded",
-                "chain: U~' arrived | output: first 16 rows of P", "chain: U~ arrived | output: P arrived", "P3 seen", "state updated",
-                "S^T stored", "S^T arrived"]
-SCAN_CONTROL = ["state operand seen", "P1 issued", "copies issued", "U~' seen", "P3 issued", "U~ and P seen", "PU issued", "copies seen",
+SCAN_CHAIN = ["loop top", "tiles seen", "P1 seen", "W S loaded", "U~' arrived", "U~ arrived", "P3 seen", "state updated", "S^T arrived", "",
+              "P3 loaded"]
+SCAN_OUTPUT = ["loop top", "QK seen", "P formed", "last chunk's O written", "PQ seen", "start of PU arrived"]
+SCAN_CONTROL = ["state operand seen", "P1, PQ issued", "QK issued", "U~' seen", "P3 issued", "U~ and P seen", "PU issued", "",
                 "", "loop top"]
 
 
@@ -96,7 +96,7 @@ def kda_phases(b, wl, inp, d):
     L = b.load()
     if not hasattr(L, "tri_inv_debug_counters"):
         raise SystemExit("%s is not a development build" % b.LIB_PATH)
-    words = (ctypes.c_int * 128)()
+    words = (ctypes.c_int * 256)()
     for _ in range(3):
         L.tri_inv_debug_counters(words)
         b.fused_kda(d["K"], d["V"], G, d["beta"], inp.C, cu_seqlens=inp.cu_seqlens, out=out)
@@ -121,18 +121,19 @@ def scan_chunk(b, wl, inp, d):
     L = b.load()
     if not hasattr(L, "tri_inv_debug_counters"):
         raise SystemExit("%s is not a development build" % b.LIB_PATH)
-    words = (ctypes.c_int * 128)()
+    words = (ctypes.c_int * 256)()
     for _ in range(3):
         L.tri_inv_debug_counters(words)
         b.chunk_scan(Q, d["K"], W, U, d["g"], inp.C, scale=0.1, cu_seqlens=inp.cu_seqlens, out=O, want_state=False)
         torch.cuda.synchronize()
     L.tri_inv_debug_counters(words)
-    w = np.array(words[:], dtype=np.int64)[8:].reshape(10, 12)
-    base = w[8, 0]
-    for i in range(8):
-        role = "chain " if (i & 3) < 2 else "output"
-        print("warp %d (%s): " % (i, role) + ", ".join("%s %d" % (n, w[i, k] - base) for k, n in enumerate(SCAN_COMPUTE) if w[i, k]))
-    print("control thread: " + ", ".join("%s %d" % (n, w[8, k] - base) for k, n in enumerate(SCAN_CONTROL) if w[8, k]))
+    w = np.array(words[:], dtype=np.int64)[8:248].reshape(20, 12)
+    control = 12
+    base = w[control, 0]
+    for i in range(control):
+        role, names = ("chain ", SCAN_CHAIN) if i < 8 else ("output", SCAN_OUTPUT)
+        print("warp %d (%s): " % (i, role) + ", ".join("%s %d" % (n, w[i, k] - base) for k, n in enumerate(names) if n and w[i, k]))
+    print("control thread: " + ", ".join("%s %d" % (n, w[control, k] - base) for k, n in enumerate(SCAN_CONTROL) if n and w[control, k]))
 
 
 if __name__ == "__main__":

@@ -152,6 +152,42 @@ def test_chunk_scan_cuda_core_kernel_other_shapes(bnd, name, B, T, H, d_k, d_v, 
         assert max_ratio(bnd.to_numpy_f64(O2), O_rec) <= 1e-5 and max_ratio(bnd.to_numpy_f64(S2), S_rec) <= 1e-5
 
 
+# all 128 value columns in one CTA: more pairs than half the SMs, with more chunks than the kernel has tile stages, a last chunk
+# of one token, one-chunk and empty sequences, and several CTAs in turn on an SM
+WIDE_CASES = [
+    ("pairs_75", 1, 7 * 64 + 1, 75, None, True),
+    ("ragged_pairs_160", 1, 0, 16, np.array([0, 64, 64, 65, 400, 401, 720, 784, 1000, 1001, 1321], np.int32), False),
+]
+
+
+@pytest.mark.parametrize("name,B,T,H,cu,with_s0", WIDE_CASES, ids=[c[0] for c in WIDE_CASES])
+def test_chunk_scan_all_columns_in_one_block(bnd, name, B, T, H, cu, with_s0):
+    test_chunk_scan_matches_its_definition(bnd, name, B, T, H, cu, with_s0)
+
+
+def test_wide_scan_waits_that_run_out(bnd):
+    """The give-up path where the first thread block holds all 128 value columns of sequence 0, head 0: its first chunk is
+    written, the other heads' output is untouched, and the next ordinary call gives the bits of the call before."""
+    inp = wl.make("wide_stall", 1, 6 * 64, 80, 128, 128, 64, wl.BF16, seed=641)
+    dev = bnd.to_device(inp)
+    Q = bnd.kv_to_torch(wl.queries(inp, seed=642))
+    _, W, U = bnd.fused(dev["K"], dev["V"], dev["beta"], dev["g"], 64, method=bnd.W_DECAY, want_A=False)
+    call = lambda: bnd.chunk_scan(Q, dev["K"], W, U, dev["g"], 64, scale=1.0, want_state=False)[0]
+    ref = call()
+    torch.cuda.synchronize()
+    assert bnd.last_device_status() == 0
+    O = torch.full_like(dev["V"], float("nan"))
+    bnd.selftest_scan_wait_timeout(Q, dev["K"], W, U, dev["g"], 64, wait_limit_ns=100_000, out=O)
+    assert bnd.last_device_status() == bnd.ERR_DEVICE_TIMEOUT
+    assert bnd.last_device_status() == 0
+    bits = lambda t: t.contiguous().view(torch.int16)
+    assert torch.equal(bits(O[:, :64, 0]), bits(ref[:, :64, 0])) and torch.equal(bits(O[:, :, 1:]), bits(ref[:, :, 1:]))
+    again = call()
+    torch.cuda.synchronize()
+    assert bnd.last_device_status() == 0
+    assert torch.equal(bits(again), bits(ref))
+
+
 # the register-tiled fp32 scan: key dimensions on both sides of its two instances (padded and full), a last value slice of
 # eight columns, one-token and empty sequences, a chunk that ends one token into the next, and the first d_k beyond it
 F32_SCAN_CASES = [
