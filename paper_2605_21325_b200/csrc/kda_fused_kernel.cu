@@ -217,9 +217,9 @@ __global__ void __launch_bounds__(NT, CTAS_PER_SM) kda_fused_kernel(const __grid
 #pragma unroll
       for (int ks = 0; ks < D / 16; ++ks) {
         const uint32_t koff = (ks >> 2) * 8192 + (ks & 3) * 32;
-        umma_bf16(tmem, umma_desc(sK + koff, 16, 1024), umma_desc(sKm + koff, 16, 1024), idesc, ks > 0);
+        umma_bf16_lane(tmem, umma_desc(sK + koff, 16, 1024), umma_desc(sKm + koff, 16, 1024), idesc, ks > 0);
       }
-      umma_commit(bar_mma);
+      umma_commit_lane(bar_mma);
     }
     wait(bar_mma, ph_mma);
     ph_mma ^= 1;
@@ -312,8 +312,8 @@ __global__ void __launch_bounds__(NT, CTAS_PER_SM) kda_fused_kernel(const __grid
     auto issue_wy = [&](uint32_t b_tile) {
 #pragma unroll
       for (int ks = 0; ks < C / 16; ++ks)
-        umma_bf16(tmem, umma_desc(sAp + ks * 32, 16, 1024), umma_desc(b_tile + ks * 2048, 8192, 1024), idesc_wy, ks > 0);
-      umma_commit(bar_mma);
+        umma_bf16_lane(tmem, umma_desc(sAp + ks * 32, 16, 1024), umma_desc(b_tile + ks * 2048, 8192, 1024), idesc_wy, ks > 0);
+      umma_commit_lane(bar_mma);
     };
     if (tid == 0 && !bad) { tc_fence_after(); issue_wy(sK); }
     wait(bar_mma, ph_mma);
@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(NT, CTAS_PER_SM) kda_fused_kernel(const __grid
     if (tid == kTidG && n_g) mbar_wait_bounded(bar_g, (n_g - 1) & 1, p.wait_limit_ns);
     if (tid == kTidV && n_v) mbar_wait_bounded(bar_v, (n_v - 1) & 1, p.wait_limit_ns);
     if (tid == 0) {
-      umma_commit(bar_exit);
+      umma_commit_lane(bar_exit);
       mbar_wait_bounded(bar_exit, 0, p.wait_limit_ns);
     }
   }

@@ -179,9 +179,9 @@ __global__ void __launch_bounds__(NT, CTAS_PER_SM) kda_build_kernel(const __grid
 #pragma unroll
       for (int ks = 0; ks < D / 16; ++ks) {
         const uint32_t koff = (ks >> 2) * 8192 + (ks & 3) * 32;
-        umma_bf16(tmem, umma_desc(sK + koff, 16, 1024), umma_desc(sKm + koff, 16, 1024), idesc, ks > 0);
+        umma_bf16_lane(tmem, umma_desc(sK + koff, 16, 1024), umma_desc(sKm + koff, 16, 1024), idesc, ks > 0);
       }
-      umma_commit(bar_mma);
+      umma_commit_lane(bar_mma);
     }
     wait(bar_mma, ph_mma);
     ph_mma ^= 1;

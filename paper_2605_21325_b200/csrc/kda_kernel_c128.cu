@@ -216,14 +216,14 @@ __global__ void __launch_bounds__(NT, 2) kda_build_kernel_c128(const __grid_cons
 #pragma unroll
       for (int ks = 0; ks < D / 16; ++ks) {
         const uint32_t ko = (ks >> 2) * K_BOX + (ks & 3) * 32, mo = (ks >> 2) * KM_BOX + (ks & 3) * 32;
-        umma_bf16(tmem, umma_desc(sK + ko, 16, 1024), umma_desc(sKm + mo, 16, 1024), idesc0, ks > 0);
+        umma_bf16_lane(tmem, umma_desc(sK + ko, 16, 1024), umma_desc(sKm + mo, 16, 1024), idesc0, ks > 0);
       }
 #pragma unroll
       for (int ks = 0; ks < D / 16; ++ks) {
         const uint32_t ko = (ks >> 2) * K_BOX + (ks & 3) * 32, mo = (ks >> 2) * KM_BOX + (ks & 3) * 32;
-        umma_bf16(tmem + 64, umma_desc(sK + 64 * 128 + ko, 16, 1024), umma_desc(sKm + 64 * 128 + mo, 16, 1024), idesc1, ks > 0);
+        umma_bf16_lane(tmem + 64, umma_desc(sK + 64 * 128 + ko, 16, 1024), umma_desc(sKm + 64 * 128 + mo, 16, 1024), idesc1, ks > 0);
       }
-      umma_commit(bar_mma);
+      umma_commit_lane(bar_mma);
     }
     wait(bar_mma, ph_mma);
     ph_mma ^= 1;

@@ -323,8 +323,8 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
         const uint32_t st = (uint32_t)((c % kStages) * cfg::STAGE) >> 4;
 #pragma unroll
         for (int ks = 0; ks < 4; ++ks)
-          umma_bf16_el(tmem + cfg::TM_QK, dQ + st + ((box * cfg::WQ_BOX + ks * 32) >> 4), dK + st + ((box * cfg::K_BOX + ks * 32) >> 4), idesc_qk, box > 0 || ks > 0);
-        if (box == 1) umma_commit_el(bar_qk);
+          umma_bf16(tmem + cfg::TM_QK, dQ + st + ((box * cfg::WQ_BOX + ks * 32) >> 4), dK + st + ((box * cfg::K_BOX + ks * 32) >> 4), idesc_qk, box > 0 || ks > 0);
+        if (box == 1) umma_commit(bar_qk);
       };
       auto issue_p1 = [&](uint32_t d_col, uint64_t b) {
 #pragma unroll
@@ -341,9 +341,9 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
         tc_fence_after();
         TL(0);
         issue_p1(cfg::TM_WS, dW + st);
-        umma_commit_el(bar_t1);
+        umma_commit(bar_t1);
         issue_p1(cfg::TM_QS, dQ + st);
-        umma_commit_el(bar_tq);
+        umma_commit(bar_tq);
         TL(1);
         // the next chunk's QK, if its tiles have landed and this chunk's QK has been read; otherwise behind this chunk's products
         const bool last = c + 1 >= n_chunks;
@@ -359,7 +359,7 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
 #pragma unroll
           for (int ks = 0; ks < C / 16; ++ks)   // 16 tokens (8 columns of the A operand, 2048 bytes of the K tile) per step
             umma_bf16_ta(tmem + cfg::TM_DS, tmem + (KDA ? cfg::TM_UT : cfg::TM_UD) + 8 * ks, dKm + st + ((ks * 2048) >> 4), idesc_p3, ks > 0);
-          umma_commit_el(bar_s);
+          umma_commit(bar_s);
         }
         TL(4);
         if (early) issue_qk_half(c + 1, 1);
@@ -369,7 +369,7 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
 #pragma unroll
         for (int ks = 0; ks < C / 16; ++ks)
           umma_bf16_ta(tmem + cfg::TM_PU, tmem + cfg::TM_UT + 8 * ks, dP + ((ks * 32) >> 4), idesc_pu, 1u);   // on top of gamma_i (Q S)^T
-        umma_commit_el(bar_pu);
+        umma_commit(bar_pu);
         TL(6);
         if (!last && !early) {
           if (!wait(bar_full + 8 * ((c + 1) % kStages), full_parity(c + 1)) || !wait(bar_qr, ph)) { failed = true; break; }
@@ -381,7 +381,7 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
       if (failed) {
         // A wait has run out and this CTA is about to give up its shared and tensor memory: every product issued so far is
         // waited for first, again with a limit (a commit on a spare barrier); the gate warp does the same for the copies.
-        umma_commit_el(bar_exit);
+        umma_commit(bar_exit);
         mbar_wait_bounded(bar_exit, 0u, lim);
       }
     }

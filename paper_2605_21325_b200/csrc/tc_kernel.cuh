@@ -147,8 +147,15 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
     bad = !mbar_wait_bounded(bar, parity, p.wait_limit_ns);
     return !bad;
   };
+  // for the warp that issues products: a wait on which all of its lanes agree, and whether no lane has given up
+  auto wait_warp = [&](uint32_t bar, uint32_t parity) -> bool {
+    wait(bar, parity);
+    if constexpr (!BO) bad = __any_sync(0xffffffffu, bad);
+    return !bad;
+  };
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = BO ? tid >> 5 : __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // not BO: uniform for the compiler
+  const bool issuer = BO ? tid == 0 : warp == 0;   // who issues the products: warp 0, or (build only) its first lane
   const int g = lane >> 2, t = lane & 3;
   CTA_MARK(0);
   CTA_MARK(3);
@@ -174,7 +181,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
   // Thread 0 requests the tiles of an item; K and V complete on separate barriers so that the Gram
   // product can start on K alone and each buffer is refilled as soon as its last reader is done.
   // The tiles of an item are requested by single threads of different warps, so that no warp carries
-  // all of the control work: K by warp 2, V by warp 3, the L2 prefetch by warp 1, the MMAs by warp 0.
+  // all of the control work: K by warp 2, V by warp 3, the L2 prefetch by warp 1; the MMAs by warp 0.
   // K and V complete on separate barriers: the Gram product starts on K alone, and each buffer is
   // refilled as soon as its last reader is done.
   constexpr int kTidL2 = 32, kTidK = 64, kTidV = 96;
@@ -243,21 +250,27 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = BO ? *tmem_slot : __shfl_sync(0xffffffffu, *tmem_slot, 0);
   const uint32_t tmem_rows = tmem + (lane_base << 16);
   uint32_t ph_k = 0, ph_v = 0, ph_mma = 0, ph_u = 0;  // parities of the next completion to wait for on each barrier
 
-  // Gram S = K K^T: D/16 MMAs of C x C x 16 into the first C columns of tensor memory (thread 0)
+  // Gram S = K K^T: D/16 MMAs of C x C x 16 into the first C columns of tensor memory (warp 0)
   auto issue_gram = [&]() {
     constexpr uint32_t idesc = umma_idesc(C, C, 0);
 #pragma unroll
     for (int ks = 0; ks < D / 16; ++ks) {
       const uint64_t dk = umma_desc(sK + (ks >> 2) * cfg::BOX_BYTES + (ks & 3) * 32, 16, 1024);
-      umma_bf16(tmem, dk, dk, idesc, ks > 0);
+      if constexpr (BO) umma_bf16_lane(tmem, dk, dk, idesc, ks > 0);
+      else umma_bf16(tmem, dk, dk, idesc, ks > 0);
     }
-    umma_commit(bar_mma);
+    if constexpr (BO) umma_commit_lane(bar_mma);
+    else umma_commit(bar_mma);
   };
-  bool gram_early = false;  // thread 0: the Gram product of the coming item was already issued at the end of the last one
+  auto k_landed = [&]() {   // called by the issuer
+    const bool landed = mbar_try_wait(bar_k, ph_k);
+    return BO ? landed : (bool)__all_sync(0xffffffffu, landed);
+  };
+  bool gram_early = false;  // warp 0: the Gram product of the coming item was already issued at the end of the last one
   // Work distribution: the first two items of a CTA are fixed (blockIdx, blockIdx + grid), every
   // later one comes from a device counter, fetched one item ahead of its use so that prefetches
   // know their target.  SMs that run faster simply take more items.  A launch without a counter
@@ -413,10 +426,10 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
 
     if (!load_a) {
       // ---- 2. Gram S = K K^T on the tensor core: one thread issues D/16 MMAs of C x C x 16 into TMEM
-      if (tid == 0 && !gram_early) {
+      if (issuer && !gram_early) {
         // self-test (kTestStall): CTA 0 leaves out the Gram product of its first item, so the wait below runs out
         const bool stall = (p.ops & kTestStall) && item == 0;
-        if (wait(bar_k, ph_k) && !stall) {
+        if (wait_warp(bar_k, ph_k) && !stall) {
           tc_fence_after();
           issue_gram();
         }
@@ -515,7 +528,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
         constexpr uint32_t idesc_h = umma_idesc_f16(C, C, 1);
 #pragma unroll 1
         for (int s = 0; s <= R; ++s) {
-          if (tid == 0 && !bad) {
+          if (warp == 0 && !__any_sync(0xffffffffu, bad)) {
             tc_fence_after();
             // Y = N^p with p = 2^s is zero within p of the diagonal: steps of sixteen k whose operands are structurally
             // zero are not issued (Y.Y: k in [p, C-1-p]; X.Y: k in [p, C-1]).
@@ -652,7 +665,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
         constexpr uint32_t idesc_s = umma_idesc_tf32(C, C, 0);
 #pragma unroll 1
         for (int s = 0; s <= R; ++s) {
-          if (tid == 0) {
+          if (warp == 0) {
             tc_fence_after();
             // Y = N^p with p = 2^s is zero within p of the diagonal: Y[i][k] needs k <= i - p, Y[k][j] needs
             // k >= j + p.  Steps of eight k whose operands are structurally zero are not issued.
@@ -865,7 +878,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
         fence_proxy_async();
         tc_fence_before();
         __syncthreads();
-        if (tid == 0) { tc_fence_after(); issue_merge(0); }
+        if (warp == 0) { tc_fence_after(); issue_merge(0); }
         wait(bar_mma, ph_mma);
         ph_mma ^= 1;
         tc_fence_after();
@@ -888,7 +901,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
         fence_proxy_async();
         tc_fence_before();
         __syncthreads();
-        if (tid == 0) { tc_fence_after(); issue_merge(64); }
+        if (warp == 0) { tc_fence_after(); issue_merge(64); }
         wait(bar_mma, ph_mma);
         ph_mma ^= 1;
         tc_fence_after();
@@ -1077,10 +1090,10 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
         }
         umma_commit(second ? bar_mma_u : bar_mma);
       };
-      if (tid == 0) {
-        if (wait(bar_k, ph_k)) { tc_fence_after(); issue_wy(sApw, sK); }
+      if (warp == 0) {
+        if (wait_warp(bar_k, ph_k)) { tc_fence_after(); issue_wy(sApw, sK); }
         if (C == 128 && need_v) {
-          if (wait(bar_v, ph_v)) { tc_fence_after(); issue_wy(sAp, sV, D, true); }
+          if (wait_warp(bar_v, ph_v)) { tc_fence_after(); issue_wy(sAp, sV, D, true); }
         }
       }
       // A goes to global memory while the W product runs (its registers are free again before W returns)
@@ -1108,8 +1121,8 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
         tmem_wait_ld();
         tc_fence_before();
         __syncthreads();  // every warp holds its rows of W in registers: U may overwrite the columns
-        if (tid == 0) {
-          if (wait(bar_v, ph_v)) { tc_fence_after(); issue_wy(sAp, sV); }
+        if (warp == 0) {
+          if (wait_warp(bar_v, ph_v)) { tc_fence_after(); issue_wy(sAp, sV); }
         }
         if (tid == kTidK && has_next) issue_k(nx_tok0, nx_h);  // K's last reader (the W product) is done
         store_frag_piece_bf16(f0, stage, lane, w_row0, row_stride, rows - row0, &tmW, h * D + 0, tok0 + row0);
@@ -1127,7 +1140,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
         ph_k ^= 1;
         ph_v ^= 1;
         if (tid == kTidV && has_next && !cfg::RELOAD) issue_v(nx_tok0, nx_h);
-        if (tid == 0 && has_next && nx_rows == C && !load_a && mbar_try_wait(bar_k, ph_k)) {
+        if (issuer && has_next && nx_rows == C && !load_a && k_landed()) {
           // the next K tile has landed and tensor memory is free: start the next Gram product now
           tc_fence_after();
           issue_gram();
@@ -1180,7 +1193,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
       ph_k ^= 1;
       ph_v ^= 1;
       if (tid == kTidK && has_next && ((p.ops & kLoadA) || cfg::RELOAD)) issue_k(nx_tok0, nx_h);  // otherwise requested after the Gram product
-      if (tid == 0 && has_next && nx_rows == C && !load_a && mbar_try_wait(bar_k, ph_k)) {
+      if (issuer && has_next && nx_rows == C && !load_a && k_landed()) {
         // the next K tile has landed and tensor memory is free: start the next Gram product now
         tc_fence_after();
         issue_gram();
@@ -1207,8 +1220,9 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
     // (bounded) chance to finish: the last copy each tile thread requested, and every product issued so far.
     if (tid == kTidK && n_issue) mbar_wait_bounded(bar_k, (n_issue - 1) & 1, p.wait_limit_ns);
     if (tid == kTidV && n_issue) mbar_wait_bounded(bar_v, (n_issue - 1) & 1, p.wait_limit_ns);
-    if (tid == 0) {
-      umma_commit(bar_exit);
+    if (issuer) {
+      if constexpr (BO) umma_commit_lane(bar_exit);
+      else umma_commit(bar_exit);
       mbar_wait_bounded(bar_exit, 0, p.wait_limit_ns);
     }
   }
