@@ -18,7 +18,7 @@
 //   P1 [DVS x 64]  = S^T . W^T                     the chain's
 //   PQ [DVS x 64]  = S^T . Q^T                     right behind it, with a commit of its own
 //   P3 [DVS x 128] = U~'^T . K                     U~' = decay-scaled U~; the K tile is read MN-major
-//   QK [64 x 64]   = Q . K^T                       both K-major tiles; needs no state: one chunk ahead, half of it while U~' is formed, half behind P3
+//   QK [64 x 64]   = Q . K^T                       both K-major tiles; needs no state: one chunk ahead, behind P3
 //   PU [DVS x 64]  = U~^T . P^T, on top of gamma_i (Q S)^T
 // The dependent chain of a chunk is  P1 -> U~' -> P3 -> S^T.
 //
@@ -319,12 +319,13 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
                      dKm = umma_desc(s0 + cfg::OFF_KT, cfg::K_BOX, 1024), dP = umma_desc(sP, 16, 1024);
       auto wait = [&](uint32_t bar, uint32_t parity) { return (bool)__all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, lim)); };
       auto seen = [&](uint32_t bar, uint32_t parity) { return (bool)__all_sync(0xffffffffu, mbar_test_wait(bar, parity)); };
-      auto issue_qk_half = [&](int c, int box) {   // 64 of the 128 features; in halves, so that the control warp is back in time for U~'
+      auto issue_qk = [&](int c) {
         const uint32_t st = (uint32_t)((c % kStages) * cfg::STAGE) >> 4;
 #pragma unroll
-        for (int ks = 0; ks < 4; ++ks)
-          umma_bf16(tmem + cfg::TM_QK, dQ + st + ((box * cfg::WQ_BOX + ks * 32) >> 4), dK + st + ((box * cfg::K_BOX + ks * 32) >> 4), idesc_qk, box > 0 || ks > 0);
-        if (box == 1) umma_commit(bar_qk);
+        for (int ks = 0; ks < D / 16; ++ks)
+          umma_bf16(tmem + cfg::TM_QK, dQ + st + (((ks >> 2) * cfg::WQ_BOX + (ks & 3) * 32) >> 4),
+                    dK + st + (((ks >> 2) * cfg::K_BOX + (ks & 3) * 32) >> 4), idesc_qk, ks > 0);
+        umma_commit(bar_qk);
       };
       auto issue_p1 = [&](uint32_t d_col, uint64_t b) {
 #pragma unroll
@@ -332,7 +333,7 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
           umma_bf16_ta(tmem + d_col, tmem + cfg::TM_S + 8 * ks, b + (((ks >> 2) * cfg::WQ_BOX + (ks & 3) * 32) >> 4), idesc_p1, ks > 0);
       };
       uint32_t ph = 0;
-      if (wait(bar_full, 0)) { issue_qk_half(0, 0); issue_qk_half(0, 1); }
+      if (wait(bar_full, 0)) issue_qk(0);
       else failed = true;
       for (int c = 0; c < n_chunks && !failed; ++c, ph ^= 1) {
         const uint32_t st = (uint32_t)((c % kStages) * cfg::STAGE) >> 4;
@@ -345,10 +346,7 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
         issue_p1(cfg::TM_QS, dQ + st);
         umma_commit(bar_tq);
         TL(1);
-        // the next chunk's QK, if its tiles have landed and this chunk's QK has been read; otherwise behind this chunk's products
         const bool last = c + 1 >= n_chunks;
-        const bool early = !last && seen(bar_full + 8 * ((c + 1) % kStages), full_parity(c + 1)) && seen(bar_qr, ph);
-        if (early) { tc_fence_after(); issue_qk_half(c + 1, 0); }
         TL(2);
         if (!wait(bar_ud, ph)) { failed = true; break; }
         tc_fence_after();
@@ -362,7 +360,9 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
           umma_commit(bar_s);
         }
         TL(4);
-        if (early) issue_qk_half(c + 1, 1);
+        // the next chunk's QK, if its tiles have landed and this chunk's QK has been read; otherwise behind PU
+        const bool early = !last && seen(bar_full + 8 * ((c + 1) % kStages), full_parity(c + 1)) && seen(bar_qr, ph);
+        if (early) { tc_fence_after(); issue_qk(c + 1); }
         if (!wait(bar_ut, ph)) { failed = true; break; }   // U~ (chain warps) and P with the start of PU (output warps)
         tc_fence_after();
         TL(5);
@@ -374,8 +374,7 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
         if (!last && !early) {
           if (!wait(bar_full + 8 * ((c + 1) % kStages), full_parity(c + 1)) || !wait(bar_qr, ph)) { failed = true; break; }
           tc_fence_after();
-          issue_qk_half(c + 1, 0);
-          issue_qk_half(c + 1, 1);
+          issue_qk(c + 1);
         }
       }
       if (failed) {
