@@ -122,10 +122,10 @@ struct ScanParams {
 cudaError_t launch_seq_offsets(int* dev_out, const tri_inv_desc* d, cudaStream_t stream);
 cudaError_t launch_chunk_scan(const ScanParams& p, const void* Q, const void* K, const void* W, long long tokens,
                               cudaStream_t stream, bool kda = false);
-// Per-channel form: the operands of the tensor-core scan from Q, K, W (bf16, [tokens,H,128]) and G, C = 64:
-// Qp = Q exp(G - G_ref), Km = K exp(G_ref - G), Wm = W exp(-G_ref) and the per-chunk vectors EL = exp(G_last),
+// Per-channel form: the operands of the tensor-core scan from Q, K (bf16, [tokens,H,128]) and G, C = 64:
+// Qp = Q exp(G - G_ref), Km = K exp(G_ref - G) and the per-chunk vectors EL = exp(G_last),
 // ER = exp(G_ref), EX = exp(G_last - G_ref) ([slots,H,128] fp32), G_ref the middle row of each chunk, G_last its last.
-cudaError_t launch_kda_scan_prep(const ScanParams& p, const void* Q, const void* K, const void* W, void* Qp, void* Km, void* Wm,
+cudaError_t launch_kda_scan_prep(const ScanParams& p, const void* Q, const void* K, void* Qp, void* Km,
                                  float* EL, float* ER, float* EX, int max_chunks_per_seq, cudaStream_t stream);
 // Single precision with a scalar gate at C = 64 and d_k <= 128 (scan_f32_kernel.cu).
 cudaError_t launch_chunk_scan_f32(const ScanParams& p, const void* Q, const void* K, const void* W, int d_k, int d_v, cudaStream_t stream);

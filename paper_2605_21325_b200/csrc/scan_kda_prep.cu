@@ -3,11 +3,11 @@
 // row and G_last its last row, the chunk form
 //     P_ij = sum_k Q_ik K_jk exp(G_ik - G_jk),   O = (Q exp G) S + P U~,   S <- diag(exp G_last) S + (K exp(G_last - G))^T U~
 // becomes the scalar-gate kernel's three products on
-//     Q+ = Q exp(G - G_ref),   K- = K exp(G_ref - G),   W- = W exp(-G_ref)
-// (each factor within exp(+-|G over 32 tokens|)), with the state operand scaled per row by exp(G_ref),
-//     [W- ; Q+] . [diag(exp G_ref) S | K-^T]  =  [W S | . ; (Q exp G) S | Q+ K-^T],
+//     Q+ = Q exp(G - G_ref),   K- = K exp(G_ref - G)
+// (each factor within exp(+-|G over 32 tokens|)), with a second copy of the state operand scaled per feature by exp(G_ref),
+//     Q+ . diag(exp G_ref) S = (Q exp G) S,     Q+ K-^T = the decayed Q K^T   (W S needs neither),
 // and the state increment taken from K- as well: (K exp(G_last - G))^T U~ = diag(exp(G_last - G_ref)) K-^T U~.
-// One pass over Q, K, W and G writes the three bf16 tensors and, per chunk, exp(G_last), exp(G_ref) and
+// One pass over Q, K and G writes the two bf16 tensors and, per chunk, exp(G_last), exp(G_ref) and
 // exp(G_last - G_ref); the exponent of each difference is taken once per element instead of once per (i, j, k).
 #include "common.cuh"
 
@@ -18,9 +18,9 @@ constexpr int C = 64, D = 128, NT = 256;
 constexpr float kLog2e = 1.4426950408889634f;
 
 struct PrepArgs {
-  const __nv_bfloat16 *Q, *K, *W;
+  const __nv_bfloat16 *Q, *K;
   const float* G;
-  __nv_bfloat16 *Qp, *Km, *Wm;
+  __nv_bfloat16 *Qp, *Km;
   float *EL, *ER, *EX;
   const int* seq_off;
   int H, T, n_seqs;
@@ -64,16 +64,12 @@ __global__ void __launch_bounds__(NT) kda_scan_prep_kernel(PrepArgs a) {
                                                                       ex2f(glast[4 * q + 2] - gref[4 * q + 2]), ex2f(glast[4 * q + 3] - gref[4 * q + 3]));
       }
     }
-    float wneg[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) wneg[e] = ex2f(-gref[e]);
 #pragma unroll
     for (int pass = 0; pass < 4; ++pass) {
       const int r = r0 + 16 * pass;
       if (r >= rows) break;
       const size_t idx = ((size_t)(tok0 + r) * a.H + h) * D + f0;
-      const uint4 qv = *reinterpret_cast<const uint4*>(a.Q + idx), kv = *reinterpret_cast<const uint4*>(a.K + idx),
-                  wv = *reinterpret_cast<const uint4*>(a.W + idx);
+      const uint4 qv = *reinterpret_cast<const uint4*>(a.Q + idx), kv = *reinterpret_cast<const uint4*>(a.K + idx);
       float g[8];
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
@@ -82,32 +78,28 @@ __global__ void __launch_bounds__(NT) kda_scan_prep_kernel(PrepArgs a) {
       }
       const uint32_t* qw = reinterpret_cast<const uint32_t*>(&qv);
       const uint32_t* kw = reinterpret_cast<const uint32_t*>(&kv);
-      const uint32_t* ww = reinterpret_cast<const uint32_t*>(&wv);
-      uint4 qo, mo, wo;
-      uint32_t *qp = reinterpret_cast<uint32_t*>(&qo), *mp = reinterpret_cast<uint32_t*>(&mo), *wp = reinterpret_cast<uint32_t*>(&wo);
+      uint4 qo, mo;
+      uint32_t *qp = reinterpret_cast<uint32_t*>(&qo), *mp = reinterpret_cast<uint32_t*>(&mo);
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
         const float2 qf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&qw[e]));
         const float2 kf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&kw[e]));
-        const float2 wf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&ww[e]));
         const float x0 = g[2 * e] - gref[2 * e], x1 = g[2 * e + 1] - gref[2 * e + 1];
         qp[e] = pack2(qf.x * ex2f(x0), qf.y * ex2f(x1));
         mp[e] = pack2(kf.x * ex2f(-x0), kf.y * ex2f(-x1));
-        wp[e] = pack2(wf.x * wneg[2 * e], wf.y * wneg[2 * e + 1]);
       }
       *reinterpret_cast<uint4*>(a.Qp + idx) = qo;
       *reinterpret_cast<uint4*>(a.Km + idx) = mo;
-      *reinterpret_cast<uint4*>(a.Wm + idx) = wo;
     }
   }
 }
 
 }  // namespace
 
-cudaError_t launch_kda_scan_prep(const ScanParams& p, const void* Q, const void* K, const void* W, void* Qp, void* Km, void* Wm,
+cudaError_t launch_kda_scan_prep(const ScanParams& p, const void* Q, const void* K, void* Qp, void* Km,
                                  float* EL, float* ER, float* EX, int max_chunks_per_seq, cudaStream_t stream) {
-  PrepArgs a{reinterpret_cast<const __nv_bfloat16*>(Q), reinterpret_cast<const __nv_bfloat16*>(K), reinterpret_cast<const __nv_bfloat16*>(W), p.G,
-             reinterpret_cast<__nv_bfloat16*>(Qp), reinterpret_cast<__nv_bfloat16*>(Km), reinterpret_cast<__nv_bfloat16*>(Wm), EL, ER, EX,
+  PrepArgs a{reinterpret_cast<const __nv_bfloat16*>(Q), reinterpret_cast<const __nv_bfloat16*>(K), p.G,
+             reinterpret_cast<__nv_bfloat16*>(Qp), reinterpret_cast<__nv_bfloat16*>(Km), EL, ER, EX,
              p.seq_off, p.H, p.T, p.n_seqs};
   const long long gx = (long long)p.n_seqs * p.H;
   if (gx > 0x7fffffffLL) return cudaErrorInvalidValue;

@@ -13,8 +13,9 @@
 // two operands on the dependent chain, S^T and U~'^T (bf16), are A operands IN tensor memory.  They go there straight
 // from the accumulator fragments that produced them (tcgen05.ld 16x256b -> arithmetic -> tcgen05.st 16x128b: the same
 // lanes, pairs of columns packed), with no trip through shared memory, no transpose and no proxy fence.  The products
-// of a chunk, with M = 128 lanes where the operand is transposed (a slice of 64 or 32 columns leaves lanes unused: an
-// instruction takes the same time at M = 64):
+// of a chunk (the transposed ones with M = 128, or for a slice of 64 or 32 columns M = 64, rows 16 q .. + 15 in lanes 0 .. 15 of
+// quadrant q: the same time per instruction, but the kernel runs at the power cap, where less work is a higher clock: 612 ->
+// 583 us back to back on 32 pairs of 512 chunks):
 //   P1 [DVS x 64]  = S^T . W^T                     the chain's
 //   PQ [DVS x 64]  = S^T . Q^T                     right behind it, with a commit of its own
 //   P3 [DVS x 128] = U~'^T . K                     U~' = decay-scaled U~; the K tile is read MN-major
@@ -49,16 +50,19 @@ constexpr float kLog2e = 1.4426950408889634f;
 
 // KDA: the per-channel form (one decay per key feature, the KDA row of Table 1).  Its decays are folded into the
 // operands beforehand (kda_scan_prep_kernel, scan_kda_prep.cu): with G_ref the middle row of a chunk and G_last its last,
-//     W- = W exp(-G_ref),  Q+ = Q exp(G - G_ref),  K- = K exp(G_ref - G),
-// P1 = (diag(exp G_ref) S)^T . [W- ; Q+]^T gives (W S)^T and ((Q exp G) S)^T, Q+ K-^T is the decayed Q K^T; P3 = U~^T K-,
+//     Q+ = Q exp(G - G_ref),  K- = K exp(G_ref - G),
+// S^T . W^T needs no decay, (diag(exp G_ref) S)^T . Q+^T gives ((Q exp G) S)^T, Q+ K-^T is the decayed Q K^T; P3 = U~^T K-,
 // scaled per column by exp(G_last - G_ref), is the state increment (K exp(G_last - G) = K- exp(G_last - G_ref): no second,
 // decay-scaled copy of U~); S decays by exp(G_last) per feature.  The kernel then differs from the scalar-gate one only in
-// where its operands come from and in a few scalings: the S^T operand is scaled per column by exp(G_ref) of the coming
-// chunk, P needs no decay, the state update has two per-column factors.
+// where its operands come from and in a few scalings: S^T is put down a second time, scaled per column by exp(G_ref) of the
+// coming chunk, as PQ's operand; P needs no decay; the state update has two per-column factors.  (A second S^T operand instead
+// of W exp(-G_ref) from the preparation pass takes a quarter of that pass's traffic away, and a rounding of W: 180.6 -> 164 us
+// for the call on B = 4, T = 4096, H = 16.)
 template <int DVS, bool KDA>
 struct ScanCfg {
   static_assert(DVS == 128 || DVS == 64 || DVS == 32, "slices of value columns");
   static constexpr int LG = DVS == 128 ? 2 : 1;          // groups of 16 tensor-memory lanes per quadrant in use
+  static constexpr int M = 64 * LG;                      // M = 64: lanes 0 .. 15 of each quadrant
   static constexpr int E = DVS == 32 ? 1 : 2;            // halves of a group of 16 lanes in use
   static constexpr int RPQ = DVS / 4;                    // value columns (rows here) per quadrant
   static constexpr int UBOX = DVS == 128 ? 2 : 1;        // 64-column boxes of U that hold the slice
@@ -73,7 +77,11 @@ struct ScanCfg {
   static constexpr int OFF_BAR = OFF_G + G_BYTES;
   static constexpr int SMEM = OFF_BAR + 160;
   // tensor-memory columns
-  static constexpr int TM_WS = 0, TM_QS = 64, TM_DS = 128, TM_PU = 256, TM_QK = 320, TM_S = 384, TM_UD = 448, TM_UT = 480;
+  // (per-channel form: the accumulators of P1 and P3 share their columns -- the chain warps have read the one before the other
+  // is issued, either way round -- and the scaled copy of S^T takes the room)
+  static constexpr int TM_WS = 0, TM_DS = KDA ? 0 : 64, TM_QS = TM_DS + 128, TM_PU = TM_QS + 64, TM_QK = TM_PU + 64, TM_S = TM_QK + 64,
+                       TM_SQ = KDA ? TM_S + 64 : TM_S, TM_UD = TM_SQ + 64, TM_UT = KDA ? TM_UD : TM_UD + 32;
+  static_assert(TM_UT + 32 <= 512, "tensor memory");
   static constexpr int TMEM_COLS = 512;
 };
 static_assert(ScanCfg<128, true>::SMEM <= 232448, "one CTA per SM");
@@ -284,20 +292,28 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
   const uint32_t tmem_w = tmem + ((uint32_t)(32 * quad) << 16);   // this warp's lanes, column 0
   bool failed = misaligned;
   // S^T as the A operand of P1: this warp's lanes, its 64 features as 32 columns of packed pairs
-  // (per-channel form: feature k times er[k], exp(G_ref) of the chunk that will read the operand)
+  // (per-channel form: a second time for PQ, feature k times er[k], exp(G_ref) of the chunk that will read the operand)
   auto write_state_operand = [&](const float* er) {
 #pragma unroll
     for (int lg = 0; lg < LG; ++lg) {
+      const uint32_t at = tmem_w + ((uint32_t)(16 * lg) << 16) + 32 * half;
       uint32_t r[16];
 #pragma unroll
       for (int nt = 0; nt < 8; ++nt) {
-        float2 f = make_float2(1.f, 1.f);
-        if constexpr (KDA) f = *reinterpret_cast<const float2*>(er + 64 * half + 8 * nt + 2 * t);
-        r[2 * nt] = KDA ? pack_bf16(f.x * S[lg][nt][0], f.y * S[lg][nt][1]) : pack_bf16(S[lg][nt][0], S[lg][nt][1]);
+        r[2 * nt] = pack_bf16(S[lg][nt][0], S[lg][nt][1]);
         r[2 * nt + 1] = 0u;
-        if constexpr (E == 2) r[2 * nt + 1] = KDA ? pack_bf16(f.x * S[lg][nt][2], f.y * S[lg][nt][3]) : pack_bf16(S[lg][nt][2], S[lg][nt][3]);
+        if constexpr (E == 2) r[2 * nt + 1] = pack_bf16(S[lg][nt][2], S[lg][nt][3]);
       }
-      tmem_st_packed32(r, tmem_w + ((uint32_t)(16 * lg) << 16) + cfg::TM_S + 32 * half);
+      tmem_st_packed32(r, at + cfg::TM_S);
+      if constexpr (KDA) {
+#pragma unroll
+        for (int nt = 0; nt < 8; ++nt) {
+          const float2 f = *reinterpret_cast<const float2*>(er + 64 * half + 8 * nt + 2 * t);
+          r[2 * nt] = pack_bf16(f.x * S[lg][nt][0], f.y * S[lg][nt][1]);
+          if constexpr (E == 2) r[2 * nt + 1] = pack_bf16(f.x * S[lg][nt][2], f.y * S[lg][nt][3]);
+        }
+        tmem_st_packed32(r, at + cfg::TM_SQ);
+      }
     }
     tmem_wait_st();
     tc_fence_before();
@@ -310,10 +326,10 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
     // code that the compiler knows to be uniform keeps them there (issued by a branch of one lane, each instruction costs 67
     // cycles of moves into them, whatever its shape).
     if (!misaligned) {
-      constexpr uint32_t idesc_p1 = umma_idesc(128, 64, 0);    // S^T, W or Q K-major
-      constexpr uint32_t idesc_p3 = umma_idesc(128, 128, 1);   // U~'^T, K MN-major
+      constexpr uint32_t idesc_p1 = umma_idesc(cfg::M, 64, 0);    // S^T, W or Q K-major
+      constexpr uint32_t idesc_p3 = umma_idesc(cfg::M, 128, 1);   // U~'^T, K MN-major
       constexpr uint32_t idesc_qk = umma_idesc(64, 64, 0);     // Q, K K-major
-      constexpr uint32_t idesc_pu = umma_idesc(128, 64, 0);    // U~^T, P K-major
+      constexpr uint32_t idesc_pu = umma_idesc(cfg::M, 64, 0);    // U~^T, P K-major
       // descriptors differ from these bases only in the address field (bits 0..13, units of 16 bytes)
       const uint64_t dW = umma_desc(s0, 16, 1024), dQ = umma_desc(s0 + 8192, 16, 1024), dK = umma_desc(s0 + cfg::OFF_KT, 16, 1024),
                      dKm = umma_desc(s0 + cfg::OFF_KT, cfg::K_BOX, 1024), dP = umma_desc(sP, 16, 1024);
@@ -327,10 +343,10 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
                     dK + st + (((ks >> 2) * cfg::K_BOX + (ks & 3) * 32) >> 4), idesc_qk, ks > 0);
         umma_commit(bar_qk);
       };
-      auto issue_p1 = [&](uint32_t d_col, uint64_t b) {
+      auto issue_p1 = [&](uint32_t d_col, uint32_t a_col, uint64_t b) {
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks)
-          umma_bf16_ta(tmem + d_col, tmem + cfg::TM_S + 8 * ks, b + (((ks >> 2) * cfg::WQ_BOX + (ks & 3) * 32) >> 4), idesc_p1, ks > 0);
+          umma_bf16_ta(tmem + d_col, tmem + a_col + 8 * ks, b + (((ks >> 2) * cfg::WQ_BOX + (ks & 3) * 32) >> 4), idesc_p1, ks > 0);
       };
       uint32_t ph = 0;
       if (wait(bar_full, 0)) issue_qk(0);
@@ -341,9 +357,9 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
         if (!wait(bar_sr, ph)) { failed = true; break; }   // (the chunk's tiles were waited for before its QK)
         tc_fence_after();
         TL(0);
-        issue_p1(cfg::TM_WS, dW + st);
+        issue_p1(cfg::TM_WS, cfg::TM_S, dW + st);
         umma_commit(bar_t1);
-        issue_p1(cfg::TM_QS, dQ + st);
+        issue_p1(cfg::TM_QS, cfg::TM_SQ, dQ + st);
         umma_commit(bar_tq);
         TL(1);
         const bool last = c + 1 >= n_chunks;
@@ -734,11 +750,13 @@ cudaError_t launch_seq_offsets(int* dev_out, const tri_inv_desc* d, cudaStream_t
 }
 
 // bf16 Q, K, W, U with d_k = d_v = 128 and C = 64.  One CTA per SM walks a (sequence, head) pair or a slice of its value
-// columns.  While every slice still gets an SM of its own, a pair is cut into four slices of 32 columns or two of 64: the
-// steps between the products get shorter with the slice.  With more pairs than that a CTA takes all 128 columns: the
+// columns.  A pair is cut into four slices of 32 columns while that takes half the SMs at most, into two of 64 while every
+// slice gets an SM of its own: the steps between the products get shorter with the slice.  (32 pairs in 128 CTAs of 32 columns
+// run at 1000 W, under the power cap, at 1.69 GHz: 583 us back to back; in 64 CTAs of 64 columns at 1.97 GHz: 548 us.)
+// With more pairs than that a CTA takes all 128 columns: the
 // products take the same time at any slice width, so each further slice would repeat them (64 packed sequences x 16 heads:
 // 265 us with 128 columns, 416 us in slices of 64 before).
-// kda selects the per-channel form: Q, K, W are then the prepared operands Q+, K-, W- (scan_kda_prep.cu), with p.EL,
+// kda selects the per-channel form: Q, K are then the prepared operands Q+, K- (scan_kda_prep.cu), with p.EL,
 // p.ER, p.EX the per-chunk vectors.
 cudaError_t launch_chunk_scan(const ScanParams& p, const void* Q, const void* K, const void* W, long long tokens,
                               cudaStream_t stream, bool kda) {
@@ -749,7 +767,7 @@ cudaError_t launch_chunk_scan(const ScanParams& p, const void* Q, const void* K,
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return cudaErrorUnknown;
   const long long pairs = (long long)p.n_seqs * p.H;
-  if (pairs * 4 <= sms) return kda ? launch_scan_one<32, true>(p, tmW, tmQ, tmK, tmU, stream) : launch_scan_one<32, false>(p, tmW, tmQ, tmK, tmU, stream);
+  if (pairs * 8 <= sms) return kda ? launch_scan_one<32, true>(p, tmW, tmQ, tmK, tmU, stream) : launch_scan_one<32, false>(p, tmW, tmQ, tmK, tmU, stream);
   if (pairs * 2 <= sms) return kda ? launch_scan_one<64, true>(p, tmW, tmQ, tmK, tmU, stream) : launch_scan_one<64, false>(p, tmW, tmQ, tmK, tmU, stream);
   return kda ? launch_scan_one<128, true>(p, tmW, tmQ, tmK, tmU, stream) : launch_scan_one<128, false>(p, tmW, tmQ, tmK, tmU, stream);
 }
