@@ -32,7 +32,9 @@ constexpr int kSliceLd = kSlice + 4;  // padded row length of the staging tile: 
 template <int C>
 struct SimtSmem {
   static constexpr int LD = C + 4;
-  static constexpr size_t floats = 3 * (size_t)C * LD + (size_t)C * kSliceLd + 4 * C;
+  // the scratch matrix also stages a slice of G in the per-channel Gram phase, whose rows are longer than LD at C = 16
+  static constexpr int Z_FLOATS = C * (LD > kSliceLd ? LD : kSliceLd);
+  static constexpr size_t floats = 2 * (size_t)C * LD + Z_FLOATS + (size_t)C * kSliceLd + 4 * C;
   static constexpr size_t bytes = floats * sizeof(float);
 };
 
@@ -152,7 +154,8 @@ __global__ void __launch_bounds__(kThreads, C <= 64 ? 2 : 1) simt_kernel(KParams
   float* Nm = smem;
   float* Xm = Nm + C * LD;
   float* Zm = Xm + C * LD;
-  float* Ks = Zm + C * LD;  // [C][kSliceLd]
+  float* Ks = Zm + SimtSmem<C>::Z_FLOATS;  // [C][kSliceLd]
+  static_assert(SimtSmem<C>::Z_FLOATS >= C * kSliceLd, "a slice of G fits into the scratch matrix");
   float* sb = Ks + C * kSliceLd;
   float* sg = sb + C;
   float* sr = sg + C;  // raw front end: 1 / |k_i|

@@ -73,7 +73,8 @@ def test_comba_layer_two_launches_against_its_recurrence(bnd):
         assert max_ratio(bnd.to_numpy_f64(O), O_ref) <= 2e-2 and max_ratio(bnd.to_numpy_f64(S), S_ref) <= 2e-2
 
 
-@pytest.mark.parametrize("C,dtype,d", [(64, wl.BF16, 128), (64, wl.F32, 64), (32, wl.BF16, 64), (128, wl.BF16, 128)])
+@pytest.mark.parametrize("C,dtype,d", [(64, wl.BF16, 128), (64, wl.F32, 64), (32, wl.BF16, 64), (128, wl.BF16, 128),
+                                       (16, wl.BF16, 128), (16, wl.F32, 40)])
 def test_per_channel_decay_through_wy_and_scan(bnd, C, dtype, d):
     """tri_inv_fused_kda (tensor-core route at bf16 / d = 128 / C = 64, CUDA cores elsewhere) against the oracle's A, W, U;
     then tri_inv_chunk_scan_kda on them against the token-by-token recurrence with one decay per key feature."""

@@ -494,7 +494,8 @@ def test_concurrent_launches_on_two_streams(bnd):
 
 # ---------------------------------------------------------------- per-channel decay (KDA row of Table 1)
 
-@pytest.mark.parametrize("C,dtype,d", [(64, wl.BF16, 128), (64, wl.F32, 64), (32, wl.BF16, 64), (128, wl.BF16, 128)])
+@pytest.mark.parametrize("C,dtype,d", [(64, wl.BF16, 128), (64, wl.F32, 64), (32, wl.BF16, 64), (128, wl.BF16, 128),
+                                       (16, wl.BF16, 128), (16, wl.F32, 40)])
 def test_build_kda(bnd, C, dtype, d):
     cu = np.array([0, 2 * C + 9, 3 * C + 9, 3 * C + 10], np.int32)
     for cu_seqlens, B, T in ((None, 2, 3 * C), (cu, 1, int(cu[-1]))):
