@@ -133,6 +133,20 @@ __device__ __forceinline__ void tmem_st_packed32(const uint32_t (&r)[16], uint32
                  "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(taddr) : "memory");
 }
 
+// A bounded wait whose outcome all lanes of the warp agree on.  A lane that has seen the phase may poll it again: the next phase
+// of every barrier of this kernel waits for something that each of its waiting warps does after its wait.  Not inlined: the
+// first polls are (below), and with the timer's loop in every wait as well the 128-column instance was 2 to 6 % slower (a vote
+// behind the per-lane wait: 1 to 6 % more); in this form calls of 1 .. 300 (sequence, head) pairs and 16 .. 512 chunks
+// take between 0.97 and 1.02 of the per-lane waits' time.
+__device__ __noinline__ bool wait_by_warp(uint32_t bar, uint32_t parity, unsigned long long limit_ns) {
+  const unsigned long long t0 = global_timer_ns();
+  for (uint32_t i = 1; i < kSpinLimit; ++i) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if ((i & 63u) == 0 && __any_sync(0xffffffffu, global_timer_ns() - t0 > limit_ns)) return false;
+  }
+  return false;
+}
+
 template <int DVS, bool KDA>
 __global__ void __launch_bounds__(kThreadsScan, 1)
 chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmQ,
@@ -291,6 +305,15 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
   const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   const uint32_t tmem_w = tmem + ((uint32_t)(32 * quad) << 16);   // this warp's lanes, column 0
   bool failed = misaligned;
+  // Every wait of the roles below is one of a whole warp (wait_by_warp): its lanes go on together or give up together.  What
+  // follows a wait (tcgen05.ld / st, ldmatrix, stmatrix, __syncwarp) takes the full warp, and lanes that polled and read the timer
+  // one by one could leave at the limit while others see the phase complete.
+  auto wait = [&](uint32_t bar, uint32_t parity) -> bool {
+#pragma unroll 1
+    for (int i = 0; i < 64; ++i)
+      if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    return wait_by_warp(bar, parity, lim);
+  };
   // S^T as the A operand of P1: this warp's lanes, its 64 features as 32 columns of packed pairs
   // (per-channel form: a second time for PQ, feature k times er[k], exp(G_ref) of the chunk that will read the operand)
   auto write_state_operand = [&](const float* er) {
@@ -333,7 +356,6 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
       // descriptors differ from these bases only in the address field (bits 0..13, units of 16 bytes)
       const uint64_t dW = umma_desc(s0, 16, 1024), dQ = umma_desc(s0 + 8192, 16, 1024), dK = umma_desc(s0 + cfg::OFF_KT, 16, 1024),
                      dKm = umma_desc(s0 + cfg::OFF_KT, cfg::K_BOX, 1024), dP = umma_desc(sP, 16, 1024);
-      auto wait = [&](uint32_t bar, uint32_t parity) { return (bool)__all_sync(0xffffffffu, mbar_wait_bounded(bar, parity, lim)); };
       auto seen = [&](uint32_t bar, uint32_t parity) { return (bool)__all_sync(0xffffffffu, mbar_test_wait(bar, parity)); };
       auto issue_qk = [&](int c) {
         const uint32_t st = (uint32_t)((c % kStages) * cfg::STAGE) >> 4;
@@ -408,13 +430,13 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
     for (int c = 0; c + 1 < n_chunks && !misaligned; ++c) {
       // stage of c + 2 = that of c - 1: its readers (the products of chunk c - 1, the chain warps' U) were done before the
       // arrivals that open chunk c
-      if (!mbar_wait_bounded(bar_sr, (uint32_t)(c & 1), lim)) { failed = true; break; }
+      if (!wait(bar_sr, (uint32_t)(c & 1))) { failed = true; break; }
       if (lane == 0 && c + 2 < n_chunks) { issue_copies(c + 2); requested = c + 2; }
       __syncwarp();
       // the factors of c - 1 have no reader left once the first product of chunk c is complete (it was issued behind the
       // arrivals of every warp that read them); bar_qr also says that every output warp has seen bar_g of chunk c, which must not
       // run two phases ahead of a warp that still waits for it
-      if (!mbar_wait_bounded(bar_t1, (uint32_t)(c & 1), lim) || !mbar_wait_bounded(bar_qr, (uint32_t)(c & 1), lim)) { failed = true; break; }
+      if (!wait(bar_t1, (uint32_t)(c & 1)) || !wait(bar_qr, (uint32_t)(c & 1))) { failed = true; break; }
       if constexpr (KDA) {
         // The vectors run one chunk further ahead than g: exp(G_ref) of chunk c + 1 is read at the end of chunk c (it
         // scales the S^T operand), so it has to be in place, and announced by an arrival, a chunk earlier.  Those of
@@ -440,9 +462,9 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
       const float* fb = sG + (c & 1) * 4 * C;
       const uint32_t sU = s0 + (c % kStages) * cfg::STAGE + cfg::OFF_UT;
       TL(0);
-      if (!mbar_wait_bounded(bar_full + 8 * (c % kStages), full_parity(c), lim)) { failed = true; break; }   // landed long ago; U is read below
+      if (!wait(bar_full + 8 * (c % kStages), full_parity(c))) { failed = true; break; }   // landed long ago; U is read below
       TL(1);
-      if (!mbar_wait_bounded(bar_t1, ph, lim)) { failed = true; break; }
+      if (!wait(bar_t1, ph)) { failed = true; break; }
       tc_fence_after();
       TL(2);
       // ---- U~ = U - W S, transposed: first the decay-scaled U~' that the chain waits for (its own arrival), then U~ itself
@@ -525,7 +547,7 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
       warp_arrive(bar_ut, lane);
       TL(5);
       // ---- state update and the bf16 operand for the next chunk
-      if (!mbar_wait_bounded(bar_s, ph, lim)) { failed = true; break; }
+      if (!wait(bar_s, ph)) { failed = true; break; }
       tc_fence_after();
       TL(6);
 #pragma unroll
@@ -604,7 +626,7 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
       const float* fb = sG + (c & 1) * 4 * C;
       TL(0);
       // ---- P = (Q K^T) * decay, lower triangle with its diagonal: rows 16 quad .. + 15 of this warp
-      if (!mbar_wait_bounded(bar_g, ph, lim) || !mbar_wait_bounded(bar_qk, ph, lim)) { failed = true; break; }
+      if (!wait(bar_g, ph) || !wait(bar_qk, ph)) { failed = true; break; }
       tc_fence_after();
       TL(1);
       uint32_t wa[8], wb[8];
@@ -641,7 +663,7 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
       // K-major operand, row i, 16-byte pieces of eight tokens j, swizzled; x4 stores of the matrices (rows +0..7, block),
       // (rows +8..15, block), and the same of block + 1
       if (c > 0) {
-        if (!mbar_wait_bounded(bar_pu, ph ^ 1, lim)) { failed = true; break; }
+        if (!wait(bar_pu, ph ^ 1)) { failed = true; break; }
         tc_fence_after();
       }
       {
@@ -652,7 +674,7 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
       }
       if (c > 0) write_output();
       TL(3);
-      if (!mbar_wait_bounded(bar_tq, ph, lim)) { failed = true; break; }
+      if (!wait(bar_tq, ph)) { failed = true; break; }
       tc_fence_after();
       TL(4);
       // ---- gamma_i (Q S)^T becomes the starting value of the PU accumulator (same lanes); in the per-channel form the
@@ -685,7 +707,7 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
       o_rows = end - tok0 < C ? end - tok0 : C;
     }
     if (!failed && !misaligned) {
-      if (mbar_wait_bounded(bar_pu, ph ^ 1, lim)) {
+      if (wait(bar_pu, ph ^ 1)) {
         tc_fence_after();
         write_output();
       } else {

@@ -101,3 +101,12 @@ def test_newer_entry_points_validate_on_the_host(lib):
     assert L.tri_inv_chunk_scan(ok, ok, ok, ok, ok, None, ok, None, scale, None, None) == binding.ERR_INVALID_ARG
     wide, _ = binding.make_desc(1, 64, 1, 512, 64, 64, binding.F32)      # d_k beyond the CUDA-core scan's state slice
     assert L.tri_inv_chunk_scan(ok, ok, ok, ok, ok, None, ok, None, scale, ctypes.byref(wide), None) == binding.ERR_UNSUPPORTED
+
+
+def test_scan_warps_wait_as_a_whole():
+    """What follows a wait in the scan kernel's warp roles takes the full warp (tcgen05.ld / st, ldmatrix, __syncwarp), so no
+    role may branch on the outcome of a wait lane by lane: each branches on wait(), whose lanes agree.  The per-lane
+    waits that are left drain a warp that has given up and are not branched on."""
+    src = open(os.path.join(ROOT, "paper_2605_21325_b200", "csrc", "scan_kernel.cu")).read()
+    roles = src[src.index("if (warp == kControl) {"):src.index("constexpr int kSeqsPerLaunch")]
+    assert not re.findall(r"if \([^;{]*mbar_(?:try_)?wait\w*\([^;{]*", roles)
