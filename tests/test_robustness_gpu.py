@@ -118,6 +118,32 @@ def test_scan_waits_that_run_out(bnd, B, H):
     assert torch.equal(again.view(torch.int16), ref.view(torch.int16))
 
 
+@pytest.mark.parametrize("d", [128, 64])
+def test_inversions_on_a_second_stream_do_not_wait_for_a_scan(bnd, d):
+    """A scan of few (sequence, head) pairs leaves most SMs free and takes all tensor memory of the others: inversions issued
+    behind it on another stream must run on the free SMs and be done long before the scan (1024 chunks: about a
+    millisecond; the inversions alone: some tens of microseconds)."""
+    a = wl.make("long_scan", 1, 1024 * 64, 4, 128, 128, 64, wl.BF16, seed=651)
+    b = wl.make("beside", 1, 64 * 64, 16, d, d, 64, wl.BF16, seed=652)
+    da, db = bnd.to_device(a), bnd.to_device(b)
+    Q = bnd.kv_to_torch(wl.queries(a, seed=653))
+    _, W, U = bnd.fused(da["K"], da["V"], da["beta"], da["g"], 64, method=bnd.W_DECAY, want_A=False)
+    O, A = torch.empty_like(da["V"]), torch.empty((b.B, b.T, b.H, 64), dtype=torch.float32, device="cuda")
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    for _ in range(2):   # the first pass sets the kernels up
+        torch.cuda.synchronize()
+        begin, scanned, built = (torch.cuda.Event(enable_timing=True) for _ in range(3))
+        begin.record(s1)
+        s2.wait_event(begin)
+        bnd.chunk_scan(Q, da["K"], W, U, da["g"], 64, out=O, want_state=False, stream=s1)
+        bnd.build(db["K"], db["beta"], db["g"], 64, out=A, stream=s2)
+        scanned.record(s1)
+        built.record(s2)
+        torch.cuda.synchronize()
+    assert bnd.last_device_status() == 0
+    assert begin.elapsed_time(built) < 0.8 * begin.elapsed_time(scanned)
+
+
 @pytest.mark.parametrize("C,with_wy", [(64, True), (64, False), (128, True)], ids=["C64_one_kernel", "C64_build", "C128_two_launches"])
 def test_per_channel_waits_that_run_out(bnd, C, with_wy):
     """The per-channel kernels' give-up path (tri_inv_selftest_kda_wait_timeout, limit 50 us): the first thread block leaves out
