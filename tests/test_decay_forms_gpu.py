@@ -154,8 +154,8 @@ def test_per_channel_scan_on_the_tensor_cores_full_size_ragged(bnd):
 
 def test_per_channel_scan_resumes_bit_for_bit(bnd):
     """Dense batch cut at a chunk boundary: the second part, started from the first part's returned state, gives the very
-    bits of the uncut run (few (sequence, head) pairs: the 32-column instance; many: the 64-column one)."""
-    for B, H in ((1, 2), (3, 20)):
+    bits of the uncut run (2, 60 and 100 (sequence, head) pairs: 32, 64 and 128 value columns per thread block)."""
+    for B, H in ((1, 2), (3, 20), (5, 20)):
         T, cut = 6 * 64 + 23, 4 * 64
         inp = wl.make("resume", B, T, H, 128, 128, 64, wl.BF16, seed=1400 + H)
         G = wl.per_channel_gate(inp, seed=66)

@@ -89,7 +89,7 @@ def test_graph_replays_overlapping_many_plain_launches(bnd):
 
 @pytest.mark.parametrize("B,H", [(1, 2), (4, 16)], ids=["narrow_slices", "wide_slices"])
 def test_scan_waits_that_run_out(bnd, B, H):
-    """The chunk-scan kernel's ten warps wait for one another through barriers only; with one product of the first thread
+    """The chunk-scan kernel's fourteen warps wait for one another through barriers only; with one product of the first thread
     block left out (tri_inv_selftest_scan_wait_timeout, limit 100 us) every one of that block's waits must give up in turn,
     the kernel must return with the status word raised once, the other blocks' output must be untouched by it, and the
     next ordinary call must give the bits of the call before."""
@@ -104,9 +104,10 @@ def test_scan_waits_that_run_out(bnd, B, H):
     bnd.selftest_scan_wait_timeout(Q, dev["K"], W, U, dev["g"], 64, wait_limit_ns=100_000, out=O)
     assert bnd.last_device_status() == bnd.ERR_DEVICE_TIMEOUT     # raised ...
     assert bnd.last_device_status() == 0                          # ... and cleared by the read
-    # the stalled block is (sequence 0, head 0, first slice of value columns: 32 or 64 wide); its first chunk was written
+    # the stalled block is (sequence 0, head 0, first slice of value columns); its first chunk was written
     # before the product was left out
-    width = 32 if B * H * 4 <= torch.cuda.get_device_properties(0).multi_processor_count else 64
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    width = 32 if B * H * 8 <= sms else 64 if B * H * 2 <= sms else 128
     r2, o2 = ref.clone(), O.clone()
     assert torch.equal(o2[0, :64, 0, :width].view(torch.int16), r2[0, :64, 0, :width].view(torch.int16))
     r2[0, 64:, 0, :width] = 0

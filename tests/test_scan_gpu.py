@@ -46,7 +46,7 @@ CASES = [
     ("dense_partial_s0", 1, 3 * 64 + 17, 2, None, True),
     ("ragged_s0", 1, 0, 2, np.array([0, 64, 65, 65, 300, 531], np.int32), True),
     ("many_heads", 5, 2 * 64, 64, None, True),   # 640 CTAs: several per SM in turn
-    # few (sequence, head) pairs run as four CTAs of 32 value columns per pair, more as two of 64: both sides of the switch
+    # two CTAs of 64 value columns per (sequence, head) pair
     ("pairs_36", 2, 3 * 64 + 9, 18, None, True),
     ("pairs_40", 2, 3 * 64 + 9, 20, None, True),
 ]
@@ -150,6 +150,66 @@ def test_chunk_scan_cuda_core_kernel_other_shapes(bnd, name, B, T, H, d_k, d_v, 
         torch.cuda.synchronize()
         O_rec, S_rec = oracle.gdn_recurrence(Q, inp.K, inp.V, inp.beta, inp.g, C, scale=0.5, S0=S0, cu_seqlens=cu)
         assert max_ratio(bnd.to_numpy_f64(O2), O_rec) <= 1e-5 and max_ratio(bnd.to_numpy_f64(S2), S_rec) <= 1e-5
+
+
+# The launch cuts a (sequence, head) pair's value columns into four slices while that takes half the SMs at most, into two while every
+# slice gets an SM, else none: the pair counts on both sides of either switch, and their slice width.
+def slice_edges():
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    return [(sms // 8, 32), (sms // 8 + 1, 64), (sms // 2, 64), (sms // 2 + 1, 128)]
+
+
+@pytest.mark.parametrize("edge", range(4))
+@pytest.mark.parametrize("per_channel", [False, True])
+def test_chunk_scan_on_both_sides_of_each_slice_width(bnd, edge, per_channel):
+    """Against the token-by-token recurrence, with a carried state and a last chunk of nine tokens."""
+    H, _ = slice_edges()[edge]
+    inp = wl.make("edge", 1, 3 * 64 + 9, H, 128, 128, 64, wl.BF16, seed=370 + edge)
+    Q, S0 = wl.queries(inp, seed=371), wl.initial_state(inp, seed=372)
+    dev = bnd.to_device(inp)
+    Qd, S0d = bnd.kv_to_torch(Q), torch.from_numpy(S0).cuda()
+    O = torch.full_like(dev["V"], float("nan"))
+    if per_channel:
+        G = wl.per_channel_gate(inp, seed=373)
+        Gd = torch.from_numpy(G).cuda()
+        _, W, U = bnd.fused_kda(dev["K"], dev["V"], Gd, dev["beta"], 64)
+        O, S = bnd.chunk_scan_kda(Qd, dev["K"], W, U, Gd, 64, scale=0.5, S0=S0d, out=O)
+        O_ref, S_ref = oracle.recurrence_ex(Q, inp.K, inp.V, inp.beta, None, 64, G=G, scale=0.5, S0=S0)
+    else:
+        _, W, U = bnd.fused(dev["K"], dev["V"], dev["beta"], dev["g"], 64, method=bnd.W_DECAY, want_A=False)
+        O, S = bnd.chunk_scan(Qd, dev["K"], W, U, dev["g"], 64, scale=0.5, S0=S0d, out=O)
+        O_ref, S_ref = oracle.gdn_recurrence(Q, inp.K, inp.V, inp.beta, inp.g, 64, scale=0.5, S0=S0)
+    torch.cuda.synchronize()
+    assert bnd.last_device_status() == 0
+    o = bnd.to_numpy_f64(O)
+    assert not np.isnan(o).any(), "a row of O was not written"
+    assert max_ratio(o, O_ref) <= TOL_LAYER and max_ratio(bnd.to_numpy_f64(S), S_ref) <= TOL_LAYER
+
+
+@pytest.mark.parametrize("per_channel", [False, True])
+def test_a_heads_result_does_not_depend_on_the_slice_width(bnd, per_channel):
+    """The same heads scanned among so many others that a CTA takes 128, 64 or 32 value columns: the same bits."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    T, few = 5 * 64 + 7, 4
+    inp = wl.make("width", 1, T, sms // 2 + 1, 128, 128, 64, wl.BF16, seed=380)
+    Q, S0 = bnd.kv_to_torch(wl.queries(inp, seed=381)), torch.from_numpy(wl.initial_state(inp, seed=382)).cuda()
+    dev = bnd.to_device(inp)
+    if per_channel:
+        g = torch.from_numpy(wl.per_channel_gate(inp, seed=383)).cuda()
+        _, W, U = bnd.fused_kda(dev["K"], dev["V"], g, dev["beta"], 64)
+    else:
+        g = dev["g"]
+        _, W, U = bnd.fused(dev["K"], dev["V"], dev["beta"], g, 64, method=bnd.W_DECAY, want_A=False)
+    results = []
+    for heads in (sms // 2 + 1, sms // 4, few):
+        cut = lambda t: t[:, :, :heads].contiguous()
+        scan = bnd.chunk_scan_kda if per_channel else bnd.chunk_scan
+        O, S = scan(cut(Q), cut(dev["K"]), cut(W), cut(U), cut(g), 64, scale=0.5, S0=S0[:, :heads].contiguous())
+        torch.cuda.synchronize()
+        results.append((O[:, :, :few].contiguous().view(torch.int16), S[:, :few].contiguous()))
+    assert bnd.last_device_status() == 0
+    for O, S in results[1:]:
+        assert torch.equal(O, results[0][0]) and torch.equal(S, results[0][1])
 
 
 # all 128 value columns in one CTA: more pairs than half the SMs, with more chunks than the kernel has tile stages, a last chunk
@@ -356,11 +416,11 @@ def test_random_layouts_layer_forward(bnd, seed):
         assert max_ratio(bnd.to_numpy_f64(O), O_ref) <= TOL_LAYER and max_ratio(bnd.to_numpy_f64(S), S_ref) <= TOL_LAYER, (it, B, T, H, cu)
 
 
-@pytest.mark.parametrize("n_seqs,H", [(9, 3), (26, 8)], ids=["narrow_slices", "wide_slices"])
+@pytest.mark.parametrize("n_seqs,H", [(5, 3), (9, 3), (26, 8)], ids=["32_columns", "64_columns", "128_columns"])
 def test_chunk_scan_repeats_bit_for_bit(bnd, n_seqs, H):
-    """The hand-offs inside a CTA (copies, products, operand writes of ten warps) are all ordered by barriers: the same
+    """The hand-offs inside a CTA (copies, products, operand writes of fourteen warps) are all ordered by barriers: the same
     launch on the same inputs gives the same bits every time.  A missing ordering would show as a difference between runs.
-    Ragged packed sequences; both slice widths (27 and 208 (sequence, head) pairs)."""
+    Ragged packed sequences; every slice width (15, 27 and 208 (sequence, head) pairs)."""
     rng = np.random.default_rng(60 + H)
     cu = np.concatenate([[0], np.cumsum(rng.integers(1, 500, size=n_seqs))]).astype(np.int32)
     inp = wl.make("repeat", 1, int(cu[-1]), H, 128, 128, 64, wl.BF16, seed=360 + H, cu_seqlens=cu)
