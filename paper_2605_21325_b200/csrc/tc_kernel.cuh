@@ -154,8 +154,11 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
     return !bad;
   };
 
-  const int tid = threadIdx.x, warp = BO ? tid >> 5 : __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // not BO: uniform for the compiler
-  const bool issuer = BO ? tid == 0 : warp == 0;   // who issues the products: warp 0, or (build only) its first lane
+  // warp_u: uniform for the compiler (not BO), for the code that issues products.  The rest uses it too, except with the refinement
+  // step, whose selection of tiles by warp costs more as branches on a uniform value than as predicates (4096 matrices: C = 64
+  // 123.8 us with, 119.2 us without; C = 128 853.8 and 800.4 us).
+  const int tid = threadIdx.x, warp_u = BO ? tid >> 5 : __shfl_sync(0xffffffffu, tid >> 5, 0), warp = REF ? tid >> 5 : warp_u, lane = tid & 31;
+  const bool issuer = BO ? tid == 0 : warp_u == 0;   // who issues the products: warp 0, or (build only) its first lane
   const int g = lane >> 2, t = lane & 3;
   CTA_MARK(0);
   CTA_MARK(3);
@@ -243,7 +246,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
     }
     if (any) bg_next = fetch_bg(tok0, rows, h);
   }
-  if (warp == 0) {
+  if (warp_u == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -528,7 +531,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
         constexpr uint32_t idesc_h = umma_idesc_f16(C, C, 1);
 #pragma unroll 1
         for (int s = 0; s <= R; ++s) {
-          if (warp == 0 && !__any_sync(0xffffffffu, bad)) {
+          if (warp_u == 0 && !__any_sync(0xffffffffu, bad)) {
             tc_fence_after();
             // Y = N^p with p = 2^s is zero within p of the diagonal: steps of sixteen k whose operands are structurally
             // zero are not issued (Y.Y: k in [p, C-1-p]; X.Y: k in [p, C-1]).
@@ -665,7 +668,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
         constexpr uint32_t idesc_s = umma_idesc_tf32(C, C, 0);
 #pragma unroll 1
         for (int s = 0; s <= R; ++s) {
-          if (warp == 0) {
+          if (warp_u == 0) {
             tc_fence_after();
             // Y = N^p with p = 2^s is zero within p of the diagonal: Y[i][k] needs k <= i - p, Y[k][j] needs
             // k >= j + p.  Steps of eight k whose operands are structurally zero are not issued.
@@ -878,7 +881,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
         fence_proxy_async();
         tc_fence_before();
         __syncthreads();
-        if (warp == 0) { tc_fence_after(); issue_merge(0); }
+        if (warp_u == 0) { tc_fence_after(); issue_merge(0); }
         wait(bar_mma, ph_mma);
         ph_mma ^= 1;
         tc_fence_after();
@@ -901,7 +904,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
         fence_proxy_async();
         tc_fence_before();
         __syncthreads();
-        if (warp == 0) { tc_fence_after(); issue_merge(64); }
+        if (warp_u == 0) { tc_fence_after(); issue_merge(64); }
         wait(bar_mma, ph_mma);
         ph_mma ^= 1;
         tc_fence_after();
@@ -1090,7 +1093,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
         }
         umma_commit(second ? bar_mma_u : bar_mma);
       };
-      if (warp == 0) {
+      if (warp_u == 0) {
         if (wait_warp(bar_k, ph_k)) { tc_fence_after(); issue_wy(sApw, sK); }
         if (C == 128 && need_v) {
           if (wait_warp(bar_v, ph_v)) { tc_fence_after(); issue_wy(sAp, sV, D, true); }
@@ -1121,7 +1124,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
         tmem_wait_ld();
         tc_fence_before();
         __syncthreads();  // every warp holds its rows of W in registers: U may overwrite the columns
-        if (warp == 0) {
+        if (warp_u == 0) {
           if (wait_warp(bar_v, ph_v)) { tc_fence_after(); issue_wy(sAp, sV); }
         }
         if (tid == kTidK && has_next) issue_k(nx_tok0, nx_h);  // K's last reader (the W product) is done
@@ -1228,7 +1231,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
   }
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
+  if (warp_u == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TMEM_COLS) : "memory");
 }
 
 // ------------------------------------------------------------------------------------------ host side
