@@ -26,6 +26,7 @@ namespace tri_inv {
 namespace {
 
 constexpr int kThreads = 256;
+constexpr long long kSMs = 148;
 constexpr int kSlice = 32;            // columns of K / V staged per pass
 constexpr int kSliceLd = kSlice + 4;  // padded row length of the staging tile: 16-byte pieces, eight rows in different banks
 
@@ -146,9 +147,9 @@ __device__ __forceinline__ void fma4(float (&acc)[4], float a, const float4& b) 
   acc[0] = fmaf(a, b.x, acc[0]); acc[1] = fmaf(a, b.y, acc[1]); acc[2] = fmaf(a, b.z, acc[2]); acc[3] = fmaf(a, b.w, acc[3]);
 }
 
-// at C <= 64 three CTAs fit an SM's shared memory; two of them at up to 128 registers keep the tiles out of local memory
-template <int C>
-__global__ void __launch_bounds__(kThreads, C <= 64 ? 2 : 1) simt_kernel(KParams p) {
+// BLOCKS: thread blocks per SM that the registers are shared out for (launch_one).
+template <int C, int BLOCKS>
+__global__ void __launch_bounds__(kThreads, BLOCKS) simt_kernel(KParams p) {
   constexpr int LD = C + 4;
   extern __shared__ float smem[];
   float* Nm = smem;
@@ -231,7 +232,7 @@ __global__ void __launch_bounds__(kThreads, C <= 64 ? 2 : 1) simt_kernel(KParams
           if (kda) gr.fetch(p.G, TRI_INV_F32, tok0, rows, p.H, h, p.d_k, ks + kSlice, tid);
         }
         if (kda) {
-#pragma unroll 1
+#pragma unroll(C <= 32 ? 8 : 1)   // small tiles: the loads of one step alone do not hide their latency
           for (int kk = 0; kk < kSlice; ++kk) {
             float ki[kB], gi[kB];
 #pragma unroll
@@ -524,16 +525,31 @@ __global__ void __launch_bounds__(kThreads, C <= 64 ? 2 : 1) simt_kernel(KParams
   }
 }
 
+template <int C, int BLOCKS>
+cudaError_t launch_blocks(const KParams& p, long long total, cudaStream_t stream) {
+  size_t bytes = SimtSmem<C>::bytes;
+  cudaError_t e = cudaFuncSetAttribute(simt_kernel<C, BLOCKS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  if (e != cudaSuccess) return e;
+  int grid = (int)(total < kSMs * 64 ? total : kSMs * 64);
+  simt_kernel<C, BLOCKS><<<grid, kThreads, bytes, stream>>>(p);
+  return cudaGetLastError();
+}
+
+// At C = 64 three blocks fit the shared memory of an SM; two of them at up to 128 registers keep the tiles out of local memory.
+// At C = 32 and 16 the products are short and the barriers between them bound a block, so with more chunks than two for each SM
+// more blocks are worth a few spilled registers.  fp32, d = 64, C = 16 with five blocks (47 registers) against two (84): 304
+// chunks fused 14.4 -> 10.3 us, 8192 chunks build 79.9 -> 49.0, fused 201 -> 116, Newton-Schulz 298 -> 172 us; C = 32 with four
+// (64) against two (124): 304 chunks fused 20.9 -> 15.6 us, 8192 chunks fused 308 -> 217, Newton-Schulz 1284 -> 928 us.  With fewer
+// chunks a block has the SM to itself or shares it with one other, and the registers shorten it: eight chunks, bf16, d = 128,
+// C = 16, fused 14.4 us with five blocks' registers, 12.3 us with two's.
 template <int C>
 cudaError_t launch_one(const KParams& p, cudaStream_t stream) {
-  size_t bytes = SimtSmem<C>::bytes;
-  cudaError_t e = cudaFuncSetAttribute(simt_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-  if (e != cudaSuccess) return e;
-  long long total = (long long)p.n_chunks * p.H;
+  const long long total = (long long)p.n_chunks * p.H;
   if (total == 0) return cudaSuccess;
-  int grid = (int)(total < 148LL * 64 ? total : 148LL * 64);
-  simt_kernel<C><<<grid, kThreads, bytes, stream>>>(p);
-  return cudaGetLastError();
+  if constexpr (C <= 32) {
+    if (total > 2 * kSMs) return launch_blocks<C, C == 16 ? 5 : 4>(p, total, stream);
+  }
+  return launch_blocks<C, C <= 64 ? 2 : 1>(p, total, stream);
 }
 
 }  // namespace

@@ -680,3 +680,29 @@ def test_decay_weighted_w_from_its_own_operand(bnd, shift, T, cu):
     assert bnd.last_device_status() == 0 and none is None
     assert torch.equal(A, A0) and torch.equal(U, U0) and torch.equal(W, W2) and torch.equal(U, U2)
     assert float((W.float() - W_ref.float()).abs().max()) <= 1e-2 * float(W_ref.float().abs().max())
+
+
+@pytest.mark.parametrize("C", [16, 32])
+@pytest.mark.parametrize("call", ["fused", "kda"])
+def test_cuda_core_kernel_on_both_sides_of_its_register_split(bnd, C, call):
+    """At C = 16 and 32 the CUDA-core kernel has an instance for up to 296 chunk matrices and one for more: 297 against the
+    oracle (1e-5, fp32), and the first 296 alone give the same bits (the sums are the same, in the same order)."""
+    inp = wl.make("split", 297, C, 1, 40, 24, C, wl.F32, seed=95 + C)
+    dev = bnd.to_device(inp)
+    G = wl.per_channel_gate(inp, seed=96)
+    Gd = torch.from_numpy(G).cuda()
+    run = (lambda n: bnd.fused(dev["K"][:n], dev["V"][:n], dev["beta"][:n], dev["g"][:n], C)) if call == "fused" else \
+          (lambda n: bnd.fused_kda(dev["K"][:n], dev["V"][:n], Gd[:n], dev["beta"][:n], C))
+    more, fewer = run(297), run(296)
+    torch.cuda.synchronize()
+    assert bnd.last_device_status() == 0
+    for a, b in zip(more, fewer):
+        assert torch.equal(a[:296], b)
+    if call == "fused":
+        A_ref, _, W_ref, U_ref = oracle_all(inp)
+    else:
+        A_ref = oracle.build_A_kda(inp.K, G, inp.beta, C)
+        W_ref, _ = oracle.wy(A_ref, inp.K.astype(np.float64) * np.exp(G.astype(np.float64)), None, inp.beta, C)
+        _, U_ref = oracle.wy(A_ref, inp.K, inp.V, inp.beta, C)
+    for x, r in zip(more, (A_ref, W_ref, U_ref)):
+        assert max_ratio(bnd.to_numpy_f64(x), r) <= 1e-5
