@@ -151,7 +151,8 @@ __device__ __forceinline__ void fma4(float (&acc)[4], float a, const float4& b) 
 template <int C, int BLOCKS>
 __global__ void __launch_bounds__(kThreads, BLOCKS) simt_kernel(KParams p) {
   constexpr int LD = C + 4;
-  extern __shared__ float smem[];
+  extern __shared__ __align__(16) float smem[];   // read and written 16 bytes at a time
+  static_assert(LD % 4 == 0 && kSliceLd % 4 == 0 && (C * LD) % 4 == 0 && SimtSmem<C>::Z_FLOATS % 4 == 0, "rows and matrices on 16-byte boundaries");
   float* Nm = smem;
   float* Xm = Nm + C * LD;
   float* Zm = Xm + C * LD;
