@@ -5,7 +5,8 @@ torch is used for device memory and streams.  There is no CPU path: if the
 library is missing or a call fails, these functions raise.
 
 Outputs that a function allocates are not filled first: the kernels write every row of every token (each token belongs to
-a sequence), all columns of it.
+a sequence), all columns of it.  After a call whose device-side wait gave up (``last_device_status`` then returns
+``ERR_DEVICE_TIMEOUT``) the rows that the thread block had not written hold whatever the memory held before, not zeros.
 
 Tensors follow the header's layouts: K/V ``[B,T,H,d]`` (bf16 or fp32), beta/g
 ``[B,T,H]`` fp32, A ``[B,T,H,C]`` fp32, W/U like K/V.  All must be contiguous

@@ -318,7 +318,9 @@ int chunk_scan_any(const void* Q, const void* K, const void* W, const void* U, c
       err = launch_chunk_scan(p, Qp, Km, W, tokens, stream, true);
     }
   } else {
-    // fp32 with a scalar gate has register-tiled products at the chunk size and key dimensions it keeps on chip
+    // fp32 with a scalar gate has register-tiled products at the chunk size and key dimensions it keeps on chip.  d_k is padded
+    // to 64 or 128 there, which pays at small d_k too (16 chunks, against the general kernel): d_k = d_v = 8, 2 / 256 pairs
+    // 404 -> 107 / 527 -> 175 us; 32: 862 -> 107 / 1302 -> 359 us; least with many narrow slices, d_k = 8, d_v = 128, 256 pairs: 1477 -> 1241 us.
     const bool f32 = !G && desc->kv_dtype == TRI_INV_F32 && desc->C == 64 && desc->d_k <= 128;
     err = (tc && !G) ? launch_chunk_scan(p, Q, K, W, tokens > 0 ? tokens : 1, stream)
           : f32      ? launch_chunk_scan_f32(p, Q, K, W, desc->d_k, desc->d_v, stream)

@@ -90,7 +90,7 @@ __device__ __forceinline__ float load_kv(const void* base, int dtype, size_t idx
 cudaError_t launch_simt(const KParams& p, int C, cudaStream_t stream);
 // Tensor-core path: returns cudaErrorNotSupported when it has no kernel for the request.
 cudaError_t launch_tc(const KParams& p, int C, cudaStream_t stream, bool* handled);
-// Instantiations of the tensor-core kernel, one group per tc_inst_*.cu file; raw = the variant that rewrites the K tile.
+// Instantiations of the tensor-core kernel, one group per tc_inst_*.cu file; raw = with a factor on each row of the keys (front end, decay-weighted W).
 cudaError_t launch_tc_c64_br(const KParams& p, cudaStream_t stream, bool raw);
 cudaError_t launch_tc_c64_series(const KParams& p, cudaStream_t stream, bool raw);
 cudaError_t launch_tc_c64_build(const KParams& p, cudaStream_t stream);

@@ -313,7 +313,7 @@ __global__ void __launch_bounds__(kThreads, BLOCKS) simt_kernel(KParams p) {
         constexpr int kLeaf = C < 16 ? C : 16;
         if (p.method & TRI_INV_LEAF_SERIES) {
           // Alg. 2: series on the leaves.  Work on a copy so N's off-diagonal blocks survive.
-          // Ks ([C][33]) is free now and holds two compact [C][16] block-diagonal matrices.
+          // Ks ([C][kSliceLd]) is free now and holds two compact [C][16] block-diagonal matrices.
           float* Yc = Ks;
           float* Y2 = Ks + C * kLeaf;
           for (int e = tid; e < C * kLeaf; e += kThreads) {

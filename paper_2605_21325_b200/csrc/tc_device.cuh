@@ -426,11 +426,10 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t saddr, uint32_t lbo_bytes
 __host__ __device__ constexpr uint32_t umma_idesc(int M, int N, int b_mn) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)b_mn << 16) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
-// tcgen05.mma and its commit are called by a whole, converged warp; one elected lane issues.  The operands of the instruction
-// are uniform registers: in code that the compiler knows to be uniform (the warp index from a shuffle, descriptors built from
-// shared-memory addresses) they are computed there, while a branch of one lane has to move them there for every
-// instruction, 67 cycles each whatever the shape.  Measured, one CTA: 8 instructions of 128 x 64 x 16 take 546 cycles to issue and
-// 658 until completion is seen from one lane, 45 and 333 from a warp; 8 of 64 x 64 x 16: 577 and 689, 95 and 370.
+// tcgen05.mma and its commit are called by a whole, converged warp from code that the compiler knows to be uniform (the warp
+// index from a shuffle, descriptors built from shared-memory addresses); one elected lane issues.  Measured, one CTA, against
+// a branch of one lane: 8 instructions of 128 x 64 x 16 take 546 cycles to issue and 658 until completion is seen from one lane,
+// 45 and 333 from a warp; 8 of 64 x 64 x 16: 577 and 689, 95 and 370 -- from one lane 67 to 72 cycles each, whatever the shape.
 __device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %4, 0;\n\telect.sync _|q, 0xffffffff;\n\t"
@@ -493,12 +492,6 @@ __device__ __forceinline__ void tmem_ld_16x32(float (&r)[4][4], uint32_t taddr) 
         "=f"(r[2][0]), "=f"(r[2][1]), "=f"(r[2][2]), "=f"(r[2][3]), "=f"(r[3][0]), "=f"(r[3][1]), "=f"(r[3][2]), "=f"(r[3][3])
       : "r"(taddr));
 }
-// 16 lanes x 16 columns -> 2 n-tiles of accumulator fragments.
-__device__ __forceinline__ void tmem_ld_16x16(float (&r)[2][4], uint32_t taddr) {
-  asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=f"(r[0][0]), "=f"(r[0][1]), "=f"(r[0][2]), "=f"(r[0][3]), "=f"(r[1][0]), "=f"(r[1][1]), "=f"(r[1][2]), "=f"(r[1][3])
-               : "r"(taddr));
-}
 // 16 lanes x 128 columns -> 16 n-tiles of accumulator fragments.
 __device__ __forceinline__ void tmem_ld_16x128(float (&r)[16][4], uint32_t taddr) {
   asm volatile(
@@ -524,11 +517,6 @@ __device__ __forceinline__ void tmem_st_16x32(const float (&r)[4][4], uint32_t t
         "f"(r[2][0]), "f"(r[2][1]), "f"(r[2][2]), "f"(r[2][3]), "f"(r[3][0]), "f"(r[3][1]), "f"(r[3][2]), "f"(r[3][3]),
         "r"(taddr)
       : "memory");
-}
-__device__ __forceinline__ void tmem_st_16x16(const float (&r)[2][4], uint32_t taddr) {
-  asm volatile("tcgen05.st.sync.aligned.16x256b.x2.b32 [%8], {%0,%1,%2,%3,%4,%5,%6,%7};"
-               ::"f"(r[0][0]), "f"(r[0][1]), "f"(r[0][2]), "f"(r[0][3]), "f"(r[1][0]), "f"(r[1][1]), "f"(r[1][2]), "f"(r[1][3]), "r"(taddr)
-               : "memory");
 }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void stmatrix_x4(uint32_t addr, uint32_t m0, uint32_t m1, uint32_t m2, uint32_t m3) {

@@ -6,7 +6,7 @@
 //      memory on separate mbarriers; the next item's tiles are prefetched into L2 an item ahead and
 //      copied as soon as a buffer's last reader has finished; beta and g travel one item ahead in a register.
 //   2. Gram S = K K^T: tcgen05.mma (kind::f16, bf16 operands straight from the TMA-written tile,
-//      fp32 accumulator in tensor memory), issued by one thread, completion through an mbarrier.
+//      fp32 accumulator in tensor memory), issued by warp 0 (build only: by its first lane), completion through an mbarrier.
 //   3. Each warp reads its 16 rows of S from tensor memory (tcgen05.ld 16x256b: the m16n8 accumulator
 //      fragment layout), applies gate + strict-lower mask, writes N to shared memory in fp32.
 //   4. Block recursion (Sec. 3.3): 16x16 leaves by forward substitution, one lane per column (Sec. 3.1),
@@ -96,8 +96,8 @@ struct Cfg {
 //
 // The factors of VAR 4 sit in the operand, not in the keys: W = (A diag(beta exp g)) K takes an operand A'' of its own, written
 // beside A' where the output staging will be (W is staged only after the product that reads A'' has completed).  That is 8 KB
-// of shared-memory stores; weighting the K tile's rows instead, as the RAW variant does, reads and writes 16 KB, takes a
-// barrier for the row factors in the gate and rounds to bf16 twice.  Without A wanted
+// of shared-memory stores; weighting the K tile's rows instead, as the RAW instances of the other schemes and of C = 128 do, reads
+// and writes 16 KB, takes a barrier for the row factors in the gate and rounds to bf16 twice.  Without A wanted
 // (L2 flushed): B = 4, T = 4096, H = 16: 80.4 -> 67.6 us; B = 1, T = 32768, H = 32: 261 -> 223 us; 64 packed sequences of up
 // to 2048 tokens, H = 16: 285 -> 240 us.
 template <int C, int D, bool SER, bool RAW, bool BO, bool REF, bool H16, int VAR>
@@ -170,8 +170,8 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
   const bool need_v = do_wy && p.V != nullptr;
   const bool load_a = VAR == 3 ? (p.ops & kLoadA) != 0 : VAR == 2;
   const bool leaf_series_on = (VAR == 3 || (VAR == 4 && RAW)) ? (p.method & TRI_INV_LEAF_SERIES) != 0 : VAR == 1;
-  // RAW compiles in the code that rewrites the K tile in shared memory before the WY step and the per-row
-  // factors of the gate.  Two run-time uses: the front end (sigmoid, log-sigmoid + chunk cumsum, key
+  // RAW compiles in the row factors of the keys and, but for VAR 4, the code that rewrites the K tile in shared memory with
+  // them before the WY step.  Two run-time uses: the front end (sigmoid, log-sigmoid + chunk cumsum, key
   // normalisation: kRaw) and the decay-weighted W (rows of K times exp(g_i): kWDecay).
   constexpr bool raw = RAW;
   const bool front = RAW && (p.ops & kRaw) != 0;
@@ -428,7 +428,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
     if (BO && has_next) bg_next = fetch_bg(nx_tok0, nx_rows, nx_h);
 
     if (!load_a) {
-      // ---- 2. Gram S = K K^T on the tensor core: one thread issues D/16 MMAs of C x C x 16 into TMEM
+      // ---- 2. Gram S = K K^T on the tensor core: the issuer's D/16 MMAs of C x C x 16 into TMEM
       if (issuer && !gram_early) {
         // self-test (kTestStall): CTA 0 leaves out the Gram product of its first item, so the wait below runs out
         const bool stall = (p.ops & kTestStall) && item == 0;

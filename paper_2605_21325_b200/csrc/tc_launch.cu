@@ -75,7 +75,7 @@ cudaError_t launch_tc(const KParams& p, int C, cudaStream_t stream, bool* handle
   const bool series = (p.method & TRI_INV_METHOD_MASK) == TRI_INV_PRODUCT_SERIES;
   if ((p.method & TRI_INV_METHOD_MASK) == TRI_INV_NEWTON_SCHULZ) return cudaSuccess;   // CUDA-core kernel only
   if (C != 64 && C != 128) return cudaSuccess;
-  const bool raw = (p.ops & (kRaw | kWDecay)) != 0;  // both need the variant that rewrites the K tile
+  const bool raw = (p.ops & (kRaw | kWDecay)) != 0;  // both put a factor on each row of the keys
   if (p.d_k == 64 && C == 64 && !series && !raw && !(p.method & (TRI_INV_REFINE | TRI_INV_OPERANDS_F16)) &&
       !((p.ops & kDoWY) && p.V && p.d_v != 64)) {
     // head dimension 64: block recursion (and series leaves) of the plain calls; everything else stays on the CUDA cores
