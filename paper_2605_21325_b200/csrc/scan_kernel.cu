@@ -32,11 +32,12 @@
 // inside the loop: one in flight would make its next tensor-memory load wait for it too.
 // What bounds it: with few (sequence, head) pairs the latencies of the chain (a chunk of 32 columns: P1 420 cycles, U~' 330, P3
 // 410, S^T 310 and the hand-overs between them: about 1,850), with more pairs than SMs the bytes.  Measured (L2 flushed)
-// against the form that kept the operands in shared memory, S as columns and issued from one lane: B = 4, T = 4096, H = 16:
-// 110 -> 84 us; B = 1, T = 32768, H = 32: 743 -> 505 .. 537 us (two boxes); 64 packed sequences of up to 2048 tokens, H = 16: 416 -> 265 us (0.9 of
-// the copy bandwidth on 82 KB per chunk and head).  Not kept: Q K^T as mma.sync in the output warps (they get what tcgen05.mma
-// leaves: 810 us on the second shape), K in P1's free lanes instead of a product of its own (the output warps become the
-// bound: 689 us, before the issue by a whole warp), eight output warps (no gain, more contention: 532 us).
+// against the form that kept the operands in shared memory, S as columns and issued from one lane, over several boxes: B = 4, T = 4096,
+// H = 16: 110 -> 78 .. 86 us; B = 1, T = 32768, H = 32: 743 -> 542 us; 64 packed sequences of up to 2048 tokens, H = 16: 416 -> 262 .. 290 us
+// (0.82 .. 0.9 of the copy bandwidth on 82 KB per chunk and head).  Not kept, on the second shape in slices of 32 columns (505 us with L2
+// flushed then): Q K^T as mma.sync in the output warps (they get what tcgen05.mma leaves: 810 us), K in P1's free lanes instead
+// of a product of its own (the output warps become the bound: 689 us, before the issue by a whole warp), eight output warps
+// (no gain, more contention: 532 us).
 // Every mbarrier wait is bounded; on expiry the CTA raises the status word, frees its tensor memory and returns.
 #include "tc_device.cuh"
 
@@ -779,11 +780,13 @@ cudaError_t launch_seq_offsets(int* dev_out, const tri_inv_desc* d, cudaStream_t
 
 // bf16 Q, K, W, U with d_k = d_v = 128 and C = 64.  One CTA per SM walks a (sequence, head) pair or a slice of its value
 // columns.  A pair is cut into four slices of 32 columns while that takes half the SMs at most, into two of 64 while every
-// slice gets an SM of its own: the steps between the products get shorter with the slice.  (32 pairs in 128 CTAs of 32 columns
-// run at 1000 W, under the power cap, at 1.69 GHz: 583 us back to back; in 64 CTAs of 64 columns at 1.97 GHz: 548 us.)
-// With more pairs than that a CTA takes all 128 columns: the
-// products take the same time at any slice width, so each further slice would repeat them (64 packed sequences x 16 heads:
-// 265 us with 128 columns, 416 us in slices of 64 before).
+// slice gets an SM of its own: the steps between the products get shorter with the slice (512 chunks, 18 pairs, one launch:
+// 498 us in slices of 32, 545 in slices of 64, 764 in one).  The first line keeps clear of the power cap, which 128 CTAs of 32 columns
+// reach back to back (512 chunks, 32 pairs: one launch 529 against 541 us in slices of 64, back to back 574 at 1.78 GHz against
+// 538 at 1.97 GHz; 37 pairs 612 against 541); from 19 to about 28 pairs the narrow slices do not reach it and would be 6 to 9 %
+// faster than what is taken (24 pairs: 500 against 542).  With more pairs than half the SMs a CTA takes all 128 columns: the
+// products take the same time at any slice width, so each further slice would repeat them in a second wave (64 chunks: 74 pairs
+// 79.9 us in slices of 64, 113 in one; 75 pairs 148 and 113).
 // kda selects the per-channel form: Q, K are then the prepared operands Q+, K- (scan_kda_prep.cu), with p.EL,
 // p.ER, p.EX the per-chunk vectors.
 cudaError_t launch_chunk_scan(const ScanParams& p, const void* Q, const void* K, const void* W, long long tokens,
