@@ -253,7 +253,8 @@ int tri_inv_chunk_scan_kda(const void* Q, const void* K, const void* W, const vo
  * o_t = scale S^T q_t.
  *   Q, K, W [B,T,H,d_k], U [B,T,H,d_v]: device, desc->kv_dtype, 16-byte aligned;  g [B,T,H] fp32 device;
  *   S0, S_out [n_sequences,H,d_k,d_v] fp32 device, each may be NULL (zero initial state / final state not wanted);
- *   O [B,T,H,d_v] device, desc->kv_dtype: rows of real tokens are written.
+ *   O [B,T,H,d_v] device, desc->kv_dtype: rows of real tokens are written; it may not overlap Q, K or W, which other
+ *   thread blocks of the same head may still have to read.
  * Dense and ragged chunking as in tri_inv_build (desc->cu_seqlens on the HOST).  bf16 with d_k = d_v = 128 and
  * C = 64 runs on the tensor cores; every other shape and fp32 storage run on the CUDA cores in fp32 (d_k <= 256,
  * else TRI_INV_ERR_UNSUPPORTED).  g is used as given (it need not decrease); the tensor-core path forms exp(g_i - g_j)

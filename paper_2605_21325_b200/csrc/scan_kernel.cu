@@ -32,7 +32,7 @@
 // inside the loop: one in flight would make its next tensor-memory load wait for it too.
 // What bounds it: with few (sequence, head) pairs the latencies of the chain (a chunk of 32 columns: P1 420 cycles, U~' 330, P3
 // 410, S^T 310 and the hand-overs between them: about 1,850), with more pairs than SMs the bytes.  Measured (L2 flushed)
-// against the form that kept the operands in shared memory, S as columns and issued from one lane, over several boxes: B = 4, T = 4096,
+// against the form that kept the operands in shared memory, S as columns and issued from one lane, over several GPUs: B = 4, T = 4096,
 // H = 16: 110 -> 78 .. 86 us; B = 1, T = 32768, H = 32: 743 -> 542 us; 64 packed sequences of up to 2048 tokens, H = 16: 416 -> 262 .. 290 us
 // (0.82 .. 0.9 of the copy bandwidth on 82 KB per chunk and head).  Not kept, on the second shape in slices of 32 columns (505 us with L2
 // flushed then): Q K^T as mma.sync in the output warps (they get what tcgen05.mma leaves: 810 us), K in P1's free lanes instead
