@@ -260,8 +260,10 @@ int tri_inv_chunk_scan_kda(const void* Q, const void* K, const void* W, const vo
  * else TRI_INV_ERR_UNSUPPORTED).  g is used as given (it need not decrease); the tensor-core path forms exp(g_i - g_j)
  * as a product of two factors around the first token of j's block of eight, so g may vary by at most about 88
  * inside eight consecutive tokens of a chunk.  Launch is asynchronous on
- * cuda_stream; nothing is allocated except, in ragged mode, n_sequences + 1 ints from the library's
- * stream-ordered pool.  A device-side wait that expires raises TRI_INV_ERR_DEVICE_TIMEOUT in the status word.
+ * cuda_stream; nothing is allocated except, from the library's stream-ordered pool, n_sequences + 1 ints in ragged mode, and at
+ * most 128 MiB of scratch (more only if a single chunk of every sequence and head needs it) for fp32 storage with C = 64 and
+ * d_k <= 128, where longer inputs go through in segments; if that scratch cannot be had, the kernel of the other shapes
+ * takes the call.  A device-side wait that expires raises TRI_INV_ERR_DEVICE_TIMEOUT in the status word.
  */
 int tri_inv_chunk_scan(const void* Q, const void* K, const void* W, const void* U, const float* g, const float* S0,
                        void* O, float* S_out, float scale, const tri_inv_desc* desc, void* cuda_stream);

@@ -289,15 +289,15 @@ int chunk_scan_any(const void* Q, const void* K, const void* W, const void* U, c
     }
     p.seq_off = dev_off;
   }
+  int max_len = desc->T;   // of the sequences
+  if (desc->cu_seqlens) {
+    max_len = 0;
+    for (int q = 0; q < desc->n_seqs; ++q) max_len = std::max(max_len, desc->cu_seqlens[q + 1] - desc->cu_seqlens[q]);
+  }
   void* work = nullptr;
   if (tc && G && tokens > 0) {
     // Per-channel gate on the tensor cores: Q+, K- (bf16, the tensors' own shape) and the per-chunk vectors
     // exp(G_last), exp(G_ref), exp(G_last - G_ref), in stream-ordered scratch memory that is released behind the scan.
-    int max_len = desc->T;
-    if (desc->cu_seqlens) {
-      max_len = 0;
-      for (int q = 0; q < desc->n_seqs; ++q) max_len = std::max(max_len, desc->cu_seqlens[q + 1] - desc->cu_seqlens[q]);
-    }
     const size_t tensor_bytes = ((size_t)tokens * desc->H * 128 * 2 + 255) & ~(size_t)255;
     const size_t slots = (size_t)(tokens / 64) + (size_t)p.n_seqs + 1;
     const size_t vec_bytes = (slots * desc->H * 128 * sizeof(float) + 255) & ~(size_t)255;
@@ -318,13 +318,23 @@ int chunk_scan_any(const void* Q, const void* K, const void* W, const void* U, c
       err = launch_chunk_scan(p, Qp, Km, W, tokens, stream, true);
     }
   } else {
-    // fp32 with a scalar gate has register-tiled products at the chunk size and key dimensions it keeps on chip.  d_k is padded
-    // to 64 or 128 there, which pays at small d_k too (16 chunks, against the general kernel): d_k = d_v = 8, 2 / 256 pairs
-    // 404 -> 107 / 527 -> 175 us; 32: 862 -> 107 / 1302 -> 359 us; least with many narrow slices, d_k = 8, d_v = 128, 256 pairs: 1477 -> 1241 us.
     const bool f32 = !G && desc->kv_dtype == TRI_INV_F32 && desc->C == 64 && desc->d_k <= 128;
-    err = (tc && !G) ? launch_chunk_scan(p, Q, K, W, tokens > 0 ? tokens : 1, stream)
-          : f32      ? launch_chunk_scan_f32(p, Q, K, W, desc->d_k, desc->d_v, stream)
-                     : launch_chunk_scan_simt(p, Q, K, W, desc->d_k, desc->d_v, desc->C, desc->kv_dtype, stream);
+    if (f32) {
+      int n_seg = 0;
+      const int max_chunks = (max_len + 63) / 64;
+      const size_t bytes = chunk_scan_f32_scratch((long long)p.n_seqs * p.H, max_chunks, desc->d_k, desc->d_v, &n_seg);
+      cudaMemPool_t pool = table_pool_for_current_device();
+      if (pool && cudaMallocFromPoolAsync(&work, bytes, pool, stream) == cudaSuccess) {
+        err = launch_chunk_scan_f32(p, Q, K, W, desc->d_k, desc->d_v, max_chunks, work, n_seg, stream);
+      } else {   // no scratch to be had: the kernel that needs none
+        (void)cudaGetLastError();
+        work = nullptr;
+        err = launch_chunk_scan_simt(p, Q, K, W, desc->d_k, desc->d_v, desc->C, desc->kv_dtype, stream);
+      }
+    } else {
+      err = (tc && !G) ? launch_chunk_scan(p, Q, K, W, tokens > 0 ? tokens : 1, stream)
+                       : launch_chunk_scan_simt(p, Q, K, W, desc->d_k, desc->d_v, desc->C, desc->kv_dtype, stream);
+    }
   }
   if (err == cudaSuccess) g_launches.fetch_add(1, std::memory_order_relaxed);
   if (work) cudaFreeAsync(work, stream);

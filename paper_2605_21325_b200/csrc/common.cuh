@@ -128,7 +128,10 @@ cudaError_t launch_chunk_scan(const ScanParams& p, const void* Q, const void* K,
 cudaError_t launch_kda_scan_prep(const ScanParams& p, const void* Q, const void* K, void* Qp, void* Km,
                                  float* EL, float* ER, float* EX, int max_chunks_per_seq, cudaStream_t stream);
 // Single precision with a scalar gate at C = 64 and d_k <= 128 (scan_f32_kernel.cu).
-cudaError_t launch_chunk_scan_f32(const ScanParams& p, const void* Q, const void* K, const void* W, int d_k, int d_v, cudaStream_t stream);
+// Its scratch for this many (sequence, head) pairs and chunks of the longest sequence; *n_seg: chunks that go through at a time.
+size_t chunk_scan_f32_scratch(long long pairs, int max_chunks, int d_k, int d_v, int* n_seg);
+cudaError_t launch_chunk_scan_f32(const ScanParams& p, const void* Q, const void* K, const void* W, int d_k, int d_v, int max_chunks,
+                                  void* scratch, int n_seg, cudaStream_t stream);
 // The same scan on the CUDA cores, for every other shape and storage type (fp32 arithmetic).
 cudaError_t launch_chunk_scan_simt(const ScanParams& p, const void* Q, const void* K, const void* W, int d_k, int d_v, int C,
                                    int kv_dtype, cudaStream_t stream);

@@ -1,34 +1,28 @@
 // Chunk scan in single precision (fp32 storage, scalar gate, C = 64, d_k <= 128): the chunk form of scan_kernel.cu with
-// every product as FFMA on register tiles.  One CTA of 256 threads per (sequence, head, slice of 16 value columns) walks
-// the chunks in order; the slice of the state S [d_k][16] stays in shared memory.  Per chunk:
-//   1. [W ; Q] S          thread: row r of both, four columns          U~ = U - W S to shared memory (plain and times
-//                                                                      exp(g_last - g_r)), Q S kept in registers
-//   2. P = (Q K^T) decay  thread: element (ty, tx) of the ten 16 x 16 blocks on and below the diagonal
-//   3. O = scale (gamma Q S + P U~)    thread: row r, four columns (those of its Q S)
-//   4. S = gamma_last S + K^T (decayed U~)   thread: four features x four columns, tokens split over JG lanes that then
-//                                            exchange their partial sums (reduce-scatter by shuffles)
-// What bounds it: shared-memory wavefronts against FFMA issue.  All operands are read 16 bytes at a time along the
-// summed index, rows 4 words apart in banks (row length d_k + 4; U~ rows of 24 words), 6 loads per 32 FMAs in step 1,
-// 8 per 40 in step 2.  The tiles of W, U, Q and K are single; each is refilled (cp.async) for the next chunk as soon as
-// its last reader of this one is done, so a copy has two or three of the four steps to land.
-// Measured (L2 flushed): B = 2, T = 2048, H = 8, d = 64: 3340 us with scan_simt_kernel (one element per thread, operands
-// from global memory), 216 us here.
-// A CTA of 16 columns repeats step 2 for each slice of a head; wider slices would leave more of the chip idle at the
-// (sequence, head) counts that fp32 is used with.
+// every product as FFMA on register tiles, in two kernels, so that only what the state depends on runs chunk after chunk:
+//   scan_f32_chain    one CTA per (sequence, head, slice of NS value columns) walks the chunks:
+//                       U~ = U - W S,   S <- gamma_last S + K^T (exp(g_last - g) U~),
+//                     and leaves U~ and the state that ENTERS each chunk in scratch memory.
+//   scan_f32_output   one CTA per (sequence, head, chunk, 64 value columns), all chunks at once:
+//                       P = (Q K^T) decay,   O = scale (gamma Q S + P U~).
+// The scratch of a call is bounded (kScratchBytes): longer inputs go through in segments of chunks, a pair of launches each,
+// the state carried in scratch between them.
+//
+// What bounds the chain: latency.  Its two products are 64 x NS x d_k and d_k x NS x 64 (32 K FMAs each at 8 columns, d_k = 64);
+// a thread holds a 4 x 4 tile of the result for one of KS parts of the summed index and the parts are joined by a
+// reduce-scatter of shuffles, so that all 256 threads work on so small a result.  16-byte shared-memory loads (8 per 64 FMAs), rows laid
+// out so that the eight lanes of a load step fall into different banks; W and K come by cp.async two chunks
+// ahead, U and g into registers one chunk ahead; the thread's part of S stays in registers beside its shared copy.
+// The output kernel is bound by FFMA issue and shared-memory loads (8 per 64 FMAs).
+// Measured (ncu, B = 2, T = 2048, H = 8, d = 64: 16 pairs of 32 chunks): 50 + 28 us; 213 us as one kernel per slice of 16 columns that also
+// formed P and O on the way (P again in each slice, all of it on the chain, 64 CTAs); the layer 262 -> 127 us.
 #include "common.cuh"
 
 namespace tri_inv {
 namespace {
 
-constexpr int kThreads = 256, kC = 64, kNS = 16, kLdP = kC + 4, kLdU = 24;
-
-template <int DK>
-struct F32Scan {
-  static constexpr int LD = DK + 4;
-  static constexpr int JG = DK == 64 ? 4 : 2;                 // token groups of step 4: (DK / 4) x 4 x JG threads
-  static constexpr int floats = 3 * kC * LD + kC * kNS + DK * kNS + 2 * kC * kLdU + kC * kLdP + 2 * kC;
-  static constexpr size_t bytes = floats * sizeof(float);
-};
+constexpr int kThreads = 256, kC = 64, kLdP = kC + 4, kNV = 64;   // kNV: value columns of an output CTA
+constexpr size_t kScratchBytes = (size_t)128 << 20;
 
 __device__ __forceinline__ void cp_async16(float* dst, const float* src, bool valid) {   // 16 bytes, zeros where not valid
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(valid ? 16 : 0) : "memory");
@@ -44,218 +38,360 @@ __device__ __forceinline__ void fma4(float (&acc)[4], float a, const float4& b) 
 struct F32Args {
   const float *Q, *K, *W, *U;
   int d_k, d_v;
+  float* slots;          // per (pair, chunk of the segment): the state that enters the chunk [d_k][d_v], then U~ [64][d_v]
+  float* carry;          // per pair: the state between segments [d_k][d_v]; unused with one segment
+  int c0, n_seg;         // this segment: chunks c0 .. c0 + n_seg - 1 of every sequence
+};
+__device__ __forceinline__ size_t slot_floats(const F32Args& a) { return (size_t)(a.d_k + kC) * a.d_v; }
+
+// rows of a [tokens, H, d] tensor into a tile of row length LD; rows past the sequence's end and columns past d become zeros
+template <int DK, int LD>
+__device__ __forceinline__ void copy_rows(float* dst, const float* src, int tok0, int rows, int H, int h, int d, int tid) {
+  constexpr int Q4 = DK / 4;
+#pragma unroll
+  for (int m = 0; m < kC * Q4 / kThreads; ++m) {
+    const int e = tid + m * kThreads, j = e / Q4, c = 4 * (e % Q4);
+    const bool ok = j < rows && c < d;
+    cp_async16(dst + j * LD + c, src + (ok ? ((size_t)(tok0 + j) * H + h) * d + c : 0), ok);
+  }
+}
+
+// The sum of v over KS neighbouring lanes, scattered: each lane keeps 16 / KS consecutive ones of the 16 values, from the
+// returned index on.
+template <int KS>
+__device__ __forceinline__ int reduce_scatter(float (&v)[16], int ks) {
+  int base = 0;
+#pragma unroll
+  for (int m = KS / 2, n = 8; m >= 1; m >>= 1, n >>= 1) {
+    const bool up = ks & m;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      if (i < n) {
+        const float give = up ? v[i] : v[n + i], keep = up ? v[n + i] : v[i];
+        v[i] = keep + __shfl_xor_sync(0xffffffffu, give, m);
+      }
+    }
+    base += up ? n : 0;
+  }
+  return base;
+}
+
+template <int DK, int NS>
+struct Chain {
+  static constexpr int LD = DK + 4;                       // row length of the W and K tiles
+  static constexpr int NG = NS / 4;                       // groups of four columns
+  static constexpr int KA = kThreads / (kC / 4 * NG);     // parts of the summed index: of W S (features) ...
+  static constexpr int KB = kThreads / (DK / 4 * NG);     // ... and of K^T U~ (tokens)
+  static_assert(KA >= 2 && KB >= 2 && KA <= 8 && KB <= 8, "a tile's parts lie in one warp");
+  static constexpr int S_BLK = 4 * NS + (NS == 8 ? 4 : 8);   // four features of S and padding: neighbouring parts in different banks
+  static constexpr int LDU = KB == 8 ? 12 : KB == 4 ? 24 : 16;   // row length of the decayed U~, for the same reason
+  static_assert(LDU >= NS, "a row of U~");
+  static constexpr int kStages = DK == 64 ? 3 : 2;
+  static constexpr int TILE = kC * LD;
+  static constexpr int floats = kStages * 2 * TILE + (DK / 4) * S_BLK + kC * LDU;
+  static constexpr size_t bytes = floats * sizeof(float);
+};
+
+template <int DK, int NS>
+__global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) scan_f32_chain(ScanParams p, F32Args a) {
+  using cfg = Chain<DK, NS>;
+  constexpr int LD = cfg::LD, KA = cfg::KA, KB = cfg::KB, NG = cfg::NG, VA = 16 / KA, VB = 16 / KB;
+  extern __shared__ __align__(16) float sm[];
+  float *tiles = sm, *S = sm + cfg::kStages * 2 * cfg::TILE, *Ud = S + (DK / 4) * cfg::S_BLK;
+  const int tid = threadIdx.x;
+  const int n_slices = (a.d_v + NS - 1) / NS;
+  const int slice = blockIdx.x % n_slices, pair = blockIdx.x / n_slices, h = pair % p.H, s = pair / p.H;
+  const int beg = p.seq_off ? p.seq_off[s] : s * p.T;
+  const int end = p.seq_off ? p.seq_off[s + 1] : (s + 1) * p.T;
+  const int n_all = (end - beg + kC - 1) / kC;
+  const int n_chunks = n_all - a.c0 < a.n_seg ? n_all - a.c0 : a.n_seg;   // of this segment
+  if (n_chunks <= 0 && a.c0 > 0) return;
+  const int col0 = slice * NS;
+  const size_t state_base = (size_t)pair * a.d_k * a.d_v;
+
+  // this thread's results: VA neighbouring columns of a row of U~, VB neighbouring columns of a feature of S
+  const int ka = tid & (KA - 1), cga = (tid / KA) % NG, rg = tid / (KA * NG);
+  const int kb = tid & (KB - 1), cgb = (tid / KB) % NG, fg = tid / (KB * NG);
+  auto base_of = [](int ks, int KS) {   // as reduce_scatter returns it
+    int b = 0;
+    for (int m = KS / 2, n = 8; m >= 1; m >>= 1, n >>= 1) b += (ks & m) ? n : 0;
+    return b;
+  };
+  const int ba = base_of(ka, KA), bb = base_of(kb, KB);
+  const int row = 4 * rg + ba / 4, ucol = 4 * cga + (ba & 3);       // VA = 2 or 4 columns from ucol on (VA = 8 does not occur)
+  const int feat = 4 * fg + bb / 4, scol = 4 * cgb + (bb & 3);      // VB = 8: two features of four columns
+  static_assert(VA <= 4 && VB <= 8, "layout of a thread's results");
+  const bool ucol_in = col0 + ucol < a.d_v, scol_in = col0 + scol < a.d_v;
+
+  float Sr[VB];
+  auto for_state = [&](auto&& f) {   // (value, feature, column of the slice)
+#pragma unroll
+    for (int i = 0; i < VB; ++i) f(Sr[i], feat + i / 4, VB == 8 ? scol + (i & 3) : scol + i);
+  };
+  const float* src = a.c0 > 0 ? a.carry : p.S0;
+  for_state([&](float& x, int k, int n) { x = (src && k < a.d_k && scol_in) ? src[state_base + (size_t)k * a.d_v + col0 + n] : 0.f; });
+  auto put_state = [&](float* dst) {   // to a [d_k][d_v] matrix in global memory
+    for_state([&](float& x, int k, int n) { if (k < a.d_k && scol_in) dst[(size_t)k * a.d_v + col0 + n] = x; });
+  };
+  if (n_chunks <= 0) {
+    if (p.S_out) put_state(p.S_out + state_base);
+    return;
+  }
+  auto share_state = [&]() {
+    for_state([&](float& x, int k, int n) { S[(k >> 2) * cfg::S_BLK + (k & 3) * NS + n] = x; });
+  };
+  auto rows_of = [&](int c) { const int left = end - beg - (a.c0 + c) * kC; return left < kC ? left : kC; };
+  auto copy_tiles = [&](int c) {
+    float* t = tiles + (c % cfg::kStages) * 2 * cfg::TILE;
+    const int tok0 = beg + (a.c0 + c) * kC, rows = rows_of(c);
+    copy_rows<DK, LD>(t, a.W, tok0, rows, p.H, h, a.d_k, tid);
+    copy_rows<DK, LD>(t + cfg::TILE, a.K, tok0, rows, p.H, h, a.d_k, tid);
+  };
+  // this thread's elements of U and its row's decay exp(g_last - g_row), and gamma_last, of a chunk
+  float u_next[VA], g_row, g_last;
+  auto fetch = [&](int c) {
+    const int tok0 = beg + (a.c0 + c) * kC, rows = rows_of(c);
+#pragma unroll
+    for (int i = 0; i < VA; ++i)
+      u_next[i] = (row < rows && ucol_in) ? a.U[((size_t)(tok0 + row) * p.H + h) * a.d_v + col0 + ucol + i] : 0.f;
+    g_row = p.g[(size_t)(tok0 + (row < rows ? row : rows - 1)) * p.H + h];
+    g_last = p.g[(size_t)(tok0 + rows - 1) * p.H + h];
+  };
+
+  for (int c = 0; c < cfg::kStages - 1; ++c) {
+    if (c < n_chunks) copy_tiles(c);
+    cp_commit();
+  }
+  fetch(0);
+  share_state();
+  float* slot = a.slots + (size_t)pair * a.n_seg * slot_floats(a);
+  put_state(slot);
+  for (int c = 0; c < n_chunks; ++c) {
+    const int rows = rows_of(c);
+    const float* Ws = tiles + (c % cfg::kStages) * 2 * cfg::TILE;
+    const float* Ks = Ws + cfg::TILE;
+    float u[VA];
+#pragma unroll
+    for (int i = 0; i < VA; ++i) u[i] = u_next[i];
+    const float f = expf(g_last - g_row), gl = expf(g_last);
+    cp_wait<cfg::kStages - 2>();   // this chunk's tiles
+    __syncthreads();               // S in place; the last chunk's tiles have been read
+    if (c + cfg::kStages - 1 < n_chunks) copy_tiles(c + cfg::kStages - 1);
+    cp_commit();
+    if (c + 1 < n_chunks) fetch(c + 1);
+    // ---- U~ = U - W S
+    {
+      float acc[4][4] = {};
+      const float *w0 = Ws + 4 * rg * LD + 4 * ka, *s0 = S + ka * cfg::S_BLK + 4 * cga;
+#pragma unroll
+      for (int i = 0; i < DK / 4 / KA; ++i) {
+        const int k = 4 * KA * i;
+        const float4 x0 = ld4(w0 + k), x1 = ld4(w0 + LD + k), x2 = ld4(w0 + 2 * LD + k), x3 = ld4(w0 + 3 * LD + k);
+        const float* sb = s0 + KA * i * cfg::S_BLK;
+        const float4 y0 = ld4(sb), y1 = ld4(sb + NS), y2 = ld4(sb + 2 * NS), y3 = ld4(sb + 3 * NS);
+        fma4(acc[0], x0.x, y0); fma4(acc[1], x1.x, y0); fma4(acc[2], x2.x, y0); fma4(acc[3], x3.x, y0);
+        fma4(acc[0], x0.y, y1); fma4(acc[1], x1.y, y1); fma4(acc[2], x2.y, y1); fma4(acc[3], x3.y, y1);
+        fma4(acc[0], x0.z, y2); fma4(acc[1], x1.z, y2); fma4(acc[2], x2.z, y2); fma4(acc[3], x3.z, y2);
+        fma4(acc[0], x0.w, y3); fma4(acc[1], x1.w, y3); fma4(acc[2], x2.w, y3); fma4(acc[3], x3.w, y3);
+      }
+      float v[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) v[i] = acc[i / 4][i & 3];
+      reduce_scatter<KA>(v, ka);
+      float* ut = slot + (size_t)a.d_k * a.d_v + (size_t)row * a.d_v + col0 + ucol;
+#pragma unroll
+      for (int i = 0; i < VA; ++i) {
+        const float x = row < rows ? u[i] - v[i] : 0.f;
+        if (ucol_in) ut[i] = x;
+        Ud[row * cfg::LDU + ucol + i] = x * f;
+      }
+    }
+    __syncthreads();   // U~ in place; S has been read
+    // ---- S
+    {
+      float acc[4][4] = {};
+      const float *k0 = Ks + kb * LD + 4 * fg, *u0 = Ud + kb * cfg::LDU + 4 * cgb;
+#pragma unroll 8
+      for (int i = 0; i < kC / KB; ++i) {
+        const float4 kv = ld4(k0 + KB * i * LD), uv = ld4(u0 + KB * i * cfg::LDU);
+        fma4(acc[0], kv.x, uv); fma4(acc[1], kv.y, uv); fma4(acc[2], kv.z, uv); fma4(acc[3], kv.w, uv);
+      }
+      float v[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) v[i] = acc[i / 4][i & 3];
+      reduce_scatter<KB>(v, kb);
+#pragma unroll
+      for (int i = 0; i < VB; ++i) Sr[i] = fmaf(gl, Sr[i], v[i]);
+    }
+    slot += slot_floats(a);
+    if (c + 1 < n_chunks) {
+      share_state();
+      put_state(slot);
+    }
+  }
+  if (a.c0 + n_chunks < n_all) put_state(a.carry + state_base);
+  else if (p.S_out) put_state(p.S_out + state_base);
+}
+
+template <int DK>
+struct Output {
+  static constexpr int LD = DK + 4, LDV = kNV + 4;
+  static constexpr int P_FLOATS = kC * (kLdP > LD ? kLdP : LD);   // P takes the place of K
+  static constexpr int floats = kC * LD + P_FLOATS + DK * LDV + kC * LDV + kC;
+  static constexpr size_t bytes = floats * sizeof(float);
 };
 
 template <int DK>
-__global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) scan_f32_kernel(ScanParams p, F32Args a) {
-  using cfg = F32Scan<DK>;
-  constexpr int LD = cfg::LD, JG = cfg::JG;
+__global__ void __launch_bounds__(kThreads, DK == 64 ? 3 : 1) scan_f32_output(ScanParams p, F32Args a) {
+  using cfg = Output<DK>;
+  constexpr int LD = cfg::LD, LDV = cfg::LDV;
   extern __shared__ __align__(16) float sm[];
-  float *Ws = sm, *Qs = Ws + kC * LD, *Ks = Qs + kC * LD;
-  float *Us = Ks + kC * LD, *S = Us + kC * kNS, *Ut = S + DK * kNS, *Ud = Ut + kC * kLdU, *P = Ud + kC * kLdU, *sg = P + kC * kLdP;
+  float *Qs = sm, *Ks = Qs + kC * LD, *P = Ks, *Ss = Ks + cfg::P_FLOATS, *Ut = Ss + DK * LDV, *sg = Ut + kC * LDV;
   const int tid = threadIdx.x;
-  const int n_slices = (a.d_v + kNS - 1) / kNS;
-  const int slice = blockIdx.x % n_slices, h = (blockIdx.x / n_slices) % p.H, s = blockIdx.x / (n_slices * p.H);
+  const int n_slices = (a.d_v + kNV - 1) / kNV;
+  const int slice = blockIdx.x % n_slices, at = blockIdx.x / n_slices, lc = at % a.n_seg, pair = at / a.n_seg, h = pair % p.H, s = pair / p.H;
   const int beg = p.seq_off ? p.seq_off[s] : s * p.T;
   const int end = p.seq_off ? p.seq_off[s + 1] : (s + 1) * p.T;
-  const int col0 = slice * kNS;
-  const size_t state_base = ((size_t)s * p.H + h) * a.d_k * a.d_v;
+  const int tok0 = beg + (a.c0 + lc) * kC;
+  if (tok0 >= end) return;
+  const int rows = end - tok0 < kC ? end - tok0 : kC;
+  const int col0 = slice * kNV;
+  const float* slot = a.slots + (size_t)at * slot_floats(a);
 
-  // state slice: rows past d_k and columns past d_v stay zero throughout (their operands are zero-filled)
-  for (int e = tid; e < DK * kNS; e += kThreads) {
-    const int k = e / kNS, n = e % kNS;
-    S[e] = (p.S0 && k < a.d_k && col0 + n < a.d_v) ? p.S0[state_base + (size_t)k * a.d_v + col0 + n] : 0.f;
+  copy_rows<DK, LD>(Qs, a.Q, tok0, rows, p.H, h, a.d_k, tid);
+  copy_rows<DK, LD>(Ks, a.K, tok0, rows, p.H, h, a.d_k, tid);
+  cp_commit();
+#pragma unroll
+  for (int m = 0; m < (DK + kC) * (kNV / 4) / kThreads; ++m) {   // the state [d_k][d_v], then U~ [64][d_v]
+    const int e = tid + m * kThreads, k = e / (kNV / 4), n = 4 * (e % (kNV / 4));
+    const bool in_state = k < DK, ok = col0 + n < a.d_v && (!in_state || k < a.d_k);
+    cp_async16(Ss + k * LDV + n, slot + (ok ? (size_t)(in_state ? k : a.d_k + k - DK) * a.d_v + col0 + n : 0), ok);
   }
-  // rows of a [tokens, H, d_k] tensor; rows past the sequence's end and columns past d_k become zeros
-  auto copy_rows = [&](float* dst, const float* src, int tok0, int rows) {
-    constexpr int Q4 = DK / 4;
-#pragma unroll
-    for (int m = 0; m < kC * Q4 / kThreads; ++m) {
-      const int e = tid + m * kThreads, j = e / Q4, c = 4 * (e % Q4);
-      const bool ok = j < rows && c < a.d_k;
-      cp_async16(dst + j * LD + c, src + (ok ? ((size_t)(tok0 + j) * p.H + h) * a.d_k + c : 0), ok);
-    }
-  };
-  auto copy_u = [&](int tok0, int rows) {
-    const int j = tid >> 2, c = 4 * (tid & 3);
-    const bool ok = j < rows && col0 + c < a.d_v;
-    cp_async16(Us + j * kNS + c, a.U + (ok ? ((size_t)(tok0 + j) * p.H + h) * a.d_v + col0 + c : 0), ok);
-  };
-  auto load_g = [&](int tok0, int rows) {   // rows past the end take the last real row's g
-    return tid < kC ? p.g[(size_t)(tok0 + (tid < rows ? tid : rows - 1)) * p.H + h] : 0.f;
-  };
-  const int nq = tid & 3, r = tid >> 2;                                                   // steps 1 and 3
-  const int ty = ((tid & 31) >> 2) + 8 * ((tid >> 5) & 1), tx = (tid & 3) + 4 * (tid >> 6);   // step 2: eight rows, four columns of a block per warp
-  const int jg = tid % JG, n4 = (tid / JG) & 3, kq = tid / (4 * JG);                      // step 4
-
-  int buf = 0;
-  if (beg < end) {
-    const int rows = end - beg < kC ? end - beg : kC;
-    copy_rows(Ws, a.W, beg, rows);
-    copy_u(beg, rows);
-    copy_rows(Qs, a.Q, beg, rows);
-    cp_commit();
-    copy_rows(Ks, a.K, beg, rows);
-    cp_commit();
-    if (tid < kC) sg[tid] = load_g(beg, rows);
-  }
-  for (int tok0 = beg; tok0 < end; tok0 += kC, buf ^= 1) {
-    const int rows = end - tok0 < kC ? end - tok0 : kC;
-    const int next0 = tok0 + kC, nrows = end - next0 < kC ? end - next0 : kC;   // of the next chunk (nrows <= 0: none)
-    const float* gb = sg + buf * kC;
-    cp_wait<1>();      // W, U, Q of this chunk; K may still be on its way
-    __syncthreads();
-    const float g_next = nrows > 0 ? load_g(next0, nrows) : 0.f;
-    // ---- 1. W S and Q S
-    float ws[4] = {0.f, 0.f, 0.f, 0.f}, qs[4] = {0.f, 0.f, 0.f, 0.f};
-    {
-      const float *wr = Ws + r * LD, *qr = Qs + r * LD, *sc = S + 4 * nq;
-#pragma unroll 4
-      for (int k = 0; k < DK; k += 4) {
-        const float4 w = ld4(wr + k), q = ld4(qr + k);
-        const float4 s0 = ld4(sc + k * kNS), s1 = ld4(sc + (k + 1) * kNS), s2 = ld4(sc + (k + 2) * kNS), s3 = ld4(sc + (k + 3) * kNS);
-        fma4(ws, w.x, s0); fma4(qs, q.x, s0);
-        fma4(ws, w.y, s1); fma4(qs, q.y, s1);
-        fma4(ws, w.z, s2); fma4(qs, q.z, s2);
-        fma4(ws, w.w, s3); fma4(qs, q.w, s3);
-      }
-      const float4 u = ld4(Us + r * kNS + 4 * nq);
-      const float f = expf(gb[rows - 1] - gb[r]);
-      float4 t = make_float4(u.x - ws[0], u.y - ws[1], u.z - ws[2], u.w - ws[3]);
-      if (r >= rows) t = make_float4(0.f, 0.f, 0.f, 0.f);
-      *reinterpret_cast<float4*>(Ut + r * kLdU + 4 * nq) = t;
-      *reinterpret_cast<float4*>(Ud + r * kLdU + 4 * nq) = make_float4(t.x * f, t.y * f, t.z * f, t.w * f);
-    }
-    cp_wait<0>();      // K of this chunk
-    __syncthreads();   // U~ in place; W and U have been read
-    if (nrows > 0) {
-      copy_rows(Ws, a.W, next0, nrows);
-      copy_u(next0, nrows);
-    }
-    cp_commit();
-    // ---- 2. P
-    {
-      float acc[4][4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+  cp_commit();
+  if (tid < kC) sg[tid] = p.g[(size_t)(tok0 + (tid < rows ? tid : rows - 1)) * p.H + h];   // rows past the end take the last real row's
+  // eight rows and four columns (groups of four columns) per warp: either operand's loads of a step touch 32 different banks
+  const int ty = ((tid & 31) >> 2) + 8 * ((tid >> 5) & 1), tx = (tid & 3) + 4 * (tid >> 6);
+  cp_wait<1>();
+  __syncthreads();
+  // ---- P: element (ty, tx) of the ten 16 x 16 blocks on and below the diagonal
+  {
+    float acc[4][4] = {};
 #pragma unroll 2
-      for (int k = 0; k < DK; k += 4) {
-        float4 q[4];
+    for (int k = 0; k < DK; k += 4) {
+      float4 q[4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) q[i] = ld4(Qs + (ty + 16 * i) * LD + k);
+      for (int i = 0; i < 4; ++i) q[i] = ld4(Qs + (ty + 16 * i) * LD + k);
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const float4 kv = ld4(Ks + (tx + 16 * j) * LD + k);
+      for (int j = 0; j < 4; ++j) {
+        const float4 kv = ld4(Ks + (tx + 16 * j) * LD + k);
 #pragma unroll
-          for (int i = 0; i < 4; ++i)
-            if (i >= j) acc[i][j] = fmaf(q[i].w, kv.w, fmaf(q[i].z, kv.z, fmaf(q[i].y, kv.y, fmaf(q[i].x, kv.x, acc[i][j]))));
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j <= i; ++j) {
-          const int ri = ty + 16 * i, cj = tx + 16 * j;
-          P[ri * kLdP + cj] = cj <= ri ? acc[i][j] * expf(gb[ri] - gb[cj]) : 0.f;
-        }
-    }
-    __syncthreads();   // P in place; Q has been read
-    if (nrows > 0) copy_rows(Qs, a.Q, next0, nrows);
-    cp_commit();
-    // ---- 3. O
-    if (r < rows && col0 + 4 * nq < a.d_v) {
-      const float gam = expf(gb[r]);
-      float o[4] = {gam * qs[0], gam * qs[1], gam * qs[2], gam * qs[3]};
-      const float *pr = P + r * kLdP, *uc = Ut + 4 * nq;
-      int j = 0;
-#pragma unroll 2
-      for (; j + 3 <= r; j += 4) {
-        const float4 pv = ld4(pr + j);
-        fma4(o, pv.x, ld4(uc + j * kLdU));
-        fma4(o, pv.y, ld4(uc + (j + 1) * kLdU));
-        fma4(o, pv.z, ld4(uc + (j + 2) * kLdU));
-        fma4(o, pv.w, ld4(uc + (j + 3) * kLdU));
-      }
-      for (; j <= r; ++j) fma4(o, pr[j], ld4(uc + j * kLdU));
-      *reinterpret_cast<float4*>((float*)p.O + ((size_t)(tok0 + r) * p.H + h) * a.d_v + col0 + 4 * nq) =
-          make_float4(p.scale * o[0], p.scale * o[1], p.scale * o[2], p.scale * o[3]);
-    }
-    // ---- 4. S (every read of the old S was before the barriers above)
-    {
-      float acc[4][4];   // [feature][column]
-#pragma unroll
-      for (int f = 0; f < 4; ++f)
-#pragma unroll
-        for (int n = 0; n < 4; ++n) acc[f][n] = 0.f;
-#pragma unroll 4
-      for (int it = 0; it < kC / JG / 2; ++it)
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const int j = it * 2 * JG + 2 * jg + q;   // two neighbouring tokens per lane group: their rows lie in different banks
-          const float4 kv = ld4(Ks + j * LD + 4 * kq), uv = ld4(Ud + j * kLdU + 4 * n4);
-          fma4(acc[0], kv.x, uv); fma4(acc[1], kv.y, uv); fma4(acc[2], kv.z, uv); fma4(acc[3], kv.w, uv);
-        }
-      // reduce-scatter over the token groups: lanes that differ in bit 0 keep two features each, then (JG = 4) one each
-      const bool up = jg & 1;
-      float two[2][4];
-#pragma unroll
-      for (int f = 0; f < 2; ++f)
-#pragma unroll
-        for (int n = 0; n < 4; ++n) {
-          const float give = up ? acc[f][n] : acc[2 + f][n], keep = up ? acc[2 + f][n] : acc[f][n];
-          two[f][n] = keep + __shfl_xor_sync(0xffffffffu, give, 1);
-        }
-      const float gl = expf(gb[rows - 1]);
-      auto update = [&](int k, const float (&v)[4]) {
-        float* sp = S + k * kNS + 4 * n4;
-        const float4 o = ld4(sp);
-        *reinterpret_cast<float4*>(sp) = make_float4(fmaf(gl, o.x, v[0]), fmaf(gl, o.y, v[1]), fmaf(gl, o.z, v[2]), fmaf(gl, o.w, v[3]));
-      };
-      if constexpr (JG == 4) {
-        const bool up2 = jg & 2;
-        float one[4];
-#pragma unroll
-        for (int n = 0; n < 4; ++n) {
-          const float give = up2 ? two[0][n] : two[1][n], keep = up2 ? two[1][n] : two[0][n];
-          one[n] = keep + __shfl_xor_sync(0xffffffffu, give, 2);
-        }
-        update(4 * kq + 2 * (jg & 1) + (jg >> 1), one);
-      } else {
-        update(4 * kq + 2 * jg, two[0]);
-        update(4 * kq + 2 * jg + 1, two[1]);
+        for (int i = 0; i < 4; ++i)
+          if (i >= j) acc[i][j] = fmaf(q[i].w, kv.w, fmaf(q[i].z, kv.z, fmaf(q[i].y, kv.y, fmaf(q[i].x, kv.x, acc[i][j]))));
       }
     }
-    if (tid < kC) sg[(buf ^ 1) * kC + tid] = g_next;
-    __syncthreads();   // S updated; K has been read
-    if (nrows > 0) copy_rows(Ks, a.K, next0, nrows);
-    cp_commit();
+    cp_wait<0>();
+    __syncthreads();   // K has been read; S and U~ have landed
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j <= i; ++j) {
+        const int ri = ty + 16 * i, cj = tx + 16 * j;
+        P[ri * kLdP + cj] = cj <= ri ? acc[i][j] * expf(sg[ri] - sg[cj]) : 0.f;
+      }
   }
-  if (p.S_out) {
-    __syncthreads();
-    for (int e = tid; e < DK * kNS; e += kThreads) {
-      const int k = e / kNS, n = e % kNS;
-      if (k < a.d_k && col0 + n < a.d_v) p.S_out[state_base + (size_t)k * a.d_v + col0 + n] = S[e];
+  // ---- O: rows ty + 16 i, four columns
+  float o[4][4] = {};
+  {
+    const float* sc = Ss + 4 * tx;
+#pragma unroll 2
+    for (int k = 0; k < DK; k += 4) {
+      const float4 s0 = ld4(sc + k * LDV), s1 = ld4(sc + (k + 1) * LDV), s2 = ld4(sc + (k + 2) * LDV), s3 = ld4(sc + (k + 3) * LDV);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float4 q = ld4(Qs + (ty + 16 * i) * LD + k);
+        fma4(o[i], q.x, s0); fma4(o[i], q.y, s1); fma4(o[i], q.z, s2); fma4(o[i], q.w, s3);
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const float gam = expf(sg[ty + 16 * i]);
+#pragma unroll
+      for (int n = 0; n < 4; ++n) o[i][n] *= gam;
+    }
+  }
+  __syncthreads();   // P in place
+#pragma unroll
+  for (int b = 0; b < 4; ++b) {   // tokens 16 b .. + 15 of the sum: rows of the blocks i >= b
+    const float *uc = Ut + 16 * b * LDV + 4 * tx, *pc = P + ty * kLdP + 16 * b;
+#pragma unroll 2
+    for (int j = 0; j < 16; j += 4) {
+      const float4 u0 = ld4(uc + j * LDV), u1 = ld4(uc + (j + 1) * LDV), u2 = ld4(uc + (j + 2) * LDV), u3 = ld4(uc + (j + 3) * LDV);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        if (i >= b) {
+          const float4 pv = ld4(pc + 16 * i * kLdP + j);
+          fma4(o[i], pv.x, u0); fma4(o[i], pv.y, u1); fma4(o[i], pv.z, u2); fma4(o[i], pv.w, u3);
+        }
+      }
+    }
+  }
+  if (col0 + 4 * tx < a.d_v) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int r = ty + 16 * i;
+      if (r < rows)
+        *reinterpret_cast<float4*>((float*)p.O + ((size_t)(tok0 + r) * p.H + h) * a.d_v + col0 + 4 * tx) =
+            make_float4(p.scale * o[i][0], p.scale * o[i][1], p.scale * o[i][2], p.scale * o[i][3]);
     }
   }
 }
 
-template <int DK>
-cudaError_t launch_one(const ScanParams& p, const F32Args& a, cudaStream_t stream) {
-  cudaError_t e = cudaFuncSetAttribute(scan_f32_kernel<DK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)F32Scan<DK>::bytes);
+template <int DK, int NS>
+cudaError_t launch_chain(const ScanParams& p, const F32Args& a, long long pairs, cudaStream_t stream) {
+  cudaError_t e = cudaFuncSetAttribute(scan_f32_chain<DK, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Chain<DK, NS>::bytes);
   if (e != cudaSuccess) return e;
-  const long long grid = (long long)p.n_seqs * p.H * ((a.d_v + kNS - 1) / kNS);
+  const long long grid = pairs * ((a.d_v + NS - 1) / NS);
   if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-  scan_f32_kernel<DK><<<(int)grid, kThreads, F32Scan<DK>::bytes, stream>>>(p, a);
+  scan_f32_chain<DK, NS><<<(int)grid, kThreads, Chain<DK, NS>::bytes, stream>>>(p, a);
   return cudaGetLastError();
+}
+
+template <int DK>
+cudaError_t launch_segments(const ScanParams& p, F32Args a, int max_chunks, cudaStream_t stream) {
+  cudaError_t e = cudaFuncSetAttribute(scan_f32_output<DK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Output<DK>::bytes);
+  if (e != cudaSuccess) return e;
+  const long long pairs = (long long)p.n_seqs * p.H;
+  // eight columns a CTA while that is no more than two CTAs for each SM: half the work on the chain; beyond it the wider slice reads
+  // W and K half as often
+  const bool wide = pairs * ((a.d_v + 7) / 8) > 2 * 148;
+  for (a.c0 = 0; a.c0 == 0 || a.c0 < max_chunks; a.c0 += a.n_seg) {
+    e = wide ? launch_chain<DK, 16>(p, a, pairs, stream) : launch_chain<DK, 8>(p, a, pairs, stream);
+    if (e != cudaSuccess) return e;
+    if (max_chunks == 0) break;
+    const long long grid = pairs * a.n_seg * ((a.d_v + kNV - 1) / kNV);
+    if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
+    scan_f32_output<DK><<<(int)grid, kThreads, Output<DK>::bytes, stream>>>(p, a);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 }  // namespace
 
-cudaError_t launch_chunk_scan_f32(const ScanParams& p, const void* Q, const void* K, const void* W, int d_k, int d_v, cudaStream_t stream) {
-  const F32Args a{(const float*)Q, (const float*)K, (const float*)W, (const float*)p.U, d_k, d_v};
-  return d_k <= 64 ? launch_one<64>(p, a, stream) : launch_one<128>(p, a, stream);
+// Chunks per segment and the scratch of a call: slots for every (pair, chunk) of a segment, and the carried state.
+size_t chunk_scan_f32_scratch(long long pairs, int max_chunks, int d_k, int d_v, int* n_seg) {
+  const size_t slot = (size_t)(d_k + kC) * d_v * sizeof(float), state = (size_t)d_k * d_v * sizeof(float);
+  long long n = (long long)(kScratchBytes / (slot * (size_t)pairs));
+  n = n < 1 ? 1 : n > max_chunks ? (max_chunks < 1 ? 1 : max_chunks) : n;
+  *n_seg = (int)n;
+  return (size_t)pairs * ((size_t)n * slot + (n < max_chunks ? state : 0));
+}
+
+cudaError_t launch_chunk_scan_f32(const ScanParams& p, const void* Q, const void* K, const void* W, int d_k, int d_v, int max_chunks,
+                                  void* scratch, int n_seg, cudaStream_t stream) {
+  F32Args a{(const float*)Q, (const float*)K, (const float*)W, (const float*)p.U, d_k, d_v, (float*)scratch, nullptr, 0, n_seg};
+  a.carry = a.slots + (size_t)p.n_seqs * p.H * n_seg * (size_t)(d_k + kC) * d_v;
+  return d_k <= 64 ? launch_segments<64>(p, a, max_chunks, stream) : launch_segments<128>(p, a, max_chunks, stream);
 }
 
 }  // namespace tri_inv

@@ -264,6 +264,25 @@ def test_chunk_scan_fp32_tiles(bnd, name, B, T, H, d_k, d_v, cu):
     test_chunk_scan_cuda_core_kernel_other_shapes(bnd, name, B, T, H, d_k, d_v, 64, wl.F32, cu)
 
 
+@pytest.mark.parametrize("H,d_k,d_v", [(40, 128, 128), (44, 64, 64)])
+def test_fp32_scan_in_segments(bnd, H, d_k, d_v):
+    """More (pair, chunk) slots than the scan's scratch holds: the state is carried between the segments, which gives the bits of
+    stopping and resuming by hand.  Also the chain's wider slices."""
+    per_slot = (d_k + 64) * d_v * 4
+    T = 64 * ((128 << 20) // per_slot // H + 3) + 9
+    inp = wl.make("segments", 1, T, H, d_k, d_v, 64, wl.F32, seed=780)
+    dev = bnd.to_device(inp)
+    Q = bnd.kv_to_torch(wl.queries(inp, seed=781))
+    W, U = 0.1 * Q, dev["V"]
+    half = T // 128 * 64
+    cut = lambda t, a, b: t[:, a:b].contiguous()
+    O, S = bnd.chunk_scan(Q, dev["K"], W, U, dev["g"], 64)
+    O1, S1 = bnd.chunk_scan(*(cut(x, 0, half) for x in (Q, dev["K"], W, U, dev["g"])), 64)
+    O2, S2 = bnd.chunk_scan(*(cut(x, half, T) for x in (Q, dev["K"], W, U, dev["g"])), 64, S0=S1)
+    torch.cuda.synchronize()
+    assert torch.equal(O, torch.cat([O1, O2], 1)) and torch.equal(S, S2)
+
+
 # ---------------------------------------------------------------- full sizes, in the launch configuration bench.py times
 
 def test_layer_full_size_config2_sampled_and_restart(bnd):
