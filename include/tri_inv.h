@@ -269,6 +269,22 @@ int tri_inv_chunk_scan(const void* Q, const void* K, const void* W, const void* 
                        void* O, float* S_out, float scale, const tri_inv_desc* desc, void* cuda_stream);
 
 /*
+ * The whole layer: the results of tri_inv_fused with TRI_INV_W_DECAY followed by tri_inv_chunk_scan, by one of two routes:
+ *   - block recursion without flags, every sequence at most 16 tokens long (a decode step, a short continuation; bf16 with
+ *     d_k = d_v = 128 and C = 64 only up to 4 tokens or few tokens in all), C >= 16, d_k <= 128: token by token in fp32, as the
+ *     recurrence under tri_inv_chunk_scan states it.
+ *   - otherwise the two calls.
+ * So a sequence continued from a returned state gives the same bits as in one go only if both are cut at chunk boundaries and neither
+ * takes the first route.  Arguments as in the two calls; O may not overlap an input.  `workspace`: device memory of at least
+ * tri_inv_gdn_forward_workspace() bytes (which may be 0: then it may be NULL), 16-byte aligned, contents arbitrary; nothing else may use it
+ * until the call has run.  Calls on different streams share no state but what the two calls share.
+ */
+int tri_inv_gdn_forward_workspace(const tri_inv_desc* desc, int method, size_t* bytes);
+int tri_inv_gdn_forward(const void* Q, const void* K, const void* V, const float* beta, const float* g, const float* S0,
+                        void* O, float* S_out, float scale, void* workspace, size_t workspace_bytes,
+                        const tri_inv_desc* desc, int method, void* cuda_stream);
+
+/*
  * Fused call with the layer's front end folded in: the kernel takes what the projections produce and
  * does the three producers that otherwise run as separate passes over memory before the inversion
  * (the gating recipe of a Gated-DeltaNet layer; in the paper these are among the kernels its fused

@@ -42,7 +42,7 @@ def ns_iters(m: int) -> int:
 FORCE_SIMT = 0x10000
 W_DECAY = 0x20000
 
-EXPORTS = ("tri_inv_build", "tri_inv_build_kda", "tri_inv_fused_kda", "tri_inv_chunk_scan_kda", "tri_inv_chunk_scan", "tri_inv_wy", "tri_inv_fused", "tri_inv_fused_raw", "tri_inv_fused_packed_static", "tri_inv_count_matrices",
+EXPORTS = ("tri_inv_build", "tri_inv_build_kda", "tri_inv_fused_kda", "tri_inv_chunk_scan_kda", "tri_inv_chunk_scan", "tri_inv_gdn_forward", "tri_inv_gdn_forward_workspace", "tri_inv_wy", "tri_inv_fused", "tri_inv_fused_raw", "tri_inv_fused_packed_static", "tri_inv_count_matrices",
            "tri_inv_fused_host", "tri_inv_fused_host_workspace", "tri_inv_selftest_wait_timeout", "tri_inv_selftest_scan_wait_timeout", "tri_inv_selftest_kda_wait_timeout", "tri_inv_selftest_bounds_check", "tri_inv_last_device_status", "tri_inv_launch_count", "tri_inv_status_string")
 
 
@@ -104,6 +104,11 @@ def load():
         if hasattr(lib, "tri_inv_selftest_wait_timeout"):
             lib.tri_inv_selftest_wait_timeout.argtypes = [vp, vp, vp, vp, vp, vp, vp, dp, ctypes.c_uint64, ctypes.POINTER(ctypes.c_int), vp]
             lib.tri_inv_selftest_wait_timeout.restype = i32
+        if hasattr(lib, "tri_inv_gdn_forward"):
+            lib.tri_inv_gdn_forward.argtypes = [vp, vp, vp, vp, vp, vp, vp, vp, ctypes.c_float, vp, ctypes.c_size_t, dp, i32, vp]
+            lib.tri_inv_gdn_forward.restype = i32
+            lib.tri_inv_gdn_forward_workspace.argtypes = [dp, i32, ctypes.POINTER(ctypes.c_size_t)]
+            lib.tri_inv_gdn_forward_workspace.restype = i32
         lib.tri_inv_count_matrices.argtypes = [dp, ctypes.POINTER(ctypes.c_int64)]
         lib.tri_inv_last_device_status.argtypes = [ctypes.POINTER(ctypes.c_int)]
         for f in ("tri_inv_build", "tri_inv_wy", "tri_inv_fused", "tri_inv_count_matrices", "tri_inv_last_device_status"):
@@ -162,14 +167,14 @@ def _p(t):
     if t is None:
         return None
     assert t.is_cuda and t.is_contiguous(), "tensors must be contiguous CUDA tensors"
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()   # an integer: the functions' argument types make the pointer of it
 
 
 def _stream(stream):
     if stream is not None:
-        return ctypes.c_void_p(stream.cuda_stream)
+        return stream.cuda_stream
     # the current stream's handle without a Stream object around it (which costs more than the rest of the marshalling)
-    return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def build(K, beta, g, C, method=BLOCK_RECURSIVE, cu_seqlens=None, out=None, stream=None):
@@ -240,9 +245,28 @@ def chunk_scan_kda(Q, K, W, U, G, C, scale=1.0, S0=None, cu_seqlens=None, out=No
 
 
 def gdn_forward(Q, K, V, beta, g, C, scale=1.0, S0=None, method=BLOCK_RECURSIVE, cu_seqlens=None, stream=None):
-    """The whole layer in two launches: fused build + inversion + WY with the decay-weighted W, then the chunk scan."""
-    _, W, U = fused(K, V, beta, g, C, method=method | W_DECAY, cu_seqlens=cu_seqlens, want_A=False, stream=stream)
-    return chunk_scan(Q, K, W, U, g, C, scale=scale, S0=S0, cu_seqlens=cu_seqlens, stream=stream)
+    """The whole layer -> (O, S_final): tri_inv_gdn_forward, which takes one kernel, or the fused call with the decay-weighted W and
+    the chunk scan, by shape."""
+    B, T, H, d_k = K.shape
+    d_v = V.shape[-1]
+    lib = load()
+    desc, keep = make_desc(B, T, H, d_k, d_v, C, _dtype_code(K), cu_seqlens)
+    need = ctypes.c_size_t(0)
+    method = int(method)
+    rc = lib.tri_inv_gdn_forward_workspace(desc, method, need)
+    if rc != OK:
+        raise TriInvError("tri_inv_gdn_forward_workspace", rc)
+    O = torch.empty_like(V)
+    S = torch.empty((B if keep is None else len(keep) - 1, H, d_k, d_v), dtype=torch.float32, device=K.device)
+    work = None
+    if need.value:
+        work = torch.empty(need.value, dtype=torch.uint8, device=K.device)
+        if stream is not None:
+            work.record_stream(stream)
+    rc = lib.tri_inv_gdn_forward(_p(Q), _p(K), _p(V), _p(beta), _p(g), _p(S0), _p(O), _p(S), float(scale), _p(work), need, desc, method, _stream(stream))
+    if rc != OK:
+        raise TriInvError("tri_inv_gdn_forward", rc)
+    return O, S
 
 
 def wy(A, K, V, beta, cu_seqlens=None, out=None, stream=None):

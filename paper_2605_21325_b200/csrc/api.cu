@@ -343,6 +343,24 @@ int chunk_scan_any(const void* Q, const void* K, const void* W, const void* U, c
 }
 }  // namespace
 
+namespace {
+// How tri_inv_gdn_forward runs a shape.  The token-by-token form is the block recursion's; any other scheme or flag
+// keeps its own inversion kernel, in two calls.
+enum LayerRoute { kTokens, kTwoCalls };
+size_t factor_bytes(const tri_inv_desc* d, int features) {
+  const size_t tokens = d->cu_seqlens ? (size_t)d->T : (size_t)d->T * d->B;
+  return (tokens * d->H * features * (d->kv_dtype == TRI_INV_BF16 ? 2 : 4) + 255) & ~(size_t)255;
+}
+LayerRoute layer_route(const tri_inv_desc* d, int method, size_t* workspace_bytes) {
+  *workspace_bytes = 0;
+  if (method == TRI_INV_BLOCK_RECURSIVE) {
+    if (recurrence_fits(d)) return kTokens;
+  }
+  *workspace_bytes = factor_bytes(d, d->d_k) + factor_bytes(d, d->d_v);
+  return kTwoCalls;
+}
+}  // namespace
+
 extern "C" {
 
 int tri_inv_chunk_scan(const void* Q, const void* K, const void* W, const void* U, const float* g, const float* S0,
@@ -355,6 +373,45 @@ int tri_inv_chunk_scan_kda(const void* Q, const void* K, const void* W, const vo
                            void* O, float* S_out, float scale, const tri_inv_desc* desc, void* cuda_stream) {
   if (!G) return TRI_INV_ERR_INVALID_ARG;
   return chunk_scan_any(Q, K, W, U, nullptr, G, S0, O, S_out, scale, desc, cuda_stream);
+}
+
+int tri_inv_gdn_forward_workspace(const tri_inv_desc* desc, int method, size_t* bytes) {
+  int rc = check_desc(desc, true);
+  if (rc) return rc;
+  if (!bytes) return TRI_INV_ERR_INVALID_ARG;
+  layer_route(desc, method, bytes);
+  return TRI_INV_OK;
+}
+
+int tri_inv_gdn_forward(const void* Q, const void* K, const void* V, const float* beta, const float* g, const float* S0,
+                        void* O, float* S_out, float scale, void* workspace, size_t workspace_bytes,
+                        const tri_inv_desc* desc, int method, void* cuda_stream) {
+  int rc = check_desc(desc, true);
+  if (rc) return rc;
+  if ((rc = check_method(method, true))) return rc;
+  size_t need = 0;
+  const LayerRoute route = layer_route(desc, method, &need);
+  if (!Q || !K || !V || !beta || !g || !O || (need && !workspace) || workspace_bytes < need) return TRI_INV_ERR_INVALID_ARG;
+  if (!aligned16(Q) || !aligned16(K) || !aligned16(V) || !aligned16(beta) || !aligned16(g) || !aligned16(O) || !aligned16(S0) ||
+      !aligned16(S_out) || !aligned16(workspace))
+    return TRI_INV_ERR_INVALID_ARG;
+  if (route == kTwoCalls) {
+    void* W = workspace;
+    void* U = reinterpret_cast<char*>(workspace) + factor_bytes(desc, desc->d_k);
+    if ((rc = tri_inv_fused(K, V, beta, g, nullptr, W, U, desc, method | TRI_INV_W_DECAY, cuda_stream))) return rc;
+    return tri_inv_chunk_scan(Q, K, W, U, g, S0, O, S_out, scale, desc, cuda_stream);
+  }
+  ScanParams p{};
+  p.g = g; p.S0 = S0; p.O = O; p.S_out = S_out; p.scale = scale;
+  p.H = desc->H; p.T = desc->T;
+  p.n_seqs = desc->cu_seqlens ? desc->n_seqs : desc->B;
+  cudaError_t err;
+  p.status = status_word_for_current_device(&err);
+  if (!p.status) return TRI_INV_ERR_CUDA;
+  if (p.n_seqs == 0 || (desc->T == 0 && !S_out)) return TRI_INV_OK;
+  err = launch_recurrence(Q, K, V, beta, g, p, desc, (cudaStream_t)cuda_stream);
+  if (err == cudaSuccess) g_launches.fetch_add(1, std::memory_order_relaxed);
+  return err == cudaSuccess ? TRI_INV_OK : TRI_INV_ERR_CUDA;
 }
 
 int tri_inv_selftest_scan_wait_timeout(const void* Q, const void* K, const void* W, const void* U, const float* g, void* O,

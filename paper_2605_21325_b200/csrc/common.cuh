@@ -122,6 +122,10 @@ struct ScanParams {
 cudaError_t launch_seq_offsets(int* dev_out, const tri_inv_desc* d, cudaStream_t stream);
 cudaError_t launch_chunk_scan(const ScanParams& p, const void* Q, const void* K, const void* W, long long tokens,
                               cudaStream_t stream, bool kda = false);
+// The layer token by token (recurrence_kernel.cu), any storage type and d_k <= 128: sequences of a few tokens.  scan: S0, O, S_out, scale, H, T, n_seqs.
+bool recurrence_fits(const tri_inv_desc* d);
+cudaError_t launch_recurrence(const void* Q, const void* K, const void* V, const float* beta, const float* g, const ScanParams& scan,
+                              const tri_inv_desc* d, cudaStream_t stream);
 // Per-channel form: the operands of the tensor-core scan from Q, K (bf16, [tokens,H,128]) and G, C = 64:
 // Qp = Q exp(G - G_ref), Km = K exp(G_ref - G) and the per-chunk vectors EL = exp(G_last),
 // ER = exp(G_ref), EX = exp(G_last - G_ref) ([slots,H,128] fp32), G_ref the middle row of each chunk, G_last its last.
