@@ -269,10 +269,13 @@ int tri_inv_chunk_scan(const void* Q, const void* K, const void* W, const void* 
                        void* O, float* S_out, float scale, const tri_inv_desc* desc, void* cuda_stream);
 
 /*
- * The whole layer: the results of tri_inv_fused with TRI_INV_W_DECAY followed by tri_inv_chunk_scan, by one of two routes:
+ * The whole layer: the results of tri_inv_fused with TRI_INV_W_DECAY followed by tri_inv_chunk_scan, by one of three routes:
  *   - block recursion without flags, every sequence at most 16 tokens long (a decode step, a short continuation; bf16 with
  *     d_k = d_v = 128 and C = 64 only up to 4 tokens or few tokens in all), C >= 16, d_k <= 128: token by token in fp32, as the
  *     recurrence under tri_inv_chunk_scan states it.
+ *   - block recursion without flags, bf16 with d_k = d_v = 128 and C = 64, few enough (sequence, head) pairs to be walked at the
+ *     same time: the two calls in ONE kernel, the scan of a pair running beside the factors of its later chunks -- their
+ *     results bit for bit.  Two launches on cuda_stream (a small one fills the workspace's words); nothing is allocated.
  *   - otherwise the two calls.
  * So a sequence continued from a returned state gives the same bits as in one go only if both are cut at chunk boundaries and neither
  * takes the first route.  Arguments as in the two calls; O may not overlap an input.  `workspace`: device memory of at least

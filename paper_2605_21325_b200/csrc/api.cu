@@ -344,9 +344,9 @@ int chunk_scan_any(const void* Q, const void* K, const void* W, const void* U, c
 }  // namespace
 
 namespace {
-// How tri_inv_gdn_forward runs a shape.  The token-by-token form is the block recursion's; any other scheme or flag
+// How tri_inv_gdn_forward runs a shape.  The token-by-token and one-kernel forms are the block recursion's; any other scheme or flag
 // keeps its own inversion kernel, in two calls.
-enum LayerRoute { kTokens, kTwoCalls };
+enum LayerRoute { kTokens, kOneKernel, kTwoCalls };
 size_t factor_bytes(const tri_inv_desc* d, int features) {
   const size_t tokens = d->cu_seqlens ? (size_t)d->T : (size_t)d->T * d->B;
   return (tokens * d->H * features * (d->kv_dtype == TRI_INV_BF16 ? 2 : 4) + 255) & ~(size_t)255;
@@ -355,6 +355,7 @@ LayerRoute layer_route(const tri_inv_desc* d, int method, size_t* workspace_byte
   *workspace_bytes = 0;
   if (method == TRI_INV_BLOCK_RECURSIVE) {
     if (recurrence_fits(d)) return kTokens;
+    if (d->kv_dtype == TRI_INV_BF16 && d->d_k == 128 && d->d_v == 128 && d->C == 64 && layer_fits(d, workspace_bytes)) return kOneKernel;
   }
   *workspace_bytes = factor_bytes(d, d->d_k) + factor_bytes(d, d->d_v);
   return kTwoCalls;
@@ -409,7 +410,8 @@ int tri_inv_gdn_forward(const void* Q, const void* K, const void* V, const float
   p.status = status_word_for_current_device(&err);
   if (!p.status) return TRI_INV_ERR_CUDA;
   if (p.n_seqs == 0 || (desc->T == 0 && !S_out)) return TRI_INV_OK;
-  err = launch_recurrence(Q, K, V, beta, g, p, desc, (cudaStream_t)cuda_stream);
+  err = route == kOneKernel ? launch_layer(Q, K, V, beta, g, p, workspace, desc, (cudaStream_t)cuda_stream)
+                            : launch_recurrence(Q, K, V, beta, g, p, desc, (cudaStream_t)cuda_stream);
   if (err == cudaSuccess) g_launches.fetch_add(1, std::memory_order_relaxed);
   return err == cudaSuccess ? TRI_INV_OK : TRI_INV_ERR_CUDA;
 }

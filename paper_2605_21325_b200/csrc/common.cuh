@@ -122,7 +122,12 @@ struct ScanParams {
 cudaError_t launch_seq_offsets(int* dev_out, const tri_inv_desc* d, cudaStream_t stream);
 cudaError_t launch_chunk_scan(const ScanParams& p, const void* Q, const void* K, const void* W, long long tokens,
                               cudaStream_t stream, bool kda = false);
-// The layer token by token (recurrence_kernel.cu), any storage type and d_k <= 128: sequences of a few tokens.  scan: S0, O, S_out, scale, H, T, n_seqs.
+// The layer in one kernel (layer_kernel.cuh): bf16, d_k = d_v = 128, C = 64.  scan: S0, O, S_out, scale, status, H, T, n_seqs.
+// layer_fits: whether that is the faster form for this shape, and the workspace it takes.
+bool layer_fits(const tri_inv_desc* d, size_t* workspace_bytes);
+cudaError_t launch_layer(const void* Q, const void* K, const void* V, const float* beta, const float* g, const ScanParams& scan,
+                         void* workspace, const tri_inv_desc* d, cudaStream_t stream);
+// The layer token by token (recurrence_kernel.cu), any storage type and d_k <= 128: sequences of a few tokens.  Same fields of scan.
 bool recurrence_fits(const tri_inv_desc* d);
 cudaError_t launch_recurrence(const void* Q, const void* K, const void* V, const float* beta, const float* g, const ScanParams& scan,
                               const tri_inv_desc* d, cudaStream_t stream);

@@ -45,7 +45,7 @@ namespace tri_inv {
 namespace {
 
 constexpr int C = 64, D = 128;
-constexpr int kChainWarps = 8, kOutWarps = 4, kControl = kChainWarps + kOutWarps, kGate = kControl + 1, kThreadsScan = (kGate + 1) * 32;
+constexpr int kChainWarps = 8, kOutWarps = 4, kControl = kChainWarps + kOutWarps, kGate = kControl + 1, kCopy = kGate + 1, kThreadsScan = (kGate + 1) * 32;
 constexpr int kStages = 3;
 constexpr float kLog2e = 1.4426950408889634f;
 
@@ -59,6 +59,31 @@ constexpr float kLog2e = 1.4426950408889634f;
 // coming chunk, as PQ's operand; P needs no decay; the state update has two per-column factors.  (A second S^T operand instead
 // of W exp(-G_ref) from the preparation pass takes a quarter of that pass's traffic away, and a rounding of W: 180.6 -> 164 us
 // for the call on B = 4, T = 4096, H = 16.)
+// How many chunks from `word` on (one word per chunk, `stride` apart, at most n) have their factors in memory; polls until it is one
+// at least, with a limit (0: it ran out).  A word counts one arrival per warp of the group that writes them.  A lane per chunk:
+// a round trip to L2 and the fence behind it cost about 1,000 cycles, too much for each chunk of a chain whose factors lie ready.
+constexpr uint32_t kReady = 4;
+__device__ __noinline__ int wait_ready(const uint32_t* word, int stride, int n, int lane, unsigned long long limit_ns) {
+  const uint32_t* mine = word + (size_t)(lane < n ? lane : 0) * stride;
+  unsigned long long t0 = 0;
+  for (uint32_t i = 0; i < kSpinLimit; ++i) {
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(mine) : "memory");
+    const uint32_t not_yet = __ballot_sync(0xffffffffu, lane >= n || v < kReady);
+    if (!(not_yet & 1u)) {
+      asm volatile("fence.proxy.async;" ::: "memory");   // the copies of these chunks (async proxy) come behind the loads above
+      __syncwarp();
+      return not_yet ? __ffs(not_yet) - 1 : 32;
+    }
+    if ((i & 63u) == 0) {
+      const unsigned long long now = global_timer_ns();
+      if (i == 0) t0 = now;
+      else if (__any_sync(0xffffffffu, now - t0 > limit_ns)) return 0;
+    }
+  }
+  return 0;
+}
+
 template <int DVS, bool KDA>
 struct ScanCfg {
   static_assert(DVS == 128 || DVS == 64 || DVS == 32, "slices of value columns");
@@ -154,13 +179,17 @@ __device__ __noinline__ bool wait_by_warp(uint32_t bar, uint32_t parity, unsigne
   return false;
 }
 
-template <int DVS, bool KDA>
-__global__ void __launch_bounds__(kThreadsScan, 1)
-chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmQ,
-                  const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmU, ScanParams p) {
+// One (sequence, head, slice) by a whole CTA; true when a wait has run out in this thread.
+// FED: W and U are being written by other CTAs of the same launch (layer_kernel.cuh).  The tile copies are then requested by a warp
+// of their own, kCopy, which first waits until the chunk's word in `ready` says that both factors are in memory; tensor memory
+// is the caller's (`tmem`).  Otherwise the gate warp requests the copies and the CTA allocates (and frees) its tensor memory.
+template <int DVS, bool KDA, bool FED>
+__device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmU,
+                                          const ScanParams& p, uint8_t* smem, int s, int h, int slice, bool first_block,
+                                          const uint32_t* ready, uint32_t tmem) {
   using cfg = ScanCfg<DVS, KDA>;
-  constexpr int LG = cfg::LG, E = cfg::E, NS = D / DVS;
-  extern __shared__ __align__(1024) uint8_t smem[];
+  constexpr int LG = cfg::LG, E = cfg::E;
+  static_assert(!(FED && KDA), "the scalar gate only");
   float* sG = reinterpret_cast<float*>(smem + cfg::OFF_G);   // scalar gate: [2][4][64]: g log2e; 2^(g_ref(j) - g_j), g_ref(j) = g of the first token of j's block of eight; 2^(g_last - g_j); 2^g_j
   float* sEl = sG;                 // per-channel form: exp(G_last) [3][128], exp(G_ref) [3][128], exp(G_last - G_ref) [3][128]
   float* sEr = sG + 3 * D;
@@ -181,7 +210,6 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
   const int quad = warp & 3, half = (warp >> 2) & 1;
   const int gq = lane >> 2, t = lane & 3, mi = lane >> 3, mr = lane & 7;
 
-  const int slice = blockIdx.x % NS, h = (blockIdx.x / NS) % p.H, s = blockIdx.x / (NS * p.H);
   const int beg = p.seq_off ? p.seq_off[s] : s * p.T;
   const int end = p.seq_off ? p.seq_off[s + 1] : (s + 1) * p.T;
   const int n_chunks = (end - beg + C - 1) / C;
@@ -210,7 +238,7 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
     float* dst = p.S_out + ((size_t)s * p.H + h) * D * D;
     for_state([&](float& x, size_t at) { dst[at] = x; });
   };
-  if (n_chunks == 0) { store_state(); return; }
+  if (n_chunks == 0) { store_state(); return false; }
   const bool misaligned = (s0 & 1023u) != 0;     // never expected; the swizzle pattern would not match the copies
 
   // every tile of chunk c, into stage c % 3
@@ -229,6 +257,10 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
     if constexpr (cfg::UBOX == 2) tma_load_2d(base + cfg::OFF_UT + 8192, &tmU, bar, h * D + 64, tok0);
   };
   auto full_parity = [](int c) { return (uint32_t)((c / kStages) & 1); };
+  int requested = -1;   // lane 0 of the warp that requests the copies: the last chunk whose copies were requested
+  auto drain_copies = [&]() {   // give-up path: the copies still on their way into this CTA's shared memory, with a limit
+    for (int c = requested - 1 > 0 ? requested - 1 : 0; c <= requested; ++c) mbar_wait_bounded(bar_full + 8 * (c % kStages), full_parity(c), lim);
+  };
   // g of a chunk, by the gate warp (lane l: tokens l and l + 32).  Rows past the sequence end take the last real
   // row's g, so that every exponent stays a difference of real values.
   auto fetch_g = [&](int c, float (&gr)[2]) {
@@ -271,19 +303,18 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
   };
   float4 e_raw[3] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
   float g_raw[2] = {0.f, 0.f};   // gate warp: g of the chunk it stores next
-  int requested = -1;            // gate warp, lane 0: last chunk whose copies were requested
   if (warp == kGate) {
     if (lane == 0) {
       prefetch_tmap(&tmW); prefetch_tmap(&tmQ); prefetch_tmap(&tmK); prefetch_tmap(&tmU);
       for (int b = 0; b < 8; ++b) mbar_init(bar_full + 8 * b, 1);   // three stages, exit, t1, s, pu, qk
-      mbar_init(bar_sr, kChainWarps + 1);
+      mbar_init(bar_sr, kChainWarps + (FED ? 2 : 1));
       mbar_init(bar_ud, kChainWarps);
       mbar_init(bar_ut, kChainWarps + kOutWarps);
       mbar_init(bar_qr, kOutWarps);
       mbar_init(bar_g, 1);
       mbar_init(bar_tq, 1);
       fence_mbar_init();
-      if (!misaligned) {
+      if (!FED && !misaligned) {
         issue_copies(0);
         if (n_chunks > 1) issue_copies(1);
         requested = n_chunks > 1 ? 1 : 0;
@@ -302,14 +333,14 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
       if (n_chunks > 1) fetch_g(1, g_raw);
     }
   }
-  if (warp == 0) {
+  if (!FED && warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(cfg::TMEM_COLS) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();   // barriers initialised, tensor memory allocated, first factors in place
   tc_fence_after();
-  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+  if (!FED) tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
   const uint32_t tmem_w = tmem + ((uint32_t)(32 * quad) << 16);   // this warp's lanes, column 0
   bool failed = misaligned;
   // Every wait of the roles below is one of a whole warp (wait_by_warp): its lanes go on together or give up together.  What
@@ -398,7 +429,7 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
         TL(3);
         // self-test (ScanParams::test_stall): the first CTA leaves out this product in its second chunk, so that the
         // waits for it, and then every other wait of the CTA, run out
-        if (!(p.test_stall && blockIdx.x == 0 && c == 1)) {
+        if (!(p.test_stall && first_block && c == 1)) {
 #pragma unroll
           for (int ks = 0; ks < C / 16; ++ks)   // 16 tokens (8 columns of the A operand, 2048 bytes of the K tile) per step
             umma_bf16_ta(tmem + cfg::TM_DS, tmem + (KDA ? cfg::TM_UT : cfg::TM_UD) + 8 * ks, dKm + st + ((ks * 2048) >> 4), idesc_p3, ks > 0);
@@ -438,7 +469,7 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
       // stage of c + 2 = that of c - 1: its readers (the products of chunk c - 1, the chain warps' U) were done before the
       // arrivals that open chunk c
       if (!wait(bar_sr, (uint32_t)(c & 1))) { failed = true; break; }
-      if (lane == 0 && c + 2 < n_chunks) { issue_copies(c + 2); requested = c + 2; }
+      if (!FED && lane == 0 && c + 2 < n_chunks) { issue_copies(c + 2); requested = c + 2; }
       __syncwarp();
       // the factors of c - 1 have no reader left once the first product of chunk c is complete (it was issued behind the
       // arrivals of every warp that read them); bar_qr also says that every output warp has seen bar_g of chunk c, which must not
@@ -457,8 +488,32 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
       if constexpr (KDA) { if (c + 3 < n_chunks) fetch_e(c + 3, e_raw); }
       else { if (c + 2 < n_chunks) fetch_g(c + 2, g_raw); }
     }
-    if (failed && lane == 0)   // the copies still on their way into this CTA's shared memory, with a limit
-      for (int c = requested - 1 > 0 ? requested - 1 : 0; c <= requested; ++c) mbar_wait_bounded(bar_full + 8 * (c % kStages), full_parity(c), lim);
+    if (!FED && failed && lane == 0) drain_copies();
+  } else if (FED && warp == kCopy) {
+    // ---------------------------------------------------------------- copy warp: tile copies of chunk c + 2, once W and U are there
+    // It arrives on bar_sr itself, after its wait for the phase before: the barrier must not run two phases ahead of it while it
+    // waits for another CTA.
+    int known = 0;   // chunks before this one have their factors in memory
+    auto request = [&](int c) -> bool {   // false: W and U did not come within the limit
+      if (c >= known) {
+        const int more = wait_ready(ready + ((size_t)((beg + c * C) / C + s) * p.H + h), p.H, n_chunks - c, lane, lim);
+        if (!more) return false;
+        known = c + more;
+      }
+      if (lane == 0) { issue_copies(c); requested = c; }
+      __syncwarp();
+      return true;
+    };
+    if (!misaligned) {
+      warp_arrive(bar_sr, lane);
+      failed = !request(0) || (n_chunks > 1 && !request(1));
+    }
+    for (int c = 0; c + 1 < n_chunks && !misaligned && !failed; ++c) {
+      if (!wait(bar_sr, (uint32_t)(c & 1))) { failed = true; break; }
+      warp_arrive(bar_sr, lane);
+      if (c + 2 < n_chunks && !request(c + 2)) { failed = true; break; }
+    }
+    if (failed && lane == 0) drain_copies();
   } else if (chain) {
     // ---------------------------------------------------------------- chain warps
     if (!misaligned) write_state_operand(sEr);
@@ -725,7 +780,20 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
   if (failed) atomicMax(p.status, TRI_INV_ERR_DEVICE_TIMEOUT);
   tc_fence_before();
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cfg::TMEM_COLS) : "memory");
+  if constexpr (!FED) {
+    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cfg::TMEM_COLS) : "memory");
+  }
+  return failed;
+}
+
+template <int DVS, bool KDA>
+__global__ void __launch_bounds__(kThreadsScan, 1)
+chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmQ,
+                  const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmU, ScanParams p) {
+  constexpr int NS = D / DVS;
+  extern __shared__ __align__(1024) uint8_t smem[];
+  const int slice = blockIdx.x % NS, h = (blockIdx.x / NS) % p.H, s = blockIdx.x / (NS * p.H);
+  scan_walk<DVS, KDA, false>(tmW, tmQ, tmK, tmU, p, smem, s, h, slice, blockIdx.x == 0, nullptr, 0u);
 }
 
 constexpr int kSeqsPerLaunch = 960;
@@ -804,3 +872,5 @@ cudaError_t launch_chunk_scan(const ScanParams& p, const void* Q, const void* K,
 }
 
 }  // namespace tri_inv
+
+#include "layer_kernel.cuh"   // the layer in one kernel walks with scan_walk as well

@@ -194,8 +194,10 @@ __device__ __forceinline__ void leaf_series(float* xblk, float* ys, int lane) {
 
 // One merge level of the block recursion: for every adjacent pair of B x B diagonal blocks,
 // X21 = -(X22 . N21) . X11.  Two warps share each 16-row slab of X21 and split its columns.
-template <int C, int B>
-__device__ __forceinline__ void merge_level(float* sX, int warp, int lane) {
+// sync: the barrier of the C / 16 warps that share the matrix (the whole CTA by default).
+struct CtaSync { __device__ __forceinline__ void operator()() const { __syncthreads(); } };
+template <int C, int B, class Sync = CtaSync>
+__device__ __forceinline__ void merge_level(float* sX, int warp, int lane, Sync sync = Sync()) {
   constexpr int LD = C + 4;
   constexpr int MT = B / 16;   // 16-row slabs per X21 block
   constexpr int NTT = B / 8;   // n-tiles (and k-steps) across a block
@@ -238,14 +240,14 @@ __device__ __forceinline__ void merge_level(float* sX, int warp, int lane) {
       }
     }
   }
-  __syncthreads();  // every warp has finished reading N21 before anyone overwrites it
+  sync();  // every warp has finished reading N21 before anyone overwrites it
 #pragma unroll
   for (int j = 0; j < NTR; ++j) {
     const int col = c0 + 8 * (nh * NTR + j) + 2 * t;
     *reinterpret_cast<float2*>(sX + (R0 + g) * LD + col) = make_float2(-R[j][0], -R[j][1]);
     *reinterpret_cast<float2*>(sX + (R0 + g + 8) * LD + col) = make_float2(-R[j][2], -R[j][3]);
   }
-  __syncthreads();
+  sync();
 }
 
 // One step of iterative refinement (Alg. 6 / Sec. 3.6) for the matrix I + N on the warp-level tensor cores:

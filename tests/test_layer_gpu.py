@@ -1,6 +1,7 @@
 """GPU tests of the layer forward's routes (tri_inv_gdn_forward).
 
-Token by token: fp32 arithmetic on the stored inputs, against the fp64 recurrence: fp32 storage 1e-5 of max|O| (at most 16
+One kernel (factors and scans side by side): the arithmetic is that of the two calls it replaces, so results are compared bit for
+bit.  Token by token: fp32 arithmetic on the stored inputs, against the fp64 recurrence: fp32 storage 1e-5 of max|O| (at most 16
 steps of sums of up to 128 terms, 2^-24 each), bf16 storage 2^-8 (the output's own rounding), the state 1e-5.
 """
 import numpy as np
@@ -35,6 +36,67 @@ def layer_inputs(bnd, name, B, T, H, d_k, d_v, dtype, cu, seed, with_s0=True):
     S0 = wl.initial_state(inp, seed=seed + 2) if with_s0 else None
     dev = bnd.to_device(inp)
     return inp, Q, S0, dev, bnd.kv_to_torch(Q), None if S0 is None else torch.from_numpy(S0).cuda()
+
+
+def two_calls(bnd, dev, Q, S0, cu, scale):
+    _, W, U = bnd.fused(dev["K"], dev["V"], dev["beta"], dev["g"], 64, method=bnd.W_DECAY, cu_seqlens=cu, want_A=False)
+    return bnd.chunk_scan(Q, dev["K"], W, U, dev["g"], 64, scale=scale, S0=S0, cu_seqlens=cu)
+
+
+# one chunk and one token over it, more chunks than tile stages, each slice width (few pairs: 32 columns, 32: 64, 75: 128), groups
+# that build one matrix and several, packed sequences with empty ones, of one token, and more of them than walk at the same time
+ONE_KERNEL = [
+    ("one_chunk", 1, 64, 1, None),
+    ("one_token_over", 1, 65, 2, None),
+    ("partial", 2, 333, 3, None),
+    ("slices_of_64", 2, 5 * 64 + 1, 16, None),
+    ("slices_of_128", 1, 40 * 64, 75, None),
+    ("many_matrices", 1, 96 * 64 + 7, 16, None),
+    ("packed", 1, 0, 16, np.array([0, 64, 64, 65, 300, 531, 540], np.int32)),
+    ("packed_many", 1, 0, 4, np.cumsum([0] + [1 + (37 * i) % 90 for i in range(24)]).astype(np.int32)),
+]
+
+
+@pytest.mark.parametrize("name,B,T,H,cu", ONE_KERNEL, ids=[c[0] for c in ONE_KERNEL])
+def test_one_kernel_gives_the_bits_of_the_two_calls(bnd, name, B, T, H, cu):
+    for with_s0 in (False, True):
+        _, _, _, dev, Q, S0 = layer_inputs(bnd, name, B, T, H, 128, 128, wl.BF16, cu, 700 + H, with_s0)
+        ref = two_calls(bnd, dev, Q, S0, cu, 0.25)
+        n0 = bnd.launch_count()
+        O, S = bnd.gdn_forward(Q, dev["K"], dev["V"], dev["beta"], dev["g"], 64, scale=0.25, S0=S0, cu_seqlens=cu)
+        torch.cuda.synchronize()
+        assert bnd.last_device_status() == 0
+        assert bnd.launch_count() == n0 + 1, "not the one-kernel route"
+        assert torch.equal(bits(O), bits(ref[0])) and torch.equal(bits(S), bits(ref[1]))
+
+
+def test_one_kernel_on_two_streams_and_in_a_graph(bnd):
+    """Two calls whose thread blocks share the chip (either may hold SMs that the other waits for), and a captured call replayed on
+    new inputs in the same buffers: the bits of a call by itself."""
+    args = [layer_inputs(bnd, "streams", 1, 20 * 64 + 5, 24, 128, 128, wl.BF16, None, 720 + 10 * i) for i in range(2)]
+    run = lambda a, st=None: bnd.gdn_forward(a[4], a[3]["K"], a[3]["V"], a[3]["beta"], a[3]["g"], 64, scale=0.5, S0=a[5], stream=st)
+    refs = [run(a) for a in args]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    outs = []
+    for _ in range(8):
+        for a, st in zip(args, streams):
+            with torch.cuda.stream(st):
+                outs.append(run(a, st))
+    torch.cuda.synchronize()
+    assert bnd.last_device_status() == 0
+    for i, o in enumerate(outs):
+        assert torch.equal(bits(o[0]), bits(refs[i % 2][0])) and torch.equal(bits(o[1]), bits(refs[i % 2][1]))
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        O, S = run(args[0])
+    for x, y in ((args[0][4], args[1][4]), (args[0][5], args[1][5])):
+        x.copy_(y)
+    for k in ("K", "V", "beta", "g"):
+        args[0][3][k].copy_(args[1][3][k])
+    graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(bits(O), bits(refs[1][0])) and torch.equal(bits(S), bits(refs[1][1]))
 
 
 # one token, the longest, features and columns on both sides of the kernel's instances and slices, an empty sequence
