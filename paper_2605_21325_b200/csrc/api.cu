@@ -160,7 +160,7 @@ int run(KParams p, const tri_inv_desc* d, void* stream_v) {
     if (dev_tab) cudaFreeAsync(dev_tab, stream);
     return TRI_INV_ERR_UNSUPPORTED;
   }
-  if (err == cudaSuccess && !handled) err = launch_simt(p, d->C, stream);
+  if (err == cudaSuccess && !handled) err = f32_factors_fit(p, d->C) ? launch_f32_factors(p, stream) : launch_simt(p, d->C, stream);
   if (err == cudaSuccess) g_launches.fetch_add(1, std::memory_order_relaxed);
   if (dev_tab) cudaFreeAsync(dev_tab, stream);
   if (log_enabled()) fprintf(stderr, "[tri_inv]   -> %s kernel, %s\n", handled ? "tensor-core" : "CUDA-core", cudaGetErrorString(err));
@@ -325,7 +325,7 @@ int chunk_scan_any(const void* Q, const void* K, const void* W, const void* U, c
       const size_t bytes = chunk_scan_f32_scratch((long long)p.n_seqs * p.H, max_chunks, desc->d_k, desc->d_v, &n_seg);
       cudaMemPool_t pool = table_pool_for_current_device();
       if (pool && cudaMallocFromPoolAsync(&work, bytes, pool, stream) == cudaSuccess) {
-        err = launch_chunk_scan_f32(p, Q, K, W, desc->d_k, desc->d_v, max_chunks, work, n_seg, stream);
+        err = launch_chunk_scan_f32(p, Q, K, W, desc->d_k, desc->d_v, max_chunks, tokens > 0 ? tokens : 1, work, n_seg, stream);
       } else {   // no scratch to be had: the kernel that needs none
         (void)cudaGetLastError();
         work = nullptr;

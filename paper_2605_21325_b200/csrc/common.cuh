@@ -88,6 +88,9 @@ __device__ __forceinline__ float load_kv(const void* base, int dtype, size_t idx
 
 // Launchers (defined next to their kernels).  Return a cudaError_t from the launch.
 cudaError_t launch_simt(const KParams& p, int C, cudaStream_t stream);
+// Single precision at C = 64, block recursion with substitution leaves, d <= 128 (f32_kernel.cu).
+bool f32_factors_fit(const KParams& p, int chunk);
+cudaError_t launch_f32_factors(const KParams& p, cudaStream_t stream);
 // Tensor-core path: returns cudaErrorNotSupported when it has no kernel for the request.
 cudaError_t launch_tc(const KParams& p, int C, cudaStream_t stream, bool* handled);
 // Instantiations of the tensor-core kernel, one group per tc_inst_*.cu file; raw = with a factor on each row of the keys (front end, decay-weighted W).
@@ -140,7 +143,7 @@ cudaError_t launch_kda_scan_prep(const ScanParams& p, const void* Q, const void*
 // Its scratch for this many (sequence, head) pairs and chunks of the longest sequence; *n_seg: chunks that go through at a time.
 size_t chunk_scan_f32_scratch(long long pairs, int max_chunks, int d_k, int d_v, int* n_seg);
 cudaError_t launch_chunk_scan_f32(const ScanParams& p, const void* Q, const void* K, const void* W, int d_k, int d_v, int max_chunks,
-                                  void* scratch, int n_seg, cudaStream_t stream);
+                                  long long tokens, void* scratch, int n_seg, cudaStream_t stream);
 // The same scan on the CUDA cores, for every other shape and storage type (fp32 arithmetic).
 cudaError_t launch_chunk_scan_simt(const ScanParams& p, const void* Q, const void* K, const void* W, int d_k, int d_v, int C,
                                    int kv_dtype, cudaStream_t stream);

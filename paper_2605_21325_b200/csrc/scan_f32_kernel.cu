@@ -10,13 +10,13 @@
 //
 // What bounds the chain: latency.  Its two products are 64 x NS x d_k and d_k x NS x 64 (32 K FMAs each at 8 columns, d_k = 64);
 // a thread holds a 4 x 4 tile of the result for one of KS parts of the summed index and the parts are joined by a
-// reduce-scatter of shuffles, so that all 256 threads work on so small a result.  16-byte shared-memory loads (8 per 64 FMAs), rows laid
-// out so that the eight lanes of a load step fall into different banks; W and K come by cp.async two chunks
-// ahead, U and g into registers one chunk ahead; the thread's part of S stays in registers beside its shared copy.
+// reduce-scatter of shuffles, so that all 256 threads work on so small a result.  16-byte shared-memory loads (8 per 64 FMAs), the
+// eight lanes of a load step in different banks (W and K by their tiles' 128-byte swizzle, S and U~ by padding); W and K come by TMA one
+// or two chunks ahead, U and g into registers one chunk ahead; the thread's part of S stays in registers beside its shared copy.
 // The output kernel is bound by FFMA issue and shared-memory loads (8 per 64 FMAs).
 // Measured (ncu, B = 2, T = 2048, H = 8, d = 64: 16 pairs of 32 chunks): 50 + 28 us; 213 us as one kernel per slice of 16 columns that also
 // formed P and O on the way (P again in each slice, all of it on the chain, 64 CTAs); the layer 262 -> 127 us.
-#include "common.cuh"
+#include "tc_device.cuh"
 
 namespace tri_inv {
 namespace {
@@ -78,7 +78,7 @@ __device__ __forceinline__ int reduce_scatter(float (&v)[16], int ks) {
 
 template <int DK, int NS>
 struct Chain {
-  static constexpr int LD = DK + 4;                       // row length of the W and K tiles
+  static constexpr int BOX = kC * 32;                     // floats in a box of 32 features x 64 tokens, 128-byte swizzle
   static constexpr int NG = NS / 4;                       // groups of four columns
   static constexpr int KA = kThreads / (kC / 4 * NG);     // parts of the summed index: of W S (features) ...
   static constexpr int KB = kThreads / (DK / 4 * NG);     // ... and of K^T U~ (tokens)
@@ -87,16 +87,18 @@ struct Chain {
   static constexpr int LDU = KB == 8 ? 12 : KB == 4 ? 24 : 16;   // row length of the decayed U~, for the same reason
   static_assert(LDU >= NS, "a row of U~");
   static constexpr int kStages = DK == 64 ? 3 : 2;
-  static constexpr int TILE = kC * LD;
-  static constexpr int floats = kStages * 2 * TILE + (DK / 4) * S_BLK + kC * LDU;
+  static constexpr int TILE = kC * DK;
+  static constexpr int floats = kStages * 2 * TILE + (DK / 4) * S_BLK + kC * LDU + 2 * kStages;   // the last: mbarriers
+  static_assert(((kStages * 2 * TILE + (DK / 4) * S_BLK + kC * LDU) & 1) == 0, "mbarriers on 8 bytes");
   static constexpr size_t bytes = floats * sizeof(float);
 };
 
 template <int DK, int NS>
-__global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) scan_f32_chain(ScanParams p, F32Args a) {
+__global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) scan_f32_chain(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ ScanParams p, const __grid_constant__ F32Args a) {
   using cfg = Chain<DK, NS>;
-  constexpr int LD = cfg::LD, KA = cfg::KA, KB = cfg::KB, NG = cfg::NG, VA = 16 / KA, VB = 16 / KB;
-  extern __shared__ __align__(16) float sm[];
+  constexpr int KA = cfg::KA, KB = cfg::KB, NG = cfg::NG, VA = 16 / KA, VB = 16 / KB;
+  extern __shared__ __align__(1024) float sm[];
+  const uint32_t bars = smem_u32(sm + cfg::floats - 2 * cfg::kStages);
   float *tiles = sm, *S = sm + cfg::kStages * 2 * cfg::TILE, *Ud = S + (DK / 4) * cfg::S_BLK;
   const int tid = threadIdx.x;
   const int n_slices = (a.d_v + NS - 1) / NS;
@@ -141,27 +143,42 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) scan_f32_chain(Sca
     for_state([&](float& x, int k, int n) { S[(k >> 2) * cfg::S_BLK + (k & 3) * NS + n] = x; });
   };
   auto rows_of = [&](int c) { const int left = end - beg - (a.c0 + c) * kC; return left < kC ? left : kC; };
-  auto copy_tiles = [&](int c) {
-    float* t = tiles + (c % cfg::kStages) * 2 * cfg::TILE;
-    const int tok0 = beg + (a.c0 + c) * kC, rows = rows_of(c);
-    copy_rows<DK, LD>(t, a.W, tok0, rows, p.H, h, a.d_k, tid);
-    copy_rows<DK, LD>(t + cfg::TILE, a.K, tok0, rows, p.H, h, a.d_k, tid);
+  auto copy_tiles = [&](int c) {   // by one thread; features past d_k are filled with zeros, rows past the sequence's end hold what follows
+    const int st = c % cfg::kStages, tok0 = beg + (a.c0 + c) * kC;
+    const uint32_t dst = smem_u32(tiles + st * 2 * cfg::TILE), bar = bars + 8 * st;
+    mbar_expect_tx(bar, 2 * cfg::TILE * 4);
+#pragma unroll
+    for (int b = 0; b < DK / 32; ++b) {
+      tma_load_3d(dst + b * cfg::BOX * 4, &tmW, bar, 32 * b, h, tok0);
+      tma_load_3d(dst + (cfg::TILE + b * cfg::BOX) * 4, &tmK, bar, 32 * b, h, tok0);
+    }
   };
+  bool bad = (smem_u32(sm) & 1023u) != 0;   // a wait has run out: this thread walks on without waiting
+  if (tid == 0) {
+    for (int st = 0; st < cfg::kStages; ++st) mbar_init(bars + 8 * st, 1);
+    fence_mbar_init();
+    if (!bad)
+      for (int c = 0; c < cfg::kStages - 1 && c < n_chunks; ++c) copy_tiles(c);
+  }
   // this thread's elements of U and its row's decay exp(g_last - g_row), and gamma_last, of a chunk
   float u_next[VA], g_row, g_last;
+  const size_t tok_first = (size_t)(beg + a.c0 * kC);
+  const float* u_at = a.U + ((tok_first + row) * p.H + h) * a.d_v + col0 + ucol;
+  const float* g_at = p.g + tok_first * p.H + h;
   auto fetch = [&](int c) {
-    const int tok0 = beg + (a.c0 + c) * kC, rows = rows_of(c);
+    const int rows = rows_of(c);
 #pragma unroll
-    for (int i = 0; i < VA; ++i)
-      u_next[i] = (row < rows && ucol_in) ? a.U[((size_t)(tok0 + row) * p.H + h) * a.d_v + col0 + ucol + i] : 0.f;
-    g_row = p.g[(size_t)(tok0 + (row < rows ? row : rows - 1)) * p.H + h];
-    g_last = p.g[(size_t)(tok0 + rows - 1) * p.H + h];
+    for (int i = 0; i < VA; ++i) u_next[i] = (row < rows && ucol_in) ? u_at[i] : 0.f;
+    g_row = g_at[(row < rows ? row : rows - 1) * p.H];
+    g_last = g_at[(rows - 1) * p.H];
+    u_at += (size_t)kC * p.H * a.d_v;
+    g_at += (size_t)kC * p.H;
   };
-
-  for (int c = 0; c < cfg::kStages - 1; ++c) {
-    if (c < n_chunks) copy_tiles(c);
-    cp_commit();
-  }
+  // where a load step finds its 16 bytes of W (rows 4 rg + q, features 4 ka ..) and of K (token kb, features 4 fg ..) in the swizzled boxes
+  int w_at[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) w_at[q] = (4 * rg + q) * 32 + ((ka ^ ((4 * rg + q) & 7)) << 2);
+  const int k_at = (fg >> 3) * cfg::BOX + kb * 32, k_chunk = (fg & 7) ^ kb;
   fetch(0);
   share_state();
   float* slot = a.slots + (size_t)pair * a.n_seg * slot_floats(a);
@@ -174,19 +191,25 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) scan_f32_chain(Sca
 #pragma unroll
     for (int i = 0; i < VA; ++i) u[i] = u_next[i];
     const float f = expf(g_last - g_row), gl = expf(g_last);
-    cp_wait<cfg::kStages - 2>();   // this chunk's tiles
-    __syncthreads();               // S in place; the last chunk's tiles have been read
-    if (c + cfg::kStages - 1 < n_chunks) copy_tiles(c + cfg::kStages - 1);
-    cp_commit();
+    __syncthreads();   // S in place; the last chunk's tiles have been read (and, before the first chunk, the barriers are initialised)
+    if (tid == 0 && c + cfg::kStages - 1 < n_chunks && !bad) copy_tiles(c + cfg::kStages - 1);
     if (c + 1 < n_chunks) fetch(c + 1);
+    if (!bad) bad = !mbar_wait_bounded(bars + 8 * (c % cfg::kStages), (uint32_t)(c / cfg::kStages) & 1u, p.wait_limit_ns ? p.wait_limit_ns : kWaitLimitNs);
+    if (rows < kC) {   // the sequence's last chunk: a neighbour's keys must not meet even a zero
+      float* kt = tiles + (c % cfg::kStages) * 2 * cfg::TILE + cfg::TILE;
+      for (int e = tid; e < (kC - rows) * DK; e += kThreads) kt[(e / 32 % (kC - rows) + rows) * 32 + (e / 32 / (kC - rows)) * cfg::BOX + e % 32] = 0.f;
+    }
     // ---- U~ = U - W S
     {
       float acc[4][4] = {};
-      const float *w0 = Ws + 4 * rg * LD + 4 * ka, *s0 = S + ka * cfg::S_BLK + 4 * cga;
+      const float* s0 = S + ka * cfg::S_BLK + 4 * cga;
 #pragma unroll
       for (int i = 0; i < DK / 4 / KA; ++i) {
-        const int k = 4 * KA * i;
-        const float4 x0 = ld4(w0 + k), x1 = ld4(w0 + LD + k), x2 = ld4(w0 + 2 * LD + k), x3 = ld4(w0 + 3 * LD + k);
+        // features 4 (ka + KA i) ..: box (ka + KA i) / 8, chunk (ka + KA i) % 8 of its rows
+        const float* wb = Ws + (KA * i / 8) * cfg::BOX;
+        constexpr int kFlip = KA == 4 ? 16 : 0;
+        const int f = (i & 1) * kFlip;
+        const float4 x0 = ld4(wb + (w_at[0] ^ f)), x1 = ld4(wb + (w_at[1] ^ f)), x2 = ld4(wb + (w_at[2] ^ f)), x3 = ld4(wb + (w_at[3] ^ f));
         const float* sb = s0 + KA * i * cfg::S_BLK;
         const float4 y0 = ld4(sb), y1 = ld4(sb + NS), y2 = ld4(sb + 2 * NS), y3 = ld4(sb + 3 * NS);
         fma4(acc[0], x0.x, y0); fma4(acc[1], x1.x, y0); fma4(acc[2], x2.x, y0); fma4(acc[3], x3.x, y0);
@@ -210,10 +233,11 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) scan_f32_chain(Sca
     // ---- S
     {
       float acc[4][4] = {};
-      const float *k0 = Ks + kb * LD + 4 * fg, *u0 = Ud + kb * cfg::LDU + 4 * cgb;
+      const float *k0 = Ks + k_at, *u0 = Ud + kb * cfg::LDU + 4 * cgb;
 #pragma unroll 8
       for (int i = 0; i < kC / KB; ++i) {
-        const float4 kv = ld4(k0 + KB * i * LD), uv = ld4(u0 + KB * i * cfg::LDU);
+        // token kb + KB i: its row's chunks are exchanged by its last three bits
+        const float4 kv = ld4(k0 + KB * i * 32 + ((k_chunk ^ ((KB * i) & 7)) << 2)), uv = ld4(u0 + KB * i * cfg::LDU);
         fma4(acc[0], kv.x, uv); fma4(acc[1], kv.y, uv); fma4(acc[2], kv.z, uv); fma4(acc[3], kv.w, uv);
       }
       float v[16];
@@ -228,6 +252,12 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) scan_f32_chain(Sca
       share_state();
       put_state(slot);
     }
+  }
+  if (bad) {   // the copies still on their way get a bounded chance to land before the CTA's shared memory is given up
+    atomicMax(p.status, TRI_INV_ERR_DEVICE_TIMEOUT);
+    if (tid == 0 && (smem_u32(sm) & 1023u) == 0)
+      for (int c = n_chunks > cfg::kStages ? n_chunks - cfg::kStages : 0; c < n_chunks; ++c)
+        mbar_wait_bounded(bars + 8 * (c % cfg::kStages), (uint32_t)(c / cfg::kStages) & 1u, p.wait_limit_ns ? p.wait_limit_ns : kWaitLimitNs);
   }
   if (a.c0 + n_chunks < n_all) put_state(a.carry + state_base);
   else if (p.S_out) put_state(p.S_out + state_base);
@@ -347,17 +377,32 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 3 : 1) scan_f32_output(Sc
 }
 
 template <int DK, int NS>
-cudaError_t launch_chain(const ScanParams& p, const F32Args& a, long long pairs, cudaStream_t stream) {
+cudaError_t launch_chain(const CUtensorMap& tmW, const CUtensorMap& tmK, const ScanParams& p, const F32Args& a, long long pairs, cudaStream_t stream) {
   cudaError_t e = cudaFuncSetAttribute(scan_f32_chain<DK, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Chain<DK, NS>::bytes);
   if (e != cudaSuccess) return e;
   const long long grid = pairs * ((a.d_v + NS - 1) / NS);
   if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-  scan_f32_chain<DK, NS><<<(int)grid, kThreads, Chain<DK, NS>::bytes, stream>>>(p, a);
+  scan_f32_chain<DK, NS><<<(int)grid, kThreads, Chain<DK, NS>::bytes, stream>>>(tmW, tmK, p, a);
   return cudaGetLastError();
 }
 
+// 3-D view [tokens, H, d] of an fp32 tensor, one box = 32 features (128 bytes, swizzled) of one head x 64 tokens; features past d are
+// outside the tensor and read as zeros.
+bool make_tmap_heads(CUtensorMap* tm, const float* base, long long tokens, int H, int d) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[3] = {(cuuint64_t)d, (cuuint64_t)H, (cuuint64_t)tokens};
+  cuuint64_t strides[2] = {(cuuint64_t)d * 4, (cuuint64_t)H * d * 4};
+  cuuint32_t box[3] = {32, 1, (cuuint32_t)kC};
+  cuuint32_t estr[3] = {1, 1, 1};
+  return fn(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 template <int DK>
-cudaError_t launch_segments(const ScanParams& p, F32Args a, int max_chunks, cudaStream_t stream) {
+cudaError_t launch_segments(const ScanParams& p, F32Args a, int max_chunks, long long tokens, cudaStream_t stream) {
+  CUtensorMap tmW, tmK;
+  if (!make_tmap_heads(&tmW, a.W, tokens, p.H, a.d_k) || !make_tmap_heads(&tmK, a.K, tokens, p.H, a.d_k)) return cudaErrorUnknown;
   cudaError_t e = cudaFuncSetAttribute(scan_f32_output<DK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Output<DK>::bytes);
   if (e != cudaSuccess) return e;
   const long long pairs = (long long)p.n_seqs * p.H;
@@ -365,7 +410,7 @@ cudaError_t launch_segments(const ScanParams& p, F32Args a, int max_chunks, cuda
   // W and K half as often
   const bool wide = pairs * ((a.d_v + 7) / 8) > 2 * 148;
   for (a.c0 = 0; a.c0 == 0 || a.c0 < max_chunks; a.c0 += a.n_seg) {
-    e = wide ? launch_chain<DK, 16>(p, a, pairs, stream) : launch_chain<DK, 8>(p, a, pairs, stream);
+    e = wide ? launch_chain<DK, 16>(tmW, tmK, p, a, pairs, stream) : launch_chain<DK, 8>(tmW, tmK, p, a, pairs, stream);
     if (e != cudaSuccess) return e;
     if (max_chunks == 0) break;
     const long long grid = pairs * a.n_seg * ((a.d_v + kNV - 1) / kNV);
@@ -388,10 +433,10 @@ size_t chunk_scan_f32_scratch(long long pairs, int max_chunks, int d_k, int d_v,
 }
 
 cudaError_t launch_chunk_scan_f32(const ScanParams& p, const void* Q, const void* K, const void* W, int d_k, int d_v, int max_chunks,
-                                  void* scratch, int n_seg, cudaStream_t stream) {
+                                  long long tokens, void* scratch, int n_seg, cudaStream_t stream) {
   F32Args a{(const float*)Q, (const float*)K, (const float*)W, (const float*)p.U, d_k, d_v, (float*)scratch, nullptr, 0, n_seg};
   a.carry = a.slots + (size_t)p.n_seqs * p.H * n_seg * (size_t)(d_k + kC) * d_v;
-  return d_k <= 64 ? launch_segments<64>(p, a, max_chunks, stream) : launch_segments<128>(p, a, max_chunks, stream);
+  return d_k <= 64 ? launch_segments<64>(p, a, max_chunks, tokens, stream) : launch_segments<128>(p, a, max_chunks, tokens, stream);
 }
 
 }  // namespace tri_inv
