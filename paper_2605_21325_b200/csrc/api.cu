@@ -324,7 +324,7 @@ int chunk_scan_any(const void* Q, const void* K, const void* W, const void* U, c
       const int max_chunks = (max_len + 63) / 64;
       const size_t bytes = chunk_scan_f32_scratch((long long)p.n_seqs * p.H, max_chunks, desc->d_k, desc->d_v, &n_seg);
       cudaMemPool_t pool = table_pool_for_current_device();
-      if (pool && cudaMallocFromPoolAsync(&work, bytes, pool, stream) == cudaSuccess) {
+      if (bytes == 0 || (pool && cudaMallocFromPoolAsync(&work, bytes, pool, stream) == cudaSuccess)) {
         err = launch_chunk_scan_f32(p, Q, K, W, desc->d_k, desc->d_v, max_chunks, tokens > 0 ? tokens : 1, work, n_seg, stream);
       } else {   // no scratch to be had: the kernel that needs none
         (void)cudaGetLastError();

@@ -49,12 +49,11 @@ __global__ void __launch_bounds__(kThreads, DT == 64 ? 4 : 2) f32_factors_kernel
     // bounds-checking build: an item outside the tensors is reduced to no rows (nothing of it is then read or stored)
     if (!TRI_INV_CHECK(p, rows >= 1 && rows <= C && tok0 >= 0 && (long long)tok0 + rows <= p.n_tokens && h >= 0 && h < p.H)) { tok0 = 0; rows = 0; h = 0; }
     if (item != (int)blockIdx.x) __syncthreads();   // the last matrix's readers are done with shared memory
-    auto copy_rows = [&](float* dst, const void* src, int d) {   // rows past the chunk and columns past d become zeros
+    auto copy_rows = [&](float* dst, const void* src, int d) {   // rows past the chunk become zeros, columns past d are left alone
 #pragma unroll
       for (int m = 0; m < C * DT / 4 / kThreads; ++m) {
         const int e = tid + m * kThreads, j = e / (DT / 4), c = 4 * (e % (DT / 4));
-        const bool ok = j < rows && c < d;
-        cp_async16(dst + j * LD + c, (const float*)src + (ok ? ((size_t)(tok0 + j) * p.H + h) * d + c : 0), ok);
+        if (c < d) cp_async16(dst + j * LD + c, (const float*)src + (j < rows ? ((size_t)(tok0 + j) * p.H + h) * d + c : 0), j < rows);
       }
       cp_commit();
     };
@@ -69,8 +68,14 @@ __global__ void __launch_bounds__(kThreads, DT == 64 ? 4 : 2) f32_factors_kernel
     // ---- Gram matrix and gate: N where i > j, in the blocks on and below the diagonal
     {
       float acc[4][4] = {};
+      if (rows <= 16) {   // one block only
+        for (int k = 0; k < p.d_k; k += 4) {
+          const float4 q = ld4(Ks + ty * LD + k), kv = ld4(Ks + tx * LD + k);
+          acc[0][0] = fmaf(q.w, kv.w, fmaf(q.z, kv.z, fmaf(q.y, kv.y, fmaf(q.x, kv.x, acc[0][0]))));
+        }
+      } else
 #pragma unroll 2
-      for (int k = 0; k < DT; k += 4) {
+      for (int k = 0; k < p.d_k; k += 4) {
         float4 q[4];
 #pragma unroll
         for (int a = 0; a < 4; ++a) q[a] = ld4(Ks + (ty + 16 * a) * LD + k);
@@ -120,6 +125,7 @@ __global__ void __launch_bounds__(kThreads, DT == 64 ? 4 : 2) f32_factors_kernel
       // ---- meanwhile: row j of K times beta_j (times exp g_j for the decay-weighted W), row j of V times beta_j
       for (int e = tid - 128; e < C * DT / 4; e += 128) {
         const int j = e / (DT / 4), c = 4 * (e % (DT / 4));
+        if (j >= rows) break;
         const float b = sb[j], f = (p.ops & kWDecay) ? b * ((gshift && j == 0) ? 1.f : expf(sg[j - gshift])) : b;
         float4* kp = reinterpret_cast<float4*>(Ks + j * LD + c);
         float4* vp = reinterpret_cast<float4*>(Vs + j * LD + c);
@@ -129,8 +135,8 @@ __global__ void __launch_bounds__(kThreads, DT == 64 ? 4 : 2) f32_factors_kernel
       }
     }
     __syncthreads();
-    // ---- merges X21 = -(X22 N21) X11, both products into registers and then over N21
-    {
+    // ---- merges X21 = -(X22 N21) X11, both products into registers and then over N21 (none where the rows are padding)
+    if (rows > 16) {
       // blocks of 16: two pairs, a thread has two neighbouring elements of a row
       const int r0 = 32 * (tid >> 7) + 16, c0 = r0 - 16, i = (tid >> 3) & 15, j = 2 * (tid & 7);
       float* out = M + (r0 + i) * LDM + c0 + j;
@@ -164,7 +170,7 @@ __global__ void __launch_bounds__(kThreads, DT == 64 ? 4 : 2) f32_factors_kernel
       *reinterpret_cast<float2*>(out) = make_float2(-s0, -s1);
       __syncthreads();
     }
-    {
+    if (rows > 32) {
       // blocks of 32: one pair, four neighbouring elements of a row
       const int i = tid >> 3, j = 4 * (tid & 7);
       float* out = M + (32 + i) * LDM + j;
@@ -231,6 +237,7 @@ __global__ void __launch_bounds__(kThreads, DT == 64 ? 4 : 2) f32_factors_kernel
         float o[4][4] = {};
 #pragma unroll
         for (int b = 0; b < 4; ++b) {
+          if (16 * b >= rows) break;
           const float *t0 = tile + 16 * b * LD, *a0 = M + ty * LDM + 16 * b;
 #pragma unroll 2
           for (int j = 0; j < 16; j += 4) {

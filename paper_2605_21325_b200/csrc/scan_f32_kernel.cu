@@ -5,6 +5,7 @@
 //                     and leaves U~ and the state that ENTERS each chunk in scratch memory.
 //   scan_f32_output   one CTA per (sequence, head, chunk, 64 value columns), all chunks at once:
 //                       P = (Q K^T) decay,   O = scale (gamma Q S + P U~).
+// (Sequences of one chunk take one kernel, scan_f32_one_chunk.)
 // The scratch of a call is bounded (kScratchBytes): longer inputs go through in segments of chunks, a pair of launches each,
 // the state carried in scratch between them.
 //
@@ -146,9 +147,11 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) scan_f32_chain(con
   auto copy_tiles = [&](int c) {   // by one thread; features past d_k are filled with zeros, rows past the sequence's end hold what follows
     const int st = c % cfg::kStages, tok0 = beg + (a.c0 + c) * kC;
     const uint32_t dst = smem_u32(tiles + st * 2 * cfg::TILE), bar = bars + 8 * st;
-    mbar_expect_tx(bar, 2 * cfg::TILE * 4);
+    const int boxes = (a.d_k + 31) / 32;
+    mbar_expect_tx(bar, 2 * boxes * cfg::BOX * 4);
 #pragma unroll
     for (int b = 0; b < DK / 32; ++b) {
+      if (b >= boxes) break;
       tma_load_3d(dst + b * cfg::BOX * 4, &tmW, bar, 32 * b, h, tok0);
       tma_load_3d(dst + (cfg::TILE + b * cfg::BOX) * 4, &tmK, bar, 32 * b, h, tok0);
     }
@@ -205,6 +208,7 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) scan_f32_chain(con
       const float* s0 = S + ka * cfg::S_BLK + 4 * cga;
 #pragma unroll
       for (int i = 0; i < DK / 4 / KA; ++i) {
+        if (4 * KA * i >= a.d_k) break;
         // features 4 (ka + KA i) ..: box (ka + KA i) / 8, chunk (ka + KA i) % 8 of its rows
         const float* wb = Ws + (KA * i / 8) * cfg::BOX;
         constexpr int kFlip = KA == 4 ? 16 : 0;
@@ -234,6 +238,7 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) scan_f32_chain(con
     {
       float acc[4][4] = {};
       const float *k0 = Ks + k_at, *u0 = Ud + kb * cfg::LDU + 4 * cgb;
+      if (4 * fg < a.d_k)
 #pragma unroll 8
       for (int i = 0; i < kC / KB; ++i) {
         // token kb + KB i: its row's chunks are exchanged by its last three bits
@@ -307,7 +312,7 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 3 : 1) scan_f32_output(Sc
   {
     float acc[4][4] = {};
 #pragma unroll 2
-    for (int k = 0; k < DK; k += 4) {
+    for (int k = 0; k < a.d_k; k += 4) {
       float4 q[4];
 #pragma unroll
       for (int i = 0; i < 4; ++i) q[i] = ld4(Qs + (ty + 16 * i) * LD + k);
@@ -334,7 +339,7 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 3 : 1) scan_f32_output(Sc
   {
     const float* sc = Ss + 4 * tx;
 #pragma unroll 2
-    for (int k = 0; k < DK; k += 4) {
+    for (int k = 0; k < a.d_k; k += 4) {
       const float4 s0 = ld4(sc + k * LDV), s1 = ld4(sc + (k + 1) * LDV), s2 = ld4(sc + (k + 2) * LDV), s3 = ld4(sc + (k + 3) * LDV);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -376,6 +381,156 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 3 : 1) scan_f32_output(Sc
   }
 }
 
+// Sequences of at most one chunk: nothing is walked, so both steps in one kernel, without scratch.  One CTA per (sequence, head, 16 value
+// columns).  Measured (graph of calls, B = 1, H = 20, d = 64): 8.8 us, 13.0 as two kernels; T = 1: 7.3 and 12.0.
+constexpr int kNS1 = 16, kLdU1 = 24;
+template <int DK>
+struct OneChunk {
+  static constexpr int LD = DK + 4;
+  static constexpr int JG = DK == 64 ? 4 : 2;                 // token groups of the state's product: (DK / 4) x 4 x JG threads
+  static constexpr int floats = 3 * kC * LD + DK * kNS1 + 2 * kC * kLdU1 + kC * kLdP + kC;
+  static constexpr size_t bytes = floats * sizeof(float);
+};
+
+template <int DK>
+__global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) scan_f32_one_chunk(const __grid_constant__ ScanParams p, const __grid_constant__ F32Args a) {
+  using cfg = OneChunk<DK>;
+  constexpr int LD = cfg::LD, JG = cfg::JG;
+  extern __shared__ __align__(16) float sm[];
+  float *Ws = sm, *Qs = Ws + kC * LD, *Ks = Qs + kC * LD, *S = Ks + kC * LD, *Ut = S + DK * kNS1, *Ud = Ut + kC * kLdU1, *P = Ud + kC * kLdU1, *sg = P + kC * kLdP;
+  const int tid = threadIdx.x;
+  const int n_slices = (a.d_v + kNS1 - 1) / kNS1;
+  const int slice = blockIdx.x % n_slices, pair = blockIdx.x / n_slices, h = pair % p.H, s = pair / p.H;
+  const int beg = p.seq_off ? p.seq_off[s] : s * p.T;
+  const int rows = (p.seq_off ? p.seq_off[s + 1] : (s + 1) * p.T) - beg;   // 0 .. 64
+  const int col0 = slice * kNS1;
+  const size_t state_base = (size_t)pair * a.d_k * a.d_v;
+  if (rows > 0) {
+    copy_rows<DK, LD>(Ws, a.W, beg, rows, p.H, h, a.d_k, tid);
+    copy_rows<DK, LD>(Qs, a.Q, beg, rows, p.H, h, a.d_k, tid);
+    cp_commit();
+    copy_rows<DK, LD>(Ks, a.K, beg, rows, p.H, h, a.d_k, tid);
+    cp_commit();
+    if (tid < kC) sg[tid] = p.g[(size_t)(beg + (tid < rows ? tid : rows - 1)) * p.H + h];   // rows past the end take the last real row's
+  }
+  // state slice: rows past d_k and columns past d_v stay zero throughout
+  for (int e = tid; e < DK * kNS1; e += kThreads) {
+    const int k = e / kNS1, n = e % kNS1;
+    S[e] = (p.S0 && k < a.d_k && col0 + n < a.d_v) ? p.S0[state_base + (size_t)k * a.d_v + col0 + n] : 0.f;
+  }
+  if (rows > 0) {
+    const int nq = tid & 3, r = tid >> 2;
+    const int ty = ((tid & 31) >> 2) + 8 * ((tid >> 5) & 1), tx = (tid & 3) + 4 * (tid >> 6);
+    const bool col_in = col0 + 4 * nq < a.d_v;
+    const float4 u = (r < rows && col_in) ? ld4(a.U + ((size_t)(beg + r) * p.H + h) * a.d_v + col0 + 4 * nq) : make_float4(0.f, 0.f, 0.f, 0.f);
+    cp_wait<1>();
+    __syncthreads();
+    // ---- W S and Q S: row r, four columns
+    float ws[4] = {0.f, 0.f, 0.f, 0.f}, qs[4] = {0.f, 0.f, 0.f, 0.f};
+    {
+      const float *wr = Ws + r * LD, *qr = Qs + r * LD, *sc = S + 4 * nq;
+      if (p.S0)
+#pragma unroll 4
+      for (int k = 0; k < a.d_k; k += 4) {
+        const float4 w = ld4(wr + k), q = ld4(qr + k);
+        const float4 s0 = ld4(sc + k * kNS1), s1 = ld4(sc + (k + 1) * kNS1), s2 = ld4(sc + (k + 2) * kNS1), s3 = ld4(sc + (k + 3) * kNS1);
+        fma4(ws, w.x, s0); fma4(qs, q.x, s0);
+        fma4(ws, w.y, s1); fma4(qs, q.y, s1);
+        fma4(ws, w.z, s2); fma4(qs, q.z, s2);
+        fma4(ws, w.w, s3); fma4(qs, q.w, s3);
+      }
+      const float f = expf(sg[rows - 1] - sg[r]);
+      float4 t = make_float4(u.x - ws[0], u.y - ws[1], u.z - ws[2], u.w - ws[3]);
+      if (r >= rows) t = make_float4(0.f, 0.f, 0.f, 0.f);
+      *reinterpret_cast<float4*>(Ut + r * kLdU1 + 4 * nq) = t;
+      *reinterpret_cast<float4*>(Ud + r * kLdU1 + 4 * nq) = make_float4(t.x * f, t.y * f, t.z * f, t.w * f);
+    }
+    cp_wait<0>();
+    __syncthreads();
+    // ---- P: element (ty, tx) of the 16 x 16 blocks on and below the diagonal
+    {
+      float acc[4][4] = {};
+#pragma unroll 2
+      for (int k = 0; k < a.d_k; k += 4) {
+        float4 q[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) q[i] = ld4(Qs + (ty + 16 * i) * LD + k);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float4 kv = ld4(Ks + (tx + 16 * j) * LD + k);
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (i >= j) acc[i][j] = fmaf(q[i].w, kv.w, fmaf(q[i].z, kv.z, fmaf(q[i].y, kv.y, fmaf(q[i].x, kv.x, acc[i][j]))));
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j <= i; ++j) {
+          const int ri = ty + 16 * i, cj = tx + 16 * j;
+          P[ri * kLdP + cj] = cj <= ri ? acc[i][j] * expf(sg[ri] - sg[cj]) : 0.f;
+        }
+    }
+    __syncthreads();
+    // ---- O
+    if (r < rows && col_in) {
+      const float gam = expf(sg[r]);
+      float o[4] = {gam * qs[0], gam * qs[1], gam * qs[2], gam * qs[3]};
+      const float *pr = P + r * kLdP, *uc = Ut + 4 * nq;
+      int j = 0;
+#pragma unroll 2
+      for (; j + 3 <= r; j += 4) {
+        const float4 pv = ld4(pr + j);
+        fma4(o, pv.x, ld4(uc + j * kLdU1));
+        fma4(o, pv.y, ld4(uc + (j + 1) * kLdU1));
+        fma4(o, pv.z, ld4(uc + (j + 2) * kLdU1));
+        fma4(o, pv.w, ld4(uc + (j + 3) * kLdU1));
+      }
+      for (; j <= r; ++j) fma4(o, pr[j], ld4(uc + j * kLdU1));
+      *reinterpret_cast<float4*>((float*)p.O + ((size_t)(beg + r) * p.H + h) * a.d_v + col0 + 4 * nq) =
+          make_float4(p.scale * o[0], p.scale * o[1], p.scale * o[2], p.scale * o[3]);
+    }
+    // ---- S: four features x four columns, tokens split over JG lanes
+    const int jg = tid % JG, n4 = (tid / JG) & 3, kq = tid / (4 * JG);
+    float v[16] = {};
+#pragma unroll 4
+    for (int i = 0; i < kC / JG; ++i) {
+      const int j = (i >> 1) * 2 * JG + 2 * jg + (i & 1);   // two neighbouring tokens per lane group: their rows lie in different banks
+      const float4 kv = ld4(Ks + j * LD + 4 * kq), uv = ld4(Ud + j * kLdU1 + 4 * n4);
+      const float k4[4] = {kv.x, kv.y, kv.z, kv.w};
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        v[4 * f] = fmaf(k4[f], uv.x, v[4 * f]); v[4 * f + 1] = fmaf(k4[f], uv.y, v[4 * f + 1]);
+        v[4 * f + 2] = fmaf(k4[f], uv.z, v[4 * f + 2]); v[4 * f + 3] = fmaf(k4[f], uv.w, v[4 * f + 3]);
+      }
+    }
+    const int base = reduce_scatter<JG>(v, jg);
+    const float gl = expf(sg[rows - 1]);
+#pragma unroll
+    for (int i = 0; i < 16 / JG; ++i) {
+      float* sp = S + (4 * kq + (base + i) / 4) * kNS1 + 4 * n4 + ((base + i) & 3);
+      *sp = fmaf(gl, *sp, v[i]);
+    }
+  }
+  if (p.S_out) {
+    __syncthreads();
+    for (int e = tid; e < DK * kNS1; e += kThreads) {
+      const int k = e / kNS1, n = e % kNS1;
+      if (k < a.d_k && col0 + n < a.d_v) p.S_out[state_base + (size_t)k * a.d_v + col0 + n] = S[e];
+    }
+  }
+}
+
+template <int DK>
+cudaError_t launch_one_chunk(const ScanParams& p, const F32Args& a, cudaStream_t stream) {
+  cudaError_t e = cudaFuncSetAttribute(scan_f32_one_chunk<DK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OneChunk<DK>::bytes);
+  if (e != cudaSuccess) return e;
+  const long long grid = (long long)p.n_seqs * p.H * ((a.d_v + kNS1 - 1) / kNS1);
+  if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
+  scan_f32_one_chunk<DK><<<(int)grid, kThreads, OneChunk<DK>::bytes, stream>>>(p, a);
+  return cudaGetLastError();
+}
+
 template <int DK, int NS>
 cudaError_t launch_chain(const CUtensorMap& tmW, const CUtensorMap& tmK, const ScanParams& p, const F32Args& a, long long pairs, cudaStream_t stream) {
   cudaError_t e = cudaFuncSetAttribute(scan_f32_chain<DK, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Chain<DK, NS>::bytes);
@@ -409,10 +564,9 @@ cudaError_t launch_segments(const ScanParams& p, F32Args a, int max_chunks, long
   // eight columns a CTA while that is no more than two CTAs for each SM: half the work on the chain; beyond it the wider slice reads
   // W and K half as often
   const bool wide = pairs * ((a.d_v + 7) / 8) > 2 * 148;
-  for (a.c0 = 0; a.c0 == 0 || a.c0 < max_chunks; a.c0 += a.n_seg) {
+  for (a.c0 = 0; a.c0 < max_chunks; a.c0 += a.n_seg) {
     e = wide ? launch_chain<DK, 16>(tmW, tmK, p, a, pairs, stream) : launch_chain<DK, 8>(tmW, tmK, p, a, pairs, stream);
     if (e != cudaSuccess) return e;
-    if (max_chunks == 0) break;
     const long long grid = pairs * a.n_seg * ((a.d_v + kNV - 1) / kNV);
     if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
     scan_f32_output<DK><<<(int)grid, kThreads, Output<DK>::bytes, stream>>>(p, a);
@@ -429,12 +583,14 @@ size_t chunk_scan_f32_scratch(long long pairs, int max_chunks, int d_k, int d_v,
   long long n = (long long)(kScratchBytes / (slot * (size_t)pairs));
   n = n < 1 ? 1 : n > max_chunks ? (max_chunks < 1 ? 1 : max_chunks) : n;
   *n_seg = (int)n;
+  if (max_chunks <= 1) return 0;
   return (size_t)pairs * ((size_t)n * slot + (n < max_chunks ? state : 0));
 }
 
 cudaError_t launch_chunk_scan_f32(const ScanParams& p, const void* Q, const void* K, const void* W, int d_k, int d_v, int max_chunks,
                                   long long tokens, void* scratch, int n_seg, cudaStream_t stream) {
   F32Args a{(const float*)Q, (const float*)K, (const float*)W, (const float*)p.U, d_k, d_v, (float*)scratch, nullptr, 0, n_seg};
+  if (max_chunks <= 1) return d_k <= 64 ? launch_one_chunk<64>(p, a, stream) : launch_one_chunk<128>(p, a, stream);
   a.carry = a.slots + (size_t)p.n_seqs * p.H * n_seg * (size_t)(d_k + kC) * d_v;
   return d_k <= 64 ? launch_segments<64>(p, a, max_chunks, tokens, stream) : launch_segments<128>(p, a, max_chunks, tokens, stream);
 }
