@@ -11,6 +11,7 @@
 // the kernels 21 / 5), 2048 pairs of one token 150 / 63 us (268 MB of state: 4.3 TB/s); fp32, d = 64: 2048 pairs of 1 / 16 tokens 291 / 316 ->
 // 21.5 / 95 us; d = 128: 993 / 1048 -> 63 / 251 us.
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -26,23 +27,26 @@ struct RecurrenceArgs {
   float* S_out;
   int H, T, d_k, d_v, bf16;
   float scale;
-  int packed, first;                  // sequences of this launch start at `first`
-  int32_t cu[kSeqsPerLaunch + 1];     // packed: their offsets
+  int first;                          // sequences of this launch start at `first`
+};
+struct PackedArgs : RecurrenceArgs {  // (dense calls do not carry four kilobytes of parameters to the device)
+  int32_t cu[kSeqsPerLaunch + 1];     // offsets of the launch's sequences
 };
 
 __device__ __forceinline__ float load_one(const void* p, int bf16, size_t i) {
   return bf16 ? __bfloat162float(((const __nv_bfloat16*)p)[i]) : ((const float*)p)[i];
 }
 
-template <int KR>   // features per warp
-__global__ void __launch_bounds__(kWarps * 32) recurrence_kernel(const __grid_constant__ RecurrenceArgs a) {
+template <int KR, class Args>   // features per warp
+__global__ void __launch_bounds__(kWarps * 32) recurrence_kernel(const __grid_constant__ Args a) {
   __shared__ float sk[kMaxTokens][kWarps * KR], sq[kMaxTokens][kWarps * KR];
   __shared__ float s_alpha[kMaxTokens], s_beta[kMaxTokens], s_kq[kMaxTokens];
   __shared__ float2 part[2][kWarps][kCols];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int n_slices = (a.d_v + kCols - 1) / kCols;
   const int slice = blockIdx.x % n_slices, h = (blockIdx.x / n_slices) % a.H, i = blockIdx.x / (n_slices * a.H), s = a.first + i;
-  const int beg = a.packed ? a.cu[i] : s * a.T, n = a.packed ? a.cu[i + 1] - beg : a.T;   // n <= kMaxTokens (checked on the host)
+  int beg = s * a.T, n = a.T;   // n <= kMaxTokens (checked on the host)
+  if constexpr (std::is_same<Args, PackedArgs>::value) { beg = a.cu[i]; n = a.cu[i + 1] - beg; }
   const int col = slice * kCols + lane;
   const bool in = col < a.d_v;
   const size_t base = ((size_t)s * a.H + h) * a.d_k * a.d_v + col;
@@ -135,21 +139,25 @@ bool recurrence_fits(const tri_inv_desc* d) {
 
 cudaError_t launch_recurrence(const void* Q, const void* K, const void* V, const float* beta, const float* g, const ScanParams& scan,
                               const tri_inv_desc* d, cudaStream_t stream) {
-  RecurrenceArgs a;
+  PackedArgs a;
   a.Q = Q; a.K = K; a.V = V; a.beta = beta; a.g = g; a.S0 = scan.S0; a.O = scan.O; a.S_out = scan.S_out;
   a.H = d->H; a.T = d->T; a.d_k = d->d_k; a.d_v = d->d_v; a.bf16 = d->kv_dtype == TRI_INV_BF16;
   a.scale = scan.scale;
-  a.packed = d->cu_seqlens != nullptr;
+  const bool packed = d->cu_seqlens != nullptr;
   const long long per_seq = (long long)d->H * ((d->d_v + kCols - 1) / kCols);
-  const long long most = std::min<long long>(a.packed ? kSeqsPerLaunch : 0x7fffffffLL, 0x7fffffffLL / per_seq);
+  const long long most = std::min<long long>(packed ? kSeqsPerLaunch : 0x7fffffffLL, 0x7fffffffLL / per_seq);
   if (most < 1) return cudaErrorInvalidValue;
   for (long long s0 = 0; s0 < scan.n_seqs; s0 += most) {
-    const int n = (int)std::min<long long>(most, scan.n_seqs - s0);
+    const int n = (int)std::min<long long>(most, scan.n_seqs - s0), grid = (int)(n * per_seq);
     a.first = (int)s0;
-    if (a.packed)
+    if (packed) {
       for (int q = 0; q <= n; ++q) a.cu[q] = d->cu_seqlens[s0 + q];
-    if (d->d_k <= 64) recurrence_kernel<8><<<(int)(n * per_seq), kWarps * 32, 0, stream>>>(a);
-    else recurrence_kernel<16><<<(int)(n * per_seq), kWarps * 32, 0, stream>>>(a);
+      if (d->d_k <= 64) recurrence_kernel<8, PackedArgs><<<grid, kWarps * 32, 0, stream>>>(a);
+      else recurrence_kernel<16, PackedArgs><<<grid, kWarps * 32, 0, stream>>>(a);
+    } else {
+      if (d->d_k <= 64) recurrence_kernel<8, RecurrenceArgs><<<grid, kWarps * 32, 0, stream>>>(a);
+      else recurrence_kernel<16, RecurrenceArgs><<<grid, kWarps * 32, 0, stream>>>(a);
+    }
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
