@@ -280,7 +280,9 @@ int chunk_scan_any(const void* Q, const void* K, const void* W, const void* U, c
   const long long tokens = desc->cu_seqlens ? (long long)desc->T : (long long)desc->T * desc->B;
   if (p.n_seqs == 0 || (tokens == 0 && !S_out)) return TRI_INV_OK;
   int* dev_off = nullptr;
-  if (desc->cu_seqlens) {
+  size_t control_bytes = 0;
+  const bool kda_one = tc && G && tokens > 0 && kda_scan_fits(desc, &control_bytes);   // makes its own copy of the offsets
+  if (desc->cu_seqlens && !kda_one) {
     cudaMemPool_t pool = table_pool_for_current_device();
     if (!pool || cudaMallocFromPoolAsync((void**)&dev_off, (size_t)(p.n_seqs + 1) * sizeof(int), pool, stream) != cudaSuccess) return TRI_INV_ERR_CUDA;
     if (launch_seq_offsets(dev_off, desc, stream) != cudaSuccess) {
@@ -302,7 +304,7 @@ int chunk_scan_any(const void* Q, const void* K, const void* W, const void* U, c
     const size_t slots = (size_t)(tokens / 64) + (size_t)p.n_seqs + 1;
     const size_t vec_bytes = (slots * desc->H * 128 * sizeof(float) + 255) & ~(size_t)255;
     cudaMemPool_t pool = table_pool_for_current_device();
-    if (!pool || cudaMallocFromPoolAsync(&work, 2 * tensor_bytes + 3 * vec_bytes, pool, stream) != cudaSuccess) {
+    if (!pool || cudaMallocFromPoolAsync(&work, 2 * tensor_bytes + 3 * vec_bytes + control_bytes, pool, stream) != cudaSuccess) {
       if (dev_off) cudaFreeAsync(dev_off, stream);
       return TRI_INV_ERR_CUDA;
     }
@@ -312,10 +314,14 @@ int chunk_scan_any(const void* Q, const void* K, const void* W, const void* U, c
     float* ER = reinterpret_cast<float*>(w + 2 * tensor_bytes + vec_bytes);
     float* EX = reinterpret_cast<float*>(w + 2 * tensor_bytes + 2 * vec_bytes);
     p.EL = EL; p.ER = ER; p.EX = EX;
-    err = launch_kda_scan_prep(p, Q, K, Qp, Km, EL, ER, EX, (max_len + 63) / 64, stream);
-    if (err == cudaSuccess) {
-      g_launches.fetch_add(1, std::memory_order_relaxed);
-      err = launch_chunk_scan(p, Qp, Km, W, tokens, stream, true);
+    if (kda_one) {
+      err = launch_kda_scan(p, Q, K, W, Qp, Km, w + 2 * tensor_bytes + 3 * vec_bytes, desc, stream);
+    } else {
+      err = launch_kda_scan_prep(p, Q, K, Qp, Km, EL, ER, EX, (max_len + 63) / 64, stream);
+      if (err == cudaSuccess) {
+        g_launches.fetch_add(1, std::memory_order_relaxed);
+        err = launch_chunk_scan(p, Qp, Km, W, tokens, stream, true);
+      }
     }
   } else {
     const bool f32 = !G && desc->kv_dtype == TRI_INV_F32 && desc->C == 64 && desc->d_k <= 128;

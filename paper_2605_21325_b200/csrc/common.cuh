@@ -139,6 +139,11 @@ cudaError_t launch_recurrence(const void* Q, const void* K, const void* V, const
 // ER = exp(G_ref), EX = exp(G_last - G_ref) ([slots,H,128] fp32), G_ref the middle row of each chunk, G_last its last.
 cudaError_t launch_kda_scan_prep(const ScanParams& p, const void* Q, const void* K, void* Qp, void* Km,
                                  float* EL, float* ER, float* EX, int max_chunks_per_seq, cudaStream_t stream);
+// The two in one kernel, the preparation beside the scan (layer_kernel.cuh): whether that is the faster form, and the bytes of its words
+// (and table, and offsets) in addition to Qp, Km and the vectors; p.EL, ER, EX point to the latter, p.seq_off is not needed.
+bool kda_scan_fits(const tri_inv_desc* d, size_t* control_bytes);
+cudaError_t launch_kda_scan(const ScanParams& p, const void* Q, const void* K, const void* W, void* Qp, void* Km, void* control,
+                            const tri_inv_desc* d, cudaStream_t stream);
 // Single precision with a scalar gate at C = 64 and d_k <= 128 (scan_f32_kernel.cu).
 // Its scratch for this many (sequence, head) pairs and chunks of the longest sequence; *n_seg: chunks that go through at a time.
 size_t chunk_scan_f32_scratch(long long pairs, int max_chunks, int d_k, int d_v, int* n_seg);

@@ -407,6 +407,156 @@ layer_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
 }
 
+// ---------------------------------------------------------------- the per-channel scan beside the preparation of its operands
+// The same split of the chip for tri_inv_chunk_scan_kda: instead of matrices the groups prepare chunks (Q+, K- and the three vectors,
+// the arithmetic of kda_scan_prep_kernel, scan_kda_prep.cu), bound by the bytes they move.
+struct KdaOperands {
+  const __nv_bfloat16 *Q, *K;
+  const float* G;
+  __nv_bfloat16 *Qp, *Km;
+  float *EL, *ER, *EX;
+};
+
+// The chunks of one group, drawn one ahead; `once`: one, and more only if no other CTA has come to prepare them.
+__device__ __forceinline__ void prepare_chunks(const LayerParams& p, const KdaOperands& a, int4* words, int group, bool once) {
+  const int tid = threadIdx.x & 127, r0 = tid >> 4, f0 = 8 * (tid & 15);
+  auto sync = [group]() { asm volatile("bar.sync %0, 128;" ::"r"(group + 1) : "memory"); };
+  int turn = 0;   // two slots in turn: a slow thread may still read the one while the next draw is left in the other
+  auto leave = [&](int x) {
+    Place q{0, 0, 0, 0};
+    if (x < p.total) q = place_of(p, x);
+    words[2 * (turn & 1)] = make_int4(q.tok0, q.rows, q.h, q.slot);
+    words[2 * (turn & 1) + 1].x = x;
+  };
+  auto take = [&](Place& q) -> int {
+    const int4 v = words[2 * (turn & 1)];
+    q = Place{v.x, v.y, v.z, v.w};
+    const int x = words[2 * (turn & 1) + 1].x;
+    ++turn;
+    return x;
+  };
+  Place at, nx;
+  if (tid == 0) leave(atomicAdd(p.counters + 1, 1));
+  sync();
+  int item = take(at);
+  if (tid == 0) leave(once ? p.total : atomicAdd(p.counters + 1, 1));
+  sync();
+  int nx_item = take(nx);
+  while (item < p.total) {
+    int ticket = p.total;
+    if (tid == 0 && nx_item < p.total) ticket = atomicAdd(p.counters + 1, 1);
+    const size_t row0 = ((size_t)at.tok0 * p.H + at.h) * D + f0, stride = (size_t)p.H * D;
+    float gref[8], glast[8];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const float4 x = *reinterpret_cast<const float4*>(a.G + row0 + (size_t)(at.rows >> 1) * stride + 4 * q);
+      const float4 y = *reinterpret_cast<const float4*>(a.G + row0 + (size_t)(at.rows - 1) * stride + 4 * q);
+      gref[4 * q] = x.x * kLog2e; gref[4 * q + 1] = x.y * kLog2e; gref[4 * q + 2] = x.z * kLog2e; gref[4 * q + 3] = x.w * kLog2e;
+      glast[4 * q] = y.x * kLog2e; glast[4 * q + 1] = y.y * kLog2e; glast[4 * q + 2] = y.z * kLog2e; glast[4 * q + 3] = y.w * kLog2e;
+    }
+    if (r0 == 0) {
+      const size_t v = ((size_t)at.slot * p.H + at.h) * D + f0;
+#pragma unroll
+      for (int q = 0; q < 8; q += 4) {
+        *reinterpret_cast<float4*>(a.EL + v + q) = make_float4(ex2_approx(glast[q]), ex2_approx(glast[q + 1]), ex2_approx(glast[q + 2]), ex2_approx(glast[q + 3]));
+        *reinterpret_cast<float4*>(a.ER + v + q) = make_float4(ex2_approx(gref[q]), ex2_approx(gref[q + 1]), ex2_approx(gref[q + 2]), ex2_approx(gref[q + 3]));
+        *reinterpret_cast<float4*>(a.EX + v + q) = make_float4(ex2_approx(glast[q] - gref[q]), ex2_approx(glast[q + 1] - gref[q + 1]),
+                                                               ex2_approx(glast[q + 2] - gref[q + 2]), ex2_approx(glast[q + 3] - gref[q + 3]));
+      }
+    }
+#pragma unroll 1
+    for (int r4 = r0; r4 < at.rows; r4 += 32) {
+      // four rows' loads first, without a branch between them (rows past the chunk: the last one again)
+      uint4 qv[4], kv[4];
+      float4 gv[4][2];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const size_t idx = row0 + (size_t)min(r4 + 8 * m, at.rows - 1) * stride;
+        qv[m] = *reinterpret_cast<const uint4*>(a.Q + idx);
+        kv[m] = *reinterpret_cast<const uint4*>(a.K + idx);
+        gv[m][0] = *reinterpret_cast<const float4*>(a.G + idx);
+        gv[m][1] = *reinterpret_cast<const float4*>(a.G + idx + 4);
+      }
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const float g[8] = {gv[m][0].x, gv[m][0].y, gv[m][0].z, gv[m][0].w, gv[m][1].x, gv[m][1].y, gv[m][1].z, gv[m][1].w};
+        const uint32_t qw[4] = {qv[m].x, qv[m].y, qv[m].z, qv[m].w}, kw[4] = {kv[m].x, kv[m].y, kv[m].z, kv[m].w};
+        uint32_t qo[4], ko[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const float x0 = g[2 * e] * kLog2e - gref[2 * e], x1 = g[2 * e + 1] * kLog2e - gref[2 * e + 1];
+          qo[e] = pack_bf16(__uint_as_float(qw[e] << 16) * ex2_approx(x0), __uint_as_float(qw[e] & 0xffff0000u) * ex2_approx(x1));
+          ko[e] = pack_bf16(__uint_as_float(kw[e] << 16) * ex2_approx(-x0), __uint_as_float(kw[e] & 0xffff0000u) * ex2_approx(-x1));
+        }
+        if (r4 + 8 * m < at.rows) {
+          const size_t idx = row0 + (size_t)(r4 + 8 * m) * stride;
+          *reinterpret_cast<uint4*>(a.Qp + idx) = make_uint4(qo[0], qo[1], qo[2], qo[3]);
+          *reinterpret_cast<uint4*>(a.Km + idx) = make_uint4(ko[0], ko[1], ko[2], ko[3]);
+        }
+      }
+    }
+    asm volatile("fence.proxy.async;" ::: "memory");   // ordinary stores, read by the scans' tile copies
+    if (tid == 0) leave(ticket);
+    sync();
+    if (tid == 0) asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p.ready + ((size_t)at.slot * p.H + at.h)), "r"(kReady) : "memory");
+    item = nx_item;
+    at = nx;
+    nx_item = take(nx);
+    if (once && item >= p.total && *(volatile int*)(p.counters + 3) == 0) {
+      if (tid == 0) leave(atomicAdd(p.counters + 1, 1));
+      sync();
+      item = take(at);
+    }
+  }
+}
+
+// as many threads as the walk has warps, whose 128-column form needs the registers; three groups prepare
+constexpr int kKdaThreads = (kCopy + 1) * 32, kKdaGroups = 3;
+template <int DVS>
+struct KdaScanCfg {
+  static constexpr int OFF_WORDS = (ScanCfg<DVS, true>::OFF_BAR + 160 + 15) / 16 * 16;
+  static constexpr int SMEM = OFF_WORDS + kKdaGroups * 64 + 16;
+};
+static_assert(KdaScanCfg<128>::SMEM <= 232448, "one CTA per SM");
+
+template <int DVS>
+__global__ void __launch_bounds__(kKdaThreads, 1)
+kda_scan_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmW,
+                const __grid_constant__ CUtensorMap tmU, const __grid_constant__ LayerParams p, const __grid_constant__ KdaOperands a,
+                const __grid_constant__ ScanParams sp) {
+  constexpr int NS = D / DVS;
+  extern __shared__ __align__(1024) uint8_t smem[];
+  int* s_word = reinterpret_cast<int*>(smem + KdaScanCfg<DVS>::SMEM - 16);
+  const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0);
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_word + 1)), "r"(512) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  if (threadIdx.x == 32) *s_word = atomicAdd(p.counters, 1);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = __shfl_sync(0xffffffffu, s_word[1], 0);
+  const int arrival = __shfl_sync(0xffffffffu, *s_word, 0);
+  unsigned smid;
+  asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
+  const bool scans_first = arrival >= p.sms || (int)smid >= p.factor_ctas;
+  if (!scans_first && threadIdx.x == 0) atomicAdd(p.counters + 3, 1);
+  if (warp < 4 * kKdaGroups)
+    prepare_chunks(p, a, reinterpret_cast<int4*>(smem + KdaScanCfg<DVS>::OFF_WORDS) + 4 * (warp >> 2), warp >> 2, scans_first);
+  __syncthreads();
+  if (threadIdx.x == 0) *s_word = atomicAdd(p.counters + 2, 1);
+  __syncthreads();
+  const int task = __shfl_sync(0xffffffffu, *s_word, 0);
+  if (task < p.scan_tasks) {
+    const int slice = task % NS, pair = task / NS;
+    scan_walk<DVS, true, true>(tmW, tmQ, tmK, tmU, sp, smem, pair / p.H, pair % p.H, slice, false, p.ready, tmem);
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+}
+
 // Before the layer kernel: its words at zero, and for packed sequences the chunks in build order and the device copy of cu_seqlens.
 // Sequences go in groups of `group` (those walked at the same time), and within a group chunk by chunk.
 constexpr int kSeqsPerPrep = 960;
@@ -499,6 +649,26 @@ Split choose_split(long long pairs, int longest, long long entries, int H, int s
   return best;
 }
 
+// The same for the per-channel scan.  Two launches / here (width, scan CTAs): 16 x 64: 95 / 91 (32, 64)   32 x 64: 119 / 104 (64, 64)
+//   48 x 64: 138 / 133 (128, 48)   64 x 64: 152 / 162 (128, 64)   75 x 64: 193 / 206 (128, 75)   8 x 128: 161 / 157 (32, 32)
+//   32 x 512: 884 / 651 (64, 64)   16 x 6: 19 / 25
+// A group prepares a chunk in about 9 us, three of them an SM (0.33 a us; the preparation by itself keeps eight CTAs an SM in flight
+// and reaches 69 chunks a us on the whole chip), so the gain is where the chain is long.
+Split choose_kda_split(long long pairs, int longest, long long entries, int H, int sms) {
+  const struct { int dvs; float here_us, alone_us; } width[3] = {{128, 1.95f, 1.9f}, {64, 1.25f, 1.27f}, {32, 1.16f, 1.15f}};
+  const float items = (float)entries * (float)H;
+  const auto& alone = width[pairs * 8 <= sms ? 2 : pairs * 2 <= sms ? 1 : 0];
+  float best_us = 10.f + items / 69.f + (float)longest * alone.alone_us;   // (only compared where all scans run at the same time)
+  Split best{0, 0};
+  for (const auto& w : width) {
+    const long long tasks = pairs * (D / w.dvs);
+    if (tasks > sms * 3 / 4) continue;
+    const float us = std::max(17.f + (float)longest * w.here_us, 12.f + items / (0.33f * (float)(sms - tasks)));
+    if (us < best_us) { best_us = us; best = Split{w.dvs, (int)tasks}; }
+  }
+  return best;
+}
+
 int longest_of(const tri_inv_desc* d) {
   int n = d->T;
   if (d->cu_seqlens) {
@@ -510,6 +680,49 @@ int longest_of(const tri_inv_desc* d) {
 
 Split split_of(const tri_inv_desc* d, const Layout& l, int sms) {
   return choose_split((long long)(d->cu_seqlens ? d->n_seqs : d->B) * d->H, longest_of(d), l.entries, d->H, sms);
+}
+
+// What both kernels' roles go by.
+void fill_params(LayerParams& p, const tri_inv_desc* d, const Layout& l, char* ws, const ScanParams& sp, const Split& split, int sms) {
+  p.counters = reinterpret_cast<int*>(ws + l.words);
+  p.ready = reinterpret_cast<uint32_t*>(ws + l.words) + 64;
+  p.status = sp.status;
+  p.H = d->H; p.T = d->T;
+  p.pairs = sp.n_seqs * d->H;
+  p.chunks = (d->T + C - 1) / C;
+  p.total = (int)(l.entries * d->H);
+  p.wait_limit_ns = sp.wait_limit_ns ? sp.wait_limit_ns : kWaitLimitNs;
+  p.factor_ctas = sms - split.scans;
+  p.sms = sms;
+  p.groups = kGroups * p.factor_ctas;
+  p.scan_tasks = p.pairs * (D / split.dvs);
+  p.wave = std::max(1, split.scans / (D / split.dvs));
+}
+
+// The words, the table and the offsets of a call's workspace (the last two for packed sequences); p.tab and sp.seq_off point to them.
+cudaError_t launch_prep(const tri_inv_desc* d, const Layout& l, char* ws, int sms, LayerParams& p, ScanParams& sp, cudaStream_t stream) {
+  PrepArgs a;
+  a.words = reinterpret_cast<uint32_t*>(p.counters);
+  a.n_words = l.n_words;
+  a.tab = nullptr; a.seq_off = nullptr; a.n = a.first = a.base = 0; a.group = 1;
+  const int blocks = (int)std::min<long long>(sms, (l.n_words + 255) / 256);
+  if (!d->cu_seqlens) {
+    layer_prep_kernel<<<blocks, 256, 0, stream>>>(a);
+  } else {
+    p.tab = a.tab = reinterpret_cast<LayerEntry*>(ws + l.tab);
+    sp.seq_off = a.seq_off = reinterpret_cast<int*>(ws + l.seq);
+    a.group = std::max(1, std::min(kSeqsPerPrep, (p.wave + d->H - 1) / d->H));
+    const int per = kSeqsPerPrep / a.group * a.group;   // whole groups per launch
+    for (int s0 = 0; s0 < d->n_seqs; s0 += per) {
+      a.first = s0;
+      a.n = std::min(per, d->n_seqs - s0);
+      for (int q = 0; q <= a.n; ++q) a.cu[q] = d->cu_seqlens[s0 + q];
+      layer_prep_kernel<<<std::max(blocks, std::min(a.n, sms)), 256, 0, stream>>>(a);
+      for (int q = 0; q < a.n; ++q) a.base += (a.cu[q + 1] - a.cu[q] + C - 1) / C;
+      a.n_words = 0;
+    }
+  }
+  return cudaGetLastError();
 }
 
 template <int DVS>
@@ -554,22 +767,10 @@ cudaError_t launch_layer(const void* Q, const void* K, const void* V, const floa
   LayerParams p{};
   p.beta = beta; p.g = g;
   p.W = reinterpret_cast<__nv_bfloat16*>(ws + l.w); p.U = reinterpret_cast<__nv_bfloat16*>(ws + l.u);
-  p.counters = reinterpret_cast<int*>(ws + l.words);
-  p.ready = reinterpret_cast<uint32_t*>(ws + l.words) + 64;
-  p.status = sp.status;
-  p.H = d->H; p.T = d->T;
-  p.pairs = sp.n_seqs * d->H;
-  p.chunks = (d->T + C - 1) / C;
-  p.total = (int)(l.entries * d->H);
-  p.wait_limit_ns = sp.wait_limit_ns ? sp.wait_limit_ns : kWaitLimitNs;
   sp.U = p.U;
   const Split split = split_of(d, l, sms);
   if (split.scans == 0) return cudaErrorInvalidValue;
-  p.factor_ctas = sms - split.scans;
-  p.sms = sms;
-  p.groups = kGroups * p.factor_ctas;
-  p.scan_tasks = p.pairs * (D / split.dvs);
-  p.wave = std::max(1, split.scans / (D / split.dvs));
+  fill_params(p, d, l, ws, sp, split, sms);
 
   CUtensorMap tm[7];
   if (!make_tmap(&tm[0], Q, tokens, d->H, D, C) || !make_tmap(&tm[1], K, tokens, d->H, D, C) || !make_tmap(&tm[2], V, tokens, d->H, D, C) ||
@@ -577,33 +778,71 @@ cudaError_t launch_layer(const void* Q, const void* K, const void* V, const floa
       !make_tmap(&tm[5], p.W, tokens, d->H, D, 16) || !make_tmap(&tm[6], p.U, tokens, d->H, D, 16))
     return cudaErrorUnknown;
 
-  PrepArgs a;
-  a.words = reinterpret_cast<uint32_t*>(p.counters);
-  a.n_words = l.n_words;
-  a.tab = nullptr; a.seq_off = nullptr; a.n = a.first = a.base = 0; a.group = 1;
-  const int blocks = (int)std::min<long long>(sms, (l.n_words + 255) / 256);
-  if (!d->cu_seqlens) {
-    layer_prep_kernel<<<blocks, 256, 0, stream>>>(a);
-  } else {
-    p.tab = a.tab = reinterpret_cast<LayerEntry*>(ws + l.tab);
-    sp.seq_off = a.seq_off = reinterpret_cast<int*>(ws + l.seq);
-    a.group = std::max(1, std::min(kSeqsPerPrep, (p.wave + d->H - 1) / d->H));
-    const int per = kSeqsPerPrep / a.group * a.group;   // whole groups per launch
-    for (int s0 = 0; s0 < d->n_seqs; s0 += per) {
-      a.first = s0;
-      a.n = std::min(per, d->n_seqs - s0);
-      for (int q = 0; q <= a.n; ++q) a.cu[q] = d->cu_seqlens[s0 + q];
-      layer_prep_kernel<<<std::max(blocks, std::min(a.n, sms)), 256, 0, stream>>>(a);
-      for (int q = 0; q < a.n; ++q) a.base += (a.cu[q + 1] - a.cu[q] + C - 1) / C;
-      a.n_words = 0;
-    }
-  }
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if ((e = launch_prep(d, l, ws, sms, p, sp, stream)) != cudaSuccess) return e;
   const int grid = std::max(sms, p.scan_tasks);   // a CTA walks once
   switch (split.dvs) {
     case 32: return launch_width<32>(tm, p, sp, grid, dev, stream);
     case 64: return launch_width<64>(tm, p, sp, grid, dev, stream);
     default: return launch_width<128>(tm, p, sp, grid, dev, stream);
+  }
+}
+
+bool kda_scan_fits(const tri_inv_desc* d, size_t* control_bytes) {
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
+  const Layout l = layout_of(d);
+  if (l.entries * d->H > 0x7fffffffLL || choose_kda_split((long long)(d->cu_seqlens ? d->n_seqs : d->B) * d->H, longest_of(d), l.entries, d->H, sms).scans == 0)
+    return false;
+  *control_bytes = l.w;
+  return true;
+}
+
+namespace {
+template <int DVS>
+cudaError_t launch_kda_width(const CUtensorMap (&tm)[4], const LayerParams& p, const KdaOperands& a, const ScanParams& sp, int grid, int dev, cudaStream_t stream) {
+  static std::mutex mu;
+  static bool ready[64] = {false};
+  {
+    std::lock_guard<std::mutex> lock(mu);
+    if (!ready[dev]) {
+      cudaError_t e;
+      if ((e = cudaFuncSetAttribute(kda_scan_kernel<DVS>, cudaFuncAttributeMaxDynamicSharedMemorySize, KdaScanCfg<DVS>::SMEM)) != cudaSuccess) return e;
+      if ((e = cudaFuncSetAttribute(kda_scan_kernel<DVS>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared)) != cudaSuccess) return e;
+      ready[dev] = true;
+    }
+  }
+  kda_scan_kernel<DVS><<<grid, kKdaThreads, KdaScanCfg<DVS>::SMEM, stream>>>(tm[0], tm[1], tm[2], tm[3], p, a, sp);
+  return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t launch_kda_scan(const ScanParams& scan, const void* Q, const void* K, const void* W, void* Qp, void* Km, void* control,
+                            const tri_inv_desc* d, cudaStream_t stream) {
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  const Layout l = layout_of(d);
+  char* ws = reinterpret_cast<char*>(control);
+  ScanParams sp = scan;
+  LayerParams p{};
+  const Split split = choose_kda_split((long long)sp.n_seqs * d->H, longest_of(d), l.entries, d->H, sms);
+  if (split.scans == 0) return cudaErrorInvalidValue;
+  fill_params(p, d, l, ws, sp, split, sms);
+  const KdaOperands a{(const __nv_bfloat16*)Q, (const __nv_bfloat16*)K, sp.G, (__nv_bfloat16*)Qp, (__nv_bfloat16*)Km,
+                      const_cast<float*>(sp.EL), const_cast<float*>(sp.ER), const_cast<float*>(sp.EX)};
+  const long long tokens = d->cu_seqlens ? (long long)d->T : (long long)d->B * d->T;
+  CUtensorMap tm[4];
+  if (!make_tmap(&tm[0], Qp, tokens, d->H, D, C) || !make_tmap(&tm[1], Km, tokens, d->H, D, C) || !make_tmap(&tm[2], W, tokens, d->H, D, C) ||
+      !make_tmap(&tm[3], sp.U, tokens, d->H, D, C))
+    return cudaErrorUnknown;
+  if ((e = launch_prep(d, l, ws, sms, p, sp, stream)) != cudaSuccess) return e;
+  const int grid = std::max(sms, p.scan_tasks);
+  switch (split.dvs) {
+    case 32: return launch_kda_width<32>(tm, p, a, sp, grid, dev, stream);
+    case 64: return launch_kda_width<64>(tm, p, a, sp, grid, dev, stream);
+    default: return launch_kda_width<128>(tm, p, a, sp, grid, dev, stream);
   }
 }
 

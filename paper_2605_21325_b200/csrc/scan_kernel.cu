@@ -180,8 +180,8 @@ __device__ __noinline__ bool wait_by_warp(uint32_t bar, uint32_t parity, unsigne
 }
 
 // One (sequence, head, slice) by a whole CTA; true when a wait has run out in this thread.
-// FED: W and U are being written by other CTAs of the same launch (layer_kernel.cuh).  The tile copies are then requested by a warp
-// of their own, kCopy, which first waits until the chunk's word in `ready` says that both factors are in memory; tensor memory
+// FED: W and U (per-channel form: Q+, K- and the chunks' vectors) are being written by other CTAs of the same launch (layer_kernel.cuh).  The tile copies are then requested by a warp
+// of their own, kCopy, which first waits until the chunk's word in `ready` says that they are in memory (the gate warp does the same for the vectors); tensor memory
 // is the caller's (`tmem`).  Otherwise the gate warp requests the copies and the CTA allocates (and frees) its tensor memory.
 template <int DVS, bool KDA, bool FED>
 __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmU,
@@ -189,7 +189,6 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
                                           const uint32_t* ready, uint32_t tmem) {
   using cfg = ScanCfg<DVS, KDA>;
   constexpr int LG = cfg::LG, E = cfg::E;
-  static_assert(!(FED && KDA), "the scalar gate only");
   float* sG = reinterpret_cast<float*>(smem + cfg::OFF_G);   // scalar gate: [2][4][64]: g log2e; 2^(g_ref(j) - g_j), g_ref(j) = g of the first token of j's block of eight; 2^(g_last - g_j); 2^g_j
   float* sEl = sG;                 // per-channel form: exp(G_last) [3][128], exp(G_ref) [3][128], exp(G_last - G_ref) [3][128]
   float* sEr = sG + 3 * D;
@@ -296,6 +295,13 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
     ev[1] = *reinterpret_cast<const float4*>(p.ER + (slot * p.H + h) * D + 4 * lane);
     ev[2] = *reinterpret_cast<const float4*>(p.EX + (slot * p.H + h) * D + 4 * lane);
   };
+  int vectors_known = 0;   // FED: the vectors of the chunks before this one are in memory
+  auto wait_vectors = [&](int c) {   // by the whole gate warp; false: they did not come within the limit
+    if (!FED || c < vectors_known) return true;
+    const int more = wait_ready(ready + ((size_t)((beg + c * C) / C + s) * p.H + h), p.H, n_chunks - c, lane, lim);
+    vectors_known = c + more;
+    return more > 0;
+  };
   auto store_e = [&](int c, const float4 (&ev)[3]) {
     *reinterpret_cast<float4*>(sEl + (c % 3) * D + 4 * lane) = ev[0];
     *reinterpret_cast<float4*>(sEr + (c % 3) * D + 4 * lane) = ev[1];
@@ -303,6 +309,7 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
   };
   float4 e_raw[3] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
   float g_raw[2] = {0.f, 0.f};   // gate warp: g of the chunk it stores next
+  bool gate_ok = true;
   if (warp == kGate) {
     if (lane == 0) {
       prefetch_tmap(&tmW); prefetch_tmap(&tmQ); prefetch_tmap(&tmK); prefetch_tmap(&tmU);
@@ -323,10 +330,11 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
     __syncwarp();
     if constexpr (KDA) {
       // the vectors of the first two chunks are in place before the loop starts, the third chunk's in registers
+      gate_ok = wait_vectors(0);
       fetch_e(0, e_raw);
       store_e(0, e_raw);
-      if (n_chunks > 1) { fetch_e(1, e_raw); store_e(1, e_raw); }
-      if (n_chunks > 2) fetch_e(2, e_raw);
+      if (n_chunks > 1) { gate_ok = gate_ok && wait_vectors(1); fetch_e(1, e_raw); store_e(1, e_raw); }
+      if (n_chunks > 2) { gate_ok = gate_ok && wait_vectors(2); fetch_e(2, e_raw); }
     } else {
       fetch_g(0, g_raw);
       store_g(0, g_raw);
@@ -465,7 +473,8 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
     // Its arrival on bar_sr tells the control thread, and through the first product's commit every reader, that
     // the chunk's factors are in place (bar_g tells the output warps, which start on a chunk earlier).
     if (!misaligned) { warp_arrive(bar_sr, lane); if (lane == 0) mbar_arrive(bar_g); }   // the first chunk's (written before the CTA barrier above)
-    for (int c = 0; c + 1 < n_chunks && !misaligned; ++c) {
+    failed |= !gate_ok;
+    for (int c = 0; c + 1 < n_chunks && !misaligned && !failed; ++c) {
       // stage of c + 2 = that of c - 1: its readers (the products of chunk c - 1, the chain warps' U) were done before the
       // arrivals that open chunk c
       if (!wait(bar_sr, (uint32_t)(c & 1))) { failed = true; break; }
@@ -485,7 +494,12 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
       }
       warp_arrive(bar_sr, lane);
       if (lane == 0) mbar_arrive(bar_g);
-      if constexpr (KDA) { if (c + 3 < n_chunks) fetch_e(c + 3, e_raw); }
+      if constexpr (KDA) {
+        if (c + 3 < n_chunks) {
+          if (!wait_vectors(c + 3)) { failed = true; break; }
+          fetch_e(c + 3, e_raw);
+        }
+      }
       else { if (c + 2 < n_chunks) fetch_g(c + 2, g_raw); }
     }
     if (!FED && failed && lane == 0) drain_copies();

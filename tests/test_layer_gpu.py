@@ -99,6 +99,37 @@ def test_one_kernel_on_two_streams_and_in_a_graph(bnd):
     assert torch.equal(bits(O), bits(refs[1][0])) and torch.equal(bits(S), bits(refs[1][1]))
 
 
+# few pairs (32 columns a slice), 32 (64), a last chunk of one token, packed sequences with an empty one
+KDA_ONE_KERNEL = [
+    ("few", 1, 130 * 64 + 1, 8, None),
+    ("slices_of_64", 1, 80 * 64, 32, None),
+    ("packed", 1, 0, 8, np.array([0, 9000, 9000, 9001, 13000], np.int32)),
+]
+
+
+@pytest.mark.parametrize("name,B,T,H,cu", KDA_ONE_KERNEL, ids=[c[0] for c in KDA_ONE_KERNEL])
+def test_per_channel_scan_in_one_kernel_gives_the_bits_of_two(bnd, name, B, T, H, cu):
+    """A head's result does not depend on how many there are: with many of them the preparation is a launch of its own."""
+    many = 160 if cu is None else 40
+    if cu is not None:
+        T = int(cu[-1])
+    inp = wl.make(name, B, T, H, 128, 128, 64, wl.BF16, seed=770 + H, cu_seqlens=cu)
+    dev = bnd.to_device(inp)
+    Q, G = bnd.kv_to_torch(wl.queries(inp, seed=771)), torch.from_numpy(wl.per_channel_gate(inp, seed=772)).cuda()
+    S0 = torch.from_numpy(wl.initial_state(inp, seed=773)).cuda()
+    _, W, U = bnd.fused_kda(dev["K"], dev["V"], G, dev["beta"], 64, cu_seqlens=cu)
+    wide = lambda t, dim: t.repeat_interleave((many + H - 1) // H, dim).contiguous()
+    n0 = bnd.launch_count()
+    ref = bnd.chunk_scan_kda(*(wide(t, 2) for t in (Q, dev["K"], W, U, G)), 64, scale=0.5, S0=wide(S0, 1), cu_seqlens=cu)
+    n1 = bnd.launch_count()
+    O, S = bnd.chunk_scan_kda(Q, dev["K"], W, U, G, 64, scale=0.5, S0=S0, cu_seqlens=cu)
+    torch.cuda.synchronize()
+    assert bnd.last_device_status() == 0
+    assert n1 == n0 + 2 and bnd.launch_count() == n1 + 1
+    k = (many + H - 1) // H
+    assert torch.equal(bits(O), bits(ref[0][:, :, ::k])) and torch.equal(bits(S), bits(ref[1][:, ::k]))
+
+
 # one token, the longest, features and columns on both sides of the kernel's instances and slices, an empty sequence
 TOKENS = [
     ("decode", 4, 1, 3, 128, 128, None),
