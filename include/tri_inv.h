@@ -289,6 +289,16 @@ int tri_inv_gdn_forward(const void* Q, const void* K, const void* V, const float
                         const tri_inv_desc* desc, int method, void* cuda_stream);
 
 /*
+ * Self-test of the one-kernel layer's give-up path: every wait limited to wait_limit_ns, and the first matrix is built but never
+ * announced, so that the scans of the first sequence's first head wait in vain, raise TRI_INV_ERR_DEVICE_TIMEOUT in the status word
+ * and leave (their rows of O undefined); all other heads' output is as usual.  Synchronises the stream.  TRI_INV_ERR_UNSUPPORTED for
+ * shapes that tri_inv_gdn_forward runs otherwise.
+ */
+int tri_inv_selftest_layer_wait_timeout(const void* Q, const void* K, const void* V, const float* beta, const float* g, void* O,
+                                        void* workspace, size_t workspace_bytes, const tri_inv_desc* desc, uint64_t wait_limit_ns,
+                                        void* cuda_stream);
+
+/*
  * Fused call with the layer's front end folded in: the kernel takes what the projections produce and
  * does the three producers that otherwise run as separate passes over memory before the inversion
  * (the gating recipe of a Gated-DeltaNet layer; in the paper these are among the kernels its fused

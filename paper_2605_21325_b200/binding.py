@@ -109,6 +109,9 @@ def load():
             lib.tri_inv_gdn_forward.restype = i32
             lib.tri_inv_gdn_forward_workspace.argtypes = [dp, i32, ctypes.POINTER(ctypes.c_size_t)]
             lib.tri_inv_gdn_forward_workspace.restype = i32
+        if hasattr(lib, "tri_inv_selftest_layer_wait_timeout"):
+            lib.tri_inv_selftest_layer_wait_timeout.argtypes = [vp, vp, vp, vp, vp, vp, vp, ctypes.c_size_t, dp, ctypes.c_uint64, vp]
+            lib.tri_inv_selftest_layer_wait_timeout.restype = i32
         lib.tri_inv_count_matrices.argtypes = [dp, ctypes.POINTER(ctypes.c_int64)]
         lib.tri_inv_last_device_status.argtypes = [ctypes.POINTER(ctypes.c_int)]
         for f in ("tri_inv_build", "tri_inv_wy", "tri_inv_fused", "tri_inv_count_matrices", "tri_inv_last_device_status"):
@@ -378,6 +381,23 @@ def selftest_scan_wait_timeout(Q, K, W, U, g, C, wait_limit_ns, out, stream=None
                                                    ctypes.c_uint64(int(wait_limit_ns)), _stream(stream))
     if rc != OK:
         raise TriInvError("tri_inv_selftest_scan_wait_timeout", rc)
+    return out
+
+
+def selftest_layer_wait_timeout(Q, K, V, beta, g, C, wait_limit_ns, out, stream=None):
+    """tri_inv_selftest_layer_wait_timeout: the one-kernel layer with short wait limits and the first matrix never announced to the
+    scans of the first head.  ``out`` = O."""
+    B, T, H, d_k = K.shape
+    desc, keep = make_desc(B, T, H, d_k, V.shape[-1], C, _dtype_code(K), None)
+    need = ctypes.c_size_t(0)
+    rc = load().tri_inv_gdn_forward_workspace(desc, BLOCK_RECURSIVE, need)
+    if rc != OK:
+        raise TriInvError("tri_inv_gdn_forward_workspace", rc)
+    work = torch.empty(need.value, dtype=torch.uint8, device=K.device)
+    rc = load().tri_inv_selftest_layer_wait_timeout(_p(Q), _p(K), _p(V), _p(beta), _p(g), _p(out), _p(work), need, desc,
+                                                    ctypes.c_uint64(int(wait_limit_ns)), _stream(stream))
+    if rc != OK:
+        raise TriInvError("tri_inv_selftest_layer_wait_timeout", rc)
     return out
 
 

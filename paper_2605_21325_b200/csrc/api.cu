@@ -422,6 +422,29 @@ int tri_inv_gdn_forward(const void* Q, const void* K, const void* V, const float
   return err == cudaSuccess ? TRI_INV_OK : TRI_INV_ERR_CUDA;
 }
 
+int tri_inv_selftest_layer_wait_timeout(const void* Q, const void* K, const void* V, const float* beta, const float* g, void* O,
+                                        void* workspace, size_t workspace_bytes, const tri_inv_desc* desc, uint64_t wait_limit_ns,
+                                        void* cuda_stream) {
+  int rc = check_desc(desc, true);
+  if (rc) return rc;
+  size_t need = 0;
+  if (layer_route(desc, TRI_INV_BLOCK_RECURSIVE, &need) != kOneKernel) return TRI_INV_ERR_UNSUPPORTED;
+  if (!Q || !K || !V || !beta || !g || !O || !workspace || workspace_bytes < need || wait_limit_ns == 0) return TRI_INV_ERR_INVALID_ARG;
+  if (!aligned16(Q) || !aligned16(K) || !aligned16(V) || !aligned16(beta) || !aligned16(g) || !aligned16(O) || !aligned16(workspace))
+    return TRI_INV_ERR_INVALID_ARG;
+  ScanParams p{};
+  p.g = g; p.O = O; p.scale = 1.f;
+  p.H = desc->H; p.T = desc->T;
+  p.n_seqs = desc->cu_seqlens ? desc->n_seqs : desc->B;
+  p.wait_limit_ns = wait_limit_ns; p.test_stall = 1;
+  cudaError_t err;
+  p.status = status_word_for_current_device(&err);
+  if (!p.status) return TRI_INV_ERR_CUDA;
+  err = launch_layer(Q, K, V, beta, g, p, workspace, desc, (cudaStream_t)cuda_stream);
+  if (err == cudaSuccess) g_launches.fetch_add(1, std::memory_order_relaxed);
+  return err == cudaSuccess && cudaStreamSynchronize((cudaStream_t)cuda_stream) == cudaSuccess ? TRI_INV_OK : TRI_INV_ERR_CUDA;
+}
+
 int tri_inv_selftest_scan_wait_timeout(const void* Q, const void* K, const void* W, const void* U, const float* g, void* O,
                                        const tri_inv_desc* desc, uint64_t wait_limit_ns, void* cuda_stream) {
   int rc = check_desc(desc, true);

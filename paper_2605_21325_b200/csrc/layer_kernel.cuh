@@ -50,6 +50,7 @@ struct LayerParams {
   int sms;
   int groups;                    // of these CTAs: four each
   unsigned long long wait_limit_ns;
+  int test_stall;           // self-test: the first matrix is never announced
 };
 
 struct Place { int tok0, rows, h, slot; };
@@ -319,7 +320,7 @@ __device__ __forceinline__ bool build_factors(const CUtensorMap& tmK, const CUte
     store_frag_piece_bf16(f0, stage, lane, p.U + out, stride, left, &tmU, h * D, tok0 + row0);
     store_frag_piece_bf16<1>(f1, sAp + warp * 2048, lane, p.U + out + 64, stride, left, &tmU, h * D + 64, tok0 + row0);
     partial = rows < C;
-    signal = bad ? nullptr : p.ready + ((size_t)at.slot * p.H + h);
+    signal = (bad || (p.test_stall && item == 0)) ? nullptr : p.ready + ((size_t)at.slot * p.H + h);
     item = nx_item;
     at = nx;
     nx_item = take(nx);   // left there before the operands' barriers
@@ -559,14 +560,14 @@ kda_scan_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
 
 // Before the layer kernel: its words at zero, and for packed sequences the chunks in build order and the device copy of cu_seqlens.
 // Sequences go in groups of `group` (those walked at the same time), and within a group chunk by chunk.
-constexpr int kSeqsPerPrep = 960;
+constexpr int kMostSeqs = 960;   // packed sequences of a call: their offsets are kernel parameters
 struct PrepArgs {
   uint32_t* words;
   long long n_words;
   LayerEntry* tab;
   int* seq_off;
-  int n, first, group, base;   // sequences first .. first + n - 1; entries before them
-  int32_t cu[kSeqsPerPrep + 1];
+  int n, group;
+  int32_t cu[kMostSeqs + 1];
 };
 __global__ void __launch_bounds__(256) layer_prep_kernel(const __grid_constant__ PrepArgs a) {
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < a.n_words; i += (long long)gridDim.x * blockDim.x) a.words[i] = 0u;
@@ -580,7 +581,7 @@ __global__ void __launch_bounds__(256) layer_prep_kernel(const __grid_constant__
     __syncthreads();
     if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = sum;
     __syncthreads();
-    int base = a.base;
+    int base = 0;
     for (int q = 0; q < 8; ++q) base += part[q];
     const int len = a.cu[s + 1] - a.cu[s], n = chunks(s);
     for (int c = threadIdx.x; c < n; c += blockDim.x) {
@@ -590,11 +591,11 @@ __global__ void __launch_bounds__(256) layer_prep_kernel(const __grid_constant__
         at += min(nq, c) + (q < s && nq > c ? 1 : 0);
       }
       const int tok0 = a.cu[s] + c * C;
-      a.tab[at] = LayerEntry{tok0, min(C, len - c * C), tok0 / C + a.first + s, 0};
+      a.tab[at] = LayerEntry{tok0, min(C, len - c * C), tok0 / C + s, 0};
     }
     if (threadIdx.x == 0) {
-      a.seq_off[a.first + s] = a.cu[s];
-      if (s == a.n - 1) a.seq_off[a.first + a.n] = a.cu[a.n];
+      a.seq_off[s] = a.cu[s];
+      if (s == a.n - 1) a.seq_off[a.n] = a.cu[a.n];
     }
   }
 }
@@ -692,6 +693,7 @@ void fill_params(LayerParams& p, const tri_inv_desc* d, const Layout& l, char* w
   p.chunks = (d->T + C - 1) / C;
   p.total = (int)(l.entries * d->H);
   p.wait_limit_ns = sp.wait_limit_ns ? sp.wait_limit_ns : kWaitLimitNs;
+  p.test_stall = sp.test_stall;
   p.factor_ctas = sms - split.scans;
   p.sms = sms;
   p.groups = kGroups * p.factor_ctas;
@@ -704,24 +706,17 @@ cudaError_t launch_prep(const tri_inv_desc* d, const Layout& l, char* ws, int sm
   PrepArgs a;
   a.words = reinterpret_cast<uint32_t*>(p.counters);
   a.n_words = l.n_words;
-  a.tab = nullptr; a.seq_off = nullptr; a.n = a.first = a.base = 0; a.group = 1;
-  const int blocks = (int)std::min<long long>(sms, (l.n_words + 255) / 256);
-  if (!d->cu_seqlens) {
-    layer_prep_kernel<<<blocks, 256, 0, stream>>>(a);
-  } else {
+  a.tab = nullptr; a.seq_off = nullptr; a.n = 0; a.group = 1;
+  int blocks = (int)std::min<long long>(sms, (l.n_words + 255) / 256);
+  if (d->cu_seqlens) {
     p.tab = a.tab = reinterpret_cast<LayerEntry*>(ws + l.tab);
     sp.seq_off = a.seq_off = reinterpret_cast<int*>(ws + l.seq);
-    a.group = std::max(1, std::min(kSeqsPerPrep, (p.wave + d->H - 1) / d->H));
-    const int per = kSeqsPerPrep / a.group * a.group;   // whole groups per launch
-    for (int s0 = 0; s0 < d->n_seqs; s0 += per) {
-      a.first = s0;
-      a.n = std::min(per, d->n_seqs - s0);
-      for (int q = 0; q <= a.n; ++q) a.cu[q] = d->cu_seqlens[s0 + q];
-      layer_prep_kernel<<<std::max(blocks, std::min(a.n, sms)), 256, 0, stream>>>(a);
-      for (int q = 0; q < a.n; ++q) a.base += (a.cu[q + 1] - a.cu[q] + C - 1) / C;
-      a.n_words = 0;
-    }
+    a.group = std::max(1, (p.wave + d->H - 1) / d->H);
+    a.n = d->n_seqs;
+    for (int q = 0; q <= a.n; ++q) a.cu[q] = d->cu_seqlens[q];
+    blocks = std::max(blocks, std::min(a.n, sms));
   }
+  layer_prep_kernel<<<blocks, 256, 0, stream>>>(a);
   return cudaGetLastError();
 }
 
@@ -748,7 +743,7 @@ bool layer_fits(const tri_inv_desc* d, size_t* workspace_bytes) {
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
   const Layout l = layout_of(d);
-  if (l.entries * d->H > 0x7fffffffLL || split_of(d, l, sms).scans == 0) return false;   // matrices are numbered in 32 bits
+  if (l.entries * d->H > 0x7fffffffLL || d->n_seqs > kMostSeqs || split_of(d, l, sms).scans == 0) return false;   // matrices are numbered in 32 bits
   *workspace_bytes = l.bytes;
   return true;
 }
@@ -791,7 +786,7 @@ bool kda_scan_fits(const tri_inv_desc* d, size_t* control_bytes) {
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return false;
   const Layout l = layout_of(d);
-  if (l.entries * d->H > 0x7fffffffLL || choose_kda_split((long long)(d->cu_seqlens ? d->n_seqs : d->B) * d->H, longest_of(d), l.entries, d->H, sms).scans == 0)
+  if (l.entries * d->H > 0x7fffffffLL || d->n_seqs > kMostSeqs || choose_kda_split((long long)(d->cu_seqlens ? d->n_seqs : d->B) * d->H, longest_of(d), l.entries, d->H, sms).scans == 0)
     return false;
   *control_bytes = l.w;
   return true;

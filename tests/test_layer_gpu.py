@@ -99,6 +99,25 @@ def test_one_kernel_on_two_streams_and_in_a_graph(bnd):
     assert torch.equal(bits(O), bits(refs[1][0])) and torch.equal(bits(S), bits(refs[1][1]))
 
 
+def test_one_kernel_waits_that_run_out(bnd):
+    """The give-up path: the scans of the first head wait for a chunk that is never announced (limit 2 ms, far above what the other
+    scans ever wait here); the status word says so once, every other head is right, and so is the next call."""
+    inp, _, _, dev, Q, _ = layer_inputs(bnd, "stall", 1, 6 * 64, 8, 128, 128, wl.BF16, None, 760, False)
+    call = lambda: bnd.gdn_forward(Q, dev["K"], dev["V"], dev["beta"], dev["g"], 64, scale=1.0)[0]
+    ref = call()
+    torch.cuda.synchronize()
+    assert bnd.last_device_status() == 0
+    O = torch.full_like(dev["V"], float("nan"))
+    bnd.selftest_layer_wait_timeout(Q, dev["K"], dev["V"], dev["beta"], dev["g"], 64, wait_limit_ns=2_000_000, out=O)
+    assert bnd.last_device_status() == bnd.ERR_DEVICE_TIMEOUT
+    assert bnd.last_device_status() == 0
+    assert torch.equal(bits(O[:, :, 1:]), bits(ref[:, :, 1:]))
+    again = call()
+    torch.cuda.synchronize()
+    assert bnd.last_device_status() == 0
+    assert torch.equal(bits(again), bits(ref))
+
+
 # few pairs (32 columns a slice), 32 (64), a last chunk of one token, packed sequences with an empty one
 KDA_ONE_KERNEL = [
     ("few", 1, 130 * 64 + 1, 8, None),
