@@ -445,7 +445,8 @@ __device__ __forceinline__ void prepare_chunks(const LayerParams& p, const KdaOp
   int nx_item = take(nx);
   while (item < p.total) {
     int ticket = p.total;
-    if (tid == 0 && nx_item < p.total) ticket = atomicAdd(p.counters + 1, 1);
+    // (one thread decides for the group: it reads a word that other CTAs write)
+    if (tid == 0 && (nx_item < p.total || (once && *(volatile int*)(p.counters + 3) == 0))) ticket = atomicAdd(p.counters + 1, 1);
     const size_t row0 = ((size_t)at.tok0 * p.H + at.h) * D + f0, stride = (size_t)p.H * D;
     float gref[8], glast[8];
 #pragma unroll
@@ -503,10 +504,10 @@ __device__ __forceinline__ void prepare_chunks(const LayerParams& p, const KdaOp
     item = nx_item;
     at = nx;
     nx_item = take(nx);
-    if (once && item >= p.total && *(volatile int*)(p.counters + 3) == 0) {
-      if (tid == 0) leave(atomicAdd(p.counters + 1, 1));
-      sync();
-      item = take(at);
+    if (once && item >= p.total) {   // not one ahead: the chunk just drawn, if any, is the next
+      item = nx_item;
+      at = nx;
+      nx_item = p.total;
     }
   }
 }
