@@ -15,8 +15,8 @@
 // eight lanes of a load step in different banks (W and K by their tiles' 128-byte swizzle, S and U~ by padding); W and K come by TMA one
 // or two chunks ahead, U and g into registers one chunk ahead; the thread's part of S stays in registers beside its shared copy.
 // The output kernel is bound by FFMA issue and shared-memory loads (8 per 64 FMAs).
-// Measured (ncu, B = 2, T = 2048, H = 8, d = 64: 16 pairs of 32 chunks): 50 + 28 us; 213 us as one kernel per slice of 16 columns that also
-// formed P and O on the way (P again in each slice, all of it on the chain, 64 CTAs); the layer 262 -> 127 us.
+// Measured (ncu, B = 2, T = 2048, H = 8, d = 64: 16 pairs of 32 chunks): 44 + 27 us (50 + 28 with the chain's tiles by cp.async); 213 us as one kernel per slice of 16 columns that also
+// formed P and O on the way (P again in each slice, all of it on the chain, 64 CTAs).
 #include "tc_device.cuh"
 
 namespace tri_inv {
