@@ -179,6 +179,14 @@ __device__ __noinline__ bool wait_by_warp(uint32_t bar, uint32_t parity, unsigne
   return false;
 }
 
+// Zeros into rows `rows` .. 63 of a tile of two boxes (128 bytes a row), by the chain warps; then visible to the products.  Not inlined: once a
+// sequence, and the 128-column walk has no register to spare.
+__device__ __noinline__ void clear_rows(uint32_t tile, int box, int rows, int tid) {
+  for (int e = tid; e < (C - rows) * 16; e += kChainWarps * 32)
+    asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(tile + ((e >> 3) & 1) * box + (rows + (e >> 4)) * 128 + (e & 7) * 16), "r"(0) : "memory");
+  fence_proxy_async();
+}
+
 // One (sequence, head, slice) by a whole CTA; true when a wait has run out in this thread.
 // FED: W and U (per-channel form: Q+, K- and the chunks' vectors) are being written by other CTAs of the same launch (layer_kernel.cuh).  The tile copies are then requested by a warp
 // of their own, kCopy, which first waits until the chunk's word in `ready` says that they are in memory (the gate warp does the same for the vectors); tensor memory
@@ -543,6 +551,12 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
       if (!wait(bar_t1, ph)) { failed = true; break; }
       tc_fence_after();
       TL(2);
+      if (rows < C) {
+        // The tile's rows past the sequence's end hold what follows it in memory: a neighbour's keys or, per channel beside the preparation,
+        // scratch that nobody may have written yet.  U~ is zero there, but zero times Inf or NaN is not: the state product must find
+        // zeros.  QK, the tile's other reader, was issued before the product just waited for.
+        clear_rows(s0 + (c % kStages) * cfg::STAGE + cfg::OFF_KT, cfg::K_BOX, rows, tid);
+      }
       // ---- U~ = U - W S, transposed: first the decay-scaled U~' that the chain waits for (its own arrival), then U~ itself
       float v[LG][4][4];
 #pragma unroll

@@ -149,6 +149,64 @@ def test_per_channel_scan_in_one_kernel_gives_the_bits_of_two(bnd, name, B, T, H
     assert torch.equal(bits(O), bits(ref[0][:, :, ::k])) and torch.equal(bits(S), bits(ref[1][:, ::k]))
 
 
+# partial last chunks in front of another sequence: packed, short ones beside long ones; a batch; all 128 columns in a block
+KDA_NEIGHBOURS = [
+    ("packed", 1, 8, np.array([0, 1, 8001, 8002, 8040, 16040], np.int32)),
+    ("batch", 3, 4, 80 * 64 + 37),
+    ("slices_of_128", 2, 26, 130 * 64 + 1),
+]
+
+
+@pytest.mark.parametrize("name,B,H,layout", KDA_NEIGHBOURS, ids=[c[0] for c in KDA_NEIGHBOURS])
+def test_per_channel_scan_does_not_depend_on_what_its_scratch_held(bnd, name, B, H, layout):
+    """A last chunk's tile reaches past its sequence, into rows of the scratch that another block prepares, maybe later.  The scratch is
+    left full of NaN by a call of the same shape on NaN keys; the next call's bits are those of the form in two launches."""
+    cu = layout if B == 1 else None
+    T = int(cu[-1]) if B == 1 else layout
+    gen = torch.Generator(device="cuda").manual_seed(790)
+    normal = lambda *s: torch.randn(*s, device="cuda", generator=gen)
+    unit = lambda x: (x / x.norm(dim=-1, keepdim=True)).to(torch.bfloat16)
+    Q, K, V = unit(normal(B, T, H, 128)), unit(normal(B, T, H, 128)), normal(B, T, H, 128).to(torch.bfloat16)
+    beta, G = torch.sigmoid(normal(B, T, H)), -0.05 * torch.rand(B, T, H, 128, device="cuda", generator=gen)
+    edges = [T * b for b in range(B + 1)] if cu is None else list(cu)
+    for a, b in zip(edges[:-1], edges[1:]):   # cumulative within the chunks of a sequence
+        for c in range(a, b, 64):
+            rows = G.reshape(B * T, H, 128)[c:min(c + 64, b)]
+            rows.copy_(rows.cumsum(0))
+    _, W, U = bnd.fused_kda(K, V, G, beta, 64, cu_seqlens=cu)
+    k = (160 + H - 1) // H
+    wide = [t.repeat_interleave(k, 2).contiguous() for t in (Q, K, W, U, G)]
+    n0 = bnd.launch_count()
+    ref = bnd.chunk_scan_kda(*wide, 64, scale=0.5, cu_seqlens=cu)
+    n1 = bnd.launch_count()
+    for _ in range(4):   # which block is late differs from run to run
+        bnd.chunk_scan_kda(*(torch.full_like(t, float("nan")) for t in (Q, K)), W, U, torch.zeros_like(G), 64, cu_seqlens=cu)
+        n2 = bnd.launch_count()
+        O, S = bnd.chunk_scan_kda(Q, K, W, U, G, 64, scale=0.5, cu_seqlens=cu)
+        torch.cuda.synchronize()
+        assert bnd.last_device_status() == 0
+        assert n1 == n0 + 2 and bnd.launch_count() == n2 + 1, "not one kernel against two"
+        assert torch.isfinite(S).all()
+        assert torch.equal(bits(O), bits(ref[0][:, :, ::k])) and torch.equal(bits(S), bits(ref[1][:, ::k]))
+
+
+def test_scan_does_not_multiply_a_neighbours_keys(bnd):
+    """Keys that are not finite stay with their sequence: the one before it, whose last chunk's tile reaches into them, keeps its bits."""
+    cu = np.array([0, 70, 200], np.int32)
+    _, _, _, dev, Q, S0 = layer_inputs(bnd, "neighbour", 1, 0, 2, 128, 128, wl.BF16, cu, 795)
+    _, W, U = bnd.fused(dev["K"], dev["V"], dev["beta"], dev["g"], 64, method=bnd.W_DECAY, cu_seqlens=cu, want_A=False)
+    outs = []
+    for value in (1.0, float("inf"), float("nan")):
+        K = dev["K"].clone()
+        K[0, 70:] *= value
+        O, S = bnd.chunk_scan(Q, K, W, U, dev["g"], 64, scale=0.5, S0=S0, cu_seqlens=cu)
+        outs.append((bits(O[:, :70]), bits(S[0])))
+    torch.cuda.synchronize()
+    assert torch.isfinite(S[0]).all()
+    for o in outs[1:]:
+        assert torch.equal(o[0], outs[0][0]) and torch.equal(o[1], outs[0][1])
+
+
 # one token, the longest, features and columns on both sides of the kernel's instances and slices, an empty sequence
 TOKENS = [
     ("decode", 4, 1, 3, 128, 128, None),
