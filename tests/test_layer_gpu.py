@@ -226,3 +226,9 @@ def test_token_by_token_against_the_recurrence(bnd, name, B, T, H, d_k, d_v, cu,
     torch.cuda.synchronize()
     assert max_ratio(bnd.to_numpy_f64(O), O_ref) <= (1e-5 if dtype == wl.F32 else 2.0 ** -8)
     assert max_ratio(bnd.to_numpy_f64(S), S_ref) <= 1e-5
+
+
+def test_smoke_runs():
+    """The entry that is run first on a machine, with its counts of launches and its comparisons."""
+    import __graft_entry__ as entry
+    entry.smoke()
