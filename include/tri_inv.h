@@ -413,7 +413,10 @@ int tri_inv_count_matrices(const tri_inv_desc* desc, int64_t* out);
  */
 int tri_inv_last_device_status(int* out);
 
-/* Kernel launches issued by this library in this process so far (host counter). */
+/*
+ * Kernel launches issued by this library in this process so far (host counter): every launch of a kernel that computes results; the
+ * small ones that fill chunk tables, sequence offsets or the words of a call's workspace are not counted.
+ */
 int64_t tri_inv_launch_count(void);
 
 /* Static string for a status code. */

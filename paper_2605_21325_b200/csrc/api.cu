@@ -161,7 +161,7 @@ int run(KParams p, const tri_inv_desc* d, void* stream_v) {
     return TRI_INV_ERR_UNSUPPORTED;
   }
   if (err == cudaSuccess && !handled) err = f32_factors_fit(p, d->C) ? launch_f32_factors(p, stream) : launch_simt(p, d->C, stream);
-  if (err == cudaSuccess) g_launches.fetch_add(1, std::memory_order_relaxed);
+  if (err == cudaSuccess) count_launch();
   if (dev_tab) cudaFreeAsync(dev_tab, stream);
   if (log_enabled()) fprintf(stderr, "[tri_inv]   -> %s kernel, %s\n", handled ? "tensor-core" : "CUDA-core", cudaGetErrorString(err));
   return err == cudaSuccess ? TRI_INV_OK : TRI_INV_ERR_CUDA;
@@ -318,10 +318,7 @@ int chunk_scan_any(const void* Q, const void* K, const void* W, const void* U, c
       err = launch_kda_scan(p, Q, K, W, Qp, Km, w + 2 * tensor_bytes + 3 * vec_bytes, desc, stream);
     } else {
       err = launch_kda_scan_prep(p, Q, K, Qp, Km, EL, ER, EX, (max_len + 63) / 64, stream);
-      if (err == cudaSuccess) {
-        g_launches.fetch_add(1, std::memory_order_relaxed);
-        err = launch_chunk_scan(p, Qp, Km, W, tokens, stream, true);
-      }
+      if (err == cudaSuccess) err = launch_chunk_scan(p, Qp, Km, W, tokens, stream, true);
     }
   } else {
     const bool f32 = !G && desc->kv_dtype == TRI_INV_F32 && desc->C == 64 && desc->d_k <= 128;
@@ -342,7 +339,6 @@ int chunk_scan_any(const void* Q, const void* K, const void* W, const void* U, c
                        : launch_chunk_scan_simt(p, Q, K, W, desc->d_k, desc->d_v, desc->C, desc->kv_dtype, stream);
     }
   }
-  if (err == cudaSuccess) g_launches.fetch_add(1, std::memory_order_relaxed);
   if (work) cudaFreeAsync(work, stream);
   if (dev_off) cudaFreeAsync(dev_off, stream);
   return err == cudaSuccess ? TRI_INV_OK : TRI_INV_ERR_CUDA;
@@ -418,7 +414,6 @@ int tri_inv_gdn_forward(const void* Q, const void* K, const void* V, const float
   if (p.n_seqs == 0 || (desc->T == 0 && !S_out)) return TRI_INV_OK;
   err = route == kOneKernel ? launch_layer(Q, K, V, beta, g, p, workspace, desc, (cudaStream_t)cuda_stream)
                             : launch_recurrence(Q, K, V, beta, g, p, desc, (cudaStream_t)cuda_stream);
-  if (err == cudaSuccess) g_launches.fetch_add(1, std::memory_order_relaxed);
   return err == cudaSuccess ? TRI_INV_OK : TRI_INV_ERR_CUDA;
 }
 
@@ -441,7 +436,6 @@ int tri_inv_selftest_layer_wait_timeout(const void* Q, const void* K, const void
   p.status = status_word_for_current_device(&err);
   if (!p.status) return TRI_INV_ERR_CUDA;
   err = launch_layer(Q, K, V, beta, g, p, workspace, desc, (cudaStream_t)cuda_stream);
-  if (err == cudaSuccess) g_launches.fetch_add(1, std::memory_order_relaxed);
   return err == cudaSuccess && cudaStreamSynchronize((cudaStream_t)cuda_stream) == cudaSuccess ? TRI_INV_OK : TRI_INV_ERR_CUDA;
 }
 

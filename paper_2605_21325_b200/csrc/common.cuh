@@ -167,6 +167,12 @@ cudaError_t work_counters_idle(bool* idle);
 
 // Adds one to the library's launch counter (tri_inv_launch_count).
 void count_launch();
+// Behind a launch, by the launchers that may make several: its error, and the count if there is none.
+inline cudaError_t launched() {
+  const cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess) count_launch();
+  return e;
+}
 
 // Address of the device status word (0 = ok) of the current device; nullptr and *err on failure.
 int* status_word_for_current_device(cudaError_t* err);

@@ -735,7 +735,7 @@ cudaError_t launch_width(const CUtensorMap (&tm)[7], const LayerParams& p, const
     }
   }
   layer_kernel<DVS><<<grid, kLayerThreads, LayerCfg<DVS>::SMEM, stream>>>(tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], tm[6], p, sp);
-  return cudaGetLastError();
+  return launched();
 }
 
 }  // namespace
@@ -808,7 +808,7 @@ cudaError_t launch_kda_width(const CUtensorMap (&tm)[4], const LayerParams& p, c
     }
   }
   kda_scan_kernel<DVS><<<grid, kKdaThreads, KdaScanCfg<DVS>::SMEM, stream>>>(tm[0], tm[1], tm[2], tm[3], p, a, sp);
-  return cudaGetLastError();
+  return launched();
 }
 }  // namespace
 

@@ -158,7 +158,7 @@ cudaError_t launch_recurrence(const void* Q, const void* K, const void* V, const
       if (d->d_k <= 64) recurrence_kernel<8, RecurrenceArgs><<<grid, kWarps * 32, 0, stream>>>(a);
       else recurrence_kernel<16, RecurrenceArgs><<<grid, kWarps * 32, 0, stream>>>(a);
     }
-    const cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launched();
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

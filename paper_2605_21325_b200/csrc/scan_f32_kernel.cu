@@ -528,7 +528,7 @@ cudaError_t launch_one_chunk(const ScanParams& p, const F32Args& a, cudaStream_t
   const long long grid = (long long)p.n_seqs * p.H * ((a.d_v + kNS1 - 1) / kNS1);
   if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
   scan_f32_one_chunk<DK><<<(int)grid, kThreads, OneChunk<DK>::bytes, stream>>>(p, a);
-  return cudaGetLastError();
+  return launched();
 }
 
 template <int DK, int NS>
@@ -538,7 +538,7 @@ cudaError_t launch_chain(const CUtensorMap& tmW, const CUtensorMap& tmK, const S
   const long long grid = pairs * ((a.d_v + NS - 1) / NS);
   if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
   scan_f32_chain<DK, NS><<<(int)grid, kThreads, Chain<DK, NS>::bytes, stream>>>(tmW, tmK, p, a);
-  return cudaGetLastError();
+  return launched();
 }
 
 // 3-D view [tokens, H, d] of an fp32 tensor, one box = 32 features (128 bytes, swizzled) of one head x 64 tokens; features past d are
@@ -570,7 +570,7 @@ cudaError_t launch_segments(const ScanParams& p, F32Args a, int max_chunks, long
     const long long grid = pairs * a.n_seg * ((a.d_v + kNV - 1) / kNV);
     if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
     scan_f32_output<DK><<<(int)grid, kThreads, Output<DK>::bytes, stream>>>(p, a);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = launched()) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }

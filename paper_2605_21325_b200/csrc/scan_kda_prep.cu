@@ -110,7 +110,7 @@ cudaError_t launch_kda_scan_prep(const ScanParams& p, const void* Q, const void*
   if (gy > want) gy = want > 0 ? want : 1;
   if (gy > 65535) gy = 65535;
   kda_scan_prep_kernel<<<dim3((unsigned)gx, (unsigned)gy), NT, 0, stream>>>(a);
-  return cudaGetLastError();
+  return launched();
 }
 
 }  // namespace tri_inv

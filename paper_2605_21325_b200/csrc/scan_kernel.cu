@@ -854,7 +854,7 @@ cudaError_t launch_scan_one(const ScanParams& p, const CUtensorMap& tmW, const C
   const long long grid = (long long)p.n_seqs * p.H * (D / DVS);
   if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
   chunk_scan_kernel<DVS, KDA><<<(int)grid, kThreadsScan, cfg::SMEM, stream>>>(tmW, tmQ, tmK, tmU, p);
-  return cudaGetLastError();
+  return launched();
 }
 
 }  // namespace

@@ -154,7 +154,7 @@ cudaError_t launch_chunk_scan_simt(const ScanParams& p, const void* Q, const voi
   if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
   if (grid == 0) return cudaSuccess;
   scan_simt_kernel<<<(int)grid, kThreads, bytes, stream>>>(p, a);
-  return cudaGetLastError();
+  return launched();
 }
 
 }  // namespace tri_inv

@@ -232,3 +232,24 @@ def test_smoke_runs():
     """The entry that is run first on a machine, with its counts of launches and its comparisons."""
     import __graft_entry__ as entry
     entry.smoke()
+
+
+def test_every_launch_that_computes_is_counted(bnd):
+    """One token each for more sequences than a launch takes; the fp32 scan of one chunk (one kernel), of several (chain and output) and in
+    segments of its scratch (as many pairs of launches); the per-channel scan in its two forms is counted above."""
+    def counted(call):
+        n0 = bnd.launch_count()
+        call()
+        torch.cuda.synchronize()
+        assert bnd.last_device_status() == 0
+        return bnd.launch_count() - n0
+
+    for n_seqs, launches in ((960, 1), (961, 2), (2000, 3)):
+        _, _, _, dev, Q, _ = layer_inputs(bnd, "count", 1, 0, 1, 16, 16, wl.F32, np.arange(n_seqs + 1, dtype=np.int32), 820, False)
+        assert counted(lambda: bnd.gdn_forward(Q, dev["K"], dev["V"], dev["beta"], dev["g"], 64, cu_seqlens=np.arange(n_seqs + 1))) == launches
+    slots = (128 << 20) // ((128 + 64) * 128 * 4)   # chunks whose state and U~ the scratch holds
+    H = 40
+    for chunks, launches in ((1, 1), (2, 2), (slots // H, 2), (slots // H + 1, 4)):
+        x = torch.zeros((1, 64 * chunks, H, 128), device="cuda")
+        g = torch.zeros((1, 64 * chunks, H), device="cuda")
+        assert counted(lambda: bnd.chunk_scan(x, x, x, x, g, 64)) == launches
