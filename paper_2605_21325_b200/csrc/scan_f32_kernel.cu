@@ -363,7 +363,13 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 3 : 1) scan_f32_output(Sc
       const float4 u0 = ld4(uc + j * LDV), u1 = ld4(uc + (j + 1) * LDV), u2 = ld4(uc + (j + 2) * LDV), u3 = ld4(uc + (j + 3) * LDV);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        if (i >= b) {
+        if (i == b) {   // the diagonal's block: a later token's U~ is not multiplied in, not even by zero
+          const float4 pv = ld4(pc + 16 * i * kLdP + j);
+          if (j <= ty) fma4(o[i], pv.x, u0);
+          if (j + 1 <= ty) fma4(o[i], pv.y, u1);
+          if (j + 2 <= ty) fma4(o[i], pv.z, u2);
+          if (j + 3 <= ty) fma4(o[i], pv.w, u3);
+        } else if (i > b) {
           const float4 pv = ld4(pc + 16 * i * kLdP + j);
           fma4(o[i], pv.x, u0); fma4(o[i], pv.y, u1); fma4(o[i], pv.z, u2); fma4(o[i], pv.w, u3);
         }

@@ -283,6 +283,28 @@ def test_fp32_scan_in_segments(bnd, H, d_k, d_v):
     assert torch.equal(O, torch.cat([O1, O2], 1)) and torch.equal(S, S2)
 
 
+@pytest.mark.parametrize("T", [60, 150])
+def test_fp32_scan_keeps_a_tokens_nan_to_later_rows(bnd, T):
+    """Rows before a token whose value is not finite are those of the sequence without it, one chunk long or several."""
+    inp = wl.make("nan", 1, T, 2, 64, 64, 64, wl.F32, seed=785)
+    dev = bnd.to_device(inp)
+    Q = bnd.kv_to_torch(wl.queries(inp, seed=786))
+    _, W, U = bnd.fused(dev["K"], dev["V"], dev["beta"], dev["g"], 64, method=bnd.W_DECAY, want_A=False)
+    scan = lambda U: bnd.chunk_scan(Q, dev["K"], W, U, dev["g"], 64)[0]
+    layer = lambda V: bnd.gdn_forward(Q, dev["K"], V, dev["beta"], dev["g"], 64)[0]
+    for call, x in ((scan, U), (layer, dev["V"])):
+        ref = call(x)
+        for t in (5, 20, 47, 63, 64, 100, 149):
+            if t >= T:
+                continue
+            y = x.clone()
+            y[0, t] = float("nan")
+            out = call(y)
+            torch.cuda.synchronize()
+            assert torch.equal(out[:, :t], ref[:, :t])
+            assert torch.isnan(out[:, t:]).all()
+
+
 # ---------------------------------------------------------------- full sizes, in the launch configuration bench.py times
 
 def test_layer_full_size_config2_sampled_and_restart(bnd):
