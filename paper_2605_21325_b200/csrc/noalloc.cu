@@ -90,7 +90,7 @@ extern "C" int tri_inv_fused_packed_static(const void* K, const void* V, const f
   bool handled = false;
   err = cudaSuccess;
   if (!(method & TRI_INV_FORCE_SIMT)) err = launch_tc(p, desc->C, stream, &handled);
-  if (err == cudaSuccess && !handled) err = launch_simt(p, desc->C, stream);
+  if (err == cudaSuccess && !handled) err = f32_factors_fit(p, desc->C) ? launch_f32_factors(p, stream) : launch_simt(p, desc->C, stream);   // as tri_inv_fused
   if (err == cudaSuccess) count_launch();
   return err == cudaSuccess ? TRI_INV_OK : TRI_INV_ERR_CUDA;
 }

@@ -70,3 +70,15 @@ def test_f32_factors_keep_a_tokens_infinity_to_later_rows(bnd):
         torch.cuda.synchronize()
         for x, r in zip(out, ref):
             assert torch.equal(x[:, :t], r[:, :t])
+
+
+def test_static_packed_call_gives_the_ordinary_calls_bits_in_fp32(bnd):
+    cu = np.array([0, 1, 65, 65, 192, 321], np.int32)
+    for d_k, d_v in ((64, 64), (128, 40), (136, 64)):   # both instances, and a dimension that they do not take
+        inp = wl.make("static", 1, 321, 3, d_k, d_v, 64, wl.F32, seed=840, cu_seqlens=cu)
+        dev = bnd.to_device(inp)
+        ref = bnd.fused(dev["K"], dev["V"], dev["beta"], dev["g"], 64, cu_seqlens=cu)
+        got = bnd.fused_packed_static(dev["K"], dev["V"], dev["beta"], dev["g"], 64, cu)
+        torch.cuda.synchronize()
+        for x, r in zip(got, ref):
+            assert torch.equal(x, r)
