@@ -37,9 +37,17 @@ __device__ __forceinline__ float load_one(const void* p, int bf16, size_t i) {
   return bf16 ? __bfloat162float(((const __nv_bfloat16*)p)[i]) : ((const float*)p)[i];
 }
 
+// k and q of the sequence's tokens, read four features at a time
+template <int KR>
+struct alignas(16) TokenRows {
+  float k[kMaxTokens][kWarps * KR], q[kMaxTokens][kWarps * KR];
+  static_assert(KR % 4 == 0, "a warp's features start on 16 bytes in every row");
+};
+
 template <int KR, class Args>   // features per warp
 __global__ void __launch_bounds__(kWarps * 32) recurrence_kernel(const __grid_constant__ Args a) {
-  __shared__ float sk[kMaxTokens][kWarps * KR], sq[kMaxTokens][kWarps * KR];
+  __shared__ TokenRows<KR> rows;
+  float (&sk)[kMaxTokens][kWarps * KR] = rows.k, (&sq)[kMaxTokens][kWarps * KR] = rows.q;
   __shared__ float s_alpha[kMaxTokens], s_beta[kMaxTokens], s_kq[kMaxTokens];
   __shared__ float2 part[2][kWarps][kCols];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;

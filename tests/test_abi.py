@@ -110,3 +110,19 @@ def test_scan_warps_wait_as_a_whole():
     src = open(os.path.join(ROOT, "paper_2605_21325_b200", "csrc", "scan_kernel.cu")).read()
     roles = src[src.index("if (warp == kControl) {"):src.index("constexpr int kSeqsPerLaunch")]
     assert not re.findall(r"if \([^;{]*mbar_(?:try_)?wait\w*\([^;{]*", roles)
+
+
+def test_shared_arrays_that_are_read_as_vectors_are_aligned():
+    """A static shared array that is read as float4 has its 16 bytes from its declaration, not from where the compiler happens to
+    put it: every __shared__ float array is declared with an alignment, or is in a type that has one, where its file reads
+    shared memory in fours."""
+    import glob
+    csrc = os.path.join(ROOT, "paper_2605_21325_b200", "csrc")
+    for path in glob.glob(os.path.join(csrc, "*.cu")) + glob.glob(os.path.join(csrc, "*.cuh")):
+        src = open(path).read()
+        for line in re.findall(r"^.*__shared__.*;", src, flags=re.M):
+            m = re.search(r"__shared__\s+(__align__\(16\)\s+)?float\s+(.*);", line)
+            if not m or m.group(1) or "extern" in line:
+                continue
+            for name in re.findall(r"(\w+)(?:\[[^\]]*\])+", m.group(2)):
+                assert not re.search(r"<(?:const )?float4\*>\(&?%s\b" % name, src), (os.path.basename(path), name)
