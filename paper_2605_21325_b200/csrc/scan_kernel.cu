@@ -548,15 +548,16 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
       TL(0);
       if (!wait(bar_full + 8 * (c % kStages), full_parity(c))) { failed = true; break; }   // landed long ago; U is read below
       TL(1);
-      if (!wait(bar_t1, ph)) { failed = true; break; }
-      tc_fence_after();
-      TL(2);
       if (rows < C) {
         // The tile's rows past the sequence's end hold what follows it in memory: a neighbour's keys or, per channel beside the preparation,
         // scratch that nobody may have written yet.  U~ is zero there, but zero times Inf or NaN is not: the state product must find
-        // zeros.  QK, the tile's other reader, was issued before the product just waited for.
+        // zeros.  After QK, the tile's other reader, and beside the first product.
+        if (!wait(bar_qk, ph)) { failed = true; break; }
         clear_rows(s0 + (c % kStages) * cfg::STAGE + cfg::OFF_KT, cfg::K_BOX, rows, tid);
       }
+      if (!wait(bar_t1, ph)) { failed = true; break; }
+      tc_fence_after();
+      TL(2);
       // ---- U~ = U - W S, transposed: first the decay-scaled U~' that the chain waits for (its own arrival), then U~ itself
       float v[LG][4][4];
 #pragma unroll
