@@ -264,7 +264,8 @@ int tri_inv_chunk_scan_kda(const void* Q, const void* K, const void* W, const vo
  * cuda_stream; nothing is allocated except, from the library's stream-ordered pool, n_sequences + 1 ints in ragged mode, and at
  * most 128 MiB of scratch (more only if a single chunk of every sequence and head needs it) for fp32 storage with C = 64 and
  * d_k <= 128, where longer inputs go through in segments; if that scratch cannot be had, the kernel of the other shapes
- * takes the call.  A device-side wait that expires raises TRI_INV_ERR_DEVICE_TIMEOUT in the status word.
+ * takes the call.  What came from the pool stays reserved there for later calls; captured in a graph, such a call is one of memory
+ * nodes (tri_inv_gdn_forward's scratch is its caller's).  A device-side wait that expires raises TRI_INV_ERR_DEVICE_TIMEOUT in the status word.
  */
 int tri_inv_chunk_scan(const void* Q, const void* K, const void* W, const void* U, const float* g, const float* S0,
                        void* O, float* S_out, float scale, const tri_inv_desc* desc, void* cuda_stream);
@@ -277,7 +278,7 @@ int tri_inv_chunk_scan(const void* Q, const void* K, const void* W, const void* 
  *   - block recursion without flags, bf16 with d_k = d_v = 128 and C = 64, few enough (sequence, head) pairs to be walked at the
  *     same time: the two calls in ONE kernel, the scan of a pair running beside the factors of its later chunks -- their
  *     results bit for bit.  Two launches on cuda_stream (a small one fills the workspace's words); nothing is allocated.
- *   - otherwise the two calls.
+ *   - otherwise the two calls, with W, U and the fp32 scan's scratch in the workspace.
  * So a sequence continued from a returned state gives the same bits as in one go only if both are cut at chunk boundaries and neither
  * takes the first route.  Arguments as in the two calls; O may not overlap an input.  `workspace`: device memory of at least
  * tri_inv_gdn_forward_workspace() bytes (which may be 0: then it may be NULL), 16-byte aligned, contents arbitrary; nothing else may use it

@@ -255,10 +255,24 @@ int tri_inv_build_kda(const void* K, const float* G, const float* beta, float* A
 }  // extern "C"
 
 namespace {
-// Shared body of the two chunk-scan entry points: exactly one of g (scalar gate) and G (per-channel gate) is given.
+int longest_sequence(const tri_inv_desc* d) {
+  if (!d->cu_seqlens) return d->T;
+  int n = 0;
+  for (int q = 0; q < d->n_seqs; ++q) n = std::max(n, d->cu_seqlens[q + 1] - d->cu_seqlens[q]);
+  return n;
+}
+
+// The register-tiled fp32 scan with a scalar gate: its shapes, and the scratch of a call.
+bool f32_scan_fits(const tri_inv_desc* d) { return d->kv_dtype == TRI_INV_F32 && d->C == 64 && d->d_k <= 128; }
+size_t f32_scan_scratch(const tri_inv_desc* d, int* n_seg) {
+  return chunk_scan_f32_scratch((long long)(d->cu_seqlens ? d->n_seqs : d->B) * d->H, (longest_sequence(d) + 63) / 64, d->d_k, d->d_v, n_seg);
+}
+
+// Shared body of the two chunk-scan entry points: exactly one of g (scalar gate) and G (per-channel gate) is given.  f32_scratch: of
+// f32_scan_scratch() bytes, the caller's; from the library's pool if it is not given.
 int chunk_scan_any(const void* Q, const void* K, const void* W, const void* U, const float* g, const float* G, const float* S0,
                    void* O, float* S_out, float scale, const tri_inv_desc* desc, void* cuda_stream,
-                   unsigned long long wait_limit_ns = 0, int test_stall = 0) {
+                   unsigned long long wait_limit_ns = 0, int test_stall = 0, void* f32_scratch = nullptr) {
   int rc = check_desc(desc, true);
   if (rc) return rc;
   if (!Q || !K || !W || !U || (!g && !G) || !O) return TRI_INV_ERR_INVALID_ARG;
@@ -291,11 +305,7 @@ int chunk_scan_any(const void* Q, const void* K, const void* W, const void* U, c
     }
     p.seq_off = dev_off;
   }
-  int max_len = desc->T;   // of the sequences
-  if (desc->cu_seqlens) {
-    max_len = 0;
-    for (int q = 0; q < desc->n_seqs; ++q) max_len = std::max(max_len, desc->cu_seqlens[q + 1] - desc->cu_seqlens[q]);
-  }
+  const int max_len = longest_sequence(desc);
   void* work = nullptr;
   if (tc && G && tokens > 0) {
     // Per-channel gate on the tensor cores: Q+, K- (bf16, the tensors' own shape) and the per-chunk vectors
@@ -321,14 +331,12 @@ int chunk_scan_any(const void* Q, const void* K, const void* W, const void* U, c
       if (err == cudaSuccess) err = launch_chunk_scan(p, Qp, Km, W, tokens, stream, true);
     }
   } else {
-    const bool f32 = !G && desc->kv_dtype == TRI_INV_F32 && desc->C == 64 && desc->d_k <= 128;
-    if (f32) {
+    if (!G && f32_scan_fits(desc)) {
       int n_seg = 0;
-      const int max_chunks = (max_len + 63) / 64;
-      const size_t bytes = chunk_scan_f32_scratch((long long)p.n_seqs * p.H, max_chunks, desc->d_k, desc->d_v, &n_seg);
-      cudaMemPool_t pool = table_pool_for_current_device();
-      if (bytes == 0 || (pool && cudaMallocFromPoolAsync(&work, bytes, pool, stream) == cudaSuccess)) {
-        err = launch_chunk_scan_f32(p, Q, K, W, desc->d_k, desc->d_v, max_chunks, tokens > 0 ? tokens : 1, work, n_seg, stream);
+      const size_t bytes = f32_scan_scratch(desc, &n_seg);
+      cudaMemPool_t pool = f32_scratch || bytes == 0 ? nullptr : table_pool_for_current_device();
+      if (f32_scratch || bytes == 0 || (pool && cudaMallocFromPoolAsync(&work, bytes, pool, stream) == cudaSuccess)) {
+        err = launch_chunk_scan_f32(p, Q, K, W, desc->d_k, desc->d_v, (max_len + 63) / 64, tokens > 0 ? tokens : 1, f32_scratch ? f32_scratch : work, n_seg, stream);
       } else {   // no scratch to be had: the kernel that needs none
         (void)cudaGetLastError();
         work = nullptr;
@@ -359,7 +367,8 @@ LayerRoute layer_route(const tri_inv_desc* d, int method, size_t* workspace_byte
     if (recurrence_fits(d)) return kTokens;
     if (d->kv_dtype == TRI_INV_BF16 && d->d_k == 128 && d->d_v == 128 && d->C == 64 && layer_fits(d, workspace_bytes)) return kOneKernel;
   }
-  *workspace_bytes = factor_bytes(d, d->d_k) + factor_bytes(d, d->d_v);
+  int n_seg;
+  *workspace_bytes = factor_bytes(d, d->d_k) + factor_bytes(d, d->d_v) + (f32_scan_fits(d) ? f32_scan_scratch(d, &n_seg) : 0);
   return kTwoCalls;
 }
 }  // namespace
@@ -401,8 +410,9 @@ int tri_inv_gdn_forward(const void* Q, const void* K, const void* V, const float
   if (route == kTwoCalls) {
     void* W = workspace;
     void* U = reinterpret_cast<char*>(workspace) + factor_bytes(desc, desc->d_k);
+    void* scratch = reinterpret_cast<char*>(U) + factor_bytes(desc, desc->d_v);
     if ((rc = tri_inv_fused(K, V, beta, g, nullptr, W, U, desc, method | TRI_INV_W_DECAY, cuda_stream))) return rc;
-    return tri_inv_chunk_scan(Q, K, W, U, g, S0, O, S_out, scale, desc, cuda_stream);
+    return chunk_scan_any(Q, K, W, U, g, nullptr, S0, O, S_out, scale, desc, cuda_stream, 0, 0, f32_scan_fits(desc) ? scratch : nullptr);
   }
   ScanParams p{};
   p.g = g; p.S0 = S0; p.O = O; p.S_out = S_out; p.scale = scale;

@@ -4,6 +4,8 @@ One kernel (factors and scans side by side): the arithmetic is that of the two c
 bit.  Token by token: fp32 arithmetic on the stored inputs, against the fp64 recurrence: fp32 storage 1e-5 of max|O| (at most 16
 steps of sums of up to 128 terms, 2^-24 each), bf16 storage 2^-8 (the output's own rounding), the state 1e-5.
 """
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -253,3 +255,51 @@ def test_every_launch_that_computes_is_counted(bnd):
         x = torch.zeros((1, 64 * chunks, H, 128), device="cuda")
         g = torch.zeros((1, 64 * chunks, H), device="cuda")
         assert counted(lambda: bnd.chunk_scan(x, x, x, x, g, 64)) == launches
+
+
+def graph_allocations(graph):
+    """Memory nodes of a captured graph."""
+    lib = ctypes.CDLL("libcuda.so.1")
+    g, n = ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t(0)
+    assert lib.cuGraphGetNodes(g, None, ctypes.byref(n)) == 0
+    nodes = (ctypes.c_void_p * n.value)()
+    assert lib.cuGraphGetNodes(g, nodes, ctypes.byref(n)) == 0
+    kind, count = ctypes.c_int(0), 0
+    for x in nodes:
+        assert lib.cuGraphNodeGetType(ctypes.c_void_p(x), ctypes.byref(kind)) == 0
+        count += kind.value == 10   # CU_GRAPH_NODE_TYPE_MEM_ALLOC
+    return count
+
+
+@pytest.mark.parametrize("scan_only", [False, True])
+def test_fp32_calls_in_a_graph(bnd, scan_only):
+    """The layer's scratch is part of its workspace: a dense call takes nothing from the library's pool, so its graph has no memory
+    nodes.  The scan by itself has them; either is replayed on new inputs in the same buffers, twice."""
+    args = [layer_inputs(bnd, "graph32", 2, 3 * 64 + 5, 3, 64, 64, wl.F32, None, 850 + 10 * i) for i in range(2)]
+    if scan_only:
+        for a in args:
+            a[3]["W"], a[3]["U"] = bnd.fused(a[3]["K"], a[3]["V"], a[3]["beta"], a[3]["g"], 64, method=bnd.W_DECAY, want_A=False)[1:]
+        run = lambda a: bnd.chunk_scan(a[4], a[3]["K"], a[3]["W"], a[3]["U"], a[3]["g"], 64, scale=0.5, S0=a[5])
+    else:
+        run = lambda a: bnd.gdn_forward(a[4], a[3]["K"], a[3]["V"], a[3]["beta"], a[3]["g"], 64, scale=0.5, S0=a[5])
+    refs = [[t.clone() for t in run(a)] for a in args]
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        out = run(args[0])
+    assert graph_allocations(graph) == (1 if scan_only else 0)
+    graph.instantiate()
+    for ref, src in ((refs[0], None), (refs[1], args[1]), (refs[1], None)):
+        if src is not None:
+            args[0][4].copy_(src[4])
+            args[0][5].copy_(src[5])
+            for k in args[0][3]:
+                if torch.is_tensor(args[0][3][k]):
+                    args[0][3][k].copy_(src[3][k])
+        for t in out:
+            t.fill_(float("nan"))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert bnd.last_device_status() == 0
+        for x, r in zip(out, ref):
+            assert torch.equal(x, r)
