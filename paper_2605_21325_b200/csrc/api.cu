@@ -408,6 +408,7 @@ int tri_inv_gdn_forward(const void* Q, const void* K, const void* V, const float
       !aligned16(S_out) || !aligned16(workspace))
     return TRI_INV_ERR_INVALID_ARG;
   if (route == kTwoCalls) {
+    if (!need) workspace = O;   // no token: neither W nor U is touched
     void* W = workspace;
     void* U = reinterpret_cast<char*>(workspace) + factor_bytes(desc, desc->d_k);
     void* scratch = reinterpret_cast<char*>(U) + factor_bytes(desc, desc->d_v);

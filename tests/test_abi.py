@@ -103,6 +103,42 @@ def test_newer_entry_points_validate_on_the_host(lib):
     assert L.tri_inv_chunk_scan(ok, ok, ok, ok, ok, None, ok, None, scale, ctypes.byref(wide), None) == binding.ERR_UNSUPPORTED
 
 
+def test_layer_call_validates_on_the_host(lib):
+    """Every call below is refused before any device work: one argument is wrong in each."""
+    L, binding = lib
+    ok, odd, scale = 4096, 4100, ctypes.c_float(1.0)
+    for dims in ((1, 640, 2, 128, 128, 64, binding.BF16), (1, 640, 2, 64, 64, 64, binding.F32), (2, 3, 2, 64, 64, 64, binding.F32)):
+        d, _ = binding.make_desc(*dims)
+        p = ctypes.byref(d)
+        need = ctypes.c_size_t(0)
+        assert L.tri_inv_gdn_forward_workspace(p, 0, ctypes.byref(need)) == binding.OK
+        assert L.tri_inv_gdn_forward_workspace(p, 0, None) == binding.ERR_INVALID_ARG
+        assert L.tri_inv_gdn_forward_workspace(None, 0, ctypes.byref(need)) == binding.ERR_INVALID_ARG
+        good = dict(Q=ok, K=ok, V=ok, beta=ok, g=ok, S0=ok, O=ok, S=ok, scale=scale, work=ok, bytes=need.value, desc=p, method=0, stream=None)
+        call = lambda **kw: L.tri_inv_gdn_forward(*dict(good, **kw).values())
+        for name in ("Q", "K", "V", "beta", "g", "O"):
+            assert call(**{name: None}) == binding.ERR_INVALID_ARG
+        for name in ("Q", "K", "V", "beta", "g", "S0", "O", "S", "work"):
+            assert call(**{name: odd}) == binding.ERR_INVALID_ARG
+        if need.value:
+            assert call(work=None) == binding.ERR_INVALID_ARG and call(bytes=need.value - 1) == binding.ERR_INVALID_ARG
+        assert call(desc=None) == binding.ERR_INVALID_ARG
+        assert call(method=7) == binding.ERR_UNSUPPORTED and call(method=binding.LEAF_SERIES | binding.PRODUCT_SERIES) == binding.ERR_UNSUPPORTED
+
+
+def test_layer_call_without_tokens(lib):
+    """No token, no workspace: not an error, whatever the scheme (nothing is launched; without a device the status says so)."""
+    L, binding = lib
+    ok = 4096
+    for method in (binding.BLOCK_RECURSIVE, binding.PRODUCT_SERIES):
+        for d_k in (128, 192):
+            d, _ = binding.make_desc(1, 0, 2, d_k, 128, 64, binding.BF16)
+            need = ctypes.c_size_t(1)
+            assert L.tri_inv_gdn_forward_workspace(ctypes.byref(d), method, ctypes.byref(need)) == binding.OK and need.value == 0
+            rc = L.tri_inv_gdn_forward(ok, ok, ok, ok, ok, None, ok, None, ctypes.c_float(1.0), None, 0, ctypes.byref(d), method, None)
+            assert rc in (binding.OK, binding.ERR_CUDA)
+
+
 def test_scan_warps_wait_as_a_whole():
     """What follows a wait in the scan kernel's warp roles takes the full warp (tcgen05.ld / st, ldmatrix, __syncwarp), so no
     role may branch on the outcome of a wait lane by lane: each branches on wait(), whose lanes agree.  The per-lane
