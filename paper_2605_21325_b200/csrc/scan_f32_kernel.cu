@@ -144,7 +144,9 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) scan_f32_chain(con
     for_state([&](float& x, int k, int n) { S[(k >> 2) * cfg::S_BLK + (k & 3) * NS + n] = x; });
   };
   auto rows_of = [&](int c) { const int left = end - beg - (a.c0 + c) * kC; return left < kC ? left : kC; };
+  int requested = -1;   // thread 0: the last chunk whose tiles it asked for
   auto copy_tiles = [&](int c) {   // by one thread; features past d_k are filled with zeros, rows past the sequence's end hold what follows
+    requested = c;
     const int st = c % cfg::kStages, tok0 = beg + (a.c0 + c) * kC;
     const uint32_t dst = smem_u32(tiles + st * 2 * cfg::TILE), bar = bars + 8 * st;
     const int boxes = (a.d_k + 31) / 32;
@@ -261,7 +263,7 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) scan_f32_chain(con
   if (bad) {   // the copies still on their way get a bounded chance to land before the CTA's shared memory is given up
     atomicMax(p.status, TRI_INV_ERR_DEVICE_TIMEOUT);
     if (tid == 0 && (smem_u32(sm) & 1023u) == 0)
-      for (int c = n_chunks > cfg::kStages ? n_chunks - cfg::kStages : 0; c < n_chunks; ++c)
+      for (int c = requested >= cfg::kStages ? requested - cfg::kStages + 1 : 0; c <= requested; ++c)   // the last of each stage
         mbar_wait_bounded(bars + 8 * (c % cfg::kStages), (uint32_t)(c / cfg::kStages) & 1u, p.wait_limit_ns ? p.wait_limit_ns : kWaitLimitNs);
   }
   if (a.c0 + n_chunks < n_all) put_state(a.carry + state_base);

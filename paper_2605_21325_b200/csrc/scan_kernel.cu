@@ -266,7 +266,7 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
   auto full_parity = [](int c) { return (uint32_t)((c / kStages) & 1); };
   int requested = -1;   // lane 0 of the warp that requests the copies: the last chunk whose copies were requested
   auto drain_copies = [&]() {   // give-up path: the copies still on their way into this CTA's shared memory, with a limit
-    for (int c = requested - 1 > 0 ? requested - 1 : 0; c <= requested; ++c) mbar_wait_bounded(bar_full + 8 * (c % kStages), full_parity(c), lim);
+    for (int c = requested >= kStages ? requested - kStages + 1 : 0; c <= requested; ++c) mbar_wait_bounded(bar_full + 8 * (c % kStages), full_parity(c), lim);
   };
   // g of a chunk, by the gate warp (lane l: tokens l and l + 32).  Rows past the sequence end take the last real
   // row's g, so that every exponent stays a difference of real values.

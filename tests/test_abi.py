@@ -148,6 +148,24 @@ def test_scan_warps_wait_as_a_whole():
     assert not re.findall(r"if \([^;{]*mbar_(?:try_)?wait\w*\([^;{]*", roles)
 
 
+@pytest.mark.parametrize("name", ["scan_kernel.cu", "scan_f32_kernel.cu"])
+def test_a_block_that_gives_up_waits_for_the_last_copy_of_every_stage(name):
+    """The loop behind a wait that has run out, as the source has it, against the copies that can be on their way: for every chunk at
+    which the requests can end, each stage's last one is waited for with its own parity (another parity's wait returns at once)."""
+    src = open(os.path.join(ROOT, "paper_2605_21325_b200", "csrc", name)).read()
+    m = re.search(r"for \(int c = (requested[^;]*|n_chunks[^;]*); c (<=?) (\w+); \+\+c\)(?: *//[^\n]*)?\s*mbar_wait_bounded\(", src)
+    cond, a, b = re.match(r"(.*) \? (.*) : (.*)", m.group(1).replace("cfg::", "")).groups()
+    for stages in (2, 3):
+        for n_chunks in (1, 2, 5, 32):
+            for requested in range(n_chunks):
+                env = dict(requested=requested, n_chunks=n_chunks, kStages=stages)
+                first = eval(a, {}, env) if eval(cond, {}, env) else eval(b, {}, env)
+                last = env[m.group(3)] if m.group(2) == "<=" else env[m.group(3)] - 1
+                waited = {(c % stages, c // stages % 2) for c in range(first, last + 1)}
+                for c in range(max(0, requested - stages + 1), requested + 1):
+                    assert (c % stages, c // stages % 2) in waited, (stages, n_chunks, requested)
+
+
 def test_shared_arrays_that_are_read_as_vectors_are_aligned():
     """A static shared array that is read as float4 has its 16 bytes from its declaration, not from where the compiler happens to
     put it: every __shared__ float array is declared with an alignment, or is in a type that has one, where its file reads
