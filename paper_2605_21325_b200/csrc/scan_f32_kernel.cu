@@ -571,7 +571,9 @@ cudaError_t launch_segments(const ScanParams& p, F32Args a, int max_chunks, long
   const long long pairs = (long long)p.n_seqs * p.H;
   // eight columns a CTA while that is no more than two CTAs for each SM: half the work on the chain; beyond it the wider slice reads
   // W and K half as often
-  const bool wide = pairs * ((a.d_v + 7) / 8) > 2 * 148;
+  int dev = 0, sms = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  const bool wide = pairs * ((a.d_v + 7) / 8) > 2 * sms;
   for (a.c0 = 0; a.c0 < max_chunks; a.c0 += a.n_seg) {
     e = wide ? launch_chain<DK, 16>(tmW, tmK, p, a, pairs, stream) : launch_chain<DK, 8>(tmW, tmK, p, a, pairs, stream);
     if (e != cudaSuccess) return e;
