@@ -299,6 +299,10 @@ int tri_inv_selftest_layer_wait_timeout(const void* Q, const void* K, const void
                                         void* workspace, size_t workspace_bytes, const tri_inv_desc* desc, uint64_t wait_limit_ns,
                                         void* cuda_stream);
 
+/* The same for the per-channel scan in one kernel: the first chunk's operands are written but never announced. */
+int tri_inv_selftest_kda_scan_wait_timeout(const void* Q, const void* K, const void* W, const void* U, const float* G, void* O,
+                                           const tri_inv_desc* desc, uint64_t wait_limit_ns, void* cuda_stream);
+
 /*
  * Fused call with the layer's front end folded in: the kernel takes what the projections produce and
  * does the three producers that otherwise run as separate passes over memory before the inversion

@@ -112,6 +112,9 @@ def load():
         if hasattr(lib, "tri_inv_selftest_layer_wait_timeout"):
             lib.tri_inv_selftest_layer_wait_timeout.argtypes = [vp, vp, vp, vp, vp, vp, vp, ctypes.c_size_t, dp, ctypes.c_uint64, vp]
             lib.tri_inv_selftest_layer_wait_timeout.restype = i32
+        if hasattr(lib, "tri_inv_selftest_kda_scan_wait_timeout"):
+            lib.tri_inv_selftest_kda_scan_wait_timeout.argtypes = [vp, vp, vp, vp, vp, vp, dp, ctypes.c_uint64, vp]
+            lib.tri_inv_selftest_kda_scan_wait_timeout.restype = i32
         lib.tri_inv_count_matrices.argtypes = [dp, ctypes.POINTER(ctypes.c_int64)]
         lib.tri_inv_last_device_status.argtypes = [ctypes.POINTER(ctypes.c_int)]
         for f in ("tri_inv_build", "tri_inv_wy", "tri_inv_fused", "tri_inv_count_matrices", "tri_inv_last_device_status"):
@@ -381,6 +384,17 @@ def selftest_scan_wait_timeout(Q, K, W, U, g, C, wait_limit_ns, out, stream=None
                                                    ctypes.c_uint64(int(wait_limit_ns)), _stream(stream))
     if rc != OK:
         raise TriInvError("tri_inv_selftest_scan_wait_timeout", rc)
+    return out
+
+
+def selftest_kda_scan_wait_timeout(Q, K, W, U, G, C, wait_limit_ns, out, stream=None):
+    """tri_inv_selftest_kda_scan_wait_timeout: the one-kernel per-channel scan with short wait limits and the first chunk never announced
+    to the scans of the first head.  ``out`` = O."""
+    B, T, H, d_k = K.shape
+    desc, keep = make_desc(B, T, H, d_k, U.shape[3], C, _dtype_code(K), None)
+    rc = load().tri_inv_selftest_kda_scan_wait_timeout(_p(Q), _p(K), _p(W), _p(U), _p(G), _p(out), desc, ctypes.c_uint64(int(wait_limit_ns)), _stream(stream))
+    if rc != OK:
+        raise TriInvError("tri_inv_selftest_kda_scan_wait_timeout", rc)
     return out
 
 

@@ -450,6 +450,19 @@ int tri_inv_selftest_layer_wait_timeout(const void* Q, const void* K, const void
   return err == cudaSuccess && cudaStreamSynchronize((cudaStream_t)cuda_stream) == cudaSuccess ? TRI_INV_OK : TRI_INV_ERR_CUDA;
 }
 
+int tri_inv_selftest_kda_scan_wait_timeout(const void* Q, const void* K, const void* W, const void* U, const float* G, void* O,
+                                           const tri_inv_desc* desc, uint64_t wait_limit_ns, void* cuda_stream) {
+  int rc = check_desc(desc, true);
+  if (rc) return rc;
+  if (!G || wait_limit_ns == 0) return TRI_INV_ERR_INVALID_ARG;
+  size_t control_bytes = 0;   // only the one-kernel form waits for another block
+  if (desc->kv_dtype != TRI_INV_BF16 || desc->d_k != 128 || desc->d_v != 128 || desc->C != 64 || !kda_scan_fits(desc, &control_bytes))
+    return TRI_INV_ERR_UNSUPPORTED;
+  rc = chunk_scan_any(Q, K, W, U, nullptr, G, nullptr, O, nullptr, 1.f, desc, cuda_stream, wait_limit_ns, 1);
+  if (rc) return rc;
+  return cudaStreamSynchronize((cudaStream_t)cuda_stream) == cudaSuccess ? TRI_INV_OK : TRI_INV_ERR_CUDA;
+}
+
 int tri_inv_selftest_scan_wait_timeout(const void* Q, const void* K, const void* W, const void* U, const float* g, void* O,
                                        const tri_inv_desc* desc, uint64_t wait_limit_ns, void* cuda_stream) {
   int rc = check_desc(desc, true);

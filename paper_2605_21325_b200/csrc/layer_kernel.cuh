@@ -50,7 +50,7 @@ struct LayerParams {
   int sms;
   int groups;                    // of these CTAs: four each
   unsigned long long wait_limit_ns;
-  int test_stall;           // self-test: the first matrix is never announced
+  int test_stall;           // self-test: the first matrix (per-channel scan: the first chunk) is never announced
 };
 
 struct Place { int tok0, rows, h, slot; };
@@ -500,7 +500,7 @@ __device__ __forceinline__ void prepare_chunks(const LayerParams& p, const KdaOp
     asm volatile("fence.proxy.async;" ::: "memory");   // ordinary stores, read by the scans' tile copies
     if (tid == 0) leave(ticket);
     sync();
-    if (tid == 0) asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p.ready + ((size_t)at.slot * p.H + at.h)), "r"(kReady) : "memory");
+    if (tid == 0 && !(p.test_stall && item == 0)) asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p.ready + ((size_t)at.slot * p.H + at.h)), "r"(kReady) : "memory");
     item = nx_item;
     at = nx;
     nx_item = take(nx);

@@ -209,6 +209,96 @@ def test_scan_does_not_multiply_a_neighbours_keys(bnd):
         assert torch.equal(o[0], outs[0][0]) and torch.equal(o[1], outs[0][1])
 
 
+def kda_operands(bnd, B, T, H, seed):
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    normal = lambda *s: torch.randn(*s, device="cuda", generator=gen)
+    unit = lambda x: (x / x.norm(dim=-1, keepdim=True)).to(torch.bfloat16)
+    Q, K, V, beta = unit(normal(B, T, H, 128)), unit(normal(B, T, H, 128)), normal(B, T, H, 128).to(torch.bfloat16), torch.sigmoid(normal(B, T, H))
+    rate = -0.05 * torch.rand(B, 1, H, 128, device="cuda", generator=gen)
+    G = rate * (1 + torch.arange(T, device="cuda") % 64)[None, :, None, None]   # cumulative within each chunk
+    _, W, U = bnd.fused_kda(K, V, G.contiguous(), beta, 64)
+    return Q, K, W, U, G.contiguous()
+
+
+@pytest.mark.parametrize("B,T,H", [(1, 130 * 64, 8), (1, 80 * 64, 32), (2, 130 * 64, 26)], ids=["32_columns", "64_columns", "128_columns"])
+def test_per_channel_one_kernel_waits_that_run_out(bnd, B, T, H):
+    """As above: the first chunk's operands are never announced, so the scans of the first sequence's first head give up."""
+    args = kda_operands(bnd, B, T, H, 796)
+    n0 = bnd.launch_count()
+    ref, S_ref = bnd.chunk_scan_kda(*args, 64)
+    torch.cuda.synchronize()
+    assert bnd.last_device_status() == 0 and bnd.launch_count() == n0 + 1
+    O = torch.full_like(args[3], float("nan"))
+    bnd.selftest_kda_scan_wait_timeout(*args, 64, wait_limit_ns=2_000_000, out=O)
+    assert bnd.last_device_status() == bnd.ERR_DEVICE_TIMEOUT
+    assert bnd.last_device_status() == 0
+    assert torch.equal(bits(O[:, :, 1:]), bits(ref[:, :, 1:])) and torch.equal(bits(O[1:]), bits(ref[1:]))
+    again, S = bnd.chunk_scan_kda(*args, 64)
+    torch.cuda.synchronize()
+    assert bnd.last_device_status() == 0
+    assert torch.equal(bits(again), bits(ref)) and torch.equal(bits(S), bits(S_ref))
+
+
+def test_per_channel_one_kernel_on_two_streams_and_in_a_graph(bnd):
+    """As the layer's test of that name."""
+    args = [kda_operands(bnd, 1, 80 * 64 + 5, 32, 797 + i) for i in range(2)]
+    refs = [bnd.chunk_scan_kda(*a, 64) for a in args]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    outs = []
+    for _ in range(6):
+        for a, st in zip(args, streams):
+            with torch.cuda.stream(st):
+                outs.append(bnd.chunk_scan_kda(*a, 64, stream=st))
+    torch.cuda.synchronize()
+    assert bnd.last_device_status() == 0
+    for i, o in enumerate(outs):
+        assert torch.equal(bits(o[0]), bits(refs[i % 2][0])) and torch.equal(bits(o[1]), bits(refs[i % 2][1]))
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        O, S = bnd.chunk_scan_kda(*args[0], 64)
+    for x, y in zip(*args):
+        x.copy_(y)
+    for _ in range(2):
+        O.fill_(float("nan"))
+        S.fill_(float("nan"))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(bits(O), bits(refs[1][0])) and torch.equal(bits(S), bits(refs[1][1]))
+
+
+# one kernel (dense, packed with partial and empty sequences); two calls (bf16 with more pairs than walk at once; fp32 in one segment)
+WORKSPACES = [
+    ("one_kernel", 2, 333, 3, 128, wl.BF16, None),
+    ("one_kernel_packed", 1, 0, 16, 128, wl.BF16, np.array([0, 64, 64, 65, 300, 531, 540], np.int32)),
+    ("two_calls", 4, 70, 64, 128, wl.BF16, None),
+    ("fp32", 2, 197, 3, 64, wl.F32, None),
+    ("fp32_packed", 1, 0, 3, 72, wl.F32, np.array([0, 64, 64, 65, 300], np.int32)),
+]
+
+
+@pytest.mark.parametrize("name,B,T,H,d,dtype,cu", WORKSPACES, ids=[c[0] for c in WORKSPACES])
+def test_workspace_contents_are_arbitrary(bnd, name, B, T, H, d, dtype, cu):
+    """Zeros, all bits set (NaN in either type, counters far from zero) and what the call before left: the same bits."""
+    inp, _, _, dev, Q, S0 = layer_inputs(bnd, name, B, T, H, d, d, dtype, cu, 860)
+    desc, keep = bnd.make_desc(inp.B, inp.T, H, d, d, 64, dtype, cu)
+    lib, need, results = bnd.load(), ctypes.c_size_t(0), []
+    assert lib.tri_inv_gdn_forward_workspace(desc, 0, need) == bnd.OK and need.value > 0
+    work = torch.zeros(need.value, dtype=torch.uint8, device="cuda")
+    for fill in (None, 255, None):
+        if fill is not None:
+            work.fill_(fill)
+        O, S = torch.full_like(dev["V"], float("nan")), torch.full_like(S0, float("nan"))
+        assert lib.tri_inv_gdn_forward(*(bnd._p(t) for t in (Q, dev["K"], dev["V"], dev["beta"], dev["g"], S0, O, S)), 0.5, bnd._p(work), need, desc, 0,
+                                       torch.cuda.current_stream().cuda_stream) == bnd.OK
+        torch.cuda.synchronize()
+        assert bnd.last_device_status() == 0
+        results.append((O, S))
+    for O, S in results[1:]:
+        assert torch.equal(bits(O), bits(results[0][0])) and torch.equal(bits(S), bits(results[0][1]))
+    assert torch.isfinite(results[0][0]).all() and torch.isfinite(results[0][1]).all()
+
+
 # one token, the longest, features and columns on both sides of the kernel's instances and slices, an empty sequence
 TOKENS = [
     ("decode", 4, 1, 3, 128, 128, None),
