@@ -264,6 +264,43 @@ def test_chunk_scan_fp32_tiles(bnd, name, B, T, H, d_k, d_v, cu):
     test_chunk_scan_cuda_core_kernel_other_shapes(bnd, name, B, T, H, d_k, d_v, 64, wl.F32, cu)
 
 
+# the chain's slices of 16 columns (more than two CTAs an SM in slices of eight): both instances, padded features and a cut last slice,
+# packed with a partial chunk, one token and an empty sequence
+F32_WIDE_CASES = [
+    ("d64", 1, 2 * 64 + 9, 40, 64, 64, None),
+    ("d128", 1, 130, 20, 128, 128, None),
+    ("d72_v24", 2, 129, 50, 72, 24, None),
+    ("d64_ragged", 1, 0, 12, 64, 64, np.array([0, 64, 64, 65, 200, 330], np.int32)),
+]
+
+
+@pytest.mark.parametrize("name,B,T,H,d_k,d_v,cu", F32_WIDE_CASES, ids=[c[0] for c in F32_WIDE_CASES])
+def test_chunk_scan_fp32_wide_slices(bnd, name, B, T, H, d_k, d_v, cu):
+    assert (B if cu is None else len(cu) - 1) * H * ((d_v + 7) // 8) > 2 * torch.cuda.get_device_properties(0).multi_processor_count
+    test_chunk_scan_cuda_core_kernel_other_shapes(bnd, name, B, T, H, d_k, d_v, 64, wl.F32, cu)
+
+
+@pytest.mark.parametrize("H,d_k,d_v", [(40, 128, 128), (44, 64, 64)])
+def test_fp32_scan_in_segments_against_its_definition(bnd, H, d_k, d_v):
+    """Two of the heads of a scan that goes through in segments, against fp64, at fp32's 1e-5; every row is written."""
+    T = 64 * ((128 << 20) // ((d_k + 64) * d_v * 4) // H + 3) + 9
+    inp = wl.make("segments", 1, T, H, d_k, d_v, 64, wl.F32, seed=790)
+    dev = bnd.to_device(inp)
+    Q = wl.queries(inp, seed=791)
+    Qd = bnd.kv_to_torch(Q)
+    _, W, U = bnd.fused(dev["K"], dev["V"], dev["beta"], dev["g"], 64, method=bnd.W_DECAY, want_A=False)
+    O = torch.full_like(dev["V"], float("nan"))
+    O, S = bnd.chunk_scan(Qd, dev["K"], W, U, dev["g"], 64, scale=0.5, out=O)
+    torch.cuda.synchronize()
+    assert bnd.last_device_status() == 0
+    assert torch.isfinite(O).all() and torch.isfinite(S).all()
+    cut = lambda x: np.ascontiguousarray(x[:, :, [0, H - 1]])
+    heads = lambda t: cut(t.cpu().numpy())
+    O_ref, S_ref = oracle.chunk_scan(cut(Q), cut(inp.K), heads(W), heads(U), cut(inp.g), 64, scale=0.5)
+    assert max_ratio(heads(O).astype(np.float64), O_ref) <= 1e-5
+    assert max_ratio(S[:, [0, H - 1]].cpu().numpy().astype(np.float64), S_ref) <= 1e-5
+
+
 @pytest.mark.parametrize("H,d_k,d_v", [(40, 128, 128), (44, 64, 64)])
 def test_fp32_scan_in_segments(bnd, H, d_k, d_v):
     """More (pair, chunk) slots than the scan's scratch holds: the state is carried between the segments, which gives the bits of
