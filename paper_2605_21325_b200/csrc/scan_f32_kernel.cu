@@ -17,6 +17,7 @@
 // The output kernel is bound by FFMA issue and shared-memory loads (8 per 64 FMAs).
 // Measured (ncu, B = 2, T = 2048, H = 8, d = 64: 16 pairs of 32 chunks): 44 + 27 us (50 + 28 with the chain's tiles by cp.async); 213 us as one kernel per slice of 16 columns that also
 // formed P and O on the way (P again in each slice, all of it on the chain, 64 CTAs).
+#include "f32_tiles.cuh"
 #include "tc_device.cuh"
 
 namespace tri_inv {
@@ -24,17 +25,6 @@ namespace {
 
 constexpr int kThreads = 256, kC = 64, kLdP = kC + 4, kNV = 64;   // kNV: value columns of an output CTA
 constexpr size_t kScratchBytes = (size_t)128 << 20;
-
-__device__ __forceinline__ void cp_async16(float* dst, const float* src, bool valid) {   // 16 bytes, zeros where not valid
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(valid ? 16 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int KEEP>
-__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(KEEP) : "memory"); }
-__device__ __forceinline__ float4 ld4(const float* p) { return *reinterpret_cast<const float4*>(p); }
-__device__ __forceinline__ void fma4(float (&acc)[4], float a, const float4& b) {
-  acc[0] = fmaf(a, b.x, acc[0]); acc[1] = fmaf(a, b.y, acc[1]); acc[2] = fmaf(a, b.z, acc[2]); acc[3] = fmaf(a, b.w, acc[3]);
-}
 
 struct F32Args {
   const float *Q, *K, *W, *U;
