@@ -308,10 +308,10 @@ int chunk_scan_any(const void* Q, const void* K, const void* W, const void* U, c
   const int max_len = longest_sequence(desc);
   void* work = nullptr;
   if (tc && G && tokens > 0) {
-    // Per-channel gate on the tensor cores: Q+, K- (bf16, the tensors' own shape) and the per-chunk vectors
+    // Per-channel gate on the tensor cores: Q+, K- (bf16) and the per-chunk vectors
     // exp(G_last), exp(G_ref), exp(G_last - G_ref), in stream-ordered scratch memory that is released behind the scan.
-    const size_t tensor_bytes = ((size_t)tokens * desc->H * 128 * 2 + 255) & ~(size_t)255;
     const size_t slots = (size_t)(tokens / 64) + (size_t)p.n_seqs + 1;
+    const size_t tensor_bytes = ((kda_one ? slots * 64 : (size_t)tokens) * desc->H * 128 * 2 + 255) & ~(size_t)255;   // one kernel: 64 rows for every chunk
     const size_t vec_bytes = (slots * desc->H * 128 * sizeof(float) + 255) & ~(size_t)255;
     cudaMemPool_t pool = table_pool_for_current_device();
     if (!pool || cudaMallocFromPoolAsync(&work, 2 * tensor_bytes + 3 * vec_bytes + control_bytes, pool, stream) != cudaSuccess) {

@@ -140,7 +140,7 @@ cudaError_t launch_recurrence(const void* Q, const void* K, const void* V, const
 cudaError_t launch_kda_scan_prep(const ScanParams& p, const void* Q, const void* K, void* Qp, void* Km,
                                  float* EL, float* ER, float* EX, int max_chunks_per_seq, cudaStream_t stream);
 // The two in one kernel, the preparation beside the scan (layer_kernel.cuh): whether that is the faster form, and the bytes of its words
-// (and table, and offsets) in addition to Qp, Km and the vectors; p.EL, ER, EX point to the latter, p.seq_off is not needed.
+// (and table, and offsets) in addition to Qp, Km (64 rows for every slot) and the vectors; p.EL, ER, EX point to the latter, p.seq_off is not needed.
 bool kda_scan_fits(const tri_inv_desc* d, size_t* control_bytes);
 cudaError_t launch_kda_scan(const ScanParams& p, const void* Q, const void* K, const void* W, void* Qp, void* Km, void* control,
                             const tri_inv_desc* d, cudaStream_t stream);

@@ -25,6 +25,8 @@
 #include <cmath>
 #include <mutex>
 
+#include "kda_operands.cuh"
+
 namespace tri_inv {
 namespace {
 
@@ -410,11 +412,11 @@ layer_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
 
 // ---------------------------------------------------------------- the per-channel scan beside the preparation of its operands
 // The same split of the chip for tri_inv_chunk_scan_kda: instead of matrices the groups prepare chunks (Q+, K- and the three vectors,
-// the arithmetic of kda_scan_prep_kernel, scan_kda_prep.cu), bound by the bytes they move.
+// as kda_scan_prep_kernel does: kda_operands.cuh), bound by the bytes they move.
 struct KdaOperands {
   const __nv_bfloat16 *Q, *K;
   const float* G;
-  __nv_bfloat16 *Qp, *Km;
+  __nv_bfloat16 *Qp, *Km;   // [slots][64][H][128]
   float *EL, *ER, *EX;
 };
 
@@ -447,24 +449,11 @@ __device__ __forceinline__ void prepare_chunks(const LayerParams& p, const KdaOp
     int ticket = p.total;
     // (one thread decides for the group: it reads a word that other CTAs write)
     if (tid == 0 && (nx_item < p.total || (once && *(volatile int*)(p.counters + 3) == 0))) ticket = atomicAdd(p.counters + 1, 1);
-    const size_t row0 = ((size_t)at.tok0 * p.H + at.h) * D + f0, stride = (size_t)p.H * D;
-    float gref[8], glast[8];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const float4 x = *reinterpret_cast<const float4*>(a.G + row0 + (size_t)(at.rows >> 1) * stride + 4 * q);
-      const float4 y = *reinterpret_cast<const float4*>(a.G + row0 + (size_t)(at.rows - 1) * stride + 4 * q);
-      gref[4 * q] = x.x * kLog2e; gref[4 * q + 1] = x.y * kLog2e; gref[4 * q + 2] = x.z * kLog2e; gref[4 * q + 3] = x.w * kLog2e;
-      glast[4 * q] = y.x * kLog2e; glast[4 * q + 1] = y.y * kLog2e; glast[4 * q + 2] = y.z * kLog2e; glast[4 * q + 3] = y.w * kLog2e;
-    }
+    const size_t row0 = ((size_t)at.tok0 * p.H + at.h) * D + f0, stride = (size_t)p.H * D, out0 = ((size_t)at.slot * C * p.H + at.h) * D + f0;
+    const DecayRefs refs = load_decay_refs(a.G + row0 + (size_t)(at.rows >> 1) * stride, a.G + row0 + (size_t)(at.rows - 1) * stride);
     if (r0 == 0) {
       const size_t v = ((size_t)at.slot * p.H + at.h) * D + f0;
-#pragma unroll
-      for (int q = 0; q < 8; q += 4) {
-        *reinterpret_cast<float4*>(a.EL + v + q) = make_float4(ex2_approx(glast[q]), ex2_approx(glast[q + 1]), ex2_approx(glast[q + 2]), ex2_approx(glast[q + 3]));
-        *reinterpret_cast<float4*>(a.ER + v + q) = make_float4(ex2_approx(gref[q]), ex2_approx(gref[q + 1]), ex2_approx(gref[q + 2]), ex2_approx(gref[q + 3]));
-        *reinterpret_cast<float4*>(a.EX + v + q) = make_float4(ex2_approx(glast[q] - gref[q]), ex2_approx(glast[q + 1] - gref[q + 1]),
-                                                               ex2_approx(glast[q + 2] - gref[q + 2]), ex2_approx(glast[q + 3] - gref[q + 3]));
-      }
+      store_decay_vectors(a.EL + v, a.ER + v, a.EX + v, refs);
     }
 #pragma unroll 1
     for (int r4 = r0; r4 < at.rows; r4 += 32) {
@@ -481,22 +470,17 @@ __device__ __forceinline__ void prepare_chunks(const LayerParams& p, const KdaOp
       }
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
-        const float g[8] = {gv[m][0].x, gv[m][0].y, gv[m][0].z, gv[m][0].w, gv[m][1].x, gv[m][1].y, gv[m][1].z, gv[m][1].w};
-        const uint32_t qw[4] = {qv[m].x, qv[m].y, qv[m].z, qv[m].w}, kw[4] = {kv[m].x, kv[m].y, kv[m].z, kv[m].w};
-        uint32_t qo[4], ko[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float x0 = g[2 * e] * kLog2e - gref[2 * e], x1 = g[2 * e + 1] * kLog2e - gref[2 * e + 1];
-          qo[e] = pack_bf16(__uint_as_float(qw[e] << 16) * ex2_approx(x0), __uint_as_float(qw[e] & 0xffff0000u) * ex2_approx(x1));
-          ko[e] = pack_bf16(__uint_as_float(kw[e] << 16) * ex2_approx(-x0), __uint_as_float(kw[e] & 0xffff0000u) * ex2_approx(-x1));
-        }
+        uint4 qo, ko;
+        decay_operands(qv[m], kv[m], gv[m][0], gv[m][1], refs, qo, ko);
         if (r4 + 8 * m < at.rows) {
-          const size_t idx = row0 + (size_t)(r4 + 8 * m) * stride;
-          *reinterpret_cast<uint4*>(a.Qp + idx) = make_uint4(qo[0], qo[1], qo[2], qo[3]);
-          *reinterpret_cast<uint4*>(a.Km + idx) = make_uint4(ko[0], ko[1], ko[2], ko[3]);
+          const size_t idx = out0 + (size_t)(r4 + 8 * m) * stride;
+          *reinterpret_cast<uint4*>(a.Qp + idx) = qo;
+          *reinterpret_cast<uint4*>(a.Km + idx) = ko;
         }
       }
     }
+    // the scan's state product multiplies the rows past the sequence's end by zeros, and may not find Inf or NaN there
+    for (int r = at.rows + r0; r < C; r += 8) *reinterpret_cast<uint4*>(a.Km + out0 + (size_t)r * stride) = make_uint4(0u, 0u, 0u, 0u);
     asm volatile("fence.proxy.async;" ::: "memory");   // ordinary stores, read by the scans' tile copies
     if (tid == 0) leave(ticket);
     sync();
@@ -828,9 +812,9 @@ cudaError_t launch_kda_scan(const ScanParams& scan, const void* Q, const void* K
   fill_params(p, d, l, ws, sp, split, sms);
   const KdaOperands a{(const __nv_bfloat16*)Q, (const __nv_bfloat16*)K, sp.G, (__nv_bfloat16*)Qp, (__nv_bfloat16*)Km,
                       const_cast<float*>(sp.EL), const_cast<float*>(sp.ER), const_cast<float*>(sp.EX)};
-  const long long tokens = d->cu_seqlens ? (long long)d->T : (long long)d->B * d->T;
+  const long long tokens = d->cu_seqlens ? (long long)d->T : (long long)d->B * d->T, rows = (tokens / C + sp.n_seqs + 1) * C;
   CUtensorMap tm[4];
-  if (!make_tmap(&tm[0], Qp, tokens, d->H, D, C) || !make_tmap(&tm[1], Km, tokens, d->H, D, C) || !make_tmap(&tm[2], W, tokens, d->H, D, C) ||
+  if (!make_tmap(&tm[0], Qp, rows, d->H, D, C) || !make_tmap(&tm[1], Km, rows, d->H, D, C) || !make_tmap(&tm[2], W, tokens, d->H, D, C) ||
       !make_tmap(&tm[3], sp.U, tokens, d->H, D, C))
     return cudaErrorUnknown;
   if ((e = launch_prep(d, l, ws, sms, p, sp, stream)) != cudaSuccess) return e;

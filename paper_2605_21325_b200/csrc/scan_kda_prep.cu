@@ -10,12 +10,12 @@
 // One pass over Q, K and G writes the two bf16 tensors and, per chunk, exp(G_last), exp(G_ref) and
 // exp(G_last - G_ref); the exponent of each difference is taken once per element instead of once per (i, j, k).
 #include "common.cuh"
+#include "kda_operands.cuh"
 
 namespace tri_inv {
 namespace {
 
 constexpr int C = 64, D = 128, NT = 256;
-constexpr float kLog2e = 1.4426950408889634f;
 
 struct PrepArgs {
   const __nv_bfloat16 *Q, *K;
@@ -25,16 +25,6 @@ struct PrepArgs {
   const int* seq_off;
   int H, T, n_seqs;
 };
-
-__device__ __forceinline__ float ex2f(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ uint32_t pack2(float a, float b) {
-  __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<uint32_t*>(&v);
-}
 
 // blockIdx.x: (sequence, head); blockIdx.y strides over the sequence's chunks.  16 threads per token row (8 features
 // each: 16 bytes of bf16, 32 of fp32), 16 rows per pass, four passes per chunk.
@@ -47,22 +37,10 @@ __global__ void __launch_bounds__(NT) kda_scan_prep_kernel(PrepArgs a) {
   for (int c = blockIdx.y; c < n_chunks; c += gridDim.y) {
     const int tok0 = beg + c * C, rows = end - tok0 < C ? end - tok0 : C;
     const size_t ref_row = ((size_t)(tok0 + (rows >> 1)) * a.H + h) * D + f0, last_row = ((size_t)(tok0 + rows - 1) * a.H + h) * D + f0;
-    float gref[8], glast[8];
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const float4 x = *reinterpret_cast<const float4*>(a.G + ref_row + 4 * q), y = *reinterpret_cast<const float4*>(a.G + last_row + 4 * q);
-      gref[4 * q] = x.x * kLog2e; gref[4 * q + 1] = x.y * kLog2e; gref[4 * q + 2] = x.z * kLog2e; gref[4 * q + 3] = x.w * kLog2e;
-      glast[4 * q] = y.x * kLog2e; glast[4 * q + 1] = y.y * kLog2e; glast[4 * q + 2] = y.z * kLog2e; glast[4 * q + 3] = y.w * kLog2e;
-    }
+    const DecayRefs refs = load_decay_refs(a.G + ref_row, a.G + last_row);
     if (r0 == 0) {
       const size_t slot = ((size_t)(tok0 / C + s) * a.H + h) * D + f0;
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        *reinterpret_cast<float4*>(a.EL + slot + 4 * q) = make_float4(ex2f(glast[4 * q]), ex2f(glast[4 * q + 1]), ex2f(glast[4 * q + 2]), ex2f(glast[4 * q + 3]));
-        *reinterpret_cast<float4*>(a.ER + slot + 4 * q) = make_float4(ex2f(gref[4 * q]), ex2f(gref[4 * q + 1]), ex2f(gref[4 * q + 2]), ex2f(gref[4 * q + 3]));
-        *reinterpret_cast<float4*>(a.EX + slot + 4 * q) = make_float4(ex2f(glast[4 * q] - gref[4 * q]), ex2f(glast[4 * q + 1] - gref[4 * q + 1]),
-                                                                      ex2f(glast[4 * q + 2] - gref[4 * q + 2]), ex2f(glast[4 * q + 3] - gref[4 * q + 3]));
-      }
+      store_decay_vectors(a.EL + slot, a.ER + slot, a.EX + slot, refs);
     }
 #pragma unroll
     for (int pass = 0; pass < 4; ++pass) {
@@ -70,24 +48,9 @@ __global__ void __launch_bounds__(NT) kda_scan_prep_kernel(PrepArgs a) {
       if (r >= rows) break;
       const size_t idx = ((size_t)(tok0 + r) * a.H + h) * D + f0;
       const uint4 qv = *reinterpret_cast<const uint4*>(a.Q + idx), kv = *reinterpret_cast<const uint4*>(a.K + idx);
-      float g[8];
-#pragma unroll
-      for (int q = 0; q < 2; ++q) {
-        const float4 x = *reinterpret_cast<const float4*>(a.G + idx + 4 * q);
-        g[4 * q] = x.x * kLog2e; g[4 * q + 1] = x.y * kLog2e; g[4 * q + 2] = x.z * kLog2e; g[4 * q + 3] = x.w * kLog2e;
-      }
-      const uint32_t* qw = reinterpret_cast<const uint32_t*>(&qv);
-      const uint32_t* kw = reinterpret_cast<const uint32_t*>(&kv);
+      const float4 g0 = *reinterpret_cast<const float4*>(a.G + idx), g1 = *reinterpret_cast<const float4*>(a.G + idx + 4);
       uint4 qo, mo;
-      uint32_t *qp = reinterpret_cast<uint32_t*>(&qo), *mp = reinterpret_cast<uint32_t*>(&mo);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const float2 qf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&qw[e]));
-        const float2 kf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&kw[e]));
-        const float x0 = g[2 * e] - gref[2 * e], x1 = g[2 * e + 1] - gref[2 * e + 1];
-        qp[e] = pack2(qf.x * ex2f(x0), qf.y * ex2f(x1));
-        mp[e] = pack2(kf.x * ex2f(-x0), kf.y * ex2f(-x1));
-      }
+      decay_operands(qv, kv, g0, g1, refs, qo, mo);
       *reinterpret_cast<uint4*>(a.Qp + idx) = qo;
       *reinterpret_cast<uint4*>(a.Km + idx) = mo;
     }

@@ -179,10 +179,10 @@ __device__ __noinline__ bool wait_by_warp(uint32_t bar, uint32_t parity, unsigne
   return false;
 }
 
-// Zeros into rows `rows` .. 63 of a tile of two boxes (128 bytes a row), by the chain warps; then visible to the products.  Not inlined: once a
+// Zeros into rows `rows` .. 63 of a tile of two boxes (128 bytes a row), by the output warps; then visible to the products.  Not inlined: once a
 // sequence, and the 128-column walk has no register to spare.
 __device__ __noinline__ void clear_rows(uint32_t tile, int box, int rows, int tid) {
-  for (int e = tid; e < (C - rows) * 16; e += kChainWarps * 32)
+  for (int e = tid; e < (C - rows) * 16; e += kOutWarps * 32)
     asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(tile + ((e >> 3) & 1) * box + (rows + (e >> 4)) * 128 + (e & 7) * 16), "r"(0) : "memory");
   fence_proxy_async();
 }
@@ -207,10 +207,11 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
   // products done (commit):  bar_t1 (P1), bar_tq (PQ), bar_s (P3), bar_qk (QK), bar_pu (PU); a commit covers every product issued before it
   // operands written:        bar_sr (S^T by the chain warps, the chunk's factors by the gate warp), bar_ud (U~'), bar_ut (U~),
   //                          bar_ut again (P and the start of PU, output warps); one arrival per warp
+  // bar_kz: the output warps have cleared the last chunk's key rows past the sequence's end (scalar gate)
   // bar_qr: the output warps have read QK;  bar_g: the gate warp has stored a chunk's factors (for the output warps, which need them early)
   const uint32_t bar_full = s0 + cfg::OFF_BAR, bar_exit = bar_full + 24, bar_t1 = bar_full + 32, bar_s = bar_full + 40, bar_pu = bar_full + 48,
                  bar_qk = bar_full + 56, bar_sr = bar_full + 64, bar_ud = bar_full + 72, bar_ut = bar_full + 80,
-                 bar_qr = bar_full + 96, bar_g = bar_full + 104, bar_tq = bar_full + 112;
+                 bar_kz = bar_full + 88, bar_qr = bar_full + 96, bar_g = bar_full + 104, bar_tq = bar_full + 112;
   const unsigned long long lim = p.wait_limit_ns ? p.wait_limit_ns : kWaitLimitNs;   // every wait of the kernel gives up after this long
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: uniform for the compiler
   const bool chain = warp < kChainWarps;
@@ -253,13 +254,16 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
     const int st = c % kStages;
     const uint32_t base = s0 + st * cfg::STAGE, bar = bar_full + 8 * st;
     const int tok0 = beg + c * C;
+    // beside the preparation Q+ and K- have 64 rows for every chunk, zeros past the sequence's end in K-: rows of a neighbour would be
+    // another group's, written maybe later
+    const int qk0 = KDA && FED ? (beg / C + s + c) * C : tok0;
     mbar_expect_tx(bar, (uint32_t)cfg::STAGE);
     tma_load_2d(base, &tmW, bar, h * D, tok0);
     tma_load_2d(base + cfg::WQ_BOX, &tmW, bar, h * D + 64, tok0);
-    tma_load_2d(base + 8192, &tmQ, bar, h * D, tok0);
-    tma_load_2d(base + cfg::WQ_BOX + 8192, &tmQ, bar, h * D + 64, tok0);
-    tma_load_2d(base + cfg::OFF_KT, &tmK, bar, h * D, tok0);
-    tma_load_2d(base + cfg::OFF_KT + cfg::K_BOX, &tmK, bar, h * D + 64, tok0);
+    tma_load_2d(base + 8192, &tmQ, bar, h * D, qk0);
+    tma_load_2d(base + cfg::WQ_BOX + 8192, &tmQ, bar, h * D + 64, qk0);
+    tma_load_2d(base + cfg::OFF_KT, &tmK, bar, h * D, qk0);
+    tma_load_2d(base + cfg::OFF_KT + cfg::K_BOX, &tmK, bar, h * D + 64, qk0);
     tma_load_2d(base + cfg::OFF_UT, &tmU, bar, h * D + (slice * DVS) / 64 * 64, tok0);
     if constexpr (cfg::UBOX == 2) tma_load_2d(base + cfg::OFF_UT + 8192, &tmU, bar, h * D + 64, tok0);
   };
@@ -326,6 +330,7 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
       mbar_init(bar_ud, kChainWarps);
       mbar_init(bar_ut, kChainWarps + kOutWarps);
       mbar_init(bar_qr, kOutWarps);
+      mbar_init(bar_kz, kOutWarps);
       mbar_init(bar_g, 1);
       mbar_init(bar_tq, 1);
       fence_mbar_init();
@@ -424,6 +429,7 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
         for (int ks = 0; ks < D / 16; ++ks)
           umma_bf16_ta(tmem + d_col, tmem + a_col + 8 * ks, b + (((ks >> 2) * cfg::WQ_BOX + (ks & 3) * 32) >> 4), idesc_p1, ks > 0);
       };
+      const bool partial = ((end - beg) & (C - 1)) != 0;
       uint32_t ph = 0;
       if (wait(bar_full, 0)) issue_qk(0);
       else failed = true;
@@ -440,6 +446,7 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
         TL(1);
         const bool last = c + 1 >= n_chunks;
         TL(2);
+        if (!KDA && last && partial && !wait(bar_kz, 0u)) { failed = true; break; }
         if (!wait(bar_ud, ph)) { failed = true; break; }
         tc_fence_after();
         TL(3);
@@ -548,13 +555,6 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
       TL(0);
       if (!wait(bar_full + 8 * (c % kStages), full_parity(c))) { failed = true; break; }   // landed long ago; U is read below
       TL(1);
-      if (rows < C) {
-        // The tile's rows past the sequence's end hold what follows it in memory: a neighbour's keys or, per channel beside the preparation,
-        // scratch that nobody may have written yet.  U~ is zero there, but zero times Inf or NaN is not: the state product must find
-        // zeros.  After QK, the tile's other reader, and beside the first product.
-        if (!wait(bar_qk, ph)) { failed = true; break; }
-        clear_rows(s0 + (c % kStages) * cfg::STAGE + cfg::OFF_KT, cfg::K_BOX, rows, tid);
-      }
       if (!wait(bar_t1, ph)) { failed = true; break; }
       tc_fence_after();
       TL(2);
@@ -720,6 +720,14 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
       if (!wait(bar_g, ph) || !wait(bar_qk, ph)) { failed = true; break; }
       tc_fence_after();
       TL(1);
+      if (!KDA && end - tok0 < C) {
+        // The tile's rows past the sequence's end hold a neighbour's keys.  U~ is zero there, but zero times Inf or NaN is not: the state
+        // product must find zeros.  QK, the tile's other reader, is done.  By these warps and not the chain's, whose loop got 1 % longer with
+        // it (512 chunks, 32 pairs: 650 -> 655 us; here 654 and 653).  The per-channel form does without: clearing in either role cost it 1 to
+        // 4 %; beside the preparation each chunk has rows of its own instead (issue_copies).
+        clear_rows(s0 + (c % kStages) * cfg::STAGE + cfg::OFF_KT, cfg::K_BOX, end - tok0, tid - kChainWarps * 32);
+        warp_arrive(bar_kz, lane);
+      }
       uint32_t wa[8], wb[8];
       {
         float qk[8][4];
