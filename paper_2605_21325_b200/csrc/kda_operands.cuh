@@ -40,9 +40,10 @@ __device__ __forceinline__ void decay_operands(const uint4& q, const uint4& k, c
   uint32_t qo[4], ko[4];
 #pragma unroll
   for (int e = 0; e < 4; ++e) {
+    const float2 qf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&qw[e])), kf = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&kw[e]));
     const float x0 = fmaf(g[2 * e], kDecayLog2e, -r.ref[2 * e]), x1 = fmaf(g[2 * e + 1], kDecayLog2e, -r.ref[2 * e + 1]);
-    qo[e] = pack_bf16(__uint_as_float(qw[e] << 16) * ex2_approx(x0), __uint_as_float(qw[e] & 0xffff0000u) * ex2_approx(x1));
-    ko[e] = pack_bf16(__uint_as_float(kw[e] << 16) * ex2_approx(-x0), __uint_as_float(kw[e] & 0xffff0000u) * ex2_approx(-x1));
+    qo[e] = pack_bf16(qf.x * ex2_approx(x0), qf.y * ex2_approx(x1));
+    ko[e] = pack_bf16(kf.x * ex2_approx(-x0), kf.y * ex2_approx(-x1));
   }
   qp = make_uint4(qo[0], qo[1], qo[2], qo[3]);
   km = make_uint4(ko[0], ko[1], ko[2], ko[3]);
