@@ -53,7 +53,7 @@ def algorithmic_bytes_per_matrix(C, d_k, d_v, elt, want_A=True, call="fused"):
         return C * d_k * elt + 2 * C * 4 + C * C * 4
     if call == "scan":  # Q, K, W, U, g read; O written
         return 3 * C * d_k * elt + C * d_v * elt + C * 4 + C * d_v * elt
-    if call == "kda_scan":  # what ONE kernel would move: Q, K, W, U and G (fp32 per channel) read; O written (the call is two launches)
+    if call == "kda_scan":  # what ONE kernel would move: Q, K, W, U and G (fp32 per channel) read; O written (the operands' preparation passes two more tensors through memory)
         return 3 * C * d_k * elt + C * d_v * elt + C * d_k * 4 + C * d_v * elt
     if call == "kda_layer":  # kda_fused without A, plus kda_scan
         return (C * d_k * elt + C * d_k * 4 + C * d_v * elt + C * 4 + C * d_k * elt + C * d_v * elt) + \
@@ -219,7 +219,8 @@ def main():
                     help="entry point timed: the fused path (default, the metric), tri_inv_build alone, tri_inv_wy alone, "
                          "tri_inv_fused_raw (front end folded in; same shapes, un-normalised keys and logits as inputs), "
                          "tri_inv_build_kda (per-channel decay), tri_inv_chunk_scan alone (W and U produced outside the timed "
-                         "region), or the layer forward (fused call with decay-weighted W, then the scan)")
+                         "region), or the layer forward as two calls (fused call with decay-weighted W, then the scan; tri_inv_gdn_forward is the "
+                         "one call)")
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-flush", action="store_true", help="skip the L2 flush between steps (profiling runs)")
@@ -447,7 +448,7 @@ def main():
         traffic = None if args.paper_T else ncu_traffic_bytes_per_matrix(args.call, args.config, args.method)
         roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                     "traffic": None if traffic is None else traffic * n_mat, "peak_source": "of " + peak_kind,
-                    "kernel": {"fused": "fused build+invert+WY", "raw": "front end + build+invert+WY", "build": "build+invert", "kda": "per-channel-decay build+invert", "kda_fused": "per-channel-decay build+invert+WY (one kernel)" if inp.C == 64 else "per-channel-decay build+invert (+ scaled keys), then WY (2 launches)", "wy": "WY apply", "scan": "chunk scan (state recurrence + output)", "layer": "fused build+invert+WY, then chunk scan (2 launches)", "kda_scan": "per-channel-decay chunk scan: operand preparation, then the scan (2 launches)", "kda_layer": "per-channel-decay build+invert+WY, operand preparation, chunk scan (3 launches)"}[args.call], "kernel_ms": kernel_ms, "kernel_ms_min": min(times_ms),
+                    "kernel": {"fused": "fused build+invert+WY", "raw": "front end + build+invert+WY", "build": "build+invert", "kda": "per-channel-decay build+invert", "kda_fused": "per-channel-decay build+invert+WY (one kernel)" if inp.C == 64 else "per-channel-decay build+invert (+ scaled keys), then WY (2 launches)", "wy": "WY apply", "scan": "chunk scan (state recurrence + output)", "layer": "fused build+invert+WY, then chunk scan (2 launches)", "kda_scan": "per-channel-decay chunk scan: operand preparation and scan (one kernel or two, by shape)", "kda_layer": "per-channel-decay build+invert+WY, then operand preparation and chunk scan (one kernel or two, by shape)"}[args.call], "kernel_ms": kernel_ms, "kernel_ms_min": min(times_ms),
                     "algorithmic_bytes_per_launch": alg_bytes * n_mat}
         cpu = None
         if world == 1 and not args.no_cpu_baseline:

@@ -281,7 +281,8 @@ int tri_inv_chunk_scan(const void* Q, const void* K, const void* W, const void* 
  *     results bit for bit.  Two launches on cuda_stream (a small one fills the workspace's words); nothing is allocated.
  *   - otherwise the two calls, with W, U and the fp32 scan's scratch in the workspace.
  * So a sequence continued from a returned state gives the same bits as in one go only if both are cut at chunk boundaries and neither
- * takes the first route.  Arguments as in the two calls; O may not overlap an input.  `workspace`: device memory of at least
+ * takes the first route.  The one kernel holds every SM until the factors are built, about two thirds of its time: a small call on another
+ * stream waits that long, longer than behind the two calls.  Arguments as in the two calls; O may not overlap an input.  `workspace`: device memory of at least
  * tri_inv_gdn_forward_workspace() bytes (which may be 0: then it may be NULL), 16-byte aligned, contents arbitrary; nothing else may use it
  * until the call has run.  Calls on different streams share no state but what the two calls share.
  */

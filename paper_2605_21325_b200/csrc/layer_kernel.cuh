@@ -18,6 +18,11 @@
 // way.  A CTA scans one task at most, so the grid has one for each: a loop over tasks would keep more in registers than the walk of
 // all 128 columns has.  All waits are bounded.
 //
+// The kernel has every SM, with all of its registers, until the factors are built: a small call on another stream waits that long, which it
+// did not behind the fused kernel and the scan as launches of their own.  A decode step of 8 x 16 pairs put on a second stream right behind 32
+// pairs x 512 chunks ends after 381 us (behind the two calls 182, alone 26), behind 64 x 64 after 95 us (28, 25); 333 tokens of 16 heads after
+// 396 (199, 50) and 108 (115, 50).  The large call itself is the faster one: 613 and 780 us, 158 and 160.
+//
 // W and U pass through scratch memory of the call; a scan reads a chunk microseconds after it was written, so mostly from L2.
 // Part of scan_kernel.cu, whose scan_walk it calls.
 #pragma once
@@ -613,6 +618,7 @@ Layout layout_of(const tri_inv_desc* d) {
 //   16 x 64: 92 / 86 (32, 64)    32 x 64: 112 / 96 (64, 64)    48 x 64: 127 / 130 (128, 48)   64 x 64: 140 / 130 (128, 64)
 //   75 x 64: 193 / 149 (128, 75)   100 x 64: 223 / 234 (128, 32)   148 x 64: 272 / 287 (128, 32)   8 x 512: 558 / 515 (32, 32)
 //   32 x 512: 762 / 589 (64, 64)   1024 x up to 32 chunks: 502 / 525   1024 x 1: 70 / 88   32 x 6: 28 / 23   128 x 2: 28 / 23
+// (the predictions agree with the faster form in all of these but 128 x 2, which they leave to two launches)
 // A scan here takes 1.8, 1.13 or 0.98 us a chunk in slices of 128, 64 or 32 columns (1.49, 1.06, 0.97 with the chip to itself), an SM
 // builds half a matrix per us.  More tasks than scan CTAs never paid, but for the few matrices of a call that is all latency:
 // both parts are then bound by bytes and power, which side by side save nothing.
@@ -638,6 +644,7 @@ Split choose_split(long long pairs, int longest, long long entries, int H, int s
 // The same for the per-channel scan.  Two launches / here (width, scan CTAs): 16 x 64: 95 / 91 (32, 64)   32 x 64: 119 / 104 (64, 64)
 //   48 x 64: 138 / 133 (128, 48)   64 x 64: 152 / 162 (128, 64)   75 x 64: 193 / 206 (128, 75)   8 x 128: 161 / 157 (32, 32)
 //   32 x 512: 884 / 651 (64, 64)   16 x 6: 19 / 25
+// (the predictions agree with the faster form in all of these but 48 x 64, which they leave to two launches: 5 us)
 // A group prepares a chunk in about 9 us, three of them an SM (0.33 a us; the preparation by itself keeps eight CTAs an SM in flight
 // and reaches 69 chunks a us on the whole chip), so the gain is where the chain is long.
 Split choose_kda_split(long long pairs, int longest, long long entries, int H, int sms) {

@@ -104,7 +104,7 @@ struct ScanCfg {
   // The 32-column slice asks for more than it uses.  Its registers and tiles would leave room on the SM for a CTA of the inversion
   // kernels (26.5 KB for the build at d = 64, 34.7 KB at d = 128), which would then sit in tcgen05.alloc with its first matrices
   // until the scan ends, because this kernel takes all of the tensor memory.  With 22 KB left they go to other
-  // SMs: three builds of 2048 matrices on a second stream beside a scan of 8 pairs x 256 chunks (262 us) end after 120 us, 323 us
+  // SMs (this kernel as a launch of its own; layer_kernel.cuh keeps other streams waiting): three builds of 2048 matrices on a second stream beside a scan of 8 pairs x 256 chunks (262 us) end after 120 us, 323 us
   // without (86 us alone).  The 64-column slice leaves them too few registers, the 128-column one too little shared memory.
   static constexpr int SMEM = DVS == 32 ? 208896 : OFF_BAR + 160;
   static_assert(SMEM >= OFF_BAR + 160, "everything up to the tensor-memory slot");
