@@ -233,7 +233,8 @@ int tri_inv_fused_kda(const void* K, const void* V, const float* G, const float*
  * exp(G_last - G_ref): |G_i - G_ref| must stay inside the fp32 exponent range, about 88 in natural-log units, and G must
  * not increase along a chunk), then the scan kernel of
  * tri_inv_chunk_scan on them; with few enough (sequence, head) pairs and long sequences the pass and the scan run side by side in
- * one kernel (same bits; a small launch before it).  The pass writes into stream-ordered scratch memory of twice the size of K (in one kernel
+ * one kernel (same bits; a small launch before it).  In two launches a partial last chunk's products also meet, times zero, the
+ * operands of the tokens behind it, which have to be finite.  The pass writes into stream-ordered scratch memory of twice the size of K (in one kernel
  * twice that of K with every chunk padded to 64 tokens; from a
  * memory pool that the library keeps per device: handed back to the pool behind the scan and reused by later calls, so
  * it stays reserved for the life of the process); TRI_INV_ERR_CUDA if it cannot be had.  Every other shape and fp32
