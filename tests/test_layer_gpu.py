@@ -192,21 +192,26 @@ def test_per_channel_scan_does_not_depend_on_what_its_scratch_held(bnd, name, B,
         assert torch.equal(bits(O), bits(ref[0][:, :, ::k])) and torch.equal(bits(S), bits(ref[1][:, ::k]))
 
 
-def test_scan_does_not_multiply_a_neighbours_keys(bnd):
-    """Keys that are not finite stay with their sequence: the one before it, whose last chunk's tile reaches into them, keeps its bits."""
+@pytest.mark.parametrize("H", [2, 16, 40], ids=["32_columns", "64_columns", "128_columns"])
+def test_scan_does_not_multiply_a_neighbours_keys(bnd, H):
+    """Keys that are not finite stay with their sequence: the one before it, whose last chunk's tile reaches into them, keeps its bits,
+    in the scan by itself and in the layer."""
     cu = np.array([0, 70, 200], np.int32)
-    _, _, _, dev, Q, S0 = layer_inputs(bnd, "neighbour", 1, 0, 2, 128, 128, wl.BF16, cu, 795)
+    _, _, _, dev, Q, S0 = layer_inputs(bnd, "neighbour", 1, 0, H, 128, 128, wl.BF16, cu, 795)
     _, W, U = bnd.fused(dev["K"], dev["V"], dev["beta"], dev["g"], 64, method=bnd.W_DECAY, cu_seqlens=cu, want_A=False)
-    outs = []
-    for value in (1.0, float("inf"), float("nan")):
-        K = dev["K"].clone()
-        K[0, 70:] *= value
-        O, S = bnd.chunk_scan(Q, K, W, U, dev["g"], 64, scale=0.5, S0=S0, cu_seqlens=cu)
-        outs.append((bits(O[:, :70]), bits(S[0])))
-    torch.cuda.synchronize()
-    assert torch.isfinite(S[0]).all()
-    for o in outs[1:]:
-        assert torch.equal(o[0], outs[0][0]) and torch.equal(o[1], outs[0][1])
+    for call in (lambda K: bnd.chunk_scan(Q, K, W, U, dev["g"], 64, scale=0.5, S0=S0, cu_seqlens=cu),
+                 lambda K: bnd.gdn_forward(Q, K, dev["V"], dev["beta"], dev["g"], 64, scale=0.5, S0=S0, cu_seqlens=cu)):
+        outs = []
+        for value in (1.0, float("inf"), float("nan")):
+            K = dev["K"].clone()
+            K[0, 70:] *= value
+            O, S = call(K)
+            outs.append((bits(O[:, :70]), bits(S[0])))
+        torch.cuda.synchronize()
+        assert bnd.last_device_status() == 0
+        assert torch.isfinite(S[0]).all()
+        for o in outs[1:]:
+            assert torch.equal(o[0], outs[0][0]) and torch.equal(o[1], outs[0][1])
 
 
 def kda_operands(bnd, B, T, H, seed):
