@@ -359,7 +359,7 @@ __device__ __forceinline__ bool build_factors(const CUtensorMap& tmK, const CUte
 
 template <int DVS>
 struct LayerCfg {
-  static constexpr int SCAN = ScanCfg<DVS, false>::OFF_BAR + 160, BUILD = kGroups * kGroupBytes;
+  static constexpr int SCAN = ScanCfg<DVS, false>::OFF_BAR + 192, BUILD = kGroups * kGroupBytes;
   static constexpr int SMEM = (SCAN > BUILD ? SCAN : BUILD) + 16;   // + the CTA's own words
 };
 static_assert(LayerCfg<128>::SMEM <= 232448, "one CTA per SM");
@@ -369,6 +369,7 @@ __global__ void __launch_bounds__(kLayerThreads, 1)
 layer_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV,
              const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmU,      // boxes of 64 tokens
              const __grid_constant__ CUtensorMap tmWs, const __grid_constant__ CUtensorMap tmUs,    // boxes of 16 tokens: a warp's stores
+             const __grid_constant__ CUtensorMap tmO,
              const __grid_constant__ LayerParams p, const __grid_constant__ ScanParams sp) {
   constexpr int NS = D / DVS;
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -408,7 +409,7 @@ layer_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
   const int task = __shfl_sync(0xffffffffu, *s_word, 0);
   if (task < p.scan_tasks) {
     const int slice = task % NS, pair = task / NS;
-    scan_walk<DVS, false, true>(tmW, tmQ, tmK, tmU, sp, smem, pair / p.H, pair % p.H, slice, false, p.ready, tmem);
+    scan_walk<DVS, false, true>(tmW, tmQ, tmK, tmU, tmO, sp, smem, pair / p.H, pair % p.H, slice, false, p.ready, tmem);
   }
   tc_fence_before();
   __syncthreads();
@@ -502,10 +503,10 @@ __device__ __forceinline__ void prepare_chunks(const LayerParams& p, const KdaOp
 }
 
 // as many threads as the walk has warps, whose 128-column form needs the registers; three groups prepare
-constexpr int kKdaThreads = (kCopy + 1) * 32, kKdaGroups = 3;
+constexpr int kKdaThreads = kThreadsScan, kKdaGroups = 3;
 template <int DVS>
 struct KdaScanCfg {
-  static constexpr int OFF_WORDS = (ScanCfg<DVS, true>::OFF_BAR + 160 + 15) / 16 * 16;
+  static constexpr int OFF_WORDS = (ScanCfg<DVS, true>::OFF_BAR + 192 + 15) / 16 * 16;
   static constexpr int SMEM = OFF_WORDS + kKdaGroups * 64 + 16;
 };
 static_assert(KdaScanCfg<128>::SMEM <= 232448, "one CTA per SM");
@@ -513,7 +514,7 @@ static_assert(KdaScanCfg<128>::SMEM <= 232448, "one CTA per SM");
 template <int DVS>
 __global__ void __launch_bounds__(kKdaThreads, 1)
 kda_scan_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmW,
-                const __grid_constant__ CUtensorMap tmU, const __grid_constant__ LayerParams p, const __grid_constant__ KdaOperands a,
+                const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUtensorMap tmO, const __grid_constant__ LayerParams p, const __grid_constant__ KdaOperands a,
                 const __grid_constant__ ScanParams sp) {
   constexpr int NS = D / DVS;
   extern __shared__ __align__(1024) uint8_t smem[];
@@ -541,7 +542,7 @@ kda_scan_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
   const int task = __shfl_sync(0xffffffffu, *s_word, 0);
   if (task < p.scan_tasks) {
     const int slice = task % NS, pair = task / NS;
-    scan_walk<DVS, true, true>(tmW, tmQ, tmK, tmU, sp, smem, pair / p.H, pair % p.H, slice, false, p.ready, tmem);
+    scan_walk<DVS, true, true>(tmW, tmQ, tmK, tmU, tmO, sp, smem, pair / p.H, pair % p.H, slice, false, p.ready, tmem);
   }
   tc_fence_before();
   __syncthreads();
@@ -713,7 +714,7 @@ cudaError_t launch_prep(const tri_inv_desc* d, const Layout& l, char* ws, int sm
 }
 
 template <int DVS>
-cudaError_t launch_width(const CUtensorMap (&tm)[7], const LayerParams& p, const ScanParams& sp, int grid, int dev, cudaStream_t stream) {
+cudaError_t launch_width(const CUtensorMap (&tm)[7], const LayerParams& p, const ScanParams& sp, long long tokens, int grid, int dev, cudaStream_t stream) {
   static std::mutex mu;
   static bool ready[64] = {false};
   {
@@ -725,7 +726,9 @@ cudaError_t launch_width(const CUtensorMap (&tm)[7], const LayerParams& p, const
       ready[dev] = true;
     }
   }
-  layer_kernel<DVS><<<grid, kLayerThreads, LayerCfg<DVS>::SMEM, stream>>>(tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], tm[6], p, sp);
+  CUtensorMap tmO;
+  if (!make_tmap_out<DVS>(&tmO, sp.O, tokens, p.H)) return cudaErrorUnknown;
+  layer_kernel<DVS><<<grid, kLayerThreads, LayerCfg<DVS>::SMEM, stream>>>(tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], tm[6], tmO, p, sp);
   return launched();
 }
 
@@ -768,9 +771,9 @@ cudaError_t launch_layer(const void* Q, const void* K, const void* V, const floa
   if ((e = launch_prep(d, l, ws, sms, p, sp, stream)) != cudaSuccess) return e;
   const int grid = std::max(sms, p.scan_tasks);   // a CTA walks once
   switch (split.dvs) {
-    case 32: return launch_width<32>(tm, p, sp, grid, dev, stream);
-    case 64: return launch_width<64>(tm, p, sp, grid, dev, stream);
-    default: return launch_width<128>(tm, p, sp, grid, dev, stream);
+    case 32: return launch_width<32>(tm, p, sp, tokens, grid, dev, stream);
+    case 64: return launch_width<64>(tm, p, sp, tokens, grid, dev, stream);
+    default: return launch_width<128>(tm, p, sp, tokens, grid, dev, stream);
   }
 }
 
@@ -786,7 +789,7 @@ bool kda_scan_fits(const tri_inv_desc* d, size_t* control_bytes) {
 
 namespace {
 template <int DVS>
-cudaError_t launch_kda_width(const CUtensorMap (&tm)[4], const LayerParams& p, const KdaOperands& a, const ScanParams& sp, int grid, int dev, cudaStream_t stream) {
+cudaError_t launch_kda_width(const CUtensorMap (&tm)[4], const LayerParams& p, const KdaOperands& a, const ScanParams& sp, long long tokens, int grid, int dev, cudaStream_t stream) {
   static std::mutex mu;
   static bool ready[64] = {false};
   {
@@ -798,7 +801,9 @@ cudaError_t launch_kda_width(const CUtensorMap (&tm)[4], const LayerParams& p, c
       ready[dev] = true;
     }
   }
-  kda_scan_kernel<DVS><<<grid, kKdaThreads, KdaScanCfg<DVS>::SMEM, stream>>>(tm[0], tm[1], tm[2], tm[3], p, a, sp);
+  CUtensorMap tmO;
+  if (!make_tmap_out<DVS>(&tmO, sp.O, tokens, p.H)) return cudaErrorUnknown;
+  kda_scan_kernel<DVS><<<grid, kKdaThreads, KdaScanCfg<DVS>::SMEM, stream>>>(tm[0], tm[1], tm[2], tm[3], tmO, p, a, sp);
   return launched();
 }
 }  // namespace
@@ -827,9 +832,9 @@ cudaError_t launch_kda_scan(const ScanParams& scan, const void* Q, const void* K
   if ((e = launch_prep(d, l, ws, sms, p, sp, stream)) != cudaSuccess) return e;
   const int grid = std::max(sms, p.scan_tasks);
   switch (split.dvs) {
-    case 32: return launch_kda_width<32>(tm, p, a, sp, grid, dev, stream);
-    case 64: return launch_kda_width<64>(tm, p, a, sp, grid, dev, stream);
-    default: return launch_kda_width<128>(tm, p, a, sp, grid, dev, stream);
+    case 32: return launch_kda_width<32>(tm, p, a, sp, tokens, grid, dev, stream);
+    case 64: return launch_kda_width<64>(tm, p, a, sp, tokens, grid, dev, stream);
+    default: return launch_kda_width<128>(tm, p, a, sp, tokens, grid, dev, stream);
   }
 }
 

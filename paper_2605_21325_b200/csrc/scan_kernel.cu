@@ -16,28 +16,33 @@
 // of a chunk (the transposed ones with M = 128, or for a slice of 64 or 32 columns M = 64, rows 16 q .. + 15 in lanes 0 .. 15 of
 // quadrant q: the same time per instruction, but the kernel runs at the power cap, where less work is a higher clock: 612 ->
 // 583 us back to back on 32 pairs of 512 chunks):
-//   P1 [DVS x 64]  = S^T . W^T                     the chain's
-//   PQ [DVS x 64]  = S^T . Q^T                     right behind it, with a commit of its own
-//   P3 [DVS x 128] = U~'^T . K                     U~' = decay-scaled U~; the K tile is read MN-major
-//   QK [64 x 64]   = Q . K^T                       both K-major tiles; needs no state: one chunk ahead, behind P3
-//   PU [DVS x 64]  = U~^T . P^T, on top of gamma_i (Q S)^T
+//   P1 [DVS x 64]  = S^T . W^T                     the chain's, as two products of 32 tokens with a commit each
+//   PQ [DVS x 64]  = S^T . Q^T                     behind it
+//   P3 [DVS x 128] = U~'^T . K                     U~' = decay-scaled U~; the K tile is read MN-major; two products of 64 features, a commit each
+//   PU [DVS x 64]  = U~^T . P^T
+//   QK [64 x 64]   = Q . K^T                       both K-major tiles; needs no state: one chunk ahead, behind PU
 // The dependent chain of a chunk is  P1 -> U~' -> P3 -> S^T.
 //
 // Warps 0..7 ("chain") work on tensor-memory lanes 32 (w & 3) .. + 31 and on half (w >> 2) of the columns: 32 tokens of
-// U~, 64 features of S (fp32, in registers for the whole sequence).  The output warps form P (a chunk
-// ahead of its use), the gamma-weighted start of PU, and write O one chunk behind.  The control warp issues every product; the
-// gate warp brings g and its factors a chunk ahead and requests the tile copies two chunks ahead, into
+// U~, 64 features of S (fp32, in registers for the whole sequence).  The halves have barriers of their own: a product's time goes by its columns
+// (N / 2 cycles for 16 of the summed index, whatever M, and about 70 until its commit is seen), so the first half of the warps starts on the next
+// step, and the next product on its first half of the summed index, 64 to 128 cycles before the whole product would be through.
+// The output warps form P and put O one chunk behind into its tile (O = gamma_i Q S + P U~ is joined there, scale in the factors); the store warp sends the
+// tile on by the copy engine.  The control warp issues every product; the gate warp brings g (cp.async, two chunks ahead) and its factors a chunk
+// ahead; the copy warp requests the tile copies two chunks ahead, into
 // three stages of {[W ; Q], K, U}.  Hand-offs are mbarriers: commits from the products, one arrival per warp after its
-// operand writes (U~' first: the product on the chain needs only that; U~ follows).  No compute warp issues a global load
-// inside the loop: one in flight would make its next tensor-memory load wait for it too.
-// What bounds it: with few (sequence, head) pairs the latencies of the chain (a chunk of 32 columns: P1 420 cycles, U~' 330, P3
-// 410, S^T 310 and the hand-overs between them: about 1,850), with more pairs than SMs the bytes.  Measured (L2 flushed)
-// against the form that kept the operands in shared memory, S as columns and issued from one lane, over several GPUs: B = 4, T = 4096,
-// H = 16: 110 -> 78 .. 86 us; B = 1, T = 32768, H = 32: 743 -> 542 us; 64 packed sequences of up to 2048 tokens, H = 16: 416 -> 262 .. 290 us
-// (0.82 .. 0.9 of the copy bandwidth on 82 KB per chunk and head).  Not kept, on the second shape in slices of 32 columns (505 us with L2
-// flushed then): Q K^T as mma.sync in the output warps (they get what tcgen05.mma leaves: 810 us), K in P1's free lanes instead
-// of a product of its own (the output warps become the bound: 689 us, before the issue by a whole warp), eight output warps
-// (no gain, more contention: 532 us).
+// operand writes (U~' first: the product on the chain needs only that; U~ follows).  No compute warp issues a global load or store
+// inside the loop: its next tensor-memory load, or the next fence for the asynchronous proxy, would wait for it.  That fence stands behind the barrier, with the
+// warp that issues the product or the copy: in the output warps, behind their stores, it took up to 400 cycles.
+// What bounds it: with few (sequence, head) pairs the chain (a chunk of 64 columns: P1 and P3 about 330 cycles each until the second half is
+// seen, U~' 320, S^T 250, the hand-overs) and the output warps, which take nearly as long a chunk; with more pairs than SMs the bytes.  The warps slow
+// each other down: code that does not fit the instruction caches (a second inlined copy of the O step: 95 -> 135 us at 100 pairs x 64 chunks), loads of tensor memory
+// beside a product that nobody waits for yet (Q S, Q K^T).
+// Measured back to back, us, (sequence, head) pairs x chunks; before: whole products, the start of PU put into tensor memory, O stored and g loaded by the
+// warps that use them: 8 x 256: 252 -> 243, 32 x 64: 74.6 -> 70.4, 32 x 256: 277 -> 259, 64 x 64: 76.6 -> 70.8, 100 x 64: 125 -> 91.5, 148 x 64: 138 -> 128;
+// per-channel form with its preparation: 8 x 256: 291 -> 266, 32 x 256: 339 -> 314, 64 x 64: 152 -> 140.  Not kept, of these (32 x 256): QK in two parts around P1 (260 .. 270), behind P1 (270), before
+// PU (276); polls without a suspended wait (286) or with a suspension hint (308); O and P 32 columns at a time (267 .. 305).  Not kept before: Q K^T as
+// mma.sync in the output warps (they get what tcgen05.mma leaves), K in P1's free lanes instead of a product of its own, eight output warps.
 // Every mbarrier wait is bounded; on expiry the CTA raises the status word, frees its tensor memory and returns.
 #include "tc_device.cuh"
 
@@ -45,7 +50,7 @@ namespace tri_inv {
 namespace {
 
 constexpr int C = 64, D = 128;
-constexpr int kChainWarps = 8, kOutWarps = 4, kControl = kChainWarps + kOutWarps, kGate = kControl + 1, kCopy = kGate + 1, kThreadsScan = (kGate + 1) * 32;
+constexpr int kChainWarps = 8, kOutWarps = 4, kControl = kChainWarps + kOutWarps, kGate = kControl + 1, kCopy = kGate + 1, kStore = kCopy + 1, kThreadsScan = (kStore + 1) * 32;
 constexpr int kStages = 3;
 constexpr float kLog2e = 1.4426950408889634f;
 
@@ -96,27 +101,29 @@ struct ScanCfg {
   static constexpr int WQ_BOX = 16384, K_BOX = 8192;
   static constexpr int OFF_KT = 2 * WQ_BOX, OFF_UT = OFF_KT + 2 * K_BOX, STAGE = OFF_UT + UBOX * 8192;
   static constexpr int OFF_P = kStages * STAGE;          // P, bf16 [64 tokens i][64 tokens j], K-major B operand of PU
-  static constexpr int OFF_O = OFF_P + 8192;             // O on its way out: per output warp [64 tokens][RPQ columns] bf16
-  static constexpr int O_WARP = C * RPQ * 2;
-  static constexpr int OFF_G = OFF_O + kOutWarps * O_WARP;
-  static constexpr int G_BYTES = KDA ? 9 * D * 4 : 2 * 4 * C * 4;   // per-channel: 3 vectors x 3 chunks; scalar: g, column factor, gamma_last / gamma, gamma of two chunks
+  static constexpr int OFF_O = OFF_P + 8192;             // O on its way out, bf16: boxes of 64 columns (32: the narrow slice) x 64 tokens, swizzled
+  static constexpr int OFF_G = OFF_O + C * DVS * 2;
+  static constexpr int G_BYTES = (KDA ? 12 * D : 19 * C) * 4;   // per-channel: 3 vectors of four chunks; scalar: g and its four factors of three, and g as it comes of four
   static constexpr int OFF_BAR = OFF_G + G_BYTES;
   // The 32-column slice asks for more than it uses.  Its registers and tiles would leave room on the SM for a CTA of the inversion
   // kernels (26.5 KB for the build at d = 64, 34.7 KB at d = 128), which would then sit in tcgen05.alloc with its first matrices
   // until the scan ends, because this kernel takes all of the tensor memory.  With 22 KB left they go to other
   // SMs (this kernel as a launch of its own; layer_kernel.cuh keeps other streams waiting): three builds of 2048 matrices on a second stream beside a scan of 8 pairs x 256 chunks (262 us) end after 120 us, 323 us
   // without (86 us alone).  The 64-column slice leaves them too few registers, the 128-column one too little shared memory.
-  static constexpr int SMEM = DVS == 32 ? 208896 : OFF_BAR + 160;
-  static_assert(SMEM >= OFF_BAR + 160, "everything up to the tensor-memory slot");
-  // tensor-memory columns
-  // (per-channel form: the accumulators of P1 and P3 share their columns -- the chain warps have read the one before the other
-  // is issued, either way round -- and the scaled copy of S^T takes the room)
-  static constexpr int TM_WS = 0, TM_DS = KDA ? 0 : 64, TM_QS = TM_DS + 128, TM_PU = TM_QS + 64, TM_QK = TM_PU + 64, TM_S = TM_QK + 64,
-                       TM_SQ = KDA ? TM_S + 64 : TM_S, TM_UD = TM_SQ + 64, TM_UT = KDA ? TM_UD : TM_UD + 32;
-  static_assert(TM_UT + 32 <= 512, "tensor memory");
+  static constexpr int SMEM = DVS == 32 ? 208896 : OFF_BAR + 192;
+  static_assert(SMEM >= OFF_BAR + 192, "everything up to the tensor-memory slot");
+  // Tensor-memory columns.  WS: P1 of the chunk's tokens 0 .. 31, then of 32 .. 63; the chain warps put U~ (UT) and the decay-scaled
+  // U~' (UD), 16 columns of packed pairs each for 32 tokens, where they have read their accumulators (per-channel form: U~ only).
+  // QS: two chunks in turn.  SQ: per-channel form, S^T scaled for PQ.
+  static constexpr int TM_WS = 0, TM_UT = TM_WS, TM_UD = KDA ? TM_UT : TM_WS + 16, TM_DS = TM_WS + 64, TM_QS = TM_DS + 128, TM_PU = TM_QS + 128,
+                       TM_QK = KDA ? TM_PU : TM_PU + 64, TM_S = TM_QK + 64, TM_SQ = KDA ? TM_S + 64 : TM_S;
+  static_assert(TM_SQ + 64 <= 512, "tensor memory");
   static constexpr int TMEM_COLS = 512;
 };
 static_assert(ScanCfg<128, true>::SMEM <= 232448, "one CTA per SM");
+template <int N> struct Width { static constexpr int value = N; };
+__device__ __forceinline__ void tmem_ld_tokens(float (&r)[4][4], uint32_t taddr) { tmem_ld_16x32(r, taddr); }
+__device__ __forceinline__ void tmem_ld_tokens(float (&r)[8][4], uint32_t taddr) { tmem_ld_16x64(r, taddr); }
 
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
@@ -188,38 +195,44 @@ __device__ __noinline__ void clear_rows(uint32_t tile, int box, int rows, int ti
 }
 
 // One (sequence, head, slice) by a whole CTA; true when a wait has run out in this thread.
-// FED: W and U (per-channel form: Q+, K- and the chunks' vectors) are being written by other CTAs of the same launch (layer_kernel.cuh).  The tile copies are then requested by a warp
-// of their own, kCopy, which first waits until the chunk's word in `ready` says that they are in memory (the gate warp does the same for the vectors); tensor memory
-// is the caller's (`tmem`).  Otherwise the gate warp requests the copies and the CTA allocates (and frees) its tensor memory.
+// FED: W and U (per-channel form: Q+, K- and the chunks' vectors) are being written by other CTAs of the same launch (layer_kernel.cuh).  The copy
+// warp then waits until the chunk's word in `ready` says that they are in memory before it requests the chunk's tiles (the gate warp does the same for the
+// vectors); tensor memory is the caller's (`tmem`).  Otherwise the first two chunks are requested ahead of the CTA's barrier, by the gate warp, and the CTA
+// allocates (and frees) its tensor memory.
 template <int DVS, bool KDA, bool FED>
-__device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmU,
+__device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmU, const CUtensorMap& tmO,
                                           const ScanParams& p, uint8_t* smem, int s, int h, int slice, bool first_block,
                                           const uint32_t* ready, uint32_t tmem) {
   using cfg = ScanCfg<DVS, KDA>;
   constexpr int LG = cfg::LG, E = cfg::E;
-  float* sG = reinterpret_cast<float*>(smem + cfg::OFF_G);   // scalar gate: [2][4][64]: g log2e; 2^(g_ref(j) - g_j), g_ref(j) = g of the first token of j's block of eight; 2^(g_last - g_j); 2^g_j
-  float* sEl = sG;                 // per-channel form: exp(G_last) [3][128], exp(G_ref) [3][128], exp(G_last - G_ref) [3][128]
-  float* sEr = sG + 3 * D;
-  float* sEx = sG + 6 * D;
+  float* sG = reinterpret_cast<float*>(smem + cfg::OFF_G);   // scalar gate: [3][5][64]: g log2e; scale 2^(g_ref(j) - g_j), g_ref(j) = g of the first token of j's block of eight; 2^(g_last - g_j); 2^g_j; scale 2^g_j
+  float* sEl = sG;                 // per-channel form: exp(G_last) [4][128], exp(G_ref) [4][128], exp(G_last - G_ref) [4][128]
+  float* sEr = sG + 4 * D;
+  float* sEx = sG + 8 * D;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + cfg::OFF_BAR + 128);
   const uint32_t s0 = smem_u32(smem), sP = s0 + cfg::OFF_P;
   // copies (TMA):            bar_full + 8 stage (W, Q, K, U of a chunk)
-  // products done (commit):  bar_t1 (P1), bar_tq (PQ), bar_s (P3), bar_qk (QK), bar_pu (PU); a commit covers every product issued before it
+  // products done (commit):  bar_t1 (P1), bar_s (P3), bar_qk (QK), bar_pu (PU); a commit covers every product issued before it
   // operands written:        bar_sr (S^T by the chain warps, the chunk's factors by the gate warp), bar_ud (U~'), bar_ut (U~),
-  //                          bar_ut again (P and the start of PU, output warps); one arrival per warp
+  //                          bar_ut again (P, output warps); one arrival per warp
+  // bar_t1, bar_s, bar_sr and bar_ud are the first half's (tokens 0 .. 31, features 0 .. 63); the second half's lie kSecond further on
+  // bar_o: O's tile is full;  bar_of: it has been read
   // bar_kz: the output warps have cleared the last chunk's key rows past the sequence's end (scalar gate)
   // bar_qr: the output warps have read QK;  bar_g: the gate warp has stored a chunk's factors (for the output warps, which need them early)
   const uint32_t bar_full = s0 + cfg::OFF_BAR, bar_exit = bar_full + 24, bar_t1 = bar_full + 32, bar_s = bar_full + 40, bar_pu = bar_full + 48,
                  bar_qk = bar_full + 56, bar_sr = bar_full + 64, bar_ud = bar_full + 72, bar_ut = bar_full + 80,
-                 bar_kz = bar_full + 88, bar_qr = bar_full + 96, bar_g = bar_full + 104, bar_tq = bar_full + 112;
+                 bar_kz = bar_full + 88, bar_qr = bar_full + 96, bar_g = bar_full + 104, bar_o = bar_full + 112, bar_of = bar_full + 120,
+                 kSecond = 104, bar_t1b = bar_t1 + kSecond, bar_sb = bar_s + kSecond, bar_srb = bar_sr + kSecond, bar_udb = bar_ud + kSecond;
   const unsigned long long lim = p.wait_limit_ns ? p.wait_limit_ns : kWaitLimitNs;   // every wait of the kernel gives up after this long
   const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;   // warp: uniform for the compiler
   const bool chain = warp < kChainWarps;
   const int quad = warp & 3, half = (warp >> 2) & 1;
   const int gq = lane >> 2, t = lane & 3, mi = lane >> 3, mr = lane & 7;
+  const uint32_t bars_half = bar_full + (half ? kSecond : 0);   // chain warps: where their half's barriers are counted from
 
-  const int beg = p.seq_off ? p.seq_off[s] : s * p.T;
-  const int end = p.seq_off ? p.seq_off[s + 1] : (s + 1) * p.T;
+  // uniform for the compiler as well: what the control warp's loop and its branches depend on
+  const int beg = __shfl_sync(0xffffffffu, p.seq_off ? p.seq_off[s] : s * p.T, 0);
+  const int end = __shfl_sync(0xffffffffu, p.seq_off ? p.seq_off[s + 1] : (s + 1) * p.T, 0);
   const int n_chunks = (end - beg + C - 1) / C;
   const int row0 = quad * cfg::RPQ;              // first value column of this warp's lanes, within the slice
 
@@ -272,21 +285,29 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
   auto drain_copies = [&]() {   // give-up path: the copies still on their way into this CTA's shared memory, with a limit
     for (int c = requested >= kStages ? requested - kStages + 1 : 0; c <= requested; ++c) mbar_wait_bounded(bar_full + 8 * (c % kStages), full_parity(c), lim);
   };
-  // g of a chunk, by the gate warp (lane l: tokens l and l + 32).  Rows past the sequence end take the last real
-  // row's g, so that every exponent stays a difference of real values.
-  auto fetch_g = [&](int c, float (&gr)[2]) {
-    const int tok0 = beg + c * C, rows = end - tok0 < C ? end - tok0 : C;
+  // g of a chunk into shared memory, by the gate warp (lane l: tokens l and l + 32), two chunks ahead of its use.  Rows past the sequence end take the last real
+  // row's g, so that every exponent stays a difference of real values.  By cp.async: a load into registers would be waited for before
+  // the next poll of a barrier, 1,400 cycles of a chunk's 2,100 with 128 CTAs at work.
+  auto cp_async = [](float* dst, const float* src, auto bytes) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(smem_u32(dst)), "l"(src), "n"(decltype(bytes)::value) : "memory");
+  };
+  auto fetch_g = [&](int c) {
+    if (c < n_chunks) {
+      const int tok0 = beg + c * C, rows = end - tok0 < C ? end - tok0 : C;
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const int i = lane + 32 * q < rows ? lane + 32 * q : rows - 1;
-      gr[q] = p.g[(size_t)(tok0 + i) * p.H + h];
+      for (int q = 0; q < 2; ++q) {
+        const int i = lane + 32 * q < rows ? lane + 32 * q : rows - 1;
+        cp_async(sG + (15 + (c & 3)) * C + lane + 32 * q, p.g + (size_t)(tok0 + i) * p.H + h, Width<4>{});
+      }
     }
+    asm volatile("cp.async.commit_group;" ::: "memory");
   };
   // g * log2(e) of a chunk and its factors.  The decay 2^(g_i - g_j) of P is formed as 2^(g_i - g_ref) * 2^(g_ref - g_j) with
   // g_ref the first token of j's block of eight -- one exponential per (row, block) instead of one per element; the
   // second factor spans at most seven tokens of decay
-  auto store_g = [&](int c, const float (&gr)[2]) {
-    float* b = sG + (c & 1) * 4 * C;
+  auto store_g = [&](int c) {   // behind the wait for the group; a lane reads what it copied itself
+    float* b = sG + (c % 3) * 5 * C;
+    const float gr[2] = {sG[(15 + (c & 3)) * C + lane], sG[(15 + (c & 3)) * C + lane + 32]};
     const float g_last = __shfl_sync(0xffffffffu, gr[1], 31) * kLog2e;
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
@@ -294,19 +315,25 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
       const float gref = __shfl_sync(0xffffffffu, gl2, lane & ~7);
       const int i = lane + 32 * q;
       b[i] = gl2;
-      b[C + i] = ex2_approx(gref - gl2);
+      b[C + i] = p.scale * ex2_approx(gref - gl2);
       b[2 * C + i] = ex2_approx(g_last - gl2);
-      b[3 * C + i] = ex2_approx(gl2);
+      const float gamma = ex2_approx(gl2);
+      b[3 * C + i] = gamma;
+      b[4 * C + i] = p.scale * gamma;
     }
   };
   // per-channel form: exp(G_last), exp(G_ref) and exp(G_last - G_ref) of a chunk (128 floats each, written by the preparation
-  // kernel at the chunk's slot), by the gate warp: lane l brings features 4 l .. 4 l + 3 of each; three chunks' worth are kept in turn
-  auto fetch_e = [&](int c, float4 (&ev)[3]) {
-    const size_t slot = (size_t)((beg + c * C) / C + s);
-    ev[0] = *reinterpret_cast<const float4*>(p.EL + (slot * p.H + h) * D + 4 * lane);
-    ev[1] = *reinterpret_cast<const float4*>(p.ER + (slot * p.H + h) * D + 4 * lane);
-    ev[2] = *reinterpret_cast<const float4*>(p.EX + (slot * p.H + h) * D + 4 * lane);
+  // kernel at the chunk's slot), by the gate warp: lane l brings features 4 l .. 4 l + 3 of each; four chunks' worth are kept in turn
+  auto fetch_e = [&](int c) {
+    if (c < n_chunks) {
+      const size_t at = ((size_t)((beg + c * C) / C + s) * p.H + h) * D + 4 * lane;
+      cp_async(sEl + (c & 3) * D + 4 * lane, p.EL + at, Width<16>{});
+      cp_async(sEr + (c & 3) * D + 4 * lane, p.ER + at, Width<16>{});
+      cp_async(sEx + (c & 3) * D + 4 * lane, p.EX + at, Width<16>{});
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
   };
+  auto fetched = [](auto keep) { asm volatile("cp.async.wait_group %0;" ::"n"(decltype(keep)::value) : "memory"); };   // all but the last `keep`
   int vectors_known = 0;   // FED: the vectors of the chunks before this one are in memory
   auto wait_vectors = [&](int c) {   // by the whole gate warp; false: they did not come within the limit
     if (!FED || c < vectors_known) return true;
@@ -314,44 +341,45 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
     vectors_known = c + more;
     return more > 0;
   };
-  auto store_e = [&](int c, const float4 (&ev)[3]) {
-    *reinterpret_cast<float4*>(sEl + (c % 3) * D + 4 * lane) = ev[0];
-    *reinterpret_cast<float4*>(sEr + (c % 3) * D + 4 * lane) = ev[1];
-    *reinterpret_cast<float4*>(sEx + (c % 3) * D + 4 * lane) = ev[2];
-  };
-  float4 e_raw[3] = {make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f)};
-  float g_raw[2] = {0.f, 0.f};   // gate warp: g of the chunk it stores next
   bool gate_ok = true;
   if (warp == kGate) {
     if (lane == 0) {
-      prefetch_tmap(&tmW); prefetch_tmap(&tmQ); prefetch_tmap(&tmK); prefetch_tmap(&tmU);
+      prefetch_tmap(&tmW); prefetch_tmap(&tmQ); prefetch_tmap(&tmK); prefetch_tmap(&tmU); prefetch_tmap(&tmO);
       for (int b = 0; b < 8; ++b) mbar_init(bar_full + 8 * b, 1);   // three stages, exit, t1, s, pu, qk
-      mbar_init(bar_sr, kChainWarps + (FED ? 2 : 1));
-      mbar_init(bar_ud, kChainWarps);
+      mbar_init(bar_sr, kChainWarps / 2 + 2);   // and the gate and the copy warp
+      mbar_init(bar_srb, kChainWarps / 2 + 2);
+      mbar_init(bar_ud, kChainWarps / 2);
+      mbar_init(bar_udb, kChainWarps / 2);
+      mbar_init(bar_t1b, 1);
+      mbar_init(bar_sb, 1);
       mbar_init(bar_ut, kChainWarps + kOutWarps);
       mbar_init(bar_qr, kOutWarps);
       mbar_init(bar_kz, kOutWarps);
       mbar_init(bar_g, 1);
-      mbar_init(bar_tq, 1);
+      mbar_init(bar_o, kOutWarps);
+      mbar_init(bar_of, 1);
       fence_mbar_init();
       if (!FED && !misaligned) {
         issue_copies(0);
         if (n_chunks > 1) issue_copies(1);
-        requested = n_chunks > 1 ? 1 : 0;
       }
     }
     __syncwarp();
     if constexpr (KDA) {
-      // the vectors of the first two chunks are in place before the loop starts, the third chunk's in registers
+      // the vectors of the first two chunks are in place before the loop starts, the third chunk's on their way
       gate_ok = wait_vectors(0);
-      fetch_e(0, e_raw);
-      store_e(0, e_raw);
-      if (n_chunks > 1) { gate_ok = gate_ok && wait_vectors(1); fetch_e(1, e_raw); store_e(1, e_raw); }
-      if (n_chunks > 2) { gate_ok = gate_ok && wait_vectors(2); fetch_e(2, e_raw); }
+      fetch_e(0);
+      if (n_chunks > 1) gate_ok = gate_ok && wait_vectors(1);
+      fetch_e(1);
+      if (n_chunks > 2) gate_ok = gate_ok && wait_vectors(2);
+      fetch_e(2);
+      fetched(Width<1>{});
     } else {
-      fetch_g(0, g_raw);
-      store_g(0, g_raw);
-      if (n_chunks > 1) fetch_g(1, g_raw);
+      fetch_g(0);
+      fetch_g(1);
+      fetched(Width<1>{});
+      store_g(0);
+      fetch_g(2);
     }
   }
   if (!FED && warp == 0) {
@@ -371,7 +399,7 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
 #pragma unroll 1
     for (int i = 0; i < 64; ++i)
       if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-    return wait_by_warp(bar, parity, lim);
+    return __all_sync(0xffffffffu, wait_by_warp(bar, parity, lim));
   };
   // S^T as the A operand of P1: this warp's lanes, its 64 features as 32 columns of packed pairs
   // (per-channel form: a second time for PQ, feature k times er[k], exp(G_ref) of the chunk that will read the operand)
@@ -399,7 +427,12 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
     }
     tmem_wait_st();
     tc_fence_before();
-    warp_arrive(bar_sr, lane);
+    warp_arrive(bars_half + (bar_sr - bar_full), lane);
+  };
+  // the gate and copy warps' arrivals, on both halves' barriers
+  auto arrive_sr = [&]() {
+    __syncwarp();
+    if (lane == 0) { mbar_arrive(bar_sr); mbar_arrive(bar_srb); }
   };
 
   if (warp == kControl) {
@@ -408,14 +441,14 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
     // code that the compiler knows to be uniform keeps them there (issued by a branch of one lane, each instruction costs 67
     // cycles of moves into them, whatever its shape).
     if (!misaligned) {
-      constexpr uint32_t idesc_p1 = umma_idesc(cfg::M, 64, 0);    // S^T, W or Q K-major
-      constexpr uint32_t idesc_p3 = umma_idesc(cfg::M, 128, 1);   // U~'^T, K MN-major
+      constexpr uint32_t idesc_p1 = umma_idesc(cfg::M, 32, 0);    // S^T, half of W's tokens K-major
+      constexpr uint32_t idesc_pq = umma_idesc(cfg::M, 64, 0);    // S^T, Q K-major
+      constexpr uint32_t idesc_p3 = umma_idesc(cfg::M, 64, 1);    // U~'^T, half of K's features MN-major
       constexpr uint32_t idesc_qk = umma_idesc(64, 64, 0);     // Q, K K-major
       constexpr uint32_t idesc_pu = umma_idesc(cfg::M, 64, 0);    // U~^T, P K-major
       // descriptors differ from these bases only in the address field (bits 0..13, units of 16 bytes)
       const uint64_t dW = umma_desc(s0, 16, 1024), dQ = umma_desc(s0 + 8192, 16, 1024), dK = umma_desc(s0 + cfg::OFF_KT, 16, 1024),
                      dKm = umma_desc(s0 + cfg::OFF_KT, cfg::K_BOX, 1024), dP = umma_desc(sP, 16, 1024);
-      auto seen = [&](uint32_t bar, uint32_t parity) { return (bool)__all_sync(0xffffffffu, mbar_test_wait(bar, parity)); };
       auto issue_qk = [&](int c) {
         const uint32_t st = (uint32_t)((c % kStages) * cfg::STAGE) >> 4;
 #pragma unroll
@@ -424,57 +457,76 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
                     dK + st + (((ks >> 2) * cfg::K_BOX + (ks & 3) * 32) >> 4), idesc_qk, ks > 0);
         umma_commit(bar_qk);
       };
-      auto issue_p1 = [&](uint32_t d_col, uint32_t a_col, uint64_t b) {
+      auto seen = [&](uint32_t bar, uint32_t parity) { return (bool)__all_sync(0xffffffffu, mbar_test_wait(bar, parity)); };
+      // half `fh` of the features (k-steps), into columns d_col
+      auto issue_s = [&](uint32_t d_col, uint32_t a_col, uint64_t b, uint32_t idesc, int fh) {
 #pragma unroll
-        for (int ks = 0; ks < D / 16; ++ks)
-          umma_bf16_ta(tmem + d_col, tmem + a_col + 8 * ks, b + (((ks >> 2) * cfg::WQ_BOX + (ks & 3) * 32) >> 4), idesc_p1, ks > 0);
+        for (int ks = 4 * fh; ks < 4 * fh + 4; ++ks)
+          umma_bf16_ta(tmem + d_col, tmem + a_col + 8 * ks, b + (((ks >> 2) * cfg::WQ_BOX + (ks & 3) * 32) >> 4), idesc, ks > 0);
+      };
+      // P3: tokens 32 th .. + 31 (k-steps of 16: 8 columns of the A operand, 2048 bytes of the K tile), features 64 fh .. + 63
+      auto issue_p3 = [&](uint64_t b, int th, int fh) {
+#pragma unroll
+        for (int ks = 2 * th; ks < 2 * th + 2; ++ks)
+          umma_bf16_ta(tmem + cfg::TM_DS + 64 * fh, tmem + cfg::TM_UD + 32 * th + 8 * (ks & 1), b + ((fh * cfg::K_BOX + ks * 2048) >> 4), idesc_p3, ks > 0);
       };
       const bool partial = ((end - beg) & (C - 1)) != 0;
       uint32_t ph = 0;
-      if (wait(bar_full, 0)) issue_qk(0);
-      else failed = true;
+      bool early = false;   // this chunk's QK has been issued
       for (int c = 0; c < n_chunks && !failed; ++c, ph ^= 1) {
         const uint32_t st = (uint32_t)((c % kStages) * cfg::STAGE) >> 4;
         TL(9);
-        if (!wait(bar_sr, ph)) { failed = true; break; }   // (the chunk's tiles were waited for before its QK)
+        // (P1 goes where U~ is, and QK where the output warps read the last chunk's)
+        if (!early && (!wait(bar_full + 8 * (c % kStages), full_parity(c)) || (c > 0 && !wait(bar_qr, ph ^ 1)))) { failed = true; break; }
+        if ((c > 0 && !wait(bar_pu, ph ^ 1)) || !wait(bar_sr, ph)) { failed = true; break; }
         tc_fence_after();
         TL(0);
-        issue_p1(cfg::TM_WS, cfg::TM_S, dW + st);
+        issue_s(cfg::TM_WS, cfg::TM_S, dW + st, idesc_p1, 0);
+        if (!wait(bar_srb, ph)) { failed = true; break; }
+        tc_fence_after();
+        issue_s(cfg::TM_WS, cfg::TM_S, dW + st, idesc_p1, 1);
         umma_commit(bar_t1);
-        issue_p1(cfg::TM_QS, cfg::TM_SQ, dQ + st);
-        umma_commit(bar_tq);
+        issue_s(cfg::TM_WS + 32, cfg::TM_S, dW + st + (4096 >> 4), idesc_p1, 0);
+        issue_s(cfg::TM_WS + 32, cfg::TM_S, dW + st + (4096 >> 4), idesc_p1, 1);
+        umma_commit(bar_t1b);
+        if (!early) issue_qk(c);
+        const uint32_t qs = cfg::TM_QS + 64 * (c & 1);
+        issue_s(qs, cfg::TM_SQ, dQ + st, idesc_pq, 0);
+        issue_s(qs, cfg::TM_SQ, dQ + st, idesc_pq, 1);
         TL(1);
         const bool last = c + 1 >= n_chunks;
         TL(2);
         if (!KDA && last && partial && !wait(bar_kz, 0u)) { failed = true; break; }
+        const bool stall = p.test_stall && first_block && c == 1;
         if (!wait(bar_ud, ph)) { failed = true; break; }
         tc_fence_after();
         TL(3);
+        if (!stall) { issue_p3(dKm + st, 0, 0); issue_p3(dKm + st, 0, 1); }
+        if (!wait(bar_udb, ph)) { failed = true; break; }
+        tc_fence_after();
         // self-test (ScanParams::test_stall): the first CTA leaves out this product in its second chunk, so that the
         // waits for it, and then every other wait of the CTA, run out
-        if (!(p.test_stall && first_block && c == 1)) {
-#pragma unroll
-          for (int ks = 0; ks < C / 16; ++ks)   // 16 tokens (8 columns of the A operand, 2048 bytes of the K tile) per step
-            umma_bf16_ta(tmem + cfg::TM_DS, tmem + (KDA ? cfg::TM_UT : cfg::TM_UD) + 8 * ks, dKm + st + ((ks * 2048) >> 4), idesc_p3, ks > 0);
+        if (!stall) {
+          issue_p3(dKm + st, 1, 0);
           umma_commit(bar_s);
+          issue_p3(dKm + st, 1, 1);
+          umma_commit(bar_sb);
         }
         TL(4);
-        // the next chunk's QK, if its tiles have landed and this chunk's QK has been read; otherwise behind PU
-        const bool early = !last && seen(bar_full + 8 * ((c + 1) % kStages), full_parity(c + 1)) && seen(bar_qr, ph);
-        if (early) { tc_fence_after(); issue_qk(c + 1); }
-        if (!wait(bar_ut, ph)) { failed = true; break; }   // U~ (chain warps) and P with the start of PU (output warps)
+        if (!wait(bar_ut, ph)) { failed = true; break; }   // U~ (chain warps) and P (output warps)
+        fence_proxy_async();   // P was written by ordinary stores; the fence is on this side because the writers took up to 400 cycles for it
         tc_fence_after();
         TL(5);
 #pragma unroll
         for (int ks = 0; ks < C / 16; ++ks)
-          umma_bf16_ta(tmem + cfg::TM_PU, tmem + cfg::TM_UT + 8 * ks, dP + ((ks * 32) >> 4), idesc_pu, 1u);   // on top of gamma_i (Q S)^T
+          umma_bf16_ta(tmem + (KDA ? qs : (uint32_t)cfg::TM_PU), tmem + cfg::TM_UT + 32 * (ks >> 1) + 8 * (ks & 1), dP + ((ks * 32) >> 4), idesc_pu,
+                       KDA || ks > 0);   // per-channel form: on top of (Q S)^T, which carries its decay
         umma_commit(bar_pu);
         TL(6);
-        if (!last && !early) {
-          if (!wait(bar_full + 8 * ((c + 1) % kStages), full_parity(c + 1)) || !wait(bar_qr, ph)) { failed = true; break; }
-          tc_fence_after();
-          issue_qk(c + 1);
-        }
+        // the next chunk's QK, if its tiles have landed and this chunk's QK has been read; otherwise behind its P1
+        early = !last && seen(bar_full + 8 * ((c + 1) % kStages), full_parity(c + 1)) && seen(bar_qr, ph);
+        if (early) { tc_fence_after(); issue_qk(c + 1); }
+        TL(11);
       }
       if (failed) {
         // A wait has run out and this CTA is about to give up its shared and tensor memory: every product issued so far is
@@ -484,47 +536,36 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
       }
     }
   } else if (warp == kGate) {
-    // ---------------------------------------------------------------- gate warp: tile copies of chunk c + 2, factors of chunk c + 1
+    // ---------------------------------------------------------------- gate warp: factors of chunk c + 1
     // Its arrival on bar_sr tells the control thread, and through the first product's commit every reader, that
     // the chunk's factors are in place (bar_g tells the output warps, which start on a chunk earlier).
-    if (!misaligned) { warp_arrive(bar_sr, lane); if (lane == 0) mbar_arrive(bar_g); }   // the first chunk's (written before the CTA barrier above)
+    if (!misaligned) { arrive_sr(); if (lane == 0) mbar_arrive(bar_g); }   // the first chunk's (written before the CTA barrier above)
     failed |= !gate_ok;
     for (int c = 0; c + 1 < n_chunks && !misaligned && !failed; ++c) {
-      // stage of c + 2 = that of c - 1: its readers (the products of chunk c - 1, the chain warps' U) were done before the
-      // arrivals that open chunk c
-      if (!wait(bar_sr, (uint32_t)(c & 1))) { failed = true; break; }
-      if (!FED && lane == 0 && c + 2 < n_chunks) { issue_copies(c + 2); requested = c + 2; }
-      __syncwarp();
-      // the factors of c - 1 have no reader left once the first product of chunk c is complete (it was issued behind the
+      // the factors of c - 2 (per-channel form: the vectors of c - 1) have no reader left once the first product of chunk c is complete (it was issued behind the
       // arrivals of every warp that read them); bar_qr also says that every output warp has seen bar_g of chunk c, which must not
       // run two phases ahead of a warp that still waits for it
-      if (!wait(bar_t1, (uint32_t)(c & 1)) || !wait(bar_qr, (uint32_t)(c & 1))) { failed = true; break; }
-      if constexpr (KDA) {
-        // The vectors run one chunk further ahead than g: exp(G_ref) of chunk c + 1 is read at the end of chunk c (it
-        // scales the S^T operand), so it has to be in place, and announced by an arrival, a chunk earlier.  Those of
-        // c + 2 go where those of c - 1 were.
-        if (c + 2 < n_chunks) store_e(c + 2, e_raw);
-      } else {
-        store_g(c + 1, g_raw);
-      }
-      warp_arrive(bar_sr, lane);
+      if (!wait(bar_t1b, (uint32_t)(c & 1)) || !wait(bar_qr, (uint32_t)(c & 1))) { failed = true; break; }
+      fetched(Width<KDA ? 0 : 1>{});
+      // The vectors run one chunk further ahead than g: exp(G_ref) of chunk c + 1 is read at the end of chunk c (it
+      // scales the S^T operand), so it has to be in place, and announced by an arrival, a chunk earlier.
+      if constexpr (!KDA) store_g(c + 1);
+      arrive_sr();
       if (lane == 0) mbar_arrive(bar_g);
       if constexpr (KDA) {
-        if (c + 3 < n_chunks) {
-          if (!wait_vectors(c + 3)) { failed = true; break; }
-          fetch_e(c + 3, e_raw);
-        }
+        if (c + 3 < n_chunks && !wait_vectors(c + 3)) { failed = true; break; }
+        fetch_e(c + 3);
+      } else {
+        fetch_g(c + 3);
       }
-      else { if (c + 2 < n_chunks) fetch_g(c + 2, g_raw); }
     }
-    if (!FED && failed && lane == 0) drain_copies();
-  } else if (FED && warp == kCopy) {
-    // ---------------------------------------------------------------- copy warp: tile copies of chunk c + 2, once W and U are there
+  } else if (warp == kCopy) {
+    // ---------------------------------------------------------------- copy warp: tile copies of chunk c + 2 (FED: once W and U are there)
     // It arrives on bar_sr itself, after its wait for the phase before: the barrier must not run two phases ahead of it while it
     // waits for another CTA.
     int known = 0;   // chunks before this one have their factors in memory
     auto request = [&](int c) -> bool {   // false: W and U did not come within the limit
-      if (c >= known) {
+      if (FED && c >= known) {
         const int more = wait_ready(ready + ((size_t)((beg + c * C) / C + s) * p.H + h), p.H, n_chunks - c, lane, lim);
         if (!more) return false;
         known = c + more;
@@ -534,12 +575,13 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
       return true;
     };
     if (!misaligned) {
-      warp_arrive(bar_sr, lane);
-      failed = !request(0) || (n_chunks > 1 && !request(1));
+      arrive_sr();
+      if constexpr (FED) failed = !request(0) || (n_chunks > 1 && !request(1));
+      else requested = n_chunks > 1 ? 1 : 0;   // by the gate warp, before the CTA barrier
     }
     for (int c = 0; c + 1 < n_chunks && !misaligned && !failed; ++c) {
-      if (!wait(bar_sr, (uint32_t)(c & 1))) { failed = true; break; }
-      warp_arrive(bar_sr, lane);
+      if (!wait(bar_sr, (uint32_t)(c & 1)) || !wait(bar_srb, (uint32_t)(c & 1))) { failed = true; break; }
+      arrive_sr();
       if (c + 2 < n_chunks && !request(c + 2)) { failed = true; break; }
     }
     if (failed && lane == 0) drain_copies();
@@ -550,12 +592,12 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
     for (int c = 0; c < n_chunks && !misaligned; ++c, ph ^= 1) {
       const int tok0 = beg + c * C;
       const int rows = end - tok0 < C ? end - tok0 : C;
-      const float* fb = sG + (c & 1) * 4 * C;
+      const float* fb = sG + (c % 3) * 5 * C;
       const uint32_t sU = s0 + (c % kStages) * cfg::STAGE + cfg::OFF_UT;
       TL(0);
       if (!wait(bar_full + 8 * (c % kStages), full_parity(c))) { failed = true; break; }   // landed long ago; U is read below
       TL(1);
-      if (!wait(bar_t1, ph)) { failed = true; break; }
+      if (!wait(bars_half + (bar_t1 - bar_full), ph)) { failed = true; break; }
       tc_fence_after();
       TL(2);
       // ---- U~ = U - W S, transposed: first the decay-scaled U~' that the chain waits for (its own arrival), then U~ itself
@@ -616,7 +658,7 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
             r[2 * nt] = pack_bf16(v[lg][nt][0] * dd[nt].x, v[lg][nt][1] * dd[nt].y);
             r[2 * nt + 1] = E == 2 ? pack_bf16(v[lg][nt][2] * dd[nt].x, v[lg][nt][3] * dd[nt].y) : 0u;
           }
-          tmem_st_packed16(r, tmem_w + ((uint32_t)(16 * lg) << 16) + cfg::TM_UD + 16 * half);
+          tmem_st_packed16(r, tmem_w + ((uint32_t)(16 * lg) << 16) + cfg::TM_UD + 32 * half);
         }
 #pragma unroll
         for (int nt = 0; nt < 4; ++nt) {
@@ -627,18 +669,18 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
       if constexpr (!KDA) {
         tmem_wait_st();
         tc_fence_before();
-        warp_arrive(bar_ud, lane);
+        warp_arrive(bars_half + (bar_ud - bar_full), lane);
       }
       TL(4);
 #pragma unroll
-      for (int lg = 0; lg < LG; ++lg) tmem_st_packed16(ut[lg], tmem_w + ((uint32_t)(16 * lg) << 16) + cfg::TM_UT + 16 * half);
+      for (int lg = 0; lg < LG; ++lg) tmem_st_packed16(ut[lg], tmem_w + ((uint32_t)(16 * lg) << 16) + cfg::TM_UT + 32 * half);
       tmem_wait_st();
       tc_fence_before();
-      if constexpr (KDA) warp_arrive(bar_ud, lane);   // U~ itself is the operand of both later products
+      if constexpr (KDA) warp_arrive(bars_half + (bar_ud - bar_full), lane);   // U~ itself is the operand of both later products
       warp_arrive(bar_ut, lane);
       TL(5);
       // ---- state update and the bf16 operand for the next chunk
-      if (!wait(bar_s, ph)) { failed = true; break; }
+      if (!wait(bars_half + (bar_s - bar_full), ph)) { failed = true; break; }
       tc_fence_after();
       TL(6);
 #pragma unroll
@@ -650,8 +692,8 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
 #pragma unroll
         for (int nt = 0; nt < 8; ++nt) {
           if constexpr (KDA) {
-            const float2 el = *reinterpret_cast<const float2*>(sEl + (c % 3) * D + 64 * half + 8 * nt + 2 * t);
-            const float2 ex = *reinterpret_cast<const float2*>(sEx + (c % 3) * D + 64 * half + 8 * nt + 2 * t);
+            const float2 el = *reinterpret_cast<const float2*>(sEl + (c & 3) * D + 64 * half + 8 * nt + 2 * t);
+            const float2 ex = *reinterpret_cast<const float2*>(sEx + (c & 3) * D + 64 * half + 8 * nt + 2 * t);
 #pragma unroll
             for (int e = 0; e < E; ++e) {
               S[lg][nt][2 * e] = fmaf(el.x, S[lg][nt][2 * e], ex.x * ds[nt][2 * e]);
@@ -664,154 +706,178 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
         }
       }
       TL(7);
-      if (c + 1 < n_chunks) write_state_operand(sEr + ((c + 1) % 3) * D);   // its last reader was P1 of this chunk
+      if (c + 1 < n_chunks) write_state_operand(sEr + ((c + 1) & 3) * D);   // its last reader was P1 of this chunk
       TL(8);
     }
     if (!failed) store_state();
   } else if (warp < kChainWarps + kOutWarps) {
     // ---------------------------------------------------------------- output warps
-    uint32_t ph = 0;
-    int o_tok0 = 0, o_rows = 0;
-    uint8_t* stage = smem + cfg::OFF_O + (warp - kChainWarps) * cfg::O_WARP;
-    const uint32_t stage_a = smem_u32(stage);
-    constexpr int PP = cfg::RPQ / 8;   // 16-byte pieces per token in this warp's staging tile
-    auto piece_at = [](int tok, int piece) {   // eight neighbouring tokens' pieces in different banks
-      const int x = PP == 4 ? piece ^ ((tok >> 1) & 3) : PP == 2 ? piece ^ ((tok >> 2) & 1) : piece;
-      return (uint32_t)(tok * PP * 16 + x * 16);
+    // 16 bytes (eight columns) of a token in O's tile: the swizzle that the copy engine undoes on the way out
+    auto o_at = [&](int tok, int col) {
+      if constexpr (DVS == 32) return s0 + cfg::OFF_O + tok * 64 + ((((col >> 3) ^ (tok >> 1)) & 3) << 4);
+      else return s0 + cfg::OFF_O + (col >> 6) * 8192 + tok * 128 + ((((col >> 3) ^ tok) & 7) << 4);
     };
-    // O = scale * (gamma_i QS + P U~) of the previous chunk (the PU accumulator starts from gamma_i QS), while the next
-    // chunk's first product runs: fragments -> [token][column] tile (stmatrix.trans) -> 16-byte stores
-    auto write_output = [&]() {   // (behind the wait for that chunk's PU)
+    // O = scale * (gamma_i QS + P U~) of a chunk out of tensor memory (behind the wait for its PU) into its tile, from where the store warp
+    // sends it on.  Accumulator fragments -> [token][column] by stmatrix.trans.
+    auto put_output = [&](int c) -> bool {
+      if (c > 0 && !wait(bar_of, (uint32_t)((c - 1) & 1))) return false;   // the last chunk's store has read the tile
+      const float* gam = sG + (c % 3) * 5 * C + 4 * C + 2 * t;
+      constexpr int NC = LG == 2 ? 4 : 8;   // blocks of eight tokens at a time: what the registers allow
 #pragma unroll
       for (int lg = 0; lg < LG; ++lg) {
-        float pu[8][4];
-        tmem_ld_16x64(pu, tmem_w + ((uint32_t)(16 * lg) << 16) + cfg::TM_PU);
-        tmem_wait_ld();
-        if constexpr (E == 2) {
 #pragma unroll
-          for (int nt = 0; nt < 8; nt += 2)
-            stmatrix_x4_trans(stage_a + piece_at(8 * (nt + (mi >> 1)) + mr, 2 * lg + (mi & 1)),
-                              pack_bf16(p.scale * pu[nt][0], p.scale * pu[nt][1]), pack_bf16(p.scale * pu[nt][2], p.scale * pu[nt][3]),
-                              pack_bf16(p.scale * pu[nt + 1][0], p.scale * pu[nt + 1][1]), pack_bf16(p.scale * pu[nt + 1][2], p.scale * pu[nt + 1][3]));
-        } else {
+        for (int n0 = 0; n0 < 8; n0 += NC) {
+          const uint32_t at = tmem_w + ((uint32_t)(16 * lg) << 16) + 8 * n0;
+          float pu[NC][4], qs[NC][4];
+          tmem_ld_tokens(pu, at + (KDA ? cfg::TM_QS + 64 * (c & 1) : cfg::TM_PU));
+          if constexpr (KDA) {
+            tmem_wait_ld();
+          } else {
+            tmem_ld_tokens(qs, at + cfg::TM_QS + 64 * (c & 1));
+            float2 y[NC];
 #pragma unroll
-          for (int nt = 0; nt < 8; nt += 4)
-            stmatrix_x4_trans(stage_a + piece_at(8 * (nt + mi) + mr, 0),
-                              pack_bf16(p.scale * pu[nt][0], p.scale * pu[nt][1]), pack_bf16(p.scale * pu[nt + 1][0], p.scale * pu[nt + 1][1]),
-                              pack_bf16(p.scale * pu[nt + 2][0], p.scale * pu[nt + 2][1]), pack_bf16(p.scale * pu[nt + 3][0], p.scale * pu[nt + 3][1]));
+            for (int nt = 0; nt < NC; ++nt) y[nt] = *reinterpret_cast<const float2*>(gam + 8 * (n0 + nt));
+            tmem_wait_ld();
+#pragma unroll
+            for (int nt = 0; nt < NC; ++nt)
+#pragma unroll
+              for (int e = 0; e < E; ++e) {
+                pu[nt][2 * e] = fmaf(y[nt].x, qs[nt][2 * e], pu[nt][2 * e]);
+                pu[nt][2 * e + 1] = fmaf(y[nt].y, qs[nt][2 * e + 1], pu[nt][2 * e + 1]);
+              }
+          }
+          if constexpr (KDA) {   // (scalar gate: the scale is in the factors)
+#pragma unroll
+            for (int nt = 0; nt < NC; ++nt)
+#pragma unroll
+              for (int q = 0; q < 2 * E; ++q) pu[nt][q] *= p.scale;
+          }
+          if constexpr (E == 2) {
+#pragma unroll
+            for (int nt = 0; nt < NC; nt += 2)
+              stmatrix_x4_trans(o_at(8 * (n0 + nt + (mi >> 1)) + mr, row0 + 16 * lg + 8 * (mi & 1)),
+                                pack_bf16(pu[nt][0], pu[nt][1]), pack_bf16(pu[nt][2], pu[nt][3]), pack_bf16(pu[nt + 1][0], pu[nt + 1][1]), pack_bf16(pu[nt + 1][2], pu[nt + 1][3]));
+          } else {
+#pragma unroll
+            for (int nt = 0; nt < NC; nt += 4)
+              stmatrix_x4_trans(o_at(8 * (n0 + nt + mi) + mr, row0),
+                                pack_bf16(pu[nt][0], pu[nt][1]), pack_bf16(pu[nt + 1][0], pu[nt + 1][1]), pack_bf16(pu[nt + 2][0], pu[nt + 2][1]), pack_bf16(pu[nt + 3][0], pu[nt + 3][1]));
+          }
         }
       }
       tc_fence_before();
-      __syncwarp();
-      __nv_bfloat16* Og = reinterpret_cast<__nv_bfloat16*>(p.O) + ((size_t)(o_tok0) * p.H + h) * D + slice * DVS + row0;
-#pragma unroll
-      for (int it = 0; it < 2 * PP; ++it) {
-        const int tok = (32 * it + lane) / PP, piece = lane % PP;
-        const uint4 w = *reinterpret_cast<const uint4*>(stage + piece_at(tok, piece));
-        if (tok < o_rows) *reinterpret_cast<uint4*>(Og + (size_t)tok * p.H * D + 8 * piece) = w;
-      }
-      __syncwarp();   // the tile has been read
+      return true;
     };
-    for (int c = 0; c < n_chunks && !misaligned; ++c, ph ^= 1) {
-      const int tok0 = beg + c * C;
-      const float* fb = sG + (c & 1) * 4 * C;
-      TL(0);
-      // ---- P = (Q K^T) * decay, lower triangle with its diagonal: rows 16 quad .. + 15 of this warp
-      if (!wait(bar_g, ph) || !wait(bar_qk, ph)) { failed = true; break; }
-      tc_fence_after();
-      TL(1);
-      if (!KDA && end - tok0 < C) {
-        // The tile's rows past the sequence's end hold a neighbour's keys.  U~ is zero there, but zero times Inf or NaN is not: the state
-        // product must find zeros.  QK, the tile's other reader, is done.  By these warps and not the chain's, whose loop got 1 % longer with
-        // it (512 chunks, 32 pairs: 650 -> 655 us; here 654 and 653).  The per-channel form does without: clearing in either role cost it 1 to
-        // 4 %; beside the preparation each chunk has rows of its own instead (issue_copies).
-        clear_rows(s0 + (c % kStages) * cfg::STAGE + cfg::OFF_KT, cfg::K_BOX, end - tok0, tid - kChainWarps * 32);
-        warp_arrive(bar_kz, lane);
-      }
-      uint32_t wa[8], wb[8];
-      {
-        float qk[8][4];
-        tmem_ld_16x64(qk, tmem_w + cfg::TM_QK);
-        tmem_wait_ld();
-        tc_fence_before();
-        warp_arrive(bar_qr, lane);
-        const int ia = 16 * quad + gq, ib = ia + 8;
-        const float g_a = KDA ? 0.f : fb[ia], g_b = KDA ? 0.f : fb[ib];
-        // No branch around a block: entries right of a row's diagonal are masked by selection, and the exponent of
-        // a row that lies above the whole block is not formed (its argument is replaced by zero).
+    // rows 16 quad .. + 15 of P's tile (K-major operand, row i, 16-byte pieces of eight tokens j, swizzled): the columns that form_p leaves out are zero
+    for (int e = lane; e < 16 * 8; e += 32)
+      asm volatile("st.shared.v4.b32 [%0], {%1, %1, %1, %1};" ::"r"(sP + 2048 * quad + 16 * e), "r"(0) : "memory");
+    __syncwarp();
+    uint32_t ph = 0;
+    // P = (Q K^T) * decay of chunk c, lower triangle with its diagonal: rows 16 quad .. + 15 and the first 8 NT columns.
+    // Its factors first, while QK is on its way.  No branch around a block: entries right of a row's diagonal are masked by
+    // selection, and the exponent of a row that lies above the whole block is not formed (its argument is replaced by zero).
+    float f[8][4];
+    const int ia = 16 * quad + gq, ib = ia + 8;
+    auto form_factors = [&](auto width, const float* fb) {
+      const float g_a = fb[ia], g_b = fb[ib];
 #pragma unroll
-        for (int nt = 0; nt < 8; ++nt) {
-          const int j0 = 8 * nt, j = j0 + 2 * t;
-          float p0, p1, p2, p3;
-          if constexpr (KDA) {   // the product carries its decay: only the mask is left
-            p0 = j <= ia ? qk[nt][0] : 0.f; p1 = j + 1 <= ia ? qk[nt][1] : 0.f;
-            p2 = j <= ib ? qk[nt][2] : 0.f; p3 = j + 1 <= ib ? qk[nt][3] : 0.f;
-          } else {
-            const float gref = fb[j0];
-            const float2 cj = *reinterpret_cast<const float2*>(fb + C + j);
-            const float ea = ex2_approx(j0 <= ia ? g_a - gref : 0.f), eb = ex2_approx(j0 <= ib ? g_b - gref : 0.f);
-            p0 = j <= ia ? qk[nt][0] * ea * cj.x : 0.f; p1 = j + 1 <= ia ? qk[nt][1] * ea * cj.y : 0.f;
-            p2 = j <= ib ? qk[nt][2] * eb * cj.x : 0.f; p3 = j + 1 <= ib ? qk[nt][3] * eb * cj.y : 0.f;
-          }
-          wa[nt] = pack_bf16(p0, p1);
-          wb[nt] = pack_bf16(p2, p3);
+      for (int nt = 0; nt < decltype(width)::value; ++nt) {
+        const float gref = fb[8 * nt];
+        const float2 cj = *reinterpret_cast<const float2*>(fb + C + 8 * nt + 2 * t);
+        const float ea = ex2_approx(8 * nt <= ia ? g_a - gref : 0.f), eb = ex2_approx(8 * nt <= ib ? g_b - gref : 0.f);
+        f[nt][0] = ea * cj.x; f[nt][1] = ea * cj.y;
+        f[nt][2] = eb * cj.x; f[nt][3] = eb * cj.y;
+      }
+    };
+    auto form_p = [&](auto width) {
+      constexpr int NT = decltype(width)::value;
+      float qk[NT][4];
+      tmem_ld_tokens(qk, tmem_w + cfg::TM_QK);
+      tmem_wait_ld();
+      tc_fence_before();
+      warp_arrive(bar_qr, lane);
+      uint32_t wa[NT], wb[NT];
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt) {
+        const int j = 8 * nt + 2 * t;
+        if constexpr (!KDA) {   // (per-channel form: the product carries its decay, only the mask is left)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) qk[nt][q] *= f[nt][q];
+        }
+        wa[nt] = pack_bf16(j <= ia ? qk[nt][0] : 0.f, j + 1 <= ia ? qk[nt][1] : 0.f);
+        wb[nt] = pack_bf16(j <= ib ? qk[nt][2] : 0.f, j + 1 <= ib ? qk[nt][3] : 0.f);
+      }
+      // x4 stores of the matrices (rows +0..7, block), (rows +8..15, block), and the same of block + 1
+      const int row = 16 * quad + 8 * (mi & 1) + mr;
+#pragma unroll
+      for (int nt = 0; nt < NT; nt += 2) stmatrix_x4(sP + row * 128 + (((nt + (mi >> 1)) ^ (row & 7)) << 4), wa[nt], wb[nt], wa[nt + 1], wb[nt + 1]);
+    };
+    const bool narrow = quad < 2;   // nothing in the right half (and on the schedulers of the control and the gate warp)
+    // Chunk c: its P, and the O of the chunk before (a last round has only that: one copy of each in the code, since the warps of a CTA run different
+    // code and what does not fit the instruction caches slows all of them down)
+    for (int c = 0; c <= n_chunks && !misaligned; ++c, ph ^= 1) {
+      TL(0);
+      const bool more = c < n_chunks;
+      if (more) {
+        // (per-channel form: waited for as well, so that bar_qr does not run two phases ahead of the gate warp)
+        if (!wait(bar_g, ph)) { failed = true; break; }
+        if constexpr (!KDA) {
+          if (narrow) form_factors(Width<4>{}, sG + (c % 3) * 5 * C);
+          else form_factors(Width<8>{}, sG + (c % 3) * 5 * C);
         }
       }
-      TL(2);
-      // PU of the last chunk has completed: P's tile is free, O can be read.  P goes first (its fence would wait for O's stores):
-      // K-major operand, row i, 16-byte pieces of eight tokens j, swizzled; x4 stores of the matrices (rows +0..7, block),
-      // (rows +8..15, block), and the same of block + 1
-      if (c > 0) {
+      if (c > 0) {   // PU of the chunk before has completed: its O can be read, and P's tile is free
         if (!wait(bar_pu, ph ^ 1)) { failed = true; break; }
         tc_fence_after();
+        if (!put_output(c - 1)) { failed = true; break; }
       }
-      {
-        const int row = 16 * quad + 8 * (mi & 1) + mr;
-#pragma unroll
-        for (int nt = 0; nt < 8; nt += 2) stmatrix_x4(sP + row * 128 + (((nt + (mi >> 1)) ^ (row & 7)) << 4), wa[nt], wb[nt], wa[nt + 1], wb[nt + 1]);
-        fence_proxy_async();
-      }
-      if (c > 0) write_output();
-      TL(3);
-      if (!wait(bar_tq, ph)) { failed = true; break; }
-      tc_fence_after();
-      TL(4);
-      // ---- gamma_i (Q S)^T becomes the starting value of the PU accumulator (same lanes); in the per-channel form the
-      // decay is inside the product already
-#pragma unroll
-      for (int lg = 0; lg < LG; ++lg) {
-        const uint32_t trow = tmem_w + ((uint32_t)(16 * lg) << 16);
-        float qs[8][4];
-        tmem_ld_16x64(qs, trow + cfg::TM_QS);
-        tmem_wait_ld();
-        if constexpr (!KDA) {
-#pragma unroll
-          for (int nt = 0; nt < 8; ++nt) {
-            const float2 y = *reinterpret_cast<const float2*>(fb + 3 * C + 8 * nt + 2 * t);
-            qs[nt][0] *= y.x; qs[nt][1] *= y.y; qs[nt][2] *= y.x; qs[nt][3] *= y.y;
-          }
-        }
-#pragma unroll
-        for (int b = 0; b < 8; b += 4) {
-          const float q4[4][4] = {{qs[b][0], qs[b][1], qs[b][2], qs[b][3]}, {qs[b + 1][0], qs[b + 1][1], qs[b + 1][2], qs[b + 1][3]},
-                                  {qs[b + 2][0], qs[b + 2][1], qs[b + 2][2], qs[b + 2][3]}, {qs[b + 3][0], qs[b + 3][1], qs[b + 3][2], qs[b + 3][3]}};
-          tmem_st_16x32(q4, trow + cfg::TM_PU + 8 * b);
-        }
-      }
-      tmem_wait_st();
-      tc_fence_before();
-      warp_arrive(bar_ut, lane);
-      TL(5);
-      o_tok0 = tok0;
-      o_rows = end - tok0 < C ? end - tok0 : C;
-    }
-    if (!failed && !misaligned) {
-      if (wait(bar_pu, ph ^ 1)) {
+      if (more) {
+        if (!wait(bar_qk, ph)) { failed = true; break; }
         tc_fence_after();
-        write_output();
-      } else {
-        failed = true;
+        TL(1);
+        if (!KDA && end - beg - c * C < C) {
+          // The tile's rows past the sequence's end hold a neighbour's keys.  U~ is zero there, but zero times Inf or NaN is not: the state
+          // product must find zeros.  QK, the tile's other reader, is done.  By these warps and not the chain's, whose loop got 1 % longer with
+          // it (512 chunks, 32 pairs: 650 -> 655 us; here 654 and 653).  The per-channel form does without: clearing in either role cost it 1 to
+          // 4 %; beside the preparation each chunk has rows of its own instead (issue_copies).
+          clear_rows(s0 + (c % kStages) * cfg::STAGE + cfg::OFF_KT, cfg::K_BOX, end - beg - c * C, tid - kChainWarps * 32);
+          warp_arrive(bar_kz, lane);
+        }
+        if (narrow) form_p(Width<4>{});
+        else form_p(Width<8>{});
+        TL(2);
       }
+      // (the fences between these ordinary stores and what reads them through the asynchronous proxy are the control and the store warp's)
+      __syncwarp();
+      if (lane == 0) {
+        if (more) mbar_arrive(bar_ut);
+        if (c > 0) mbar_arrive(bar_o);
+      }
+      TL(5);
+    }
+  } else if (warp == kStore) {
+    // ---------------------------------------------------------------- store warp: O's tile to memory
+    // By the copy engine, whose stores cost the output warps nothing and write whole rows of 128 bytes; the rows of a partial chunk by ordinary ones.
+    for (int c = 0; c < n_chunks && !misaligned; ++c) {
+      if (!wait(bar_o, (uint32_t)(c & 1))) { failed = true; break; }
+      const int tok0 = beg + c * C;
+      if (end - tok0 >= C) {
+        if (lane == 0) {
+          fence_proxy_async();   // the tile was written by ordinary stores
+          tma_store_2d(&tmO, s0 + cfg::OFF_O, h * D + slice * DVS, tok0);
+          if constexpr (DVS == 128) tma_store_2d(&tmO, s0 + cfg::OFF_O + 8192, h * D + 64, tok0);
+          bulk_commit();
+          bulk_wait_read();
+        }
+      } else {
+        __nv_bfloat16* Og = reinterpret_cast<__nv_bfloat16*>(p.O) + ((size_t)tok0 * p.H + h) * D + slice * DVS;
+        for (int e = lane; e < (end - tok0) * (DVS / 8); e += 32) {
+          const int tok = e / (DVS / 8), pc = e % (DVS / 8);
+          const int at = DVS == 32 ? tok * 64 + (((pc ^ (tok >> 1)) & 3) << 4) : (pc >> 3) * 8192 + tok * 128 + (((pc ^ tok) & 7) << 4);
+          *reinterpret_cast<uint4*>(Og + (size_t)tok * p.H * D + 8 * pc) = *reinterpret_cast<const uint4*>(smem + cfg::OFF_O + at);
+        }
+      }
+      warp_arrive(bar_of, lane);
     }
   }
   if (failed) atomicMax(p.status, TRI_INV_ERR_DEVICE_TIMEOUT);
@@ -826,11 +892,11 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
 template <int DVS, bool KDA>
 __global__ void __launch_bounds__(kThreadsScan, 1)
 chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmQ,
-                  const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmU, ScanParams p) {
+                  const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUtensorMap tmO, ScanParams p) {
   constexpr int NS = D / DVS;
   extern __shared__ __align__(1024) uint8_t smem[];
   const int slice = blockIdx.x % NS, h = (blockIdx.x / NS) % p.H, s = blockIdx.x / (NS * p.H);
-  scan_walk<DVS, KDA, false>(tmW, tmQ, tmK, tmU, p, smem, s, h, slice, blockIdx.x == 0, nullptr, 0u);
+  scan_walk<DVS, KDA, false>(tmW, tmQ, tmK, tmU, tmO, p, smem, s, h, slice, blockIdx.x == 0, nullptr, 0u);
 }
 
 constexpr int kSeqsPerLaunch = 960;
@@ -842,9 +908,22 @@ __global__ void __launch_bounds__(256) seq_offsets_kernel(int* out, const __grid
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i <= b.n; i += gridDim.x * blockDim.x) out[b.first + i] = b.cu[i];
 }
 
+// O as the scans store it: boxes of 64 tokens x 64 columns, or 32 of the narrow slice
+template <int DVS>
+bool make_tmap_out(CUtensorMap* tm, const void* base, long long tokens, int H) {
+  EncodeTiledFn fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[2] = {(cuuint64_t)H * D, (cuuint64_t)tokens};
+  cuuint64_t strides[1] = {(cuuint64_t)H * D * 2};
+  cuuint32_t box[2] = {DVS == 32 ? 32 : 64, (cuuint32_t)C};
+  cuuint32_t estr[2] = {1, 1};
+  return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+            DVS == 32 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 template <int DVS, bool KDA>
 cudaError_t launch_scan_one(const ScanParams& p, const CUtensorMap& tmW, const CUtensorMap& tmQ, const CUtensorMap& tmK,
-                            const CUtensorMap& tmU, cudaStream_t stream) {
+                            const CUtensorMap& tmU, long long tokens, cudaStream_t stream) {
   using cfg = ScanCfg<DVS, KDA>;
   static std::mutex mu;
   static bool ready[64] = {false};
@@ -862,7 +941,9 @@ cudaError_t launch_scan_one(const ScanParams& p, const CUtensorMap& tmW, const C
   }
   const long long grid = (long long)p.n_seqs * p.H * (D / DVS);
   if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-  chunk_scan_kernel<DVS, KDA><<<(int)grid, kThreadsScan, cfg::SMEM, stream>>>(tmW, tmQ, tmK, tmU, p);
+  CUtensorMap tmO;
+  if (!make_tmap_out<DVS>(&tmO, p.O, tokens, p.H)) return cudaErrorUnknown;
+  chunk_scan_kernel<DVS, KDA><<<(int)grid, kThreadsScan, cfg::SMEM, stream>>>(tmW, tmQ, tmK, tmU, tmO, p);
   return launched();
 }
 
@@ -903,9 +984,9 @@ cudaError_t launch_chunk_scan(const ScanParams& p, const void* Q, const void* K,
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return cudaErrorUnknown;
   const long long pairs = (long long)p.n_seqs * p.H;
-  if (pairs * 8 <= sms) return kda ? launch_scan_one<32, true>(p, tmW, tmQ, tmK, tmU, stream) : launch_scan_one<32, false>(p, tmW, tmQ, tmK, tmU, stream);
-  if (pairs * 2 <= sms) return kda ? launch_scan_one<64, true>(p, tmW, tmQ, tmK, tmU, stream) : launch_scan_one<64, false>(p, tmW, tmQ, tmK, tmU, stream);
-  return kda ? launch_scan_one<128, true>(p, tmW, tmQ, tmK, tmU, stream) : launch_scan_one<128, false>(p, tmW, tmQ, tmK, tmU, stream);
+  if (pairs * 8 <= sms) return kda ? launch_scan_one<32, true>(p, tmW, tmQ, tmK, tmU, tokens, stream) : launch_scan_one<32, false>(p, tmW, tmQ, tmK, tmU, tokens, stream);
+  if (pairs * 2 <= sms) return kda ? launch_scan_one<64, true>(p, tmW, tmQ, tmK, tmU, tokens, stream) : launch_scan_one<64, false>(p, tmW, tmQ, tmK, tmU, tokens, stream);
+  return kda ? launch_scan_one<128, true>(p, tmW, tmQ, tmK, tmU, tokens, stream) : launch_scan_one<128, false>(p, tmW, tmQ, tmK, tmU, tokens, stream);
 }
 
 }  // namespace tri_inv
