@@ -16,6 +16,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import warnings
 
 import numpy as np
 import torch
@@ -125,6 +126,26 @@ def load():
         lib.tri_inv_status_string.argtypes = [i32]
         _lib = lib
     return _lib
+
+
+_native_layer = None
+
+
+def load_native():
+    """The extension that marshals gdn_forward's ordinary calls, bound to the loaded library (once).  Where it has not been built the calls are
+    marshalled in Python as the other functions' are: the same kernels, 7 us more of host time."""
+    global _native_layer
+    if _native_layer is None:
+        lib = load()
+        try:
+            from . import _native
+            addr = lambda f: ctypes.cast(f, ctypes.c_void_p).value   # noqa: E731
+            _native.bind(addr(lib.tri_inv_gdn_forward_workspace), addr(lib.tri_inv_gdn_forward))
+            _native_layer = _native.gdn_forward
+        except ImportError as e:
+            warnings.warn("%s: gdn_forward is marshalled in Python (build it with `python -m paper_2605_21325_b200.build`)" % e)
+            _native_layer = lambda *args: None   # noqa: E731
+    return _native_layer
 
 
 def status_string(status: int) -> str:
@@ -253,6 +274,12 @@ def chunk_scan_kda(Q, K, W, U, G, C, scale=1.0, S0=None, cu_seqlens=None, out=No
 def gdn_forward(Q, K, V, beta, g, C, scale=1.0, S0=None, method=BLOCK_RECURSIVE, cu_seqlens=None, stream=None):
     """The whole layer -> (O, S_final): tri_inv_gdn_forward, which takes one kernel, or the fused call with the decay-weighted W and
     the chunk scan, by shape."""
+    if stream is None:   # plain contiguous CUDA tensors on the current stream: marshalled in native code
+        out = (_native_layer or load_native())(Q, K, V, beta, g, C, scale, S0, method, cu_seqlens)
+        if out.__class__ is tuple:
+            return out
+        if out is not None:
+            raise TriInvError("tri_inv_gdn_forward" if out < 256 else "tri_inv_gdn_forward_workspace", out & 255)
     B, T, H, d_k = K.shape
     d_v = V.shape[-1]
     lib = load()

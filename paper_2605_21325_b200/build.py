@@ -5,6 +5,9 @@ nvcc cross-compiles for sm_100a without a GPU.  The result,
 an object file of its own (in parallel, rebuilt only when it or a header changed) and the objects are
 linked into the shared library.
 
+The marshalling of one call is native too: ``csrc/py_layer.cpp``, a CPython extension against torch's headers
+(``paper_2605_21325_b200/_native.so``, ``build_native``).
+
 ``build(debug=True)`` makes a second library, ``libtri_inv_debug.so``, from the same sources with
 ``-DTRI_INV_DEBUG``: every shared-memory offset and global store of the kernels is bounds-checked and
 mbarrier parities are tracked; a violation raises the device status word (never a trap).
@@ -21,6 +24,7 @@ PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 LIB = os.path.join(PKG, "libtri_inv.so")
 LIB_DEBUG = os.path.join(PKG, "libtri_inv_debug.so")
+NATIVE = os.path.join(PKG, "_native.so")
 LIB_DEV = os.path.join(PKG, "libtri_inv_dev.so")   # development build with phase clocks (-DTRI_INV_PHASE_CLOCKS)
 
 
@@ -81,5 +85,23 @@ def build(force: bool = False, verbose: bool = False, debug: bool = False, dev: 
     return lib
 
 
+def build_native(force: bool = False) -> str:
+    """The CPython extension (host code only).  It binds to the C ABI library at run time, by address."""
+    src = os.path.join(PKG, "csrc", "py_layer.cpp")
+    if not force and not _newer([src] + headers(), NATIVE):
+        return NATIVE
+    import sysconfig
+
+    import torch
+    root = os.path.dirname(torch.__file__)
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-D_GLIBCXX_USE_CXX11_ABI=%d" % int(torch._C._GLIBCXX_USE_CXX11_ABI),
+           "-I", os.path.join(ROOT, "include"), "-I", os.path.join(root, "include"), "-I", os.path.join(root, "include", "torch", "csrc", "api", "include"),
+           "-I", os.path.join(os.environ.get("CUDA_HOME", "/usr/local/cuda"), "include"), "-I", sysconfig.get_paths()["include"],
+           src, "-o", NATIVE, "-L", os.path.join(root, "lib"), "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+    subprocess.check_call(cmd)
+    return NATIVE
+
+
 if __name__ == "__main__":
+    build_native(force="--force" in sys.argv)
     print(build(force="--force" in sys.argv, verbose="-v" in sys.argv, debug="--debug" in sys.argv, dev="--dev" in sys.argv))

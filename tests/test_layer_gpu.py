@@ -398,3 +398,31 @@ def test_fp32_calls_in_a_graph(bnd, scan_only):
         assert bnd.last_device_status() == 0
         for x, r in zip(out, ref):
             assert torch.equal(x, r)
+
+
+@pytest.mark.parametrize("case", ["decode", "decode_fp32", "short", "packed_list", "packed_tuple"])
+def test_native_marshalling_gives_the_python_bodys_bits(bnd, case):
+    """A call with a stream is marshalled in Python, one without in native code; other containers and number types take the Python body."""
+    import importlib
+    assert bnd.load_native() is importlib.import_module("paper_2605_21325_b200._native").gdn_forward
+    cu = [0, 1, 1, 70, 200] if case.startswith("packed") else None
+    B, T, dt, d = {"decode": (3, 1, wl.BF16, 128), "decode_fp32": (3, 2, wl.F32, 64), "short": (2, 130, wl.BF16, 128)}.get(case, (1, 200, wl.BF16, 128))
+    inp = wl.make(case, B, T, 2, d, d, 64, dt, seed=880, cu_seqlens=None if cu is None else np.array(cu, np.int32))
+    dev, Q = bnd.to_device(inp), bnd.kv_to_torch(wl.queries(inp, seed=881))
+    S0 = torch.from_numpy(wl.initial_state(inp, seed=882)).cuda()
+    args = (Q, dev["K"], dev["V"], dev["beta"], dev["g"], 64)
+    cu = tuple(cu) if case == "packed_tuple" else cu
+    for s0 in (None, S0):
+        ref = bnd.gdn_forward(*args, scale=0.5, S0=s0, cu_seqlens=cu, stream=torch.cuda.current_stream())
+        odd = bnd.gdn_forward(*args, scale=np.float32(0.5), S0=s0, cu_seqlens=None if cu is None else np.array(cu, np.int64))
+        out = bnd.gdn_forward(*args, scale=0.5, S0=s0, cu_seqlens=cu)
+        torch.cuda.synchronize()
+        for r, x, y in zip(ref, odd, out):
+            assert x.shape == r.shape and y.shape == r.shape and y.dtype == r.dtype and torch.equal(x, r) and torch.equal(y, r)
+    assert bnd.last_device_status() == 0
+    with pytest.raises(bnd.TriInvError):
+        bnd.gdn_forward(Q, dev["K"], dev["V"], dev["beta"], dev["g"], 48)
+    with pytest.raises(AssertionError):
+        bnd.gdn_forward(Q.cpu(), dev["K"], dev["V"], dev["beta"], dev["g"], 64)
+    with pytest.raises(AssertionError):
+        bnd.gdn_forward(Q, dev["K"].repeat_interleave(2, -1)[..., ::2], dev["V"], dev["beta"], dev["g"], 64)
