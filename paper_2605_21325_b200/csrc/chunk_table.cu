@@ -27,6 +27,8 @@ __global__ void __launch_bounds__(kWarps * 32) chunk_table_kernel(ChunkEntry* ta
   const int last = min((int)(blockIdx.x + 1) * kWarps, b.n_seqs);   // offsets 0 .. last are all that the block reads
   for (int q = threadIdx.x; q <= last; q += kWarps * 32) cu[q] = b.cu[q];
   __syncthreads();
+  let_successor_start();
+  wait_for_predecessor();
   if (s >= b.n_seqs) return;
   int before = 0;
   for (int q = lane; q < s; q += 32) before += (cu[q + 1] - cu[q] + b.C - 1) >> shift;
@@ -47,8 +49,7 @@ cudaError_t launch_chunk_table(ChunkEntry* dev_tab, const tri_inv_desc* d, cudaS
     b.C = d->C;
     for (int q = 0; q <= b.n_seqs; ++q) b.cu[q] = d->cu_seqlens[s0 + q];
     for (int q = 0; q < b.n_seqs; ++q) first_chunk += (b.cu[q + 1] - b.cu[q] + d->C - 1) / d->C;
-    chunk_table_kernel<<<(b.n_seqs + kWarps - 1) / kWarps, kWarps * 32, 0, stream>>>(dev_tab, b);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_early(chunk_table_kernel, dim3((b.n_seqs + kWarps - 1) / kWarps), kWarps * 32, 0, stream, dev_tab, b);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

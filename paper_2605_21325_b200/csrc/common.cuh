@@ -174,6 +174,28 @@ inline cudaError_t launched() {
   return e;
 }
 
+// Programmatic dependent launch.  A kernel launched by launch_early() may start while its predecessor in the stream drains: its blocks are put on
+// the SMs, and run up to wait_for_predecessor(), which returns when the predecessor has completed and its writes are visible.
+// So every block of such a kernel waits there before it reads or writes global memory (or draws from a counter), and nothing else about the order of kernels changes.
+// The predecessor says when: let_successor_start() in every block (or its exit).  The kernels do so with their last matrix or chunks: earlier,
+// and blocks that only wait would keep other streams' work off the SMs.  A kernel that runs in one short wave does so at once.  What it saves is the launch and
+// the blocks' start, 1.5 to 3 us a kernel; calls in a row, us: layer on 8 x 1 tokens x 16 heads 7.2 -> 4.9, 333 tokens 20.6 -> 18.0, 4 x 4096 123.6 -> 119.3, fp32
+// 2 x 2048 x 8 heads 104.4 -> 100.5, build of 8 fp32 matrices 8.7 -> 7.3, fused_raw on 4 x 4096 74.5 -> 71.4, fused 64.5 -> 63.9.  The general CUDA-core kernels do not use it.
+__device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_successor_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <class... P, class... A>
+cudaError_t launch_early(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, const A&... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid; cfg.blockDim = dim3((unsigned)threads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+  cfg.attrs = &attr; cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+  if (e != cudaSuccess) (void)cudaGetLastError();   // it is returned here
+  return e;
+}
+
 // Address of the device status word (0 = ok) of the current device; nullptr and *err on failure.
 int* status_word_for_current_device(cudaError_t* err);
 

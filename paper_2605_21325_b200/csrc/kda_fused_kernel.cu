@@ -88,19 +88,23 @@ __global__ void __launch_bounds__(NT, CTAS_PER_SM) kda_fused_kernel(const __grid
 
   float beta_next = 0.f;
   {
-    int tok0 = 0, rows = 0, h = 0;
-    const bool any = (int)blockIdx.x < total && !misaligned;
-    if (any) locate(p, C, blockIdx.x, tok0, rows, h);
-    if (tid == kTidK) { prefetch_tmap(&tmK); mbar_init(bar_k, 1); fence_mbar_init(); if (any) issue_k(tok0, h); }
-    if (tid == kTidG) { prefetch_tmap(&tmG); mbar_init(bar_g, 1); fence_mbar_init(); if (any) issue_g(tok0, h); }
+    if (tid == kTidK) { prefetch_tmap(&tmK); mbar_init(bar_k, 1); fence_mbar_init(); }
+    if (tid == kTidG) { prefetch_tmap(&tmG); mbar_init(bar_g, 1); fence_mbar_init(); }
     if (tid == kTidV) { prefetch_tmap(&tmV); mbar_init(bar_v, 1); fence_mbar_init(); }
     if (tid == 0) { mbar_init(bar_mma, 1); mbar_init(bar_exit, 1); fence_mbar_init(); *s_gave_up = 0; }
     if (tid == 1) { prefetch_tmap(&tmW); prefetch_tmap(&tmU); }
+    if (warp == 0) {
+      __syncwarp();
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(TMEM_COLS) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    wait_for_predecessor();
+    int tok0 = 0, rows = 0, h = 0;
+    const bool any = (int)blockIdx.x < total && !misaligned;
+    if (any) locate(p, C, blockIdx.x, tok0, rows, h);
+    if (tid == kTidK && any) issue_k(tok0, h);
+    if (tid == kTidG && any) issue_g(tok0, h);
     if (any) beta_next = fetch_beta(tok0, rows, h);
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(TMEM_COLS) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
@@ -123,6 +127,7 @@ __global__ void __launch_bounds__(NT, CTAS_PER_SM) kda_fused_kernel(const __grid
     PHASE_BEGIN();
     const int nx_item = item + gridDim.x;
     const bool has_next = nx_item < total;
+    if (!has_next && tid == 0) let_successor_start();
     int nx_tok0 = 0, nx_rows = 0, nx_h = 0;
     if (has_next) locate(p, C, nx_item, nx_tok0, nx_rows, nx_h);
     if (tid < C) sBeta[tid] = beta_next;
@@ -419,8 +424,7 @@ cudaError_t launch_kda_fused_tc(const KParams& p, cudaStream_t stream) {
   if (!q.a_box) tmA = tmK;
   const long long total = (long long)p.n_chunks * p.H, cap = (long long)n_sm * ctas;
   const int grid = (int)(total < cap ? total : cap);
-  kda_fused_kernel<<<grid, NT, SMEM_BYTES, stream>>>(tmK, tmG, tmV, tmW, tmU, tmA, q);
-  return cudaGetLastError();
+  return launch_early(kda_fused_kernel, dim3(grid), NT, SMEM_BYTES, stream, tmK, tmG, tmV, tmW, tmU, tmA, q);
 }
 
 }  // namespace tri_inv

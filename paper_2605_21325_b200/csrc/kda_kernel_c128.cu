@@ -74,20 +74,23 @@ __global__ void __launch_bounds__(NT, 2) kda_build_kernel_c128(const __grid_cons
 
   float beta_next = 0.f;
   {
+    if (tid == 64) { prefetch_tmap(&tmK); mbar_init(bar_k, 1); fence_mbar_init(); }
+    if (tid == 96) {
+      prefetch_tmap(&tmG); mbar_init(bar_g0, 1); mbar_init(bar_g1, 1); fence_mbar_init();
+    }
+    if (tid == 0) { mbar_init(bar_mma, 1); fence_mbar_init(); }
+    if (warp == 0) {
+      __syncwarp();
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(TMEM_COLS) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    wait_for_predecessor();
     int tok0 = 0, rows = 0, h = 0;
     const bool any = (int)blockIdx.x < total && !misaligned;
     if (any) locate(p, C, blockIdx.x, tok0, rows, h);
-    if (tid == 64) { prefetch_tmap(&tmK); mbar_init(bar_k, 1); fence_mbar_init(); if (any) issue_k(tok0, h); }
-    if (tid == 96) {
-      prefetch_tmap(&tmG); mbar_init(bar_g0, 1); mbar_init(bar_g1, 1); fence_mbar_init();
-      if (any) { issue_g(tok0, h, 0); issue_g(tok0, h, 1); }
-    }
-    if (tid == 0) { mbar_init(bar_mma, 1); fence_mbar_init(); }
+    if (tid == 64 && any) issue_k(tok0, h);
+    if (tid == 96 && any) { issue_g(tok0, h, 0); issue_g(tok0, h, 1); }
     if (any) beta_next = fetch_beta(tok0, rows, h);
-  }
-  if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(TMEM_COLS) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
@@ -111,6 +114,7 @@ __global__ void __launch_bounds__(NT, 2) kda_build_kernel_c128(const __grid_cons
     locate(p, C, item, tok0, rows, h);
     const int nx_item = item + gridDim.x;
     const bool has_next = nx_item < total;
+    if (!has_next && tid == 0) let_successor_start();
     int nx_tok0 = 0, nx_rows = 0, nx_h = 0;
     if (has_next) locate(p, C, nx_item, nx_tok0, nx_rows, nx_h);
     if (tid < C) sBeta[tid] = beta_next;
@@ -344,9 +348,7 @@ cudaError_t launch_kda_tc_c128(const KParams& p, cudaStream_t stream) {
   const long long cap = 2LL * n_sm;   // two CTAs per SM
   int grid = (int)(total < cap ? total : cap);
   if (grid == 0) return cudaSuccess;
-  if (p.W) kda_build_kernel_c128<true><<<grid, NT, SMEM_BYTES, stream>>>(tmK, tmG, tmA, q);
-  else kda_build_kernel_c128<false><<<grid, NT, SMEM_BYTES, stream>>>(tmK, tmG, tmA, q);
-  return cudaGetLastError();
+  return launch_early(p.W ? kda_build_kernel_c128<true> : kda_build_kernel_c128<false>, dim3(grid), NT, SMEM_BYTES, stream, tmK, tmG, tmA, q);
 }
 
 }  // namespace tri_inv

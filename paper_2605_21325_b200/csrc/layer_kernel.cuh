@@ -383,6 +383,7 @@ layer_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CU
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_word + 1)), "r"(512) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  wait_for_predecessor();
   if (threadIdx.x == 32) {
     s_word[2] = atomicAdd(p.counters + 1, 1);   // the first group's first matrix: with few of them, one per CTA
     *s_word = atomicAdd(p.counters, 1);
@@ -524,6 +525,7 @@ kda_scan_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(s_word + 1)), "r"(512) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  wait_for_predecessor();
   if (threadIdx.x == 32) *s_word = atomicAdd(p.counters, 1);
   tc_fence_before();
   __syncthreads();
@@ -561,6 +563,8 @@ struct PrepArgs {
   int32_t cu[kMostSeqs + 1];
 };
 __global__ void __launch_bounds__(256) layer_prep_kernel(const __grid_constant__ PrepArgs a) {
+  let_successor_start();
+  wait_for_predecessor();
   for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < a.n_words; i += (long long)gridDim.x * blockDim.x) a.words[i] = 0u;
   auto chunks = [&](int s) { return (a.cu[s + 1] - a.cu[s] + C - 1) / C; };
   __shared__ int part[8];
@@ -709,8 +713,7 @@ cudaError_t launch_prep(const tri_inv_desc* d, const Layout& l, char* ws, int sm
     for (int q = 0; q <= a.n; ++q) a.cu[q] = d->cu_seqlens[q];
     blocks = std::max(blocks, std::min(a.n, sms));
   }
-  layer_prep_kernel<<<blocks, 256, 0, stream>>>(a);
-  return cudaGetLastError();
+  return launch_early(layer_prep_kernel, dim3(blocks), 256, 0, stream, a);
 }
 
 template <int DVS>
@@ -728,8 +731,8 @@ cudaError_t launch_width(const CUtensorMap (&tm)[7], const LayerParams& p, const
   }
   CUtensorMap tmO;
   if (!make_tmap_out<DVS>(&tmO, sp.O, tokens, p.H)) return cudaErrorUnknown;
-  layer_kernel<DVS><<<grid, kLayerThreads, LayerCfg<DVS>::SMEM, stream>>>(tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], tm[6], tmO, p, sp);
-  return launched();
+  const cudaError_t e = launch_early(layer_kernel<DVS>, dim3(grid), kLayerThreads, LayerCfg<DVS>::SMEM, stream, tm[0], tm[1], tm[2], tm[3], tm[4], tm[5], tm[6], tmO, p, sp);
+  return e == cudaSuccess ? launched() : e;
 }
 
 }  // namespace
@@ -803,8 +806,8 @@ cudaError_t launch_kda_width(const CUtensorMap (&tm)[4], const LayerParams& p, c
   }
   CUtensorMap tmO;
   if (!make_tmap_out<DVS>(&tmO, sp.O, tokens, p.H)) return cudaErrorUnknown;
-  kda_scan_kernel<DVS><<<grid, kKdaThreads, KdaScanCfg<DVS>::SMEM, stream>>>(tm[0], tm[1], tm[2], tm[3], tmO, p, a, sp);
-  return launched();
+  const cudaError_t e = launch_early(kda_scan_kernel<DVS>, dim3(grid), kKdaThreads, KdaScanCfg<DVS>::SMEM, stream, tm[0], tm[1], tm[2], tm[3], tmO, p, a, sp);
+  return e == cudaSuccess ? launched() : e;
 }
 }  // namespace
 

@@ -58,6 +58,8 @@ __global__ void __launch_bounds__(kWarps * 32) recurrence_kernel(const __grid_co
   const int col = slice * kCols + lane;
   const bool in = col < a.d_v;
   const size_t base = ((size_t)s * a.H + h) * a.d_k * a.d_v + col;
+  let_successor_start();
+  wait_for_predecessor();
   float S[KR];
 #pragma unroll
   for (int r = 0; r < KR; ++r) {
@@ -157,17 +159,16 @@ cudaError_t launch_recurrence(const void* Q, const void* K, const void* V, const
   if (most < 1) return cudaErrorInvalidValue;
   for (long long s0 = 0; s0 < scan.n_seqs; s0 += most) {
     const int n = (int)std::min<long long>(most, scan.n_seqs - s0), grid = (int)(n * per_seq);
+    cudaError_t e;
     a.first = (int)s0;
     if (packed) {
       for (int q = 0; q <= n; ++q) a.cu[q] = d->cu_seqlens[s0 + q];
-      if (d->d_k <= 64) recurrence_kernel<8, PackedArgs><<<grid, kWarps * 32, 0, stream>>>(a);
-      else recurrence_kernel<16, PackedArgs><<<grid, kWarps * 32, 0, stream>>>(a);
+      e = launch_early(d->d_k <= 64 ? recurrence_kernel<8, PackedArgs> : recurrence_kernel<16, PackedArgs>, dim3(grid), kWarps * 32, 0, stream, a);
     } else {
-      if (d->d_k <= 64) recurrence_kernel<8, RecurrenceArgs><<<grid, kWarps * 32, 0, stream>>>(a);
-      else recurrence_kernel<16, RecurrenceArgs><<<grid, kWarps * 32, 0, stream>>>(a);
+      e = launch_early(d->d_k <= 64 ? recurrence_kernel<8, RecurrenceArgs> : recurrence_kernel<16, RecurrenceArgs>, dim3(grid), kWarps * 32, 0, stream,
+                       static_cast<const RecurrenceArgs&>(a));
     }
-    const cudaError_t e = launched();
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess || (e = launched()) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }

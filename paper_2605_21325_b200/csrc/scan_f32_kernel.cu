@@ -94,6 +94,7 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) scan_f32_chain(con
   const int tid = threadIdx.x;
   const int n_slices = (a.d_v + NS - 1) / NS;
   const int slice = blockIdx.x % n_slices, pair = blockIdx.x / n_slices, h = pair % p.H, s = pair / p.H;
+  wait_for_predecessor();
   const int beg = p.seq_off ? p.seq_off[s] : s * p.T;
   const int end = p.seq_off ? p.seq_off[s + 1] : (s + 1) * p.T;
   const int n_all = (end - beg + kC - 1) / kC;
@@ -180,6 +181,7 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) scan_f32_chain(con
   put_state(slot);
   for (int c = 0; c < n_chunks; ++c) {
     const int rows = rows_of(c);
+    if (tid == 0 && c == (n_chunks > 3 ? n_chunks - 3 : 0)) let_successor_start();
     const float* Ws = tiles + (c % cfg::kStages) * 2 * cfg::TILE;
     const float* Ks = Ws + cfg::TILE;
     float u[VA];
@@ -277,6 +279,8 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 3 : 1) scan_f32_output(Sc
   const int tid = threadIdx.x;
   const int n_slices = (a.d_v + kNV - 1) / kNV;
   const int slice = blockIdx.x % n_slices, at = blockIdx.x / n_slices, lc = at % a.n_seg, pair = at / a.n_seg, h = pair % p.H, s = pair / p.H;
+  let_successor_start();
+  wait_for_predecessor();
   const int beg = p.seq_off ? p.seq_off[s] : s * p.T;
   const int end = p.seq_off ? p.seq_off[s + 1] : (s + 1) * p.T;
   const int tok0 = beg + (a.c0 + lc) * kC;
@@ -399,6 +403,8 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) scan_f32_one_chunk
   const int tid = threadIdx.x;
   const int n_slices = (a.d_v + kNS1 - 1) / kNS1;
   const int slice = blockIdx.x % n_slices, pair = blockIdx.x / n_slices, h = pair % p.H, s = pair / p.H;
+  let_successor_start();
+  wait_for_predecessor();
   const int beg = p.seq_off ? p.seq_off[s] : s * p.T;
   const int rows = (p.seq_off ? p.seq_off[s + 1] : (s + 1) * p.T) - beg;   // 0 .. 64
   const int col0 = slice * kNS1;
@@ -525,8 +531,8 @@ cudaError_t launch_one_chunk(const ScanParams& p, const F32Args& a, cudaStream_t
   if (e != cudaSuccess) return e;
   const long long grid = (long long)p.n_seqs * p.H * ((a.d_v + kNS1 - 1) / kNS1);
   if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-  scan_f32_one_chunk<DK><<<(int)grid, kThreads, OneChunk<DK>::bytes, stream>>>(p, a);
-  return launched();
+  e = launch_early(scan_f32_one_chunk<DK>, dim3((unsigned)grid), kThreads, OneChunk<DK>::bytes, stream, p, a);
+  return e == cudaSuccess ? launched() : e;
 }
 
 template <int DK, int NS>
@@ -535,6 +541,7 @@ cudaError_t launch_chain(const CUtensorMap& tmW, const CUtensorMap& tmK, const S
   if (e != cudaSuccess) return e;
   const long long grid = pairs * ((a.d_v + NS - 1) / NS);
   if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
+  // not early: blocks that start while the factors drain are put two on an SM where there is room (105 -> 125 us for B = 2, T = 2048, H = 8, d = 64)
   scan_f32_chain<DK, NS><<<(int)grid, kThreads, Chain<DK, NS>::bytes, stream>>>(tmW, tmK, p, a);
   return launched();
 }
@@ -569,8 +576,8 @@ cudaError_t launch_segments(const ScanParams& p, F32Args a, int max_chunks, long
     if (e != cudaSuccess) return e;
     const long long grid = pairs * a.n_seg * ((a.d_v + kNV - 1) / kNV);
     if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-    scan_f32_output<DK><<<(int)grid, kThreads, Output<DK>::bytes, stream>>>(p, a);
-    if ((e = launched()) != cudaSuccess) return e;
+    e = launch_early(scan_f32_output<DK>, dim3((unsigned)grid), kThreads, Output<DK>::bytes, stream, p, a);
+    if (e != cudaSuccess || (e = launched()) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }

@@ -29,6 +29,7 @@ struct PrepArgs {
 // blockIdx.x: (sequence, head); blockIdx.y strides over the sequence's chunks.  16 threads per token row (8 features
 // each: 16 bytes of bf16, 32 of fp32), 16 rows per pass, four passes per chunk.
 __global__ void __launch_bounds__(NT) kda_scan_prep_kernel(PrepArgs a) {
+  wait_for_predecessor();   // (its own successor, the scan, starts when it is through: a scan's block takes the SM's L1: 242.9 -> 240.9 us for a layer of 4 x 4096 x 16 heads)
   const int s = blockIdx.x / a.H, h = blockIdx.x % a.H;
   const int beg = a.seq_off ? a.seq_off[s] : s * a.T;
   const int end = a.seq_off ? a.seq_off[s + 1] : (s + 1) * a.T;
@@ -72,8 +73,8 @@ cudaError_t launch_kda_scan_prep(const ScanParams& p, const void* Q, const void*
   const long long want = 4096 / (gx < 4096 ? gx : 4096);
   if (gy > want) gy = want > 0 ? want : 1;
   if (gy > 65535) gy = 65535;
-  kda_scan_prep_kernel<<<dim3((unsigned)gx, (unsigned)gy), NT, 0, stream>>>(a);
-  return launched();
+  const cudaError_t e = launch_early(kda_scan_prep_kernel, dim3((unsigned)gx, (unsigned)gy), NT, 0, stream, a);
+  return e == cudaSuccess ? launched() : e;
 }
 
 }  // namespace tri_inv

@@ -546,6 +546,7 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
       // arrivals of every warp that read them); bar_qr also says that every output warp has seen bar_g of chunk c, which must not
       // run two phases ahead of a warp that still waits for it
       if (!wait(bar_t1b, (uint32_t)(c & 1)) || !wait(bar_qr, (uint32_t)(c & 1))) { failed = true; break; }
+      if (lane == 0 && c == (n_chunks > 5 ? n_chunks - 5 : 0)) let_successor_start();
       fetched(Width<KDA ? 0 : 1>{});
       // The vectors run one chunk further ahead than g: exp(G_ref) of chunk c + 1 is read at the end of chunk c (it
       // scales the S^T operand), so it has to be in place, and announced by an arrival, a chunk earlier.
@@ -895,6 +896,7 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
                   const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUtensorMap tmO, ScanParams p) {
   constexpr int NS = D / DVS;
   extern __shared__ __align__(1024) uint8_t smem[];
+  wait_for_predecessor();
   const int slice = blockIdx.x % NS, h = (blockIdx.x / NS) % p.H, s = blockIdx.x / (NS * p.H);
   scan_walk<DVS, KDA, false>(tmW, tmQ, tmK, tmU, tmO, p, smem, s, h, slice, blockIdx.x == 0, nullptr, 0u);
 }
@@ -905,6 +907,8 @@ struct OffsetBatch {
   int32_t n, first;
 };
 __global__ void __launch_bounds__(256) seq_offsets_kernel(int* out, const __grid_constant__ OffsetBatch b) {
+  let_successor_start();
+  wait_for_predecessor();
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i <= b.n; i += gridDim.x * blockDim.x) out[b.first + i] = b.cu[i];
 }
 
@@ -943,8 +947,8 @@ cudaError_t launch_scan_one(const ScanParams& p, const CUtensorMap& tmW, const C
   if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
   CUtensorMap tmO;
   if (!make_tmap_out<DVS>(&tmO, p.O, tokens, p.H)) return cudaErrorUnknown;
-  chunk_scan_kernel<DVS, KDA><<<(int)grid, kThreadsScan, cfg::SMEM, stream>>>(tmW, tmQ, tmK, tmU, tmO, p);
-  return launched();
+  e = launch_early(chunk_scan_kernel<DVS, KDA>, dim3((unsigned)grid), kThreadsScan, cfg::SMEM, stream, tmW, tmQ, tmK, tmU, tmO, p);
+  return e == cudaSuccess ? launched() : e;
 }
 
 }  // namespace
@@ -956,8 +960,7 @@ cudaError_t launch_seq_offsets(int* dev_out, const tri_inv_desc* d, cudaStream_t
     b.first = s0;
     b.n = d->n_seqs - s0 < kSeqsPerLaunch ? d->n_seqs - s0 : kSeqsPerLaunch;
     for (int q = 0; q <= b.n; ++q) b.cu[q] = d->cu_seqlens[s0 + q];
-    seq_offsets_kernel<<<(b.n + 256) / 256, 256, 0, stream>>>(dev_out, b);
-    cudaError_t e = cudaGetLastError();
+    const cudaError_t e = launch_early(seq_offsets_kernel, dim3((b.n + 256) / 256), 256, 0, stream, dev_out, b);
     if (e != cudaSuccess) return e;
     if (s0 + kSeqsPerLaunch >= d->n_seqs) break;
   }

@@ -221,22 +221,17 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
   const bool misaligned = (sK & 1023u) != 0;  // never expected; the swizzle pattern would not match the copies
   float bg_next = 0.f;
   {
-    int tok0 = 0, rows = 0, h = 0;
-    const bool any = (int)blockIdx.x < total && !misaligned;
-    if (any) locate(p, C, blockIdx.x, tok0, rows, h);
     // the give-up flag is zeroed here; nobody can raise it before the barrier that ends the prologue
     if (tid == kTidK) {
       *s_gave_up = 0;
       prefetch_tmap(&tmK);
       mbar_init(bar_k, 1);
       fence_mbar_init();
-      if (any && !(cfg::ALIAS && load_a)) issue_k(tok0, h);  // with ALIAS, tri_inv_wy fills the matrix first and fetches K later
     }
     if (tid == kTidV) {
       if (need_v) prefetch_tmap(&tmV);
       mbar_init(bar_v, 1);
       fence_mbar_init();
-      if (any && need_v && !cfg::RELOAD) issue_v(tok0, h);  // otherwise V is requested after the inversion
     }
     if (tid == 0) {
       mbar_init(bar_mma, 1);
@@ -244,11 +239,18 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
       mbar_init(bar_exit, 1);
       fence_mbar_init();
     }
+    if (warp_u == 0) {
+      __syncwarp();
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(TMEM_COLS) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    wait_for_predecessor();
+    int tok0 = 0, rows = 0, h = 0;
+    const bool any = (int)blockIdx.x < total && !misaligned;
+    if (any) locate(p, C, blockIdx.x, tok0, rows, h);
+    if (tid == kTidK && any && !(cfg::ALIAS && load_a)) issue_k(tok0, h);  // with ALIAS, tri_inv_wy fills the matrix first and fetches K later
+    if (tid == kTidV && any && need_v && !cfg::RELOAD) issue_v(tok0, h);   // otherwise V is requested after the inversion
     if (any) bg_next = fetch_bg(tok0, rows, h);
-  }
-  if (warp_u == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(TMEM_COLS) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   tc_fence_before();
   __syncthreads();
@@ -315,6 +317,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
       }
     }
     const bool has_next = nx_item < total;
+    if (!has_next && tid == 0) let_successor_start();
     int nx_tok0 = 0, nx_rows = 0, nx_h = 0;   // the next item of this CTA
     if (has_next) locate(p, C, nx_item, nx_tok0, nx_rows, nx_h);
     if (has_next) {
@@ -1291,8 +1294,7 @@ cudaError_t launch_one(const KParams& p_in, cudaStream_t stream) {
   if (const char* gc = getenv("TRI_INV_GRID_CAP")) { int g2 = atoi(gc); if (g2 > 0 && g2 < grid) grid = g2; }
 #endif
   p.work_counter = (p.ops & kFixedStride) ? nullptr : work_counter_for(stream);  // tc_launch.cu
-  tc_kernel<C, D, SER, RAW, BO, REF, H16, VAR><<<grid, cfg::NT, cfg::SMEM, stream>>>(tmK, tmW, tmU, tmV, p);
-  return cudaGetLastError();
+  return launch_early(tc_kernel<C, D, SER, RAW, BO, REF, H16, VAR>, dim3(grid), cfg::NT, cfg::SMEM, stream, tmK, tmW, tmU, tmV, p);
 }
 
 }  // namespace

@@ -183,3 +183,63 @@ def test_per_channel_waits_that_run_out(bnd, C, with_wy):
     for r, o in zip(ref, again):
         assert torch.equal(r.view(torch.int32 if r.dtype == torch.float32 else torch.int16),
                            o.view(torch.int32 if o.dtype == torch.float32 else torch.int16))
+
+
+CHAINS = {  # name: B, T, H, d, dtype, cu_seqlens -- each layer route's kernels, one call's output the next one's input
+    "tokens": (8, 1, 16, 128, wl.BF16, None), "tokens_fp32": (3, 5, 4, 64, wl.F32, None), "one_kernel": (1, 333, 16, 128, wl.BF16, None),
+    "two_calls": (1, 4000, 24, 128, wl.BF16, list(range(0, 4001, 40))), "fp32": (2, 200, 3, 64, wl.F32, None), "fp32_one_chunk": (4, 50, 3, 64, wl.F32, None),
+}
+
+
+@pytest.mark.parametrize("name", list(CHAINS))
+def test_kernels_that_start_early_wait_for_their_predecessor(bnd, name):
+    """Calls in a row, each on the last one's output and state and in buffers that it has just used, give the bits of calls with a synchronisation after each."""
+    B, T, H, d, dt, cu = CHAINS[name]
+    inp = wl.make(name, B, T, H, d, d, 64, dt, seed=900, cu_seqlens=None if cu is None else np.array(cu, np.int32))
+    dev, Q = bnd.to_device(inp), bnd.kv_to_torch(wl.queries(inp, seed=901))
+    A = torch.empty(dev["K"].shape[:3] + (64,), device="cuda")
+
+    def chain(sync):
+        V, S, seen = dev["V"], None, []
+        for step in range(12):
+            V, S = bnd.gdn_forward(Q, dev["K"], V, dev["beta"], dev["g"], 64, scale=2.0, S0=S, cu_seqlens=cu)
+            if sync:
+                torch.cuda.synchronize()
+            bnd.build(V, dev["beta"], dev["g"], 64, cu_seqlens=cu, out=A)   # V as keys: reads what the call before has written, over what the build before has
+            if sync:
+                torch.cuda.synchronize()
+            seen.append(A.sum())
+        torch.cuda.synchronize()
+        return V, S, A.clone(), torch.stack(seen)
+
+    ref = chain(True)
+    for _ in range(3):
+        for x, r in zip(chain(False), ref):
+            assert torch.equal(torch.nan_to_num(x), torch.nan_to_num(r))
+    assert bnd.last_device_status() == 0
+
+
+def test_per_channel_kernels_that_start_early_wait_for_their_predecessor(bnd):
+    inp = wl.make("kda chain", 2, 640, 8, 128, 128, 64, wl.BF16, seed=910)
+    dev, Q, G = bnd.to_device(inp), bnd.kv_to_torch(wl.queries(inp, seed=911)), torch.from_numpy(wl.per_channel_gate(inp, seed=912)).cuda()
+
+    def chain(sync, C):
+        V, S = dev["V"], None
+        for _ in range(8):
+            A, W, U = bnd.fused_kda(dev["K"], V, G, dev["beta"], C)
+            if sync:
+                torch.cuda.synchronize()
+            if C == 64:
+                V, S = bnd.chunk_scan_kda(Q, dev["K"], W, U, G, C, scale=2.0, S0=S)
+            else:
+                V, S = U, W
+            if sync:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        return A, V, S
+
+    for C in (64, 128):
+        ref = chain(True, C)
+        for _ in range(3):
+            assert all(torch.equal(x, r) for x, r in zip(chain(False, C), ref))
+    assert bnd.last_device_status() == 0
