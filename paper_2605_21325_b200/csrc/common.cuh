@@ -177,7 +177,7 @@ inline cudaError_t launched() {
 // Programmatic dependent launch.  A kernel launched by launch_early() may start while its predecessor in the stream drains: its blocks are put on
 // the SMs, and run up to wait_for_predecessor(), which returns when the predecessor has completed and its writes are visible.
 // So every block of such a kernel waits there before it reads or writes global memory (or draws from a counter), and nothing else about the order of kernels changes.
-// The predecessor says when: let_successor_start() in every block (or its exit).  The kernels do so with their last matrix or chunks: earlier,
+// The predecessor says when: let_successor_start() in every block (or its exit).  The factor kernels do so with their last matrix: earlier,
 // and blocks that only wait would keep other streams' work off the SMs.  A kernel that runs in one short wave does so at once.  What it saves is the launch and
 // the blocks' start, 1.5 to 3 us a kernel; calls in a row, us: layer on 8 x 1 tokens x 16 heads 7.2 -> 4.9, 333 tokens 20.6 -> 18.0, 4 x 4096 123.6 -> 119.3, fp32
 // 2 x 2048 x 8 heads 104.4 -> 100.5, build of 8 fp32 matrices 8.7 -> 7.3, fused_raw on 4 x 4096 74.5 -> 71.4, fused 64.5 -> 63.9.  The general CUDA-core kernels do not use it.

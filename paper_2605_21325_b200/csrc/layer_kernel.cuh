@@ -458,10 +458,6 @@ __device__ __forceinline__ void prepare_chunks(const LayerParams& p, const KdaOp
     if (tid == 0 && (nx_item < p.total || (once && *(volatile int*)(p.counters + 3) == 0))) ticket = atomicAdd(p.counters + 1, 1);
     const size_t row0 = ((size_t)at.tok0 * p.H + at.h) * D + f0, stride = (size_t)p.H * D, out0 = ((size_t)at.slot * C * p.H + at.h) * D + f0;
     const DecayRefs refs = load_decay_refs(a.G + row0 + (size_t)(at.rows >> 1) * stride, a.G + row0 + (size_t)(at.rows - 1) * stride);
-    if (r0 == 0) {
-      const size_t v = ((size_t)at.slot * p.H + at.h) * D + f0;
-      store_decay_vectors(a.EL + v, a.ER + v, a.EX + v, refs);
-    }
 #pragma unroll 1
     for (int r4 = r0; r4 < at.rows; r4 += 32) {
       // four rows' loads first, without a branch between them (rows past the chunk: the last one again)
@@ -474,6 +470,10 @@ __device__ __forceinline__ void prepare_chunks(const LayerParams& p, const KdaOp
         kv[m] = *reinterpret_cast<const uint4*>(a.K + idx);
         gv[m][0] = *reinterpret_cast<const float4*>(a.G + idx);
         gv[m][1] = *reinterpret_cast<const float4*>(a.G + idx + 4);
+      }
+      if (r4 == 0) {   // (behind the loads of the first rows)
+        const size_t v = ((size_t)at.slot * p.H + at.h) * D + f0;
+        store_decay_vectors(a.EL + v, a.ER + v, a.EX + v, refs);
       }
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
@@ -503,8 +503,8 @@ __device__ __forceinline__ void prepare_chunks(const LayerParams& p, const KdaOp
   }
 }
 
-// as many threads as the walk has warps, whose 128-column form needs the registers; three groups prepare
-constexpr int kKdaThreads = kThreadsScan, kKdaGroups = 3;
+// as many threads as the walk has warps; every four of them prepare as a group (the fourth: 313 -> 306 us at 32 pairs x 256 chunks)
+constexpr int kKdaThreads = kThreadsScan, kKdaGroups = kKdaThreads / 128;
 template <int DVS>
 struct KdaScanCfg {
   static constexpr int OFF_WORDS = (ScanCfg<DVS, true>::OFF_BAR + 192 + 15) / 16 * 16;

@@ -546,7 +546,6 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
       // arrivals of every warp that read them); bar_qr also says that every output warp has seen bar_g of chunk c, which must not
       // run two phases ahead of a warp that still waits for it
       if (!wait(bar_t1b, (uint32_t)(c & 1)) || !wait(bar_qr, (uint32_t)(c & 1))) { failed = true; break; }
-      if (lane == 0 && c == (n_chunks > 5 ? n_chunks - 5 : 0)) let_successor_start();
       fetched(Width<KDA ? 0 : 1>{});
       // The vectors run one chunk further ahead than g: exp(G_ref) of chunk c + 1 is read at the end of chunk c (it
       // scales the S^T operand), so it has to be in place, and announced by an arrival, a chunk earlier.
@@ -896,7 +895,7 @@ chunk_scan_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant
                   const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmU, const __grid_constant__ CUtensorMap tmO, ScanParams p) {
   constexpr int NS = D / DVS;
   extern __shared__ __align__(1024) uint8_t smem[];
-  wait_for_predecessor();
+  wait_for_predecessor();   // (its successor starts when it is through: with a signal in the gate warp's loop 100 pairs x 64 chunks took 100 us, 95 without)
   const int slice = blockIdx.x % NS, h = (blockIdx.x / NS) % p.H, s = blockIdx.x / (NS * p.H);
   scan_walk<DVS, KDA, false>(tmW, tmQ, tmK, tmU, tmO, p, smem, s, h, slice, blockIdx.x == 0, nullptr, 0u);
 }
