@@ -17,6 +17,8 @@
 // The output kernel is bound by FFMA issue and shared-memory loads (8 per 64 FMAs).
 // Measured (ncu, B = 2, T = 2048, H = 8, d = 64: 16 pairs of 32 chunks): 44 + 27 us (50 + 28 with the chain's tiles by cp.async); 213 us as one kernel per slice of 16 columns that also
 // formed P and O on the way (P again in each slice, all of it on the chain, 64 CTAs).
+#include <algorithm>
+
 #include "f32_tiles.cuh"
 #include "tc_device.cuh"
 
@@ -536,13 +538,20 @@ cudaError_t launch_one_chunk(const ScanParams& p, const F32Args& a, cudaStream_t
 }
 
 template <int DK, int NS>
-cudaError_t launch_chain(const CUtensorMap& tmW, const CUtensorMap& tmK, const ScanParams& p, const F32Args& a, long long pairs, cudaStream_t stream) {
-  cudaError_t e = cudaFuncSetAttribute(scan_f32_chain<DK, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Chain<DK, NS>::bytes);
-  if (e != cudaSuccess) return e;
+cudaError_t launch_chain(const CUtensorMap& tmW, const CUtensorMap& tmK, const ScanParams& p, const F32Args& a, long long pairs, int sms, cudaStream_t stream) {
   const long long grid = pairs * ((a.d_v + NS - 1) / NS);
   if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-  // not early: blocks that start while the factors drain are put two on an SM where there is room (105 -> 125 us for B = 2, T = 2048, H = 8, d = 64)
-  scan_f32_chain<DK, NS><<<(int)grid, kThreads, Chain<DK, NS>::bytes, stream>>>(tmW, tmK, p, a);
+  // With an SM for every block they ask for more than half of an SM's shared memory: blocks that start while the factors drain would else be put two on
+  // an SM where there is room first (B = 2, T = 2048, H = 8, d = 64: 105 -> 125 us).  With more blocks the launch is an ordinary one, for the same reason.
+  const bool one_each = grid <= sms;
+  const size_t bytes = one_each ? std::max(Chain<DK, NS>::bytes, (size_t)118 << 10) : Chain<DK, NS>::bytes;
+  cudaError_t e = cudaFuncSetAttribute(scan_f32_chain<DK, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max(Chain<DK, NS>::bytes, (size_t)118 << 10));
+  if (e != cudaSuccess) return e;
+  if (one_each) {
+    e = launch_early(scan_f32_chain<DK, NS>, dim3((unsigned)grid), kThreads, bytes, stream, tmW, tmK, p, a);
+    return e == cudaSuccess ? launched() : e;
+  }
+  scan_f32_chain<DK, NS><<<(int)grid, kThreads, bytes, stream>>>(tmW, tmK, p, a);
   return launched();
 }
 
@@ -572,7 +581,7 @@ cudaError_t launch_segments(const ScanParams& p, F32Args a, int max_chunks, long
   if ((e = cudaGetDevice(&dev)) != cudaSuccess || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const bool wide = pairs * ((a.d_v + 7) / 8) > 2 * sms;
   for (a.c0 = 0; a.c0 < max_chunks; a.c0 += a.n_seg) {
-    e = wide ? launch_chain<DK, 16>(tmW, tmK, p, a, pairs, stream) : launch_chain<DK, 8>(tmW, tmK, p, a, pairs, stream);
+    e = wide ? launch_chain<DK, 16>(tmW, tmK, p, a, pairs, sms, stream) : launch_chain<DK, 8>(tmW, tmK, p, a, pairs, sms, stream);
     if (e != cudaSuccess) return e;
     const long long grid = pairs * a.n_seg * ((a.d_v + kNV - 1) / kNV);
     if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
