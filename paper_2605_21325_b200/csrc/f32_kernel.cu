@@ -265,12 +265,14 @@ __global__ void __launch_bounds__(kThreads, DT == 64 ? 4 : 2) f32_factors_kernel
 template <int DT, bool WY>
 cudaError_t launch_one(const KParams& p, cudaStream_t stream) {
   const int bytes = F32Cfg<DT>::floats(WY) * (int)sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(f32_factors_kernel<DT, WY>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  cudaError_t e = cudaFuncSetAttribute(f32_factors_kernel<DT, WY>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes > kSpreadMost ? bytes : kSpreadMost);
   if (e != cudaSuccess) return e;
+  int dev = 0, sms = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const long long total = (long long)p.n_chunks * p.H;
   if (total == 0) return cudaSuccess;
   const int grid = (int)(total < (1 << 20) ? total : (1 << 20));
-  return launch_early(f32_factors_kernel<DT, WY>, dim3(grid), kThreads, bytes, stream, p);
+  return launch_early(f32_factors_kernel<DT, WY>, dim3(grid), kThreads, spread_smem(bytes, grid, sms), stream, p);
 }
 
 }  // namespace

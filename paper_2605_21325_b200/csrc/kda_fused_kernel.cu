@@ -399,7 +399,7 @@ cudaError_t launch_kda_fused_tc(const KParams& p, cudaStream_t stream) {
   {
     std::lock_guard<std::mutex> lock(mu);
     if (!n_sm_of[dev]) {
-      if ((e = cudaFuncSetAttribute(kda_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES)) != cudaSuccess) return e;
+      if ((e = cudaFuncSetAttribute(kda_fused_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpreadMost)) != cudaSuccess) return e;
       if ((e = cudaFuncSetAttribute(kda_fused_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared)) != cudaSuccess) return e;
       int sms = 0, smem_per_sm = 0;
       if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
@@ -424,7 +424,7 @@ cudaError_t launch_kda_fused_tc(const KParams& p, cudaStream_t stream) {
   if (!q.a_box) tmA = tmK;
   const long long total = (long long)p.n_chunks * p.H, cap = (long long)n_sm * ctas;
   const int grid = (int)(total < cap ? total : cap);
-  return launch_early(kda_fused_kernel, dim3(grid), NT, SMEM_BYTES, stream, tmK, tmG, tmV, tmW, tmU, tmA, q);
+  return launch_early(kda_fused_kernel, dim3(grid), NT, spread_smem(SMEM_BYTES, grid, n_sm), stream, tmK, tmG, tmV, tmW, tmU, tmA, q);
 }
 
 }  // namespace tri_inv

@@ -291,7 +291,7 @@ cudaError_t launch_kda_tc(const KParams& p, int Cc, cudaStream_t stream, bool* h
   {
     std::lock_guard<std::mutex> lock(mu);
     if (!n_sm_of[dev]) {
-      if ((e = cudaFuncSetAttribute(kda_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES)) != cudaSuccess) return e;
+      if ((e = cudaFuncSetAttribute(kda_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpreadMost)) != cudaSuccess) return e;
       if ((e = cudaFuncSetAttribute(kda_build_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared)) != cudaSuccess) return e;
       int sms = 0, smem_per_sm = 0;
       if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
@@ -313,7 +313,7 @@ cudaError_t launch_kda_tc(const KParams& p, int Cc, cudaStream_t stream, bool* h
   if (!q.a_box) tmA = tmK;
   long long total = (long long)p.n_chunks * p.H, cap = (long long)n_sm * ctas;
   int grid = (int)(total < cap ? total : cap);
-  return launch_early(kda_build_kernel, dim3(grid), NT, SMEM_BYTES, stream, tmK, tmG, tmA, q);
+  return launch_early(kda_build_kernel, dim3(grid), NT, spread_smem(SMEM_BYTES, grid, n_sm), stream, tmK, tmG, tmA, q);
 }
 
 }  // namespace tri_inv

@@ -327,8 +327,8 @@ cudaError_t launch_kda_tc_c128(const KParams& p, cudaStream_t stream) {
   {
     std::lock_guard<std::mutex> lock(mu);
     if (!n_sm_of[dev]) {
-      if ((e = cudaFuncSetAttribute(kda_build_kernel_c128<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES)) != cudaSuccess) return e;
-      if ((e = cudaFuncSetAttribute(kda_build_kernel_c128<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES)) != cudaSuccess) return e;
+      if ((e = cudaFuncSetAttribute(kda_build_kernel_c128<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES > kSpreadMost ? SMEM_BYTES : kSpreadMost)) != cudaSuccess) return e;
+      if ((e = cudaFuncSetAttribute(kda_build_kernel_c128<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES > kSpreadMost ? SMEM_BYTES : kSpreadMost)) != cudaSuccess) return e;
       if ((e = cudaFuncSetAttribute(kda_build_kernel_c128<false>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared)) != cudaSuccess) return e;
       if ((e = cudaFuncSetAttribute(kda_build_kernel_c128<true>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared)) != cudaSuccess) return e;
       int sms = 0;
@@ -348,7 +348,7 @@ cudaError_t launch_kda_tc_c128(const KParams& p, cudaStream_t stream) {
   const long long cap = 2LL * n_sm;   // two CTAs per SM
   int grid = (int)(total < cap ? total : cap);
   if (grid == 0) return cudaSuccess;
-  return launch_early(p.W ? kda_build_kernel_c128<true> : kda_build_kernel_c128<false>, dim3(grid), NT, SMEM_BYTES, stream, tmK, tmG, tmA, q);
+  return launch_early(p.W ? kda_build_kernel_c128<true> : kda_build_kernel_c128<false>, dim3(grid), NT, spread_smem(SMEM_BYTES, grid, n_sm), stream, tmK, tmG, tmA, q);
 }
 
 }  // namespace tri_inv

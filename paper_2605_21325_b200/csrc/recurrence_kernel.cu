@@ -129,6 +129,18 @@ __global__ void __launch_bounds__(kWarps * 32) recurrence_kernel(const __grid_co
   }
 }
 
+// The blocks evenly over the SMs (spread_smem: shared memory that nothing uses; fp32, 11 x 10 tokens x 4 heads, d = 128: 12.7 -> 8.5 us, 10.4 with ordinary launches)
+template <int KR, class Args>
+cudaError_t launch_spread(const Args& a, int grid, int sms, cudaStream_t stream) {
+  constexpr int used = (int)sizeof(TokenRows<KR>) + 3 * kMaxTokens * 4 + 2 * kWarps * kCols * 8;   // the kernel's own
+  const int more = spread_smem(used, grid, sms) - used;
+  if (used + more > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(recurrence_kernel<KR, Args>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpreadMost - used);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_early(recurrence_kernel<KR, Args>, dim3(grid), kWarps * 32, (size_t)more, stream, a);
+}
+
 }  // namespace
 
 // Whether the token-by-token kernel takes the call: every sequence inside one chunk and no longer than kMaxTokens; where the other
@@ -154,6 +166,8 @@ cudaError_t launch_recurrence(const void* Q, const void* K, const void* V, const
   a.H = d->H; a.T = d->T; a.d_k = d->d_k; a.d_v = d->d_v; a.bf16 = d->kv_dtype == TRI_INV_BF16;
   a.scale = scan.scale;
   const bool packed = d->cu_seqlens != nullptr;
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return cudaErrorUnknown;
   const long long per_seq = (long long)d->H * ((d->d_v + kCols - 1) / kCols);
   const long long most = std::min<long long>(packed ? kSeqsPerLaunch : 0x7fffffffLL, 0x7fffffffLL / per_seq);
   if (most < 1) return cudaErrorInvalidValue;
@@ -163,10 +177,9 @@ cudaError_t launch_recurrence(const void* Q, const void* K, const void* V, const
     a.first = (int)s0;
     if (packed) {
       for (int q = 0; q <= n; ++q) a.cu[q] = d->cu_seqlens[s0 + q];
-      e = launch_early(d->d_k <= 64 ? recurrence_kernel<8, PackedArgs> : recurrence_kernel<16, PackedArgs>, dim3(grid), kWarps * 32, 0, stream, a);
+      e = d->d_k <= 64 ? launch_spread<8, PackedArgs>(a, grid, sms, stream) : launch_spread<16, PackedArgs>(a, grid, sms, stream);
     } else {
-      e = launch_early(d->d_k <= 64 ? recurrence_kernel<8, RecurrenceArgs> : recurrence_kernel<16, RecurrenceArgs>, dim3(grid), kWarps * 32, 0, stream,
-                       static_cast<const RecurrenceArgs&>(a));
+      e = d->d_k <= 64 ? launch_spread<8, RecurrenceArgs>(a, grid, sms, stream) : launch_spread<16, RecurrenceArgs>(a, grid, sms, stream);
     }
     if (e != cudaSuccess || (e = launched()) != cudaSuccess) return e;
   }

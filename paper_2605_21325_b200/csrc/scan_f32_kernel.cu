@@ -17,8 +17,6 @@
 // The output kernel is bound by FFMA issue and shared-memory loads (8 per 64 FMAs).
 // Measured (ncu, B = 2, T = 2048, H = 8, d = 64: 16 pairs of 32 chunks): 44 + 27 us (50 + 28 with the chain's tiles by cp.async); 213 us as one kernel per slice of 16 columns that also
 // formed P and O on the way (P again in each slice, all of it on the chain, 64 CTAs).
-#include <algorithm>
-
 #include "f32_tiles.cuh"
 #include "tc_device.cuh"
 
@@ -183,7 +181,6 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) scan_f32_chain(con
   put_state(slot);
   for (int c = 0; c < n_chunks; ++c) {
     const int rows = rows_of(c);
-    if (tid == 0 && c == (n_chunks > 3 ? n_chunks - 3 : 0)) let_successor_start();
     const float* Ws = tiles + (c % cfg::kStages) * 2 * cfg::TILE;
     const float* Ks = Ws + cfg::TILE;
     float u[VA];
@@ -529,30 +526,26 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) scan_f32_one_chunk
 
 template <int DK>
 cudaError_t launch_one_chunk(const ScanParams& p, const F32Args& a, cudaStream_t stream) {
-  cudaError_t e = cudaFuncSetAttribute(scan_f32_one_chunk<DK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)OneChunk<DK>::bytes);
+  constexpr int bytes = (int)OneChunk<DK>::bytes;
+  cudaError_t e = cudaFuncSetAttribute(scan_f32_one_chunk<DK>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes > kSpreadMost ? bytes : kSpreadMost);
   if (e != cudaSuccess) return e;
+  int dev = 0, sms = 0;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const long long grid = (long long)p.n_seqs * p.H * ((a.d_v + kNS1 - 1) / kNS1);
   if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-  e = launch_early(scan_f32_one_chunk<DK>, dim3((unsigned)grid), kThreads, OneChunk<DK>::bytes, stream, p, a);
+  e = launch_early(scan_f32_one_chunk<DK>, dim3((unsigned)grid), kThreads, spread_smem(bytes, grid, sms), stream, p, a);
   return e == cudaSuccess ? launched() : e;
 }
 
 template <int DK, int NS>
 cudaError_t launch_chain(const CUtensorMap& tmW, const CUtensorMap& tmK, const ScanParams& p, const F32Args& a, long long pairs, int sms, cudaStream_t stream) {
+  constexpr int bytes = (int)Chain<DK, NS>::bytes;
+  cudaError_t e = cudaFuncSetAttribute(scan_f32_chain<DK, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes > kSpreadMost ? bytes : kSpreadMost);
+  if (e != cudaSuccess) return e;
   const long long grid = pairs * ((a.d_v + NS - 1) / NS);
   if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-  // With an SM for every block they ask for more than half of an SM's shared memory: blocks that start while the factors drain would else be put two on
-  // an SM where there is room first (B = 2, T = 2048, H = 8, d = 64: 105 -> 125 us).  With more blocks the launch is an ordinary one, for the same reason.
-  const bool one_each = grid <= sms;
-  const size_t bytes = one_each ? std::max(Chain<DK, NS>::bytes, (size_t)118 << 10) : Chain<DK, NS>::bytes;
-  cudaError_t e = cudaFuncSetAttribute(scan_f32_chain<DK, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)std::max(Chain<DK, NS>::bytes, (size_t)118 << 10));
-  if (e != cudaSuccess) return e;
-  if (one_each) {
-    e = launch_early(scan_f32_chain<DK, NS>, dim3((unsigned)grid), kThreads, bytes, stream, tmW, tmK, p, a);
-    return e == cudaSuccess ? launched() : e;
-  }
-  scan_f32_chain<DK, NS><<<(int)grid, kThreads, bytes, stream>>>(tmW, tmK, p, a);
-  return launched();
+  e = launch_early(scan_f32_chain<DK, NS>, dim3((unsigned)grid), kThreads, spread_smem(bytes, grid, sms), stream, tmW, tmK, p, a);
+  return e == cudaSuccess ? launched() : e;
 }
 
 // 3-D view [tokens, H, d] of an fp32 tensor, one box = 32 features (128 bytes, swizzled) of one head x 64 tokens; features past d are
@@ -572,7 +565,8 @@ template <int DK>
 cudaError_t launch_segments(const ScanParams& p, F32Args a, int max_chunks, long long tokens, cudaStream_t stream) {
   CUtensorMap tmW, tmK;
   if (!make_tmap_heads(&tmW, a.W, tokens, p.H, a.d_k) || !make_tmap_heads(&tmK, a.K, tokens, p.H, a.d_k)) return cudaErrorUnknown;
-  cudaError_t e = cudaFuncSetAttribute(scan_f32_output<DK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Output<DK>::bytes);
+  constexpr int out_bytes = (int)Output<DK>::bytes;
+  cudaError_t e = cudaFuncSetAttribute(scan_f32_output<DK>, cudaFuncAttributeMaxDynamicSharedMemorySize, out_bytes > kSpreadMost ? out_bytes : kSpreadMost);
   if (e != cudaSuccess) return e;
   const long long pairs = (long long)p.n_seqs * p.H;
   // eight columns a CTA while that is no more than two CTAs for each SM: half the work on the chain; beyond it the wider slice reads
@@ -585,7 +579,7 @@ cudaError_t launch_segments(const ScanParams& p, F32Args a, int max_chunks, long
     if (e != cudaSuccess) return e;
     const long long grid = pairs * a.n_seg * ((a.d_v + kNV - 1) / kNV);
     if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-    e = launch_early(scan_f32_output<DK>, dim3((unsigned)grid), kThreads, Output<DK>::bytes, stream, p, a);
+    e = launch_early(scan_f32_output<DK>, dim3((unsigned)grid), kThreads, spread_smem(out_bytes, grid, sms), stream, p, a);
     if (e != cudaSuccess || (e = launched()) != cudaSuccess) return e;
   }
   return cudaSuccess;

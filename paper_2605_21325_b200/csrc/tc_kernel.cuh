@@ -1253,7 +1253,7 @@ cudaError_t launch_one(const KParams& p_in, cudaStream_t stream) {
   {
     std::lock_guard<std::mutex> lock(mu);
     if (!ctas_per_sm_of[dev]) {
-      e = cudaFuncSetAttribute(tc_kernel<C, D, SER, RAW, BO, REF, H16, VAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, cfg::SMEM);
+      e = cudaFuncSetAttribute(tc_kernel<C, D, SER, RAW, BO, REF, H16, VAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, cfg::SMEM > kSpreadMost ? cfg::SMEM : kSpreadMost);
       if (e != cudaSuccess) return e;
       e = cudaFuncSetAttribute(tc_kernel<C, D, SER, RAW, BO, REF, H16, VAR>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
       if (e != cudaSuccess) return e;
@@ -1294,7 +1294,7 @@ cudaError_t launch_one(const KParams& p_in, cudaStream_t stream) {
   if (const char* gc = getenv("TRI_INV_GRID_CAP")) { int g2 = atoi(gc); if (g2 > 0 && g2 < grid) grid = g2; }
 #endif
   p.work_counter = (p.ops & kFixedStride) ? nullptr : work_counter_for(stream);  // tc_launch.cu
-  return launch_early(tc_kernel<C, D, SER, RAW, BO, REF, H16, VAR>, dim3(grid), cfg::NT, cfg::SMEM, stream, tmK, tmW, tmU, tmV, p);
+  return launch_early(tc_kernel<C, D, SER, RAW, BO, REF, H16, VAR>, dim3(grid), cfg::NT, spread_smem(cfg::SMEM, grid, n_sm), stream, tmK, tmW, tmU, tmV, p);
 }
 
 }  // namespace
