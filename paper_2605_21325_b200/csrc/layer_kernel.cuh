@@ -618,20 +618,18 @@ Layout layout_of(const tri_inv_desc* d) {
 }
 
 // Which slices and how many CTAs for the scans, and whether this kernel is the better form at all: predicted times in us, from
-// what was measured with each form and width forced (SM clock and power as they come, inputs in turn; pairs x chunks: two launches / here,
-// width and scan CTAs):
-//   16 x 64: 92 / 86 (32, 64)    32 x 64: 112 / 96 (64, 64)    48 x 64: 127 / 130 (128, 48)   64 x 64: 140 / 130 (128, 64)
-//   75 x 64: 193 / 149 (128, 75)   100 x 64: 223 / 234 (128, 32)   148 x 64: 272 / 287 (128, 32)   8 x 512: 558 / 515 (32, 32)
-//   32 x 512: 762 / 589 (64, 64)   1024 x up to 32 chunks: 502 / 525   1024 x 1: 70 / 88   32 x 6: 28 / 23   128 x 2: 28 / 23
-// (the predictions agree with the faster form in all of these but 128 x 2, which they leave to two launches)
-// A scan here takes 1.8, 1.13 or 0.98 us a chunk in slices of 128, 64 or 32 columns (1.49, 1.06, 0.97 with the chip to itself), an SM
+// what was measured with each form and width forced (back to back; pairs x chunks: two calls / here in slices of 32, 64, 128 columns):
+//   16 x 64: 89 / 79, 83, 108    32 x 64: 103 / -, 87, 109    48 x 64: 119 / -, 130, 112   64 x 64: 139 / -, -, 122   75 x 64: 162 / -, -, 157
+//   100 x 64: 184 / -, -, 277    8 x 512: 577 / 476, 508, 697   32 x 512: 753 / -, 538, 712    32 x 6: 20 / -, 21, 24
+//   (before the scan's half products: 1024 x up to 32 chunks: 502 / 525; since: 474 / 503 .. 657 with 48 .. 96 SMs that scan)
+// A scan here takes 1.53, 1.02 or 0.9 us a chunk in slices of 128, 64 or 32 columns (1.3, 0.98, 0.93 with the chip to itself), an SM
 // builds half a matrix per us.  More tasks than scan CTAs never paid, but for the few matrices of a call that is all latency:
 // both parts are then bound by bytes and power, which side by side save nothing.
 struct Split { int dvs, scans; };   // scans 0: two launches
 Split choose_split(long long pairs, int longest, long long entries, int H, int sms) {
-  const struct { int dvs; float here_us, alone_us; } width[3] = {{128, 1.8f, 1.49f}, {64, 1.13f, 1.06f}, {32, 0.98f, 0.97f}};
+  const struct { int dvs; float start_us, here_us, alone_us; } width[3] = {{128, 19.f, 1.53f, 1.3f}, {64, 15.f, 1.02f, 0.98f}, {32, 15.f, 0.9f, 0.93f}};
   const float items = (float)entries * (float)H;
-  const auto& alone = width[pairs * 8 <= sms ? 2 : pairs * 2 <= sms ? 1 : 0];
+  const auto& alone = width[pairs * 4 <= sms ? 2 : pairs * 2 <= sms ? 1 : 0];
   const float waves = std::max(1.f, std::ceil((float)pairs / (float)sms)), mean = pairs > 0 ? items / (float)pairs : 0.f;
   float best_us = 18.f + items / (0.55f * (float)sms) + std::max((float)longest * alone.alone_us, waves > 1.f ? waves * (4.f + mean * alone.alone_us) : 0.f);
   Split best{0, 0};
@@ -640,7 +638,7 @@ Split choose_split(long long pairs, int longest, long long entries, int H, int s
     const bool few = w.dvs == 128 && items <= (float)(kGroups * sms) && tasks <= sms;
     if (tasks > sms * 3 / 4 && !few) continue;
     const int n = (int)std::min<long long>(tasks, sms * 3 / 4);
-    const float us = std::max(15.f + (float)longest * w.here_us, 12.f + items / (0.5f * (float)(sms - n)));
+    const float us = std::max(w.start_us + (float)longest * w.here_us, 12.f + items / (0.5f * (float)(sms - n)));
     if (us < best_us) { best_us = us; best = Split{w.dvs, n}; }
   }
   return best;
