@@ -34,8 +34,9 @@
  * other, so every stream gets a pair of its own; 64 pairs exist per device.  Launches on a 65th and
  * further streams, and every launch made while its stream is being captured into a CUDA graph, use a
  * fixed work distribution instead: same results, slightly less even load.  Neither case is an error.
- * (Programmatic dependent launch, which lets kernels of one stream overlap, must not be enabled on
- * this library's launches.)
+ * The kernels (but for the general CUDA-core ones) are programmatic dependents of what precedes them in their
+ * stream: their blocks may be placed while it drains, and wait for it to complete before they draw an item or
+ * touch global memory, so kernels of one stream never overlap in what they read and write.
  *
  * Tensor layouts (contiguous, row-major, flat token index t in [0, B*T)):
  *   K     [B, T, H, d_k]   kv_dtype (fp32, or bf16 as 16-bit patterns)

@@ -20,8 +20,8 @@
 //
 // The kernel has every SM, with all of its registers, until the factors are built: a small call on another stream waits that long, which it
 // did not behind the fused kernel and the scan as launches of their own.  A decode step of 8 x 16 pairs put on a second stream right behind 32
-// pairs x 512 chunks ends after 381 us (behind the two calls 182, alone 26), behind 64 x 64 after 95 us (28, 25); 333 tokens of 16 heads after
-// 396 (199, 50) and 108 (115, 50).  The large call itself is the faster one: 613 and 780 us, 158 and 160.
+// pairs x 512 chunks ends after 389 us (behind the two calls 178, alone 25), behind 64 x 64 after 97 us (54, 25); 333 tokens of 16 heads after
+// 415 (214, 51) and 122 (108, 50).  The large call itself is the faster one: 571 and 744 us, 152 and 159.
 //
 // W and U pass through scratch memory of the call; a scan reads a chunk microseconds after it was written, so mostly from L2.
 // Part of scan_kernel.cu, whose scan_walk it calls.
@@ -622,14 +622,14 @@ Layout layout_of(const tri_inv_desc* d) {
 //   16 x 64: 89 / 79, 83, 108    32 x 64: 103 / -, 87, 109    48 x 64: 119 / -, 130, 112   64 x 64: 139 / -, -, 122   75 x 64: 162 / -, -, 157
 //   100 x 64: 184 / -, -, 277    8 x 512: 577 / 476, 508, 697   32 x 512: 753 / -, 538, 712    32 x 6: 20 / -, 21, 24
 //   (before the scan's half products: 1024 x up to 32 chunks: 502 / 525; since: 474 / 503 .. 657 with 48 .. 96 SMs that scan)
-// A scan here takes 1.53, 1.02 or 0.9 us a chunk in slices of 128, 64 or 32 columns (1.3, 0.98, 0.93 with the chip to itself), an SM
+// A scan here takes 1.56, 1.02 or 0.9 us a chunk in slices of 128, 64 or 32 columns (1.3, 0.98, 0.93 with the chip to itself), an SM
 // builds half a matrix per us.  More tasks than scan CTAs never paid, but for the few matrices of a call that is all latency:
 // both parts are then bound by bytes and power, which side by side save nothing.
 struct Split { int dvs, scans; };   // scans 0: two launches
 Split choose_split(long long pairs, int longest, long long entries, int H, int sms) {
-  const struct { int dvs; float start_us, here_us, alone_us; } width[3] = {{128, 19.f, 1.53f, 1.3f}, {64, 15.f, 1.02f, 0.98f}, {32, 15.f, 0.9f, 0.93f}};
+  const struct { int dvs; float start_us, here_us, alone_us; } width[3] = {{128, 18.2f, 1.56f, 1.3f}, {64, 15.f, 1.02f, 0.98f}, {32, 15.f, 0.9f, 0.93f}};
   const float items = (float)entries * (float)H;
-  const auto& alone = width[pairs * 4 <= sms ? 2 : pairs * 2 <= sms ? 1 : 0];
+  const auto& alone = width[pairs * 8 <= sms ? 2 : pairs * 2 <= sms ? 1 : 0];
   const float waves = std::max(1.f, std::ceil((float)pairs / (float)sms)), mean = pairs > 0 ? items / (float)pairs : 0.f;
   float best_us = 18.f + items / (0.55f * (float)sms) + std::max((float)longest * alone.alone_us, waves > 1.f ? waves * (4.f + mean * alone.alone_us) : 0.f);
   Split best{0, 0};
@@ -638,7 +638,8 @@ Split choose_split(long long pairs, int longest, long long entries, int H, int s
     const bool few = w.dvs == 128 && items <= (float)(kGroups * sms) && tasks <= sms;
     if (tasks > sms * 3 / 4 && !few) continue;
     const int n = (int)std::min<long long>(tasks, sms * 3 / 4);
-    const float us = std::max(w.start_us + (float)longest * w.here_us, 12.f + items / (0.5f * (float)(sms - n)));
+    const float start_us = items <= (float)(kGroups * sms) ? 15.f : w.start_us;   // (where every matrix has a group at once)
+    const float us = std::max(start_us + (float)longest * w.here_us, 12.f + items / (0.5f * (float)(sms - n)));
     if (us < best_us) { best_us = us; best = Split{w.dvs, n}; }
   }
   return best;

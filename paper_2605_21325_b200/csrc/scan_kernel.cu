@@ -967,11 +967,13 @@ cudaError_t launch_seq_offsets(int* dev_out, const tri_inv_desc* d, cudaStream_t
 }
 
 // bf16 Q, K, W, U with d_k = d_v = 128 and C = 64.  One CTA per SM walks a (sequence, head) pair or a slice of its value
-// columns.  A pair is cut into four slices of 32 columns, or two of 64, while every slice gets an SM of its own: the steps between the products get shorter
-// with the slice (512 chunks, 24 pairs, back to back: 473 us in slices of 32, 499 in slices of 64, 656 in one; 37 pairs 495, 500, 664).  With more
-// slices than SMs a CTA takes all 128 columns: the
+// columns.  A pair is cut into four slices of 32 columns while that takes half the SMs at most, into two of 64 while every
+// slice gets an SM of its own: the steps between the products get shorter with the slice (512 chunks, 18 pairs, back to back: 473 us in slices of 32, 498 in
+// slices of 64, 651 in one).  The first line keeps clear of the power cap: by itself the scan of 24 or 32 pairs x 512 chunks would be 5 % faster in slices of 32 (473 and
+// 499 us), behind the factors' kernel, which leaves the chip hot, 32 pairs x 512 take 807 us in all so and 762 in slices of 64.  With more
+// slices of 64 than SMs a CTA takes all 128 columns: the
 // products take the same time at any slice width, so each further slice would repeat them in a second wave (64 chunks: 74 pairs
-// 76 us in slices of 64, 90 in one; 75 pairs 133 and 90).  The per-channel form keeps to slices of 64 from 19 pairs on: its narrow slices were not measured there.
+// 76 us in slices of 64, 90 in one; 75 pairs 133 and 90).
 // kda selects the per-channel form: Q, K are then the prepared operands Q+, K- (scan_kda_prep.cu), with p.EL,
 // p.ER, p.EX the per-chunk vectors.
 cudaError_t launch_chunk_scan(const ScanParams& p, const void* Q, const void* K, const void* W, long long tokens,
@@ -983,7 +985,7 @@ cudaError_t launch_chunk_scan(const ScanParams& p, const void* Q, const void* K,
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return cudaErrorUnknown;
   const long long pairs = (long long)p.n_seqs * p.H;
-  if (pairs * (kda ? 8 : 4) <= sms) return kda ? launch_scan_one<32, true>(p, tmW, tmQ, tmK, tmU, tokens, stream) : launch_scan_one<32, false>(p, tmW, tmQ, tmK, tmU, tokens, stream);
+  if (pairs * 8 <= sms) return kda ? launch_scan_one<32, true>(p, tmW, tmQ, tmK, tmU, tokens, stream) : launch_scan_one<32, false>(p, tmW, tmQ, tmK, tmU, tokens, stream);
   if (pairs * 2 <= sms) return kda ? launch_scan_one<64, true>(p, tmW, tmQ, tmK, tmU, tokens, stream) : launch_scan_one<64, false>(p, tmW, tmQ, tmK, tmU, tokens, stream);
   return kda ? launch_scan_one<128, true>(p, tmW, tmQ, tmK, tmU, tokens, stream) : launch_scan_one<128, false>(p, tmW, tmQ, tmK, tmU, tokens, stream);
 }
