@@ -27,7 +27,7 @@
 // U~, 64 features of S (fp32, in registers for the whole sequence).  The halves have barriers of their own: a product's time goes by its columns
 // (N / 2 cycles for 16 of the summed index, whatever M, and about 70 until its commit is seen), so the first half of the warps starts on the next
 // step, and the next product on its first half of the summed index, 64 to 128 cycles before the whole product would be through.
-// The output warps form P and put O one chunk behind into its tile (O = gamma_i Q S + P U~ is joined there, scale in the factors); the store warp sends the
+// The output warps form P and put O one chunk behind into its tile (O = gamma_i Q S + P U~ is joined there and scaled, both in fp32); the store warp sends the
 // tile on by the copy engine.  The control warp issues every product; the gate warp brings g (cp.async, two chunks ahead) and its factors a chunk
 // ahead; the copy warp requests the tile copies two chunks ahead, into
 // three stages of {[W ; Q], K, U}.  Hand-offs are mbarriers: commits from the products, one arrival per warp after its
@@ -103,7 +103,7 @@ struct ScanCfg {
   static constexpr int OFF_P = kStages * STAGE;          // P, bf16 [64 tokens i][64 tokens j], K-major B operand of PU
   static constexpr int OFF_O = OFF_P + 8192;             // O on its way out, bf16: boxes of 64 columns (32: the narrow slice) x 64 tokens, swizzled
   static constexpr int OFF_G = OFF_O + C * DVS * 2;
-  static constexpr int G_BYTES = (KDA ? 12 * D : 19 * C) * 4;   // per-channel: 3 vectors of four chunks; scalar: g and its four factors of three, and g as it comes of four
+  static constexpr int G_BYTES = (KDA ? 12 * D : 16 * C) * 4;   // per-channel: 3 vectors of four chunks; scalar: g and its three factors of three, and g as it comes of four
   static constexpr int OFF_BAR = OFF_G + G_BYTES;
   // The 32-column slice asks for more than it uses.  Its registers and tiles would leave room on the SM for a CTA of the inversion
   // kernels (26.5 KB for the build at d = 64, 34.7 KB at d = 128), which would then sit in tcgen05.alloc with its first matrices
@@ -172,6 +172,15 @@ __device__ __forceinline__ void tmem_st_packed32(const uint32_t (&r)[16], uint32
                  "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(taddr) : "memory");
 }
 
+// Two elements in one instruction, each rounded as by fmaf and by a multiplication
+__device__ __forceinline__ void fma_pair(float& d0, float& d1, float2 a, float b0, float b1) {   // d += a b
+  asm("{\n\t.reg .b64 d, a, b;\n\tmov.b64 d, {%0, %1};\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\tfma.rn.f32x2 d, a, b, d;\n\tmov.b64 {%0, %1}, d;\n\t}"
+      : "+f"(d0), "+f"(d1) : "f"(a.x), "f"(a.y), "f"(b0), "f"(b1));
+}
+__device__ __forceinline__ void mul_pair(float& d0, float& d1, float a) {
+  asm("{\n\t.reg .b64 d, a;\n\tmov.b64 d, {%0, %1};\n\tmov.b64 a, {%2, %2};\n\tmul.rn.f32x2 d, d, a;\n\tmov.b64 {%0, %1}, d;\n\t}" : "+f"(d0), "+f"(d1) : "f"(a));
+}
+
 // A bounded wait whose outcome all lanes of the warp agree on.  A lane that has seen the phase may poll it again: the next phase
 // of every barrier of this kernel waits for something that each of its waiting warps does after its wait.  Not inlined: the
 // first polls are (below), and with the timer's loop in every wait as well the 128-column instance was 2 to 6 % slower (a vote
@@ -205,7 +214,7 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
                                           const uint32_t* ready, uint32_t tmem) {
   using cfg = ScanCfg<DVS, KDA>;
   constexpr int LG = cfg::LG, E = cfg::E;
-  float* sG = reinterpret_cast<float*>(smem + cfg::OFF_G);   // scalar gate: [3][5][64]: g log2e; scale 2^(g_ref(j) - g_j), g_ref(j) = g of the first token of j's block of eight; 2^(g_last - g_j); 2^g_j; scale 2^g_j
+  float* sG = reinterpret_cast<float*>(smem + cfg::OFF_G);   // scalar gate: [3][4][64]: g log2e; 2^(g_ref(j) - g_j), g_ref(j) = g of the first token of j's block of eight; 2^(g_last - g_j); 2^g_j
   float* sEl = sG;                 // per-channel form: exp(G_last) [4][128], exp(G_ref) [4][128], exp(G_last - G_ref) [4][128]
   float* sEr = sG + 4 * D;
   float* sEx = sG + 8 * D;
@@ -297,7 +306,7 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
 #pragma unroll
       for (int q = 0; q < 2; ++q) {
         const int i = lane + 32 * q < rows ? lane + 32 * q : rows - 1;
-        cp_async(sG + (15 + (c & 3)) * C + lane + 32 * q, p.g + (size_t)(tok0 + i) * p.H + h, Width<4>{});
+        cp_async(sG + (12 + (c & 3)) * C + lane + 32 * q, p.g + (size_t)(tok0 + i) * p.H + h, Width<4>{});
       }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
@@ -306,8 +315,8 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
   // g_ref the first token of j's block of eight -- one exponential per (row, block) instead of one per element; the
   // second factor spans at most seven tokens of decay
   auto store_g = [&](int c) {   // behind the wait for the group; a lane reads what it copied itself
-    float* b = sG + (c % 3) * 5 * C;
-    const float gr[2] = {sG[(15 + (c & 3)) * C + lane], sG[(15 + (c & 3)) * C + lane + 32]};
+    float* b = sG + (c % 3) * 4 * C;
+    const float gr[2] = {sG[(12 + (c & 3)) * C + lane], sG[(12 + (c & 3)) * C + lane + 32]};
     const float g_last = __shfl_sync(0xffffffffu, gr[1], 31) * kLog2e;
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
@@ -315,11 +324,9 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
       const float gref = __shfl_sync(0xffffffffu, gl2, lane & ~7);
       const int i = lane + 32 * q;
       b[i] = gl2;
-      b[C + i] = p.scale * ex2_approx(gref - gl2);
+      b[C + i] = ex2_approx(gref - gl2);
       b[2 * C + i] = ex2_approx(g_last - gl2);
-      const float gamma = ex2_approx(gl2);
-      b[3 * C + i] = gamma;
-      b[4 * C + i] = p.scale * gamma;
+      b[3 * C + i] = ex2_approx(gl2);
     }
   };
   // per-channel form: exp(G_last), exp(G_ref) and exp(G_last - G_ref) of a chunk (128 floats each, written by the preparation
@@ -592,7 +599,7 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
     for (int c = 0; c < n_chunks && !misaligned; ++c, ph ^= 1) {
       const int tok0 = beg + c * C;
       const int rows = end - tok0 < C ? end - tok0 : C;
-      const float* fb = sG + (c % 3) * 5 * C;
+      const float* fb = sG + (c % 3) * 4 * C;
       const uint32_t sU = s0 + (c % kStages) * cfg::STAGE + cfg::OFF_UT;
       TL(0);
       if (!wait(bar_full + 8 * (c % kStages), full_parity(c))) { failed = true; break; }   // landed long ago; U is read below
@@ -721,7 +728,7 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
     // sends it on.  Accumulator fragments -> [token][column] by stmatrix.trans.
     auto put_output = [&](int c) -> bool {
       if (c > 0 && !wait(bar_of, (uint32_t)((c - 1) & 1))) return false;   // the last chunk's store has read the tile
-      const float* gam = sG + (c % 3) * 5 * C + 4 * C + 2 * t;
+      const float* gam = sG + (c % 3) * 4 * C + 3 * C + 2 * t;
       constexpr int NC = 4;   // blocks of eight tokens at a time: what the registers of 128 columns allow, and faster for 64 (32768 tokens, 32 heads: 571 -> 545 us)
 #pragma unroll
       for (int lg = 0; lg < LG; ++lg) {
@@ -741,17 +748,14 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
 #pragma unroll
             for (int nt = 0; nt < NC; ++nt)
 #pragma unroll
-              for (int e = 0; e < E; ++e) {
-                pu[nt][2 * e] = fmaf(y[nt].x, qs[nt][2 * e], pu[nt][2 * e]);
-                pu[nt][2 * e + 1] = fmaf(y[nt].y, qs[nt][2 * e + 1], pu[nt][2 * e + 1]);
-              }
+              for (int e = 0; e < E; ++e) fma_pair(pu[nt][2 * e], pu[nt][2 * e + 1], y[nt], qs[nt][2 * e], qs[nt][2 * e + 1]);
           }
-          if constexpr (KDA) {   // (scalar gate: the scale is in the factors)
+          // The scale last, on the fp32 sum, and not in P's and gamma's factors: P is rounded to bf16, elsewhere with a scale in it (3.2e-3 of O).  In pairs it takes the
+          // instructions that the join alone took (32768 tokens, 32 heads: 608 us, 608 with the scale in the factors, 614 one by one).
 #pragma unroll
-            for (int nt = 0; nt < NC; ++nt)
+          for (int nt = 0; nt < NC; ++nt)
 #pragma unroll
-              for (int q = 0; q < 2 * E; ++q) pu[nt][q] *= p.scale;
-          }
+            for (int e = 0; e < E; ++e) mul_pair(pu[nt][2 * e], pu[nt][2 * e + 1], p.scale);
           if constexpr (E == 2) {
 #pragma unroll
             for (int nt = 0; nt < NC; nt += 2)
@@ -822,8 +826,8 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
         // (per-channel form: waited for as well, so that bar_qr does not run two phases ahead of the gate warp)
         if (!wait(bar_g, ph)) { failed = true; break; }
         if constexpr (!KDA) {
-          if (narrow) form_factors(Width<4>{}, sG + (c % 3) * 5 * C);
-          else form_factors(Width<8>{}, sG + (c % 3) * 5 * C);
+          if (narrow) form_factors(Width<4>{}, sG + (c % 3) * 4 * C);
+          else form_factors(Width<8>{}, sG + (c % 3) * 4 * C);
         }
       }
       if (c > 0) {   // PU of the chunk before has completed: its O can be read, and P's tile is free

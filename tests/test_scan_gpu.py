@@ -520,3 +520,22 @@ def test_chunk_scan_repeats_bit_for_bit(bnd, n_seqs, H):
             assert max_ratio(bnd.to_numpy_f64(O), O_ref) <= TOL_SCAN and max_ratio(bnd.to_numpy_f64(S), S_ref) <= TOL_SCAN
         else:
             assert torch.equal(O.view(torch.int16), first[0].view(torch.int16)) and torch.equal(S, first[1])
+
+
+@pytest.mark.parametrize("n_seqs,H", [(2, 2), (3, 11), (26, 3)], ids=["32_columns", "64_columns", "128_columns"])
+@pytest.mark.parametrize("scale", [128 ** -0.5, 0.3, 768.0])
+def test_chunk_scan_scale_is_applied_to_the_unrounded_sum(bnd, scale, n_seqs, H):
+    """O is the bf16 rounding of scale times an fp32 sum that does not depend on the scale: each element lies within its own rounding and that of
+    the call with scale 1 (half a unit in the last place: 2^-8 of the value at most; 2^-20 for the fp32 multiplication) of scale times the latter.  A scale that
+    entered before P is rounded to bf16 would move elements in which large terms cancel further than that."""
+    cu = np.concatenate([[0], np.cumsum([150 + 7 * i for i in range(n_seqs)])]).astype(np.int32)
+    inp = wl.make("scale", 1, int(cu[-1]), H, 128, 128, 64, wl.BF16, seed=370 + H, cu_seqlens=cu)
+    dev, Q = bnd.to_device(inp), bnd.kv_to_torch(wl.queries(inp, seed=371))
+    S0 = torch.from_numpy(wl.initial_state(inp, seed=372)).cuda()
+    _, W, U = bnd.fused(dev["K"], dev["V"], dev["beta"], dev["g"], 64, method=bnd.W_DECAY, cu_seqlens=cu, want_A=False)
+    one, S1 = bnd.chunk_scan(Q, dev["K"], W, U, dev["g"], 64, scale=1.0, S0=S0, cu_seqlens=cu)
+    out, S = bnd.chunk_scan(Q, dev["K"], W, U, dev["g"], 64, scale=scale, S0=S0, cu_seqlens=cu)
+    torch.cuda.synchronize()
+    assert bnd.last_device_status() == 0 and torch.equal(S, S1)
+    a, b = out.double(), one.double() * float(np.float32(scale))
+    assert torch.isfinite(a).all() and bool(((a - b).abs() <= (2.0 ** -8 + 2.0 ** -20) * (a.abs() + b.abs())).all())
