@@ -50,8 +50,11 @@ struct KParams {
   int32_t ops;                  // kStoreA | kDoWY | kLoadA | ...
   unsigned long long wait_limit_ns;  // per bounded device-side wait (run() fills in the default of two seconds)
   int32_t a_box;                // build-only tensor-core kernel: 1 when the W tensor-map slot carries the 3-D map of A (whole-matrix store)
+  int32_t signal;               // tensor-core kernel: kSignal*, when a CTA lets the next kernel start; 0: at its exit
   long long n_tokens;           // flat tokens of the tensors (B * T, or T when packed): the bound the debug build checks rows against
 };
+
+constexpr int32_t kSignalLast = 1, kSignalInverted = 2;   // KParams::signal: with its last matrix; when its (only) matrix is inverted
 
 // Bounds-checking build (-DTRI_INV_DEBUG, libtri_inv_debug.so): TRI_INV_CHECK(p, cond) raises TRI_INV_ERR_DEBUG_CHECK in
 // the device status word when cond is false and evaluates to cond, so that the guarded access can be skipped; in the
@@ -177,10 +180,15 @@ inline cudaError_t launched() {
 // Programmatic dependent launch.  A kernel launched by launch_early() may start while its predecessor in the stream drains: its blocks are put on
 // the SMs, and run up to wait_for_predecessor(), which returns when the predecessor has completed and its writes are visible.
 // So every block of such a kernel waits there before it reads or writes global memory (or draws from a counter), and nothing else about the order of kernels changes.
-// The predecessor says when: let_successor_start() in every block (or its exit).  The factor kernels do so with their last matrix: earlier,
-// and blocks that only wait would keep other streams' work off the SMs.  A kernel that runs in one short wave does so at once.  What it saves is the launch and
-// the blocks' start, 1.5 to 3 us a kernel; calls in a row, us: layer on 8 x 1 tokens x 16 heads 7.2 -> 4.9, 333 tokens 20.6 -> 18.0, 4 x 4096 123.6 -> 119.3, fp32
-// 2 x 2048 x 8 heads 104.4 -> 100.5, build of 8 fp32 matrices 8.7 -> 7.3, fused_raw on 4 x 4096 74.5 -> 71.4, fused 64.5 -> 63.9.  The general CUDA-core kernels do not use it.
+// The predecessor says when: let_successor_start() in every block, or the block's exit.  The rule: where the block has little left to do, so that the successor's
+// blocks are placed on a chip that empties, evenly, and blocks that only wait take no room from other streams for long.  Factor kernels of one matrix a block signal when it is
+// inverted; the other large kernels and the fp32 ones leave it to the exit.  Signals at the start of a kernel that does not fill the chip
+// are worse both ways: blocks pile up on the SMs that the predecessor left idle (fp32 builds of 128 matrices in a row 7.3 -> 15.1 us, fp32 layers of 2 x 2048 x 8 heads 98 -> 123), and the piles
+// can be kept flat only by shared memory that nothing uses, which shuts other streams out: a build of 148 matrices on each of two streams took 10.0 us a pair so, 6.0 now (7.3 with ordinary launches;
+// on one stream 5.4, 5.3 and 6.2), fused calls of 148 13.1 and 10.2 (9.5), decode steps of 4 x 8 heads 4.5 and 3.6 (4.4), fp32 layers of 2 x 512 x 4 heads 38.7 and 31.9 (33.9).
+// The tables and the layer's preparation, a few blocks each, signal at once.  What it saves is the launch and
+// the blocks' start, 0.5 to 3 us a kernel; calls in a row, us, ordinary -> this: layer on 8 x 1 tokens x 16 heads 5.6 -> 4.7 (in a graph), 333 tokens 20.5 -> 17.9, fp32
+// 2 x 2048 x 8 heads 104.7 -> 99.7, build of 8 fp32 matrices 7.5 -> 6.9.  The general CUDA-core kernels do not use it.
 __device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void let_successor_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <class... P, class... A>
@@ -194,17 +202,6 @@ cudaError_t launch_early(void (*kernel)(P...), dim3 grid, int threads, size_t sm
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
   if (e != cudaSuccess) (void)cudaGetLastError();   // it is returned here
   return e;
-}
-
-// Shared memory for a block of a launch that has fewer blocks than the chip takes: so much that no SM takes more than its share of them.  Blocks that start
-// while the predecessor drains would else be put where there is room first, several on one SM beside idle ones (fp32 layer on 9 x 35 tokens x 4 heads,
-// d = 64: 22.6 us with ordinary launches, 28.0 early without this; B = 2, T = 2048, H = 8: the 128 blocks of the chain 105 and 125).
-constexpr int kSmemPerSm = 228 * 1024, kSpreadMost = kSmemPerSm / 2 - 768;   // what it returns at most, or `bytes`: 1 KiB a block is the system's
-inline int spread_smem(int bytes, long long blocks, int sms) {
-  const long long share = sms > 0 ? (blocks + sms - 1) / sms : 1, fit = kSmemPerSm / (bytes + 1024);
-  if (share < 1 || share >= fit) return bytes;
-  const int want = kSmemPerSm / (int)(share + 1) - 1024 + 256;   // share + 1 of them are too much, share are not
-  return want > bytes ? want : bytes;
 }
 
 // Address of the device status word (0 = ok) of the current device; nullptr and *err on failure.

@@ -31,7 +31,6 @@ __global__ void __launch_bounds__(kThreads, DT == 64 ? 4 : 2) f32_factors_kernel
   const int ty = (lane >> 2) + 8 * (warp & 1), tx = (lane & 3) + 4 * (warp >> 1);
   const int gshift = (p.method & TRI_INV_GATE_SHIFTED) ? 1 : 0;   // Comba row: row i decays from the token before it
   const int total = p.n_chunks * p.H;
-  let_successor_start();
   wait_for_predecessor();
 
   for (int item = blockIdx.x; item < total; item += gridDim.x) {
@@ -265,14 +264,12 @@ __global__ void __launch_bounds__(kThreads, DT == 64 ? 4 : 2) f32_factors_kernel
 template <int DT, bool WY>
 cudaError_t launch_one(const KParams& p, cudaStream_t stream) {
   const int bytes = F32Cfg<DT>::floats(WY) * (int)sizeof(float);
-  cudaError_t e = cudaFuncSetAttribute(f32_factors_kernel<DT, WY>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes > kSpreadMost ? bytes : kSpreadMost);
+  cudaError_t e = cudaFuncSetAttribute(f32_factors_kernel<DT, WY>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const long long total = (long long)p.n_chunks * p.H;
   if (total == 0) return cudaSuccess;
   const int grid = (int)(total < (1 << 20) ? total : (1 << 20));
-  return launch_early(f32_factors_kernel<DT, WY>, dim3(grid), kThreads, spread_smem(bytes, grid, sms), stream, p);
+  return launch_early(f32_factors_kernel<DT, WY>, dim3(grid), kThreads, bytes, stream, p);
 }
 
 }  // namespace

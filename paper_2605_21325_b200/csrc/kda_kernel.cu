@@ -105,7 +105,6 @@ __global__ void __launch_bounds__(NT, CTAS_PER_SM) kda_build_kernel(const __grid
     locate(p, C, item, tok0, rows, h);
     const int nx_item = item + gridDim.x;
     const bool has_next = nx_item < total;
-    if (!has_next && tid == 0) let_successor_start();
     int nx_tok0 = 0, nx_rows = 0, nx_h = 0;
     if (has_next) locate(p, C, nx_item, nx_tok0, nx_rows, nx_h);
     if (tid < C) sBeta[tid] = beta_next;
@@ -253,6 +252,7 @@ __global__ void __launch_bounds__(NT, CTAS_PER_SM) kda_build_kernel(const __grid
     __syncthreads();   // the fp32 matrix has been read by everyone: the next G tile may land in its space
     if (s_gave_up) break;   // uniform: every thread reads the flag behind the same barrier
     ph ^= 1;
+    if (total <= (int)gridDim.x && tid == 0) let_successor_start();   // with more matrices than CTAs the exit does (as in kda_fused_kernel.cu)
     if (tid == 96 && has_next) issue_g(nx_tok0, nx_h);
   }
   if (bad || misaligned) atomicMax(p.status, TRI_INV_ERR_DEVICE_TIMEOUT);
@@ -291,7 +291,7 @@ cudaError_t launch_kda_tc(const KParams& p, int Cc, cudaStream_t stream, bool* h
   {
     std::lock_guard<std::mutex> lock(mu);
     if (!n_sm_of[dev]) {
-      if ((e = cudaFuncSetAttribute(kda_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSpreadMost)) != cudaSuccess) return e;
+      if ((e = cudaFuncSetAttribute(kda_build_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES)) != cudaSuccess) return e;
       if ((e = cudaFuncSetAttribute(kda_build_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared)) != cudaSuccess) return e;
       int sms = 0, smem_per_sm = 0;
       if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
@@ -313,7 +313,7 @@ cudaError_t launch_kda_tc(const KParams& p, int Cc, cudaStream_t stream, bool* h
   if (!q.a_box) tmA = tmK;
   long long total = (long long)p.n_chunks * p.H, cap = (long long)n_sm * ctas;
   int grid = (int)(total < cap ? total : cap);
-  return launch_early(kda_build_kernel, dim3(grid), NT, spread_smem(SMEM_BYTES, grid, n_sm), stream, tmK, tmG, tmA, q);
+  return launch_early(kda_build_kernel, dim3(grid), NT, SMEM_BYTES, stream, tmK, tmG, tmA, q);
 }
 
 }  // namespace tri_inv

@@ -114,7 +114,6 @@ __global__ void __launch_bounds__(NT, 2) kda_build_kernel_c128(const __grid_cons
     locate(p, C, item, tok0, rows, h);
     const int nx_item = item + gridDim.x;
     const bool has_next = nx_item < total;
-    if (!has_next && tid == 0) let_successor_start();
     int nx_tok0 = 0, nx_rows = 0, nx_h = 0;
     if (has_next) locate(p, C, nx_item, nx_tok0, nx_rows, nx_h);
     if (tid < C) sBeta[tid] = beta_next;
@@ -301,6 +300,7 @@ __global__ void __launch_bounds__(NT, 2) kda_build_kernel_c128(const __grid_cons
     __syncthreads();   // the fp32 matrix has been read by everyone: the next G tile may land in its space
     if (*gave_up) break;   // uniform: every thread reads the flag behind the same barrier
     ph ^= 1;
+    if (total <= (int)gridDim.x && tid == 0) let_successor_start();   // with more matrices than CTAs the exit does (as in kda_fused_kernel.cu)
     if (tid == 96 && has_next) { issue_g(nx_tok0, nx_h, 0); issue_g(nx_tok0, nx_h, 1); }
   }
   if (bad || misaligned) atomicMax(p.status, TRI_INV_ERR_DEVICE_TIMEOUT);
@@ -327,8 +327,8 @@ cudaError_t launch_kda_tc_c128(const KParams& p, cudaStream_t stream) {
   {
     std::lock_guard<std::mutex> lock(mu);
     if (!n_sm_of[dev]) {
-      if ((e = cudaFuncSetAttribute(kda_build_kernel_c128<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES > kSpreadMost ? SMEM_BYTES : kSpreadMost)) != cudaSuccess) return e;
-      if ((e = cudaFuncSetAttribute(kda_build_kernel_c128<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES > kSpreadMost ? SMEM_BYTES : kSpreadMost)) != cudaSuccess) return e;
+      if ((e = cudaFuncSetAttribute(kda_build_kernel_c128<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES)) != cudaSuccess) return e;
+      if ((e = cudaFuncSetAttribute(kda_build_kernel_c128<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES)) != cudaSuccess) return e;
       if ((e = cudaFuncSetAttribute(kda_build_kernel_c128<false>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared)) != cudaSuccess) return e;
       if ((e = cudaFuncSetAttribute(kda_build_kernel_c128<true>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared)) != cudaSuccess) return e;
       int sms = 0;
@@ -348,7 +348,7 @@ cudaError_t launch_kda_tc_c128(const KParams& p, cudaStream_t stream) {
   const long long cap = 2LL * n_sm;   // two CTAs per SM
   int grid = (int)(total < cap ? total : cap);
   if (grid == 0) return cudaSuccess;
-  return launch_early(p.W ? kda_build_kernel_c128<true> : kda_build_kernel_c128<false>, dim3(grid), NT, spread_smem(SMEM_BYTES, grid, n_sm), stream, tmK, tmG, tmA, q);
+  return launch_early(p.W ? kda_build_kernel_c128<true> : kda_build_kernel_c128<false>, dim3(grid), NT, SMEM_BYTES, stream, tmK, tmG, tmA, q);
 }
 
 }  // namespace tri_inv

@@ -20,8 +20,10 @@
 //
 // The kernel has every SM, with all of its registers, until the factors are built: a small call on another stream waits that long, which it
 // did not behind the fused kernel and the scan as launches of their own.  A decode step of 8 x 16 pairs put on a second stream right behind 32
-// pairs x 512 chunks ends after 389 us (behind the two calls 178, alone 25), behind 64 x 64 after 97 us (54, 25); 333 tokens of 16 heads after
-// 415 (214, 51) and 122 (108, 50).  The large call itself is the faster one: 571 and 744 us, 152 and 159.
+// pairs x 512 chunks ends after 384 us (behind the two calls 178, alone 25), behind 64 x 64 after 95 us (27, 25); 333 tokens of 16 heads after
+// 406 (211, 50) and 111 (106, 50).  The large call itself is the faster one: 566 and 766 us, 150 and 149.  (Before the scan's half products 377 (180), 92 (28), 394 (196) and 108 (114): the
+// scans, which are faster now, leave the factors built beside them a smaller share; and a layer kernel whose blocks are placed early takes SMs from the scan that follows the fused call, where it runs with
+// more of its blocks on fewer SMs: 199 instead of 211 if it is launched the ordinary way, which costs the call of 333 tokens by itself 2.5 us of 18.)
 //
 // W and U pass through scratch memory of the call; a scan reads a chunk microseconds after it was written, so mostly from L2.
 // Part of scan_kernel.cu, whose scan_walk it calls.

@@ -278,7 +278,6 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 3 : 1) scan_f32_output(Sc
   const int tid = threadIdx.x;
   const int n_slices = (a.d_v + kNV - 1) / kNV;
   const int slice = blockIdx.x % n_slices, at = blockIdx.x / n_slices, lc = at % a.n_seg, pair = at / a.n_seg, h = pair % p.H, s = pair / p.H;
-  let_successor_start();
   wait_for_predecessor();
   const int beg = p.seq_off ? p.seq_off[s] : s * p.T;
   const int end = p.seq_off ? p.seq_off[s + 1] : (s + 1) * p.T;
@@ -402,7 +401,6 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) scan_f32_one_chunk
   const int tid = threadIdx.x;
   const int n_slices = (a.d_v + kNS1 - 1) / kNS1;
   const int slice = blockIdx.x % n_slices, pair = blockIdx.x / n_slices, h = pair % p.H, s = pair / p.H;
-  let_successor_start();
   wait_for_predecessor();
   const int beg = p.seq_off ? p.seq_off[s] : s * p.T;
   const int rows = (p.seq_off ? p.seq_off[s + 1] : (s + 1) * p.T) - beg;   // 0 .. 64
@@ -527,24 +525,22 @@ __global__ void __launch_bounds__(kThreads, DK == 64 ? 2 : 1) scan_f32_one_chunk
 template <int DK>
 cudaError_t launch_one_chunk(const ScanParams& p, const F32Args& a, cudaStream_t stream) {
   constexpr int bytes = (int)OneChunk<DK>::bytes;
-  cudaError_t e = cudaFuncSetAttribute(scan_f32_one_chunk<DK>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes > kSpreadMost ? bytes : kSpreadMost);
+  cudaError_t e = cudaFuncSetAttribute(scan_f32_one_chunk<DK>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e != cudaSuccess) return e;
-  int dev = 0, sms = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const long long grid = (long long)p.n_seqs * p.H * ((a.d_v + kNS1 - 1) / kNS1);
   if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-  e = launch_early(scan_f32_one_chunk<DK>, dim3((unsigned)grid), kThreads, spread_smem(bytes, grid, sms), stream, p, a);
+  e = launch_early(scan_f32_one_chunk<DK>, dim3((unsigned)grid), kThreads, bytes, stream, p, a);
   return e == cudaSuccess ? launched() : e;
 }
 
 template <int DK, int NS>
-cudaError_t launch_chain(const CUtensorMap& tmW, const CUtensorMap& tmK, const ScanParams& p, const F32Args& a, long long pairs, int sms, cudaStream_t stream) {
+cudaError_t launch_chain(const CUtensorMap& tmW, const CUtensorMap& tmK, const ScanParams& p, const F32Args& a, long long pairs, cudaStream_t stream) {
   constexpr int bytes = (int)Chain<DK, NS>::bytes;
-  cudaError_t e = cudaFuncSetAttribute(scan_f32_chain<DK, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes > kSpreadMost ? bytes : kSpreadMost);
+  cudaError_t e = cudaFuncSetAttribute(scan_f32_chain<DK, NS>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   if (e != cudaSuccess) return e;
   const long long grid = pairs * ((a.d_v + NS - 1) / NS);
   if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-  e = launch_early(scan_f32_chain<DK, NS>, dim3((unsigned)grid), kThreads, spread_smem(bytes, grid, sms), stream, tmW, tmK, p, a);
+  e = launch_early(scan_f32_chain<DK, NS>, dim3((unsigned)grid), kThreads, bytes, stream, tmW, tmK, p, a);
   return e == cudaSuccess ? launched() : e;
 }
 
@@ -566,7 +562,7 @@ cudaError_t launch_segments(const ScanParams& p, F32Args a, int max_chunks, long
   CUtensorMap tmW, tmK;
   if (!make_tmap_heads(&tmW, a.W, tokens, p.H, a.d_k) || !make_tmap_heads(&tmK, a.K, tokens, p.H, a.d_k)) return cudaErrorUnknown;
   constexpr int out_bytes = (int)Output<DK>::bytes;
-  cudaError_t e = cudaFuncSetAttribute(scan_f32_output<DK>, cudaFuncAttributeMaxDynamicSharedMemorySize, out_bytes > kSpreadMost ? out_bytes : kSpreadMost);
+  cudaError_t e = cudaFuncSetAttribute(scan_f32_output<DK>, cudaFuncAttributeMaxDynamicSharedMemorySize, out_bytes);
   if (e != cudaSuccess) return e;
   const long long pairs = (long long)p.n_seqs * p.H;
   // eight columns a CTA while that is no more than two CTAs for each SM: half the work on the chain; beyond it the wider slice reads
@@ -575,11 +571,11 @@ cudaError_t launch_segments(const ScanParams& p, F32Args a, int max_chunks, long
   if ((e = cudaGetDevice(&dev)) != cudaSuccess || (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const bool wide = pairs * ((a.d_v + 7) / 8) > 2 * sms;
   for (a.c0 = 0; a.c0 < max_chunks; a.c0 += a.n_seg) {
-    e = wide ? launch_chain<DK, 16>(tmW, tmK, p, a, pairs, sms, stream) : launch_chain<DK, 8>(tmW, tmK, p, a, pairs, sms, stream);
+    e = wide ? launch_chain<DK, 16>(tmW, tmK, p, a, pairs, stream) : launch_chain<DK, 8>(tmW, tmK, p, a, pairs, stream);
     if (e != cudaSuccess) return e;
     const long long grid = pairs * a.n_seg * ((a.d_v + kNV - 1) / kNV);
     if (grid > 0x7fffffffLL) return cudaErrorInvalidValue;
-    e = launch_early(scan_f32_output<DK>, dim3((unsigned)grid), kThreads, spread_smem(out_bytes, grid, sms), stream, p, a);
+    e = launch_early(scan_f32_output<DK>, dim3((unsigned)grid), kThreads, out_bytes, stream, p, a);
     if (e != cudaSuccess || (e = launched()) != cudaSuccess) return e;
   }
   return cudaSuccess;

@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
       }
     }
     const bool has_next = nx_item < total;
-    if (!has_next && tid == 0) let_successor_start();
+    if (p.signal == kSignalLast && !has_next && tid == 0) let_successor_start();
     int nx_tok0 = 0, nx_rows = 0, nx_h = 0;   // the next item of this CTA
     if (has_next) locate(p, C, nx_item, nx_tok0, nx_rows, nx_h);
     if (has_next) {
@@ -1050,6 +1050,7 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
       }
     }
     // the item after next (read after this item's last barrier): by ticket, or by a fixed stride without a counter pair
+    if (p.signal == kSignalInverted && tid == 0) let_successor_start();
     if (tid == kTidL2) *s_next_item = !has_next ? total : (p.work_counter ? 2 * (int)gridDim.x + ticket : nx_item + (int)gridDim.x);
     PHASE(6);
 
@@ -1253,7 +1254,7 @@ cudaError_t launch_one(const KParams& p_in, cudaStream_t stream) {
   {
     std::lock_guard<std::mutex> lock(mu);
     if (!ctas_per_sm_of[dev]) {
-      e = cudaFuncSetAttribute(tc_kernel<C, D, SER, RAW, BO, REF, H16, VAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, cfg::SMEM > kSpreadMost ? cfg::SMEM : kSpreadMost);
+      e = cudaFuncSetAttribute(tc_kernel<C, D, SER, RAW, BO, REF, H16, VAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, cfg::SMEM);
       if (e != cudaSuccess) return e;
       e = cudaFuncSetAttribute(tc_kernel<C, D, SER, RAW, BO, REF, H16, VAR>, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
       if (e != cudaSuccess) return e;
@@ -1293,8 +1294,12 @@ cudaError_t launch_one(const KParams& p_in, cudaStream_t stream) {
 #ifdef TRI_INV_PHASE_CLOCKS
   if (const char* gc = getenv("TRI_INV_GRID_CAP")) { int g2 = atoi(gc); if (g2 > 0 && g2 < grid) grid = g2; }
 #endif
+  // When CTAs let the next kernel start (launch_early).  One matrix a CTA: when it is inverted.  More of them: at the exit; fused calls of 4096 in a row take 69.5 us so and 70.4 with a signal
+  // at the last matrix, of C = 128, 2048: 105.0 and 106.1, and the scan behind a fused call is then placed on SMs in pairs (32 pairs x 512 chunks, both: 711 and 764).  The build of
+  // 64 x 64 matrices, with six small CTAs an SM, signals with its last ones (1600: 14.8 us, 16.6 at the exit; 16,384 from memory: 133.0 and 132.9).
+  p.signal = total <= cap ? kSignalInverted : BO ? kSignalLast : 0;
   p.work_counter = (p.ops & kFixedStride) ? nullptr : work_counter_for(stream);  // tc_launch.cu
-  return launch_early(tc_kernel<C, D, SER, RAW, BO, REF, H16, VAR>, dim3(grid), cfg::NT, spread_smem(cfg::SMEM, grid, n_sm), stream, tmK, tmW, tmU, tmV, p);
+  return launch_early(tc_kernel<C, D, SER, RAW, BO, REF, H16, VAR>, dim3(grid), cfg::NT, cfg::SMEM, stream, tmK, tmW, tmU, tmV, p);
 }
 
 }  // namespace
