@@ -621,9 +621,10 @@ Layout layout_of(const tri_inv_desc* d) {
 
 // Which slices and how many CTAs for the scans, and whether this kernel is the better form at all: predicted times in us, from
 // what was measured with each form and width forced (back to back; pairs x chunks: two calls / here in slices of 32, 64, 128 columns):
-//   16 x 64: 89 / 79, 83, 108    32 x 64: 103 / -, 87, 109    48 x 64: 119 / -, 130, 112   64 x 64: 139 / -, -, 122   75 x 64: 162 / -, -, 157
-//   100 x 64: 184 / -, -, 277    8 x 512: 577 / 476, 508, 697   32 x 512: 753 / -, 538, 712    32 x 6: 20 / -, 21, 24
+//   16 x 64: 82 / 78, 82, 109    32 x 64: 100 / -, 85, 109    48 x 64: 125 / -, 129, 116    64 x 64: 151 / -, -, 132    75 x 64: 176 / -, -, 167
+//   100 x 64: 213 / -, -, 276    8 x 512: 527 / 478, 505, 704    32 x 512: 728 / -, 592, 718    64 x 256: 583 / -, -, 486    32 x 6: 19.7 / -, 21.0, 24
 //   (before the scan's half products: 1024 x up to 32 chunks: 502 / 525; since: 474 / 503 .. 657 with 48 .. 96 SMs that scan)
+// (Since kernels start early the two calls are also the faster form of short calls that the predictions leave here: 64 x 2 15.8 and 17.2 us, 64 x 16 42 and 46, 48 x 24 51 and 57, 16 x 6 17.2 and 17.8.)
 // A scan here takes 1.56, 1.02 or 0.9 us a chunk in slices of 128, 64 or 32 columns (1.3, 0.98, 0.93 with the chip to itself), an SM
 // builds half a matrix per us.  More tasks than scan CTAs never paid, but for the few matrices of a call that is all latency:
 // both parts are then bound by bytes and power, which side by side save nothing.
@@ -647,22 +648,25 @@ Split choose_split(long long pairs, int longest, long long entries, int H, int s
   return best;
 }
 
-// The same for the per-channel scan.  Two launches / here (width, scan CTAs): 16 x 64: 95 / 91 (32, 64)   32 x 64: 119 / 104 (64, 64)
-//   48 x 64: 138 / 133 (128, 48)   64 x 64: 152 / 162 (128, 64)   75 x 64: 193 / 206 (128, 75)   8 x 128: 161 / 157 (32, 32)
-//   32 x 512: 884 / 651 (64, 64)   16 x 6: 19 / 25
-// (the predictions agree with the faster form in all of these but 48 x 64, which they leave to two launches: 5 us)
-// A group prepares a chunk in about 9 us, three of them an SM (0.33 a us; the preparation by itself keeps eight CTAs an SM in flight
-// and reaches 69 chunks a us on the whole chip), so the gain is where the chain is long.
+// The same for the per-channel scan, each form and width forced, back to back on three sets of inputs; two launches / here in slices of 32, 64, 128 columns:
+//   16 x 32: 40.8 / 48.0, 51, 66    16 x 64: 79 / 81, 87, 116    16 x 96: 115 / 110, 119, 162    8 x 128: 135 / 137, 149, 205    8 x 512: 520 / 488, 532, 752
+//   24 x 64: 93 / 84, 89, 116    32 x 16: 28.6 / -, 35.9, 44    32 x 32: 54 / -, 57, 71    32 x 48: 78 / -, 74, 93    32 x 64: 99 / -, 92, 116    32 x 512: 764 / -, 649, 761
+//   40 x 64: 109 / -, 113, 117    40 x 256: 430 / -, 431, 412    48 x 64: 121 / -, 156, 121    48 x 128: 241 / -, 307, 226    56 x 64: 134 / -, -, 138
+//   56 x 256: 531 / -, -, 508    64 x 64: 148 / -, -, 159    64 x 256: 581 / -, -, 596    75 x 64: 181 / -, -, 199    100 x 128: 433 / -, -, 704    16 x 6: 17.3 / 19.6, 20, 24
+// (of 60 such points the predictions miss the faster form in three, by 1.6 % at most)
+// Two launches: the preparation takes 79 chunks a us, a scan 0.95, 1.07 or 1.8 us a chunk at its own widths (launch_chunk_scan), in slices of 64 columns more with each pair beyond 32: bytes
+// and power.  Here: 0.89, 1.02 or 1.41 us a chunk, and an SM's four groups prepare 0.39 chunks a us (0.36 beside slices of 128), all of them 25.5 (28.5) at most: a group's chunk is a
+// chain of latencies of about 9 us, so the gain is where the scan's chain is long.
 Split choose_kda_split(long long pairs, int longest, long long entries, int H, int sms) {
-  const struct { int dvs; float here_us, alone_us; } width[3] = {{128, 1.95f, 1.9f}, {64, 1.25f, 1.27f}, {32, 1.16f, 1.15f}};
+  const struct { int dvs; float start_us, here_us, per_sm, most; } width[3] = {{128, 27.f, 1.41f, 0.36f, 28.5f}, {64, 23.f, 1.02f, 0.39f, 25.5f}, {32, 20.f, 0.89f, 0.39f, 25.5f}};
   const float items = (float)entries * (float)H;
-  const auto& alone = width[pairs * 8 <= sms ? 2 : pairs * 2 <= sms ? 1 : 0];
-  float best_us = 10.f + items / 69.f + (float)longest * alone.alone_us;   // (only compared where all scans run at the same time)
+  const float alone_us = pairs * 8 <= sms ? 0.95f : pairs * 2 <= sms ? 1.07f + 0.0115f * (float)std::max(0LL, pairs - 32) : 1.8f;
+  float best_us = 3.f + items / 79.f + (float)longest * alone_us;   // (only compared where all scans run at the same time)
   Split best{0, 0};
   for (const auto& w : width) {
     const long long tasks = pairs * (D / w.dvs);
     if (tasks > sms * 3 / 4) continue;
-    const float us = std::max(17.f + (float)longest * w.here_us, 12.f + items / (0.33f * (float)(sms - tasks)));
+    const float us = std::max(w.start_us + (float)longest * w.here_us, 12.f + items / std::min(w.per_sm * (float)(sms - tasks), w.most));
     if (us < best_us) { best_us = us; best = Split{w.dvs, (int)tasks}; }
   }
   return best;

@@ -325,6 +325,29 @@ def test_token_by_token_against_the_recurrence(bnd, name, B, T, H, d_k, d_v, cu,
     assert max_ratio(bnd.to_numpy_f64(S), S_ref) <= 1e-5
 
 
+# (pairs, chunks, launches that compute): points at which the slower form takes 5 to 25 % longer (figures beside choose_kda_split)
+KDA_ROUTES = [(16, 32, 2), (32, 16, 2), (20, 32, 2), (16, 6, 2), (75, 64, 2), (64, 64, 2), (16, 128, 1), (32, 64, 1), (48, 128, 1), (8, 256, 1)]
+
+
+def test_per_channel_scan_takes_the_form_that_was_measured_faster(bnd):
+    x = torch.zeros((1, 64 * 256 * 8, 1, 128), dtype=torch.bfloat16, device="cuda")
+    G = torch.zeros(x.shape, device="cuda")
+    cut = lambda t, P, N: t.reshape(-1)[:64 * N * P * 128].reshape(1, 64 * N, P, 128)   # noqa: E731
+    took = []
+    for P, N, launches in KDA_ROUTES:
+        if 64 * N * P > x.shape[1]:
+            x = torch.zeros((1, 64 * N * P, 1, 128), dtype=torch.bfloat16, device="cuda")
+            G = torch.zeros(x.shape, device="cuda")
+        n0 = bnd.launch_count()
+        t = cut(x, P, N)
+        O, S = bnd.chunk_scan_kda(t, t, t, t, cut(G, P, N), 64)
+        torch.cuda.synchronize()
+        took.append((P, N, bnd.launch_count() - n0))
+        assert not O.any() and not S.any()
+    assert bnd.last_device_status() == 0
+    assert took == KDA_ROUTES
+
+
 def test_smoke_runs():
     """The entry that is run first on a machine, with its counts of launches and its comparisons."""
     import __graft_entry__ as entry
