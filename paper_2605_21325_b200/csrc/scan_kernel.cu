@@ -566,6 +566,7 @@ __device__ __forceinline__ bool scan_walk(const CUtensorMap& tmW, const CUtensor
         fetch_g(c + 3);
       }
     }
+    if (failed) fetched(Width<0>{});   // give-up path: its copies too are through before the CTA gives up its shared memory
   } else if (warp == kCopy) {
     // ---------------------------------------------------------------- copy warp: tile copies of chunk c + 2 (FED: once W and U are there)
     // It arrives on bar_sr itself, after its wait for the phase before: the barrier must not run two phases ahead of it while it

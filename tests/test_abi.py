@@ -166,6 +166,18 @@ def test_a_block_that_gives_up_waits_for_the_last_copy_of_every_stage(name):
                     assert (c % stages, c // stages % 2) in waited, (stages, n_chunks, requested)
 
 
+def test_scan_roles_that_copy_wait_for_their_copies_when_they_give_up():
+    """The scan's roles that issue asynchronous copies and leave their loop where a wait has run out: the last statement of each waits for what it has
+    on its way (the gate warp's cp.async groups, the copy warp's bulk loads), and the store warp waits inside the loop, ahead of its next wait."""
+    src = open(os.path.join(ROOT, "paper_2605_21325_b200", "csrc", "scan_kernel.cu")).read()
+    role = lambda a, b: re.sub(r"//[^\n]*", "", src[src.index("} else if (warp == %s) {" % a):src.index(b)]).strip()   # noqa: E731
+    gate, copy = role("kGate", "} else if (warp == kCopy) {"), role("kCopy", "} else if (chain) {")
+    assert gate.endswith("if (failed) fetched(Width<0>{});") and "fetch_g(" in gate and "fetch_e(" in gate
+    assert copy.endswith("if (failed && lane == 0) drain_copies();") and "issue_copies(" in copy
+    store = role("kStore", "if (failed) atomicMax(p.status")
+    assert store.index("tma_store_2d(") < store.index("bulk_commit();") < store.index("bulk_wait_read();") < store.index("warp_arrive(bar_of, lane);")
+
+
 def test_shared_arrays_that_are_read_as_vectors_are_aligned():
     """A static shared array that is read as float4 has its 16 bytes from its declaration, not from where the compiler happens to
     put it: every __shared__ float array is declared with an alignment, or is in a type that has one, where its file reads
