@@ -191,31 +191,92 @@ CHAINS = {  # name: B, T, H, d, dtype, cu_seqlens -- each layer route's kernels,
 }
 
 
+def same_chains(chain, times=3):
+    """A chain of calls with nothing between them against the same with a synchronisation after each: same bits, all finite."""
+    ref = chain(torch.cuda.synchronize)
+    torch.cuda.synchronize()
+    assert all(torch.isfinite(r).all() for r in ref)
+    for _ in range(times):
+        out = chain(lambda: None)
+        torch.cuda.synchronize()
+        assert len(out) == len(ref) and all(torch.equal(x, r) for x, r in zip(out, ref))
+    return ref
+
+
 @pytest.mark.parametrize("name", list(CHAINS))
 def test_kernels_that_start_early_wait_for_their_predecessor(bnd, name):
-    """Calls in a row, each on the last one's output and state and in buffers that it has just used, give the bits of calls with a synchronisation after each."""
+    """Calls in a row with no other kernel between them -- layer behind layer, build behind layer, build behind build, layer behind build -- each on the last one's
+    output and state and in buffers that it has just used, give the bits of calls with a synchronisation after each."""
     B, T, H, d, dt, cu = CHAINS[name]
     inp = wl.make(name, B, T, H, d, d, 64, dt, seed=900, cu_seqlens=None if cu is None else np.array(cu, np.int32))
     dev, Q = bnd.to_device(inp), bnd.kv_to_torch(wl.queries(inp, seed=901))
-    A = torch.empty(dev["K"].shape[:3] + (64,), device="cuda")
 
-    def chain(sync):
+    def chain(between):
+        shared, own = torch.empty(dev["K"].shape[:3] + (64,), device="cuda"), torch.empty((6,) + tuple(dev["K"].shape[:3]) + (64,), device="cuda")
         V, S, seen = dev["V"], None, []
-        for step in range(12):
-            V, S = bnd.gdn_forward(Q, dev["K"], V, dev["beta"], dev["g"], 64, scale=2.0, S0=S, cu_seqlens=cu)
-            if sync:
-                torch.cuda.synchronize()
-            bnd.build(V, dev["beta"], dev["g"], 64, cu_seqlens=cu, out=A)   # V as keys: reads what the call before has written, over what the build before has
-            if sync:
-                torch.cuda.synchronize()
-            seen.append(A.sum())
-        torch.cuda.synchronize()
-        return V, S, A.clone(), torch.stack(seen)
+        for step in range(6):
+            for _ in range(2):
+                V, S = bnd.gdn_forward(Q, dev["K"], V, dev["beta"], dev["g"], 64, scale=2.0, S0=S, cu_seqlens=cu)
+                between()
+            seen += [V, S]
+            bnd.build(V, dev["beta"], dev["g"], 64, cu_seqlens=cu, out=shared)   # V as keys: reads what the call before has written, over what the last step's build has
+            between()
+            bnd.build(V, dev["beta"], dev["g"], 64, cu_seqlens=cu, out=own[step])
+            between()
+        return seen + [shared, own]
 
-    ref = chain(True)
-    for _ in range(3):
-        for x, r in zip(chain(False), ref):
-            assert torch.equal(torch.nan_to_num(x), torch.nan_to_num(r))
+    same_chains(chain)
+    assert bnd.last_device_status() == 0
+
+
+FACTOR_CHAINS = {"C64": (9600, 16, 64), "C64_few": (640, 6, 64), "C128": (9600, 16, 128), "C128_few": (1280, 6, 128)}   # T, H, C; 2400, 60, 1200, 60 matrices: several a block, so that the counter is drawn, or one
+
+
+@pytest.mark.parametrize("name", list(FACTOR_CHAINS))
+def test_factor_calls_directly_behind_one_another(bnd, name):
+    """build, wy, fused, fused_raw (and the scan at C = 64) in a row with no other kernel between them, on one pair of work counters, each reading what the
+    one before has written and writing over what the step before has read; then captured in a graph and replayed on other values."""
+    T, H, C = FACTOR_CHAINS[name]
+    inp = wl.make(name, 1, T, H, 128, 128, C, wl.BF16, seed=930 + C)
+    dev, Q = bnd.to_device(inp), bnd.kv_to_torch(wl.queries(inp, seed=931))
+    gen = torch.Generator(device="cuda").manual_seed(932)
+    logits = [torch.randn((1, T, H), device="cuda", generator=gen) for _ in range(2)]
+    start = dev["V"].clone()
+
+    def chain(between, steps=4):
+        A, W, U, X, Y = torch.empty((1, T, H, C), device="cuda"), *(torch.empty_like(start) for _ in range(4))
+        V, S, seen = start, None, []
+        for step in range(steps):
+            bnd.build(dev["K"], dev["beta"], dev["g"], C, out=A)
+            between()
+            bnd.wy(A, dev["K"], V, dev["beta"], out=(W, U))
+            between()
+            bnd.fused(dev["K"], U, dev["beta"], dev["g"], C, out=(A, X, Y))
+            between()
+            bnd.fused(dev["K"], Y, dev["beta"], dev["g"], C, method=bnd.W_DECAY, want_A=False, out=(None, W, U))
+            between()
+            bnd.fused_raw(dev["K"], U, *logits, C, want_A=False, out=(None, X, Y, None, None))
+            between()
+            if C == 64:
+                V, S = bnd.chunk_scan(Q, dev["K"], W, Y, dev["g"], C, scale=2.0, S0=S)
+                between()
+                seen += [V, S]
+            else:
+                V, Y = Y, torch.empty_like(Y)
+                seen.append(V)
+        return seen + [A, W, X]
+
+    ref = same_chains(chain)
+    if C == 64:
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            out = chain(lambda: None)
+        for replay in range(2):   # flipped values, then the first ones again
+            start.copy_(start.flip(1))
+            other = chain(torch.cuda.synchronize)
+            graph.replay()
+            torch.cuda.synchronize()
+            assert all(torch.equal(x, r) for x, r in zip(out, other)) and torch.equal(other[0], ref[0]) == (replay == 1)
     assert bnd.last_device_status() == 0
 
 
@@ -223,25 +284,22 @@ def test_per_channel_kernels_that_start_early_wait_for_their_predecessor(bnd):
     inp = wl.make("kda chain", 2, 640, 8, 128, 128, 64, wl.BF16, seed=910)
     dev, Q, G = bnd.to_device(inp), bnd.kv_to_torch(wl.queries(inp, seed=911)), torch.from_numpy(wl.per_channel_gate(inp, seed=912)).cuda()
 
-    def chain(sync, C):
+    def chain(between, C):
         V, S = dev["V"], None
         for _ in range(8):
             A, W, U = bnd.fused_kda(dev["K"], V, G, dev["beta"], C)
-            if sync:
-                torch.cuda.synchronize()
+            between()
             if C == 64:
                 V, S = bnd.chunk_scan_kda(Q, dev["K"], W, U, G, C, scale=2.0, S0=S)
             else:
                 V, S = U, W
-            if sync:
-                torch.cuda.synchronize()
-        torch.cuda.synchronize()
+            between()
+            bnd.build_kda(dev["K"], G, dev["beta"], C, out=A)
+            between()
         return A, V, S
 
     for C in (64, 128):
-        ref = chain(True, C)
-        for _ in range(3):
-            assert all(torch.equal(x, r) for x, r in zip(chain(False, C), ref))
+        same_chains(lambda between: chain(between, C))
     assert bnd.last_device_status() == 0
 
 
