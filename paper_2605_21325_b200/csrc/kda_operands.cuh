@@ -11,14 +11,17 @@ constexpr float kDecayLog2e = 1.4426950408889634f;
 
 struct DecayRefs { float ref[8], last[8]; };   // times log2 e
 
-__device__ __forceinline__ DecayRefs load_decay_refs(const float* ref_row, const float* last_row) {
-  DecayRefs r;
+__device__ __forceinline__ void load_decay_row(float (&x)[8], const float* row) {
 #pragma unroll
   for (int q = 0; q < 8; q += 4) {
-    const float4 x = *reinterpret_cast<const float4*>(ref_row + q), y = *reinterpret_cast<const float4*>(last_row + q);
-    r.ref[q] = x.x * kDecayLog2e; r.ref[q + 1] = x.y * kDecayLog2e; r.ref[q + 2] = x.z * kDecayLog2e; r.ref[q + 3] = x.w * kDecayLog2e;
-    r.last[q] = y.x * kDecayLog2e; r.last[q + 1] = y.y * kDecayLog2e; r.last[q + 2] = y.z * kDecayLog2e; r.last[q + 3] = y.w * kDecayLog2e;
+    const float4 y = *reinterpret_cast<const float4*>(row + q);
+    x[q] = y.x * kDecayLog2e; x[q + 1] = y.y * kDecayLog2e; x[q + 2] = y.z * kDecayLog2e; x[q + 3] = y.w * kDecayLog2e;
   }
+}
+__device__ __forceinline__ DecayRefs load_decay_refs(const float* ref_row, const float* last_row) {
+  DecayRefs r;
+  load_decay_row(r.ref, ref_row);
+  load_decay_row(r.last, last_row);
   return r;
 }
 

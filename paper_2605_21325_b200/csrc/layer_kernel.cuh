@@ -459,7 +459,13 @@ __device__ __forceinline__ void prepare_chunks(const LayerParams& p, const KdaOp
     // (one thread decides for the group: it reads a word that other CTAs write)
     if (tid == 0 && (nx_item < p.total || (once && *(volatile int*)(p.counters + 3) == 0))) ticket = atomicAdd(p.counters + 1, 1);
     const size_t row0 = ((size_t)at.tok0 * p.H + at.h) * D + f0, stride = (size_t)p.H * D, out0 = ((size_t)at.slot * C * p.H + at.h) * D + f0;
-    const DecayRefs refs = load_decay_refs(a.G + row0 + (size_t)(at.rows >> 1) * stride, a.G + row0 + (size_t)(at.rows - 1) * stride);
+    DecayRefs refs;
+    load_decay_row(refs.ref, a.G + row0 + (size_t)(at.rows >> 1) * stride);
+    if (r0 == 0) {   // the chunk's vectors, ahead of the rows: with the last row's values kept beside the rows of the loop, 128 registers are not enough (48 to 84 bytes spilled; 56 pairs x 256 chunks 493 -> 471 us, 37 x 256 376 -> 364)
+      const size_t v = ((size_t)at.slot * p.H + at.h) * D + f0;
+      load_decay_row(refs.last, a.G + row0 + (size_t)(at.rows - 1) * stride);
+      store_decay_vectors(a.EL + v, a.ER + v, a.EX + v, refs);
+    }
 #pragma unroll 1
     for (int r4 = r0; r4 < at.rows; r4 += 32) {
       // four rows' loads first, without a branch between them (rows past the chunk: the last one again)
@@ -472,10 +478,6 @@ __device__ __forceinline__ void prepare_chunks(const LayerParams& p, const KdaOp
         kv[m] = *reinterpret_cast<const uint4*>(a.K + idx);
         gv[m][0] = *reinterpret_cast<const float4*>(a.G + idx);
         gv[m][1] = *reinterpret_cast<const float4*>(a.G + idx + 4);
-      }
-      if (r4 == 0) {   // (behind the loads of the first rows)
-        const size_t v = ((size_t)at.slot * p.H + at.h) * D + f0;
-        store_decay_vectors(a.EL + v, a.ER + v, a.EX + v, refs);
       }
 #pragma unroll
       for (int m = 0; m < 4; ++m) {
