@@ -974,8 +974,9 @@ cudaError_t launch_seq_offsets(int* dev_out, const tri_inv_desc* d, cudaStream_t
 // bf16 Q, K, W, U with d_k = d_v = 128 and C = 64.  One CTA per SM walks a (sequence, head) pair or a slice of its value
 // columns.  A pair is cut into four slices of 32 columns while that takes half the SMs at most, into two of 64 while every
 // slice gets an SM of its own: the steps between the products get shorter with the slice (512 chunks, 18 pairs, back to back: 473 us in slices of 32, 498 in
-// slices of 64, 651 in one).  The first line keeps clear of the power cap: by itself the scan of 24 or 32 pairs x 512 chunks would be 5 % faster in slices of 32 (473 and
-// 499 us), behind the factors' kernel, which leaves the chip hot, 32 pairs x 512 take 807 us in all so and 762 in slices of 64.  With more
+// slices of 64, 651 in one).  The first line keeps clear of the power cap, which 112 and more CTAs of 32 columns reach: 28 x 256 254 us in slices of 32 and 250 in slices of 64, 32 x 64 68 and 66,
+// 32 x 512 532 to 558 and 499, 37 x 512 593 and 506.  Between the line and there (19 to 27 pairs) the narrow slices are 4 to 5 % faster by themselves (24 x 64: 62.5 and 65.2; 24 x 512: 472 and 497) and
+// behind a fused call that is not long (24 x 64: 90 and 93, 24 x 128: 167 and 173), and slower behind a long one, which leaves the chip hot (24 x 512: 671 and 657); the layer call takes one kernel for these shapes.  With more
 // slices of 64 than SMs a CTA takes all 128 columns: the
 // products take the same time at any slice width, so each further slice would repeat them in a second wave (64 chunks: 74 pairs
 // 76 us in slices of 64, 90 in one; 75 pairs 133 and 90).

@@ -216,8 +216,8 @@ __global__ void __launch_bounds__(Cfg<C, D, SER, BO, REF, H16>::NT, Cfg<C, D, SE
     const float* src = tid < C ? p.beta : p.g;
     return (i < rows && src && TRI_INV_CHECK(p, (long long)tok0 + i < p.n_tokens)) ? src[(size_t)(tok0 + i) * p.H + h] : 0.f;
   };
-  // Prologue.  The threads that own the K and V barriers initialise them and request the first
-  // item's tiles at once, so that the copies run while tensor memory is being allocated.
+  // Prologue.  Barriers and tensor memory first, while the kernel before may still be running (launch_early); then the wait for it, and only behind that wait
+  // anything that reads or writes global memory: the first item's tiles, by the threads that own their barriers, beta and g, and the first draw from the work counter.
   const bool misaligned = (sK & 1023u) != 0;  // never expected; the swizzle pattern would not match the copies
   float bg_next = 0.f;
   {

@@ -9,9 +9,10 @@ namespace tri_inv {
 namespace {
 
 // Work counters: a launch draws its later items from a {next item, finished CTAs} pair in a static device
-// array, which the last CTA out returns to zero.  A pair must serve ONE launch at a time.  Kernels launched
-// into the same stream run one after the other, so each stream gets a pair of its own (by the stream's unique
-// id) and nothing has to be tracked: no event, no flag, no synchronisation.  There are kCounterSlots pairs per
+// array, which the last CTA out returns to zero.  A pair must serve ONE launch at a time.  CTAs of a kernel may be
+// on the chip before the kernel ahead of them in the stream has ended (launch_early), but each waits for its end
+// (wait_for_predecessor) before it draws: that wait is what keeps a pair exclusive.  So each stream gets a pair of its
+// own (by the stream's unique id) and nothing has to be tracked: no event, no flag.  There are kCounterSlots pairs per
 // device; launches on further streams, and every launch made during stream capture (a captured launch is
 // replayed later on whatever stream the graph is launched into), get no pair at all and walk their items with
 // a fixed stride instead: same results, slightly less even load.

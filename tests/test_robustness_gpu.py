@@ -89,7 +89,7 @@ def test_graph_replays_overlapping_many_plain_launches(bnd):
 
 @pytest.mark.parametrize("B,H", [(1, 2), (4, 16)], ids=["narrow_slices", "wide_slices"])
 def test_scan_waits_that_run_out(bnd, B, H):
-    """The chunk-scan kernel's fourteen warps wait for one another through barriers only; with one product of the first thread
+    """The chunk-scan kernel's sixteen warps wait for one another through barriers only; with one product of the first thread
     block left out (tri_inv_selftest_scan_wait_timeout, limit 100 us) every one of that block's waits must give up in turn,
     the kernel must return with the status word raised once, the other blocks' output must be untouched by it, and the
     next ordinary call must give the bits of the call before."""

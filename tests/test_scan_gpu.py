@@ -496,7 +496,7 @@ def test_random_layouts_layer_forward(bnd, seed):
 
 @pytest.mark.parametrize("n_seqs,H", [(5, 3), (9, 3), (26, 8)], ids=["32_columns", "64_columns", "128_columns"])
 def test_chunk_scan_repeats_bit_for_bit(bnd, n_seqs, H):
-    """The hand-offs inside a CTA (copies, products, operand writes of fourteen warps) are all ordered by barriers: the same
+    """The hand-offs inside a CTA (copies, products, operand writes of sixteen warps) are all ordered by barriers: the same
     launch on the same inputs gives the same bits every time.  A missing ordering would show as a difference between runs.
     Ragged packed sequences; every slice width (15, 27 and 208 (sequence, head) pairs)."""
     rng = np.random.default_rng(60 + H)
